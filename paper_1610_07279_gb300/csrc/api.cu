@@ -146,7 +146,7 @@ size_t carve(gt_system *s, char *base, int64_t n, const gt_params *p, int nsm, i
     s->bbox_partial = L.take<float>(base, 6 * (size_t)s->bbox_blocks);
     s->walk_blocks = walk_blocks;
     s->walk_warps = walk_blocks * gt_walk_warps_per_block();
-    s->queue_entries = own_queue ? (int64_t)s->walk_warps * p->walk_queue : 0;
+    s->queue_entries = own_queue ? (int64_t)(s->walk_warps * gt_queue_words(p->walk_queue)) : 0;
     s->queue = own_queue ? L.take<uint32_t>(base, (size_t)s->queue_entries) : nullptr;
     return (L.off + ALIGN - 1) / ALIGN * ALIGN;
 }

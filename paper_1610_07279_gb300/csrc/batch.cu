@@ -56,7 +56,7 @@ size_t plan(int nsys, const int64_t *n, const gt_params *prm, int n_prm, int nsm
     off = align_up(off + (size_t)nsys * sizeof(DevCtl *));
     off = align_up(off + (size_t)(nsys + 1) * sizeof(uint32_t));
     off = align_up(off + sizeof(unsigned int));
-    off = align_up(off + warps * (size_t)qcap * sizeof(uint32_t));
+    off = align_up(off + warps * gt_queue_words(qcap) * sizeof(uint32_t));
     if (member_bytes) member_bytes->clear();
     for (int k = 0; k < nsys; k++) {
         gt_system tmp;
@@ -130,13 +130,15 @@ void enqueue(gt_batch *b, int bootstrap, cudaStream_t st) {
     join(b, st);
     if (bootstrap) {
         gt_launch_walk_batch(b->d_ctls, b->d_args, b->nsys, b->d_gprefix, b->d_next, b->queue, b->qcap,
-                             GT_MAC_OPENING_ANGLE, b->walk_blocks, st);
+                             GT_MAC_OPENING_ANGLE, false, b->walk_blocks, st);
         fork(b, st);
         for (int k = 0; k < b->nsys; k++)
             if (b->sys[k]->n > 0) gt_sys_aold_from_acc(b->sys[k], b->streams[k % nstreams(b)]);
         join(b, st);
     }
-    gt_launch_walk_batch(b->d_ctls, b->d_args, b->nsys, b->d_gprefix, b->d_next, b->queue, b->qcap, -1,
+    bool all_acc = true;
+    for (const gt_system *s : b->sys) all_acc = all_acc && s->prm.mac == GT_MAC_ACCELERATION;
+    gt_launch_walk_batch(b->d_ctls, b->d_args, b->nsys, b->d_gprefix, b->d_next, b->queue, b->qcap, -1, all_acc,
                          b->walk_blocks, st);
 }
 
@@ -187,7 +189,7 @@ int gt_batch_create(gt_batch **out, int nsys, const int64_t *n, const gt_params 
     off = align_up(off + sizeof(unsigned int));
     const size_t warps = (size_t)b->walk_blocks * (size_t)gt_walk_warps_per_block();
     b->queue = (uint32_t *)(base + off);
-    off = align_up(off + warps * (size_t)b->qcap * sizeof(uint32_t));
+    off = align_up(off + warps * gt_queue_words(b->qcap) * sizeof(uint32_t));
     std::vector<DevCtl *> ctls(nsys);
     b->sys.assign(nsys, nullptr);
     b->h_args.resize(nsys);
@@ -200,7 +202,7 @@ int gt_batch_create(gt_batch **out, int nsys, const int64_t *n, const gt_params 
             return rc;
         }
         s->queue = b->queue;  // the batch's queue serves the member's own walks too
-        s->queue_entries = (int64_t)(warps * (size_t)b->qcap);
+        s->queue_entries = (int64_t)(warps * gt_queue_words(b->qcap));
         ctls[k] = s->ctl;
         off = align_up(off + mb[k]);
     }

@@ -336,6 +336,12 @@ struct WalkArgs {
     int sphere;              // pseudo i-particle: 0 GEO centre, 1 Ritter's efficient bounding sphere
     float theta, delta_acc, eps2, G, inv_eps;
 };
+// A warp's cell queue: a ring of (first child, number of children) pairs, one for every opened cell.
+// walk_queue bounds the cells in it; from 8 x pairs > walk_queue - (the depth-first reserve) on the
+// newest pairs are taken first, which keeps at most ~700 more, so half as many pairs as cells (and
+// 1024 for the smallest queues) hold every walk that walk_queue admits.
+__host__ __device__ inline uint32_t gt_queue_ring(int qcap) { return qcap >= 2048 ? (uint32_t)qcap / 2u : 1024u; }
+__host__ __device__ inline size_t gt_queue_words(int qcap) { return 2 * (size_t)gt_queue_ring(qcap); }
 int gt_walk_blocks(int nsm);
 // tuner.cu
 // On-line Brent minimisation (one abscissa out, its cost back) for the critical
@@ -353,7 +359,8 @@ extern "C" int gt_rebuild_interval(const double *t_walk, int n, double t_make, i
                                    double *n_opt_out, double *coef_out);
 int gt_walk_warps_per_block();
 void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st);
-// one launch over the groups of nsys systems (args, ctls: device arrays of nsys entries)
+// one launch over the groups of nsys systems (args, ctls: device arrays of nsys entries); all_acc: every
+// system uses the acceleration MAC
 void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, uint32_t *gprefix,
-                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, int nblocks,
+                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, int nblocks,
                           cudaStream_t st);

@@ -119,7 +119,10 @@ void batched_walk(gt_server *v, const TickList &L) {
     if (L.n == 0) return;
     { k_select_args<<<1, 128, 0, v->main>>>(L, v->d_pool, v->d_ctl_pool, v->d_tick_args, v->d_tick_ctls);
       gt_note_launches(1); }
-    gt_launch_walk_batch(v->d_tick_ctls, v->d_tick_args, L.n, v->d_gprefix, v->d_next, v->queue, v->qcap, -1,
+    bool all_acc = true;
+    for (int k = 0; k < L.n; k++)
+        all_acc = all_acc && L.variant[k] != V_BOOT && v->slots[L.slot[k]].sys->prm.mac == GT_MAC_ACCELERATION;
+    gt_launch_walk_batch(v->d_tick_ctls, v->d_tick_args, L.n, v->d_gprefix, v->d_next, v->queue, v->qcap, -1, all_acc,
                          v->walk_blocks, v->main);
     v->walk_launches++;
 }
@@ -273,7 +276,7 @@ int gt_server_create(gt_server **out, size_t hbm_cap, int max_slots, int walk_qu
     const size_t o_tctl = off; off = align_up(off + (size_t)max_slots * sizeof(DevCtl *));
     const size_t o_gpre = off; off = align_up(off + (size_t)(max_slots + 1) * sizeof(uint32_t));
     const size_t o_next = off; off = align_up(off + sizeof(unsigned int));
-    const size_t o_queue = off; off = align_up(off + warps * (size_t)walk_queue * sizeof(uint32_t));
+    const size_t o_queue = off; off = align_up(off + warps * gt_queue_words(walk_queue) * sizeof(uint32_t));
     if (off > hbm_cap) { delete v; return GT_ENOMEM; }
     v->region = alloc_fn(off, ctx);
     if (!v->region || ((uintptr_t)v->region) % GT_WS_ALIGN) {
@@ -360,7 +363,7 @@ int gt_submit(gt_server *v, const gt_request *req, uint64_t *ticket) {
     v->by_ticket[sl.ticket] = k;
     if ((rc = gt_sys_init(s, req->n, &prm, ws, bytes, false, v->admit))) { release(v, k); return rc; }
     s->queue = v->queue;
-    s->queue_entries = (int64_t)v->walk_blocks * gt_walk_warps_per_block() * v->qcap;
+    s->queue_entries = (int64_t)((size_t)v->walk_blocks * gt_walk_warps_per_block() * gt_queue_words(v->qcap));
     sl.phase = PH_START;
     sl.nsteps = req->nsteps;
     sl.steps_enq = 0;

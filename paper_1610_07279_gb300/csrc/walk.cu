@@ -6,29 +6,38 @@
 // range of the active list: the actives of one tree cell (Sec. 2.4 reading) or a run
 // of group_max.  Per group:
 //   * S lanes per member (Sec. 2.5): fixed, or 32 / (members rounded up to a power of
-//     two) so that small groups still fill the warp;
+//     two) so that small groups still fill the warp; the members above 32 share the lanes
+//     a second time in the same way;
 //   * pseudo i-particle: the sphere about the centre of the members' bounding box
 //     (Appendix B, "GEO"), the FP32 radius widened by (1 + 2^-20); |a_old| of the
 //     group is the smallest of its members';
-//   * breadth-first traversal: a ring-buffer queue of cells in a per-warp slice of
-//     global memory (when the queue fills up, the newest cells are taken first, i.e.
-//     depth-first, which bounds its size; the order of the interactions does not change
-//     the set of interactions); 32 queued cells are tested at once, one per lane, with the MAC at
-//     distance lambda r_JI (Eqs. 2, 5-7) in FP32 with explicit rounding (so the decision
-//     is reproducible); accepted cells join the shared-memory interaction list,
-//     rejected cells push their children, rejected leaves copy their particles into the
-//     list with asynchronous global-to-shared copies (cp.async), waited for only when the
-//     list is flushed -- both spread over the whole warp (a warp prefix sum, then each
-//     lane finds the owner of its entry by a binary search over the lanes);
+//   * breadth-first traversal: a ring-buffer queue in a per-warp slice of global memory, one
+//     entry (first child, number of children) per opened cell.  An octree cell of more than
+//     leaf_max particles has nearly always all eight children (7.5 to 7.95 on average on the
+//     models here), so four entries fill a batch of 32 lanes without any search for the
+//     lanes' cells, their records are read in runs, and an opened cell costs one queue
+//     store.  When the queue fills up, the newest entries are taken first, i.e.
+//     depth-first, which bounds its size (the order does not change the set of
+//     interactions).  The cells are tested with the MAC at distance lambda r_JI (Eqs. 2, 5-7)
+//     in FP32 with explicit rounding (so the decision is reproducible); accepted cells and the
+//     particles of opened leaves join the shared-memory interaction list in the cells'
+//     order, the particles by asynchronous global-to-shared copies (cp.async), waited for
+//     only when the list is summed;
 //   * the list is kept as structure of arrays (x, y, z, m), so two consecutive entries
-//     load as packed pairs; it is flushed through Eq. (1) whenever it fills: each
-//     i-particle is held by S lanes that take every S-th pair of entries on the packed
-//     FP32 pipe (f32x2 add, mul and fma: two interactions per instruction; rsqrt on the
-//     SFU), the two halves and the S lanes summed at the end (an odd list gets a
-//     massless last entry).  The potential is accumulated too; the member's own term
-//     -G m_i/eps is removed at the end (Eq. 1 excludes j = i).
-// Bound: FP32 ALU (the force loop: 3 FADD, 3 FMUL, 7 FFMA and one MUFU rsqrt per
-// interaction); the node records (32 B per cell) stay resident in L2.
+//     load as packed pairs; every 128 entries are summed through Eq. (1) from zero and the
+//     partial sums added in order (so the result does not depend on when, or by which warp,
+//     a chunk is summed): each i-particle is held by S lanes that take every S-th quad of
+//     entries on the packed FP32 pipe (f32x2 add, mul and fma: two interactions per
+//     instruction; rsqrt on the SFU), the two halves and the S lanes summed at the end.
+//     The potential is accumulated too; the member's own term -G m_i/eps is removed at the
+//     end (Eq. 1 excludes j = i).
+// Bound: instruction issue and the FP32 pipe (per quad of entries 24 packed operations of two
+// cycles, 4 rsqrt, 4 loads); the node records (32 B per cell) stay in L2.  80 registers and
+// 48 KB of shared memory at three blocks per SM; members and sums wait in shared memory
+// during the traversal (held in registers they spill, and a spilling force loop costs 15 %;
+// two blocks at 95 registers 12 % more time, four at 64 10 %).  The full walk of the
+// Andromeda-like model at 2^22, leaves of 32: 2.60 ms, 0.67 warp instructions per interaction
+// (3.03 ms and 0.81 with a queue of single cells).
 #include <math.h>
 
 #include "gt_internal.cuh"
@@ -38,16 +47,22 @@ namespace {
 #ifndef GT_WALK_MINB
 #define GT_WALK_MINB 3            // resident blocks per SM the register budget is sized for
 #endif
-constexpr int WT = 256;           // threads per block
+constexpr int WT = 256;             // threads per block
 constexpr int NWARP = WT / 32;
-constexpr int LIST_CAP = 384;     // interaction-list entries per warp
-constexpr int FLUSH_AT = 256;     // flush once the list holds this many
+constexpr uint32_t LIST_CAP = 256;  // interaction-list entries per warp
+constexpr uint32_t CHUNK = 128;     // entries whose forces are summed from zero before they join a member's sums
+constexpr uint32_t WARP_SM = 4 * LIST_CAP + 4 * 4 * 32;  // the list, then the lanes' members and sums
 // Depth-first reserve of the queue: popping the newest 32 cells and pushing at most
 // 8 children each grows the queue by <= 224 per tree level, <= ~22 x 256 in all.
 constexpr int LIFO_ROOM = 6144;
 
-__device__ __forceinline__ bool mac_accept(int mac, float theta, float dacc_amin, float delta, float G, float cx,
+// MAC >= 0: the criterion is known at compile time; MAC_ANY takes the argument's
+constexpr int MAC_ANY = -1;
+
+template <int MAC>
+__device__ __forceinline__ bool mac_accept(int mac_arg, float theta, float dacc_amin, float delta, float G, float cx,
                                            float cy, float cz, float bI, float4 jp, float bJ, float B2) {
+    const int mac = MAC == MAC_ANY ? mac_arg : MAC;
     const float dx = __fsub_rn(jp.x, cx);
     const float dy = __fsub_rn(jp.y, cy);
     const float dz = __fsub_rn(jp.z, cz);
@@ -111,16 +126,16 @@ __device__ __forceinline__ void warp_arg_ext(float &v, int &m, bool want_max) {
 // first diameter joins the extreme members of the axis whose pair is farthest apart; the
 // sphere then grows towards the first member outside it (member order) until none is,
 // at most cnt times.  FP32, every operation rounded as written.  Member k < 32 is the
-// first member of the lane holding slot k (pi), member 32 + l the second of lane l (pi2).
-__device__ __forceinline__ void ebs_centre(float4 pi, float4 pi2, bool mine1, bool mine2, int slot, int lane,
-                                           int logS, uint32_t cnt, float &cx, float &cy, float &cz) {
+// first member of the lanes holding slot k (pi), the others the second of the lanes holding slot2 (pi2).
+__device__ __forceinline__ void ebs_centre(float4 pi, float4 pi2, bool mine1, bool mine2, int slot, int slot2,
+                                           int logS, int logS2, uint32_t cnt, float &cx, float &cy, float &cz) {
     const unsigned FULL = 0xffffffffu;
     const float INF = __int_as_float(0x7f800000);
     auto coord = [](const float4 &p, int a) { return a == 0 ? p.x : (a == 1 ? p.y : p.z); };
     // the member's position, fetched from the lane that holds it
     auto fetch = [&](int m, float &x, float &y, float &z) {
         const bool second = m >= 32;
-        const int src = second ? m - 32 : (m << logS);
+        const int src = second ? (m - 32) << logS2 : (m << logS);
         const float4 a1 = make_float4(__shfl_sync(FULL, pi.x, src), __shfl_sync(FULL, pi.y, src),
                                       __shfl_sync(FULL, pi.z, src), 0.f);
         const float4 a2 = make_float4(__shfl_sync(FULL, pi2.x, src), __shfl_sync(FULL, pi2.y, src),
@@ -133,8 +148,8 @@ __device__ __forceinline__ void ebs_centre(float4 pi, float4 pi2, bool mine1, bo
         int mmin = mine1 ? slot : 1 << 20, mmax = mmin;
         if (mine2) {
             const float v2 = coord(pi2, ax);
-            if (v2 < vmin) { vmin = v2; mmin = lane + 32; }  // the second member has the larger index
-            if (v2 > vmax) { vmax = v2; mmax = lane + 32; }
+            if (v2 < vmin) { vmin = v2; mmin = slot2; }  // the second member has the larger index
+            if (v2 > vmax) { vmax = v2; mmax = slot2; }
         }
         warp_arg_ext(vmin, mmin, false);
         warp_arg_ext(vmax, mmax, true);
@@ -159,7 +174,7 @@ __device__ __forceinline__ void ebs_centre(float4 pi, float4 pi2, bool mine1, bo
         const unsigned b2 = __ballot_sync(FULL, mine2 && outside(pi2));
         int m;
         if (b1) m = (__ffs(b1) - 1) >> logS;
-        else if (b2) m = 32 + __ffs(b2) - 1;
+        else if (b2) m = 32 + ((__ffs(b2) - 1) >> logS2);
         else break;
         float px, py, pz;
         fetch(m, px, py, pz);
@@ -174,53 +189,57 @@ __device__ __forceinline__ void ebs_centre(float4 pi, float4 pi2, bool mine1, bo
     }
 }
 
-// One group g of system a (Sec. 2.3): pseudo i-particle, traversal, force loop.  The
-// warp's interaction and MAC-test counts are added to n_inter and n_tests.
-__device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx,
-                                           uint32_t *q, unsigned long long &n_inter,
-                                           unsigned long long &n_tests) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t qmask = (uint32_t)a.qcap - 1u;
-    const int lifo_at = a.qcap - LIFO_ROOM;
+// members [a0, a1) of group g in the active list
+__device__ __forceinline__ void group_range(const WalkArgs &a, uint32_t g, uint32_t ngroups, uint32_t &a0, uint32_t &a1) {
     const uint32_t na = a.ctl->n_active;
-    const uint32_t gmax = (uint32_t)a.gmax;
-    const unsigned FULL = 0xffffffffu;
-    const unsigned lt = lanemask_lt();
-    uint32_t a0, a1;
     if (a.gstart) {
         a0 = a.gstart[g];
         a1 = g + 1 < ngroups ? a.gstart[g + 1] : na;
     } else {
-        a0 = g * gmax;
-        a1 = min(a0 + gmax, na);
+        a0 = g * (uint32_t)a.gmax;
+        a1 = min(a0 + (uint32_t)a.gmax, na);
     }
-    const uint32_t cnt = a1 - a0;
-    // a group of more than 32 gives every lane a second member (lane + 32), one lane each
+}
+
+// The i-particle of active position k; an index outside the system is reported and particle 0 walked instead.
+__device__ __forceinline__ uint32_t member_of(const WalkArgs &a, uint32_t k) {
+    uint32_t i = a.active ? a.active[k] : k;
+    if (i >= a.n) {
+        gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
+        i = 0u;
+    }
+    return i;
+}
+
+struct Pseudo {
+    float x, y, z, b, dacc_amin;  // centre and radius of the group's sphere; Delta_acc times its smallest |a_old|
+};
+
+// A group's pseudo i-particle, and the lane's members in shared memory: mem[0], [32] the first and second,
+// negated, with the first quad and the quad step of the lane's share in the fourth word; mem[64], [96] their
+// sums, zero.  False for a malformed group.
+__device__ __forceinline__ bool group_setup(const WalkArgs &a, uint32_t a0, uint32_t cnt, float4 *mem, Pseudo &ps) {
+    const int lane = threadIdx.x & 31;
+    const unsigned FULL = 0xffffffffu;
+    // a group of more than 32: member k < 32 has lane k, the others share the lanes a second time
     const bool two = cnt > 32u;
-    if (cnt == 0u || cnt > 64u || (two && a.ij_share > 1)) {  // a malformed group: report it, skip
-        if (lane == 0) gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
-        return;
-    }
+    if (cnt == 0u || cnt > 64u || (two && a.ij_share > 1)) return false;
     const int S = two ? 1 : (a.ij_share ? a.ij_share : 32 >> (cnt <= 1 ? 0 : 32 - __clz(cnt - 1)));
     const int logS = __ffs(S) - 1;
     const int slot = lane >> logS, sub = lane & (S - 1);
     const bool have = (uint32_t)slot < cnt;
-    const bool have2 = two && (uint32_t)(lane + 32) < cnt;
-    const uint32_t kk = a0 + (have ? (uint32_t)slot : 0u);
-    const uint32_t kk2 = a0 + (have2 ? (uint32_t)(lane + 32) : 0u);
-    uint32_t i = a.active ? a.active[kk] : kk;
-    uint32_t i2 = have2 ? (a.active ? a.active[kk2] : kk2) : i;
-    if (i >= a.n || i2 >= a.n) {  // an index outside the system: report it, walk particle 0 instead
-        gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
-        i = i >= a.n ? 0u : i;
-        i2 = i2 >= a.n ? 0u : i2;
-    }
+    // lanes of one second member: like S, as many as their count (1 to 32) leaves, so that they don't idle
+    const int logS2 = (two && !a.ij_share) ? 5 - (cnt <= 33u ? 0 : 32 - __clz(cnt - 33u)) : 0;
+    const int slot2 = 32 + (lane >> logS2), sub2 = lane & ((1 << logS2) - 1);
+    const bool have2 = two && (uint32_t)slot2 < cnt;
+    const uint32_t i = member_of(a, a0 + (have ? (uint32_t)slot : 0u));
+    const uint32_t i2 = have2 ? member_of(a, a0 + (uint32_t)slot2) : i;
     const float4 pi = a.posm[i];
     const float4 pi2 = have2 ? a.posm[i2] : pi;
     float ao = have ? (a.aold ? a.aold[i] : 0.0f) : INFINITY;
     if (have2) ao = fminf(ao, a.aold ? a.aold[i2] : 0.0f);
 
-    // pseudo i-particle (lanes without a member repeat member 0: no effect on the box)
+    // lanes without a member repeat member 0: no effect on the box
     float mnx = fminf(pi.x, pi2.x), mny = fminf(pi.y, pi2.y), mnz = fminf(pi.z, pi2.z);
     float mxx = fmaxf(pi.x, pi2.x), mxy = fmaxf(pi.y, pi2.y), mxz = fmaxf(pi.z, pi2.z);
 #pragma unroll
@@ -236,7 +255,7 @@ __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32
     float cx = __fmul_rn(0.5f, __fadd_rn(mnx, mxx));
     float cy = __fmul_rn(0.5f, __fadd_rn(mny, mxy));
     float cz = __fmul_rn(0.5f, __fadd_rn(mnz, mxz));
-    if (a.sphere == 1) ebs_centre(pi, pi2, have && sub == 0, have2, slot, lane, logS, cnt, cx, cy, cz);
+    if (a.sphere == 1) ebs_centre(pi, pi2, have && sub == 0, have2 && sub2 == 0, slot, slot2, logS, logS2, cnt, cx, cy, cz);
     const float ddx = __fsub_rn(pi.x, cx), ddy = __fsub_rn(pi.y, cy), ddz = __fsub_rn(pi.z, cz);
     float d2 = __fadd_rn(__fadd_rn(__fmul_rn(ddx, ddx), __fmul_rn(ddy, ddy)), __fmul_rn(ddz, ddz));
     {
@@ -245,271 +264,382 @@ __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) d2 = fmaxf(d2, __shfl_xor_sync(FULL, d2, o));
-    const float bI = __fmul_rn(__fsqrt_rn(d2), GT_RADIUS_MARGIN);
-    const float dacc_amin = __fmul_rn(a.delta_acc, ao);
+    ps = Pseudo{cx, cy, cz, __fmul_rn(__fsqrt_rn(d2), GT_RADIUS_MARGIN), __fmul_rn(a.delta_acc, ao)};
+    mem[0] = make_float4(-pi.x, -pi.y, -pi.z, __uint_as_float((uint32_t)sub | (1u << logS << 8)));
+    mem[32] = make_float4(-pi2.x, -pi2.y, -pi2.z, __uint_as_float((uint32_t)sub2 | (1u << logS2 << 8)));
+    mem[64] = mem[96] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return true;
+}
 
-    float ax = 0.f, ay = 0.f, az = 0.f, ph = 0.f;
-    float bx = 0.f, by = 0.f, bz = 0.f, qh = 0.f;  // the second member's sums
-    int list_n = 0;
-    // the list, structure of arrays: x, y, z, m of entry e at lx[e], ly[e], lz[e], lw[e]
-    float *ly = lx + LIST_CAP, *lz = lx + 2 * LIST_CAP, *lw = lx + 3 * LIST_CAP;
+// Forces of quads [k0, k1) of a list (arrays of `cap` entries) on one member of every lane, summed from zero.
+__device__ __forceinline__ float4 chunk_force(const float *lx, uint32_t cap, float4 p, float eps2, uint32_t k0,
+                                              uint32_t k1) {
+    const float4 *px = (const float4 *)lx, *py = (const float4 *)(lx + cap), *pz = (const float4 *)(lx + 2 * cap),
+                 *pw = (const float4 *)(lx + 3 * cap);
+    const uint32_t share = __float_as_uint(p.w), step = share >> 8;
+    const float2 e2 = make_float2(eps2, eps2);
+    const float2 nx = make_float2(p.x, p.x), ny = make_float2(p.y, p.y), nz = make_float2(p.z, p.z);
+    float2 sx = make_float2(0.f, 0.f), sy = sx, sz = sx, sp = sx;
+#pragma unroll 1
+    for (uint32_t k = k0 + (share & 0xffu); k < k1; k += step) {
+        const float4 X = px[k], Y = py[k], Z = pz[k], W = pw[k];
+        interact_pairs(make_float2(X.x, X.y), make_float2(Y.x, Y.y), make_float2(Z.x, Z.y), make_float2(W.x, W.y),
+                       nx, ny, nz, e2, sx, sy, sz, sp);
+        interact_pairs(make_float2(X.z, X.w), make_float2(Y.z, Y.w), make_float2(Z.z, Z.w), make_float2(W.z, W.w),
+                       nx, ny, nz, e2, sx, sy, sz, sp);
+    }
+    return make_float4(__fadd_rn(sx.x, sx.y), __fadd_rn(sy.x, sy.y), __fadd_rn(sz.x, sz.y), __fadd_rn(sp.x, sp.y));
+}
+
+__device__ __forceinline__ void add_force(float4 &sum, float4 f) {
+    float4 t = sum;
+    t.x = __fadd_rn(t.x, f.x); t.y = __fadd_rn(t.y, f.y); t.z = __fadd_rn(t.z, f.z); t.w = __fsub_rn(t.w, f.w);
+    sum = t;
+}
+
+// Massless entries behind the last of a list up to a multiple of four: they add exactly nothing.
+__device__ __forceinline__ void pad_list(float *lx, uint32_t cap, uint32_t list_n) {
+    const uint32_t lane = threadIdx.x & 31u;
+    if (lane < ((0u - list_n) & 3u)) {
+        float *e = lx + list_n + lane;
+        e[0] = e[cap] = e[2 * cap] = e[3 * cap] = 0.f;
+    }
+    __syncwarp();
+}
+
+// The first list_n (< CHUNK) entries from quad `from` on moved to the front of the list, by one warp.
+__device__ __forceinline__ void move_rest(float *lx, uint32_t cap, uint32_t list_n, uint32_t from) {
+    const uint32_t lane = threadIdx.x & 31u;
+    if (4u * lane < list_n) {
+        float4 *q = (float4 *)lx;
+#pragma unroll
+        for (uint32_t c = 0; c < 4; c++) q[c * (cap / 4) + lane] = q[c * (cap / 4) + from + lane];
+    }
+}
+
+struct Batch {
+    float4 jp;
+    uint32_t l0, mine;  // first child or first particle; entries for the list: one, a leaf's particles, none
+    uint32_t nch;       // children of an opened cell
+    bool ok;            // accepted
+};
+
+// One batch: the children of nb (at most four) queue entries from `base` on, one per lane, and what the MAC says.
+template <int MAC>
+__device__ __forceinline__ Batch test_batch(const WalkArgs &a, const Pseudo &ps, const uint2 *q, uint32_t base,
+                                            uint32_t nb, uint32_t qmask, uint32_t &tests) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint2 sib = q[(base + (lane >> 3)) & qmask];
+    bool valid = (lane >> 3) < nb && (lane & 7u) < sib.y;
+    uint32_t node = valid ? sib.x + (lane & 7u) : 0u;
+#if GT_DEBUG
+    const uint32_t nnodes = a.ctl->level_start[GT_TREE_LEVELS];
+    if (node >= nnodes) {
+        gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
+        valid = false;
+        node = 0u;
+    }
+#endif
+    Batch t;
+    t.jp = a.jpos[node];
+    const float4 wk = a.walk[node];
+    const uint32_t l1 = __float_as_uint(wk.z);
+    const bool leaf = (l1 & GT_LEAF_FLAG) != 0u;
+    t.l0 = __float_as_uint(wk.y);
+#if GT_DEBUG
+    if (valid && (unsigned long long)t.l0 + (l1 & ~GT_LEAF_FLAG) > (leaf ? a.n : nnodes)) {
+        gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
+        valid = false;
+    }
+#endif
+    tests += valid ? 1u : 0u;
+    t.ok = valid && mac_accept<MAC>(a.mac, a.theta, ps.dacc_amin, a.delta_acc, a.G, ps.x, ps.y, ps.z, ps.b, t.jp, wk.x,
+                                    wk.w);
+    const bool opened = valid && !t.ok;
+    t.nch = opened && !leaf ? l1 : 0u;
+    t.mine = opened && leaf ? (l1 & ~GT_LEAF_FLAG) : (t.ok ? 1u : 0u);
+    return t;
+}
+
+// The entries of a batch with index in [w0, w1) into the list: entry e goes to slot to + e.  `excl`: the index
+// of the lane's first; lm: lanes with an opened leaf.
+__device__ __forceinline__ void write_entries(const WalkArgs &a, const Batch &t, uint32_t excl, unsigned lm, float *lx,
+                                              uint32_t cap, uint32_t to, uint32_t w0, uint32_t w1) {
+    const unsigned FULL = 0xffffffffu;
+    if (t.ok && excl >= w0 && excl < w1) {
+        float *e = lx + to + excl;
+        e[0] = t.jp.x; e[cap] = t.jp.y; e[2 * cap] = t.jp.z; e[3 * cap] = t.jp.w;
+    }
+    // opened leaves next to each other among one cell's children hold one range of particles: a run of them is
+    // copied at a time, asynchronously
+    const unsigned starts = lm & ~((lm << 1) & 0xfefefefeu);
+    for (unsigned m = starts; m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const int end = min(src + __ffs(~((lm >> src) & 0xffu)) - 2, src | 7);  // the run's last lane
+        const uint32_t le = __shfl_sync(FULL, excl, src);
+        const uint32_t e1 = min(__shfl_sync(FULL, excl + t.mine, end), w1);
+        const float4 *p = a.posm + __shfl_sync(FULL, t.l0, src);
+        for (uint32_t e = max(le, w0) + (threadIdx.x & 31u); e < e1; e += 32) {
+            const float *from = (const float *)&p[e - le];
+            float *d = lx + to + e;
+            cp_async4(d, from);
+            cp_async4(d + cap, from + 1);
+            cp_async4(d + 2 * cap, from + 2);
+            cp_async4(d + 3 * cap, from + 3);
+        }
+    }
+}
+
+// The members' sums, reduced over their lanes, to the caller's accelerations.
+__device__ __forceinline__ void store_group(const WalkArgs &a, uint32_t a0, uint32_t a1, const float4 *mem) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t who = 0; who < a1 - a0; who += 32) {
+        const uint32_t share = __float_as_uint(mem[who].w), S = share >> 8;
+        float4 sum = mem[64 + who];
+        for (uint32_t o = 1; o < S; o <<= 1) {
+            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
+            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
+            sum.z += __shfl_xor_sync(0xffffffffu, sum.z, o);
+            sum.w += __shfl_xor_sync(0xffffffffu, sum.w, o);
+        }
+        const uint32_t k = a0 + who + lane / S;
+        if ((share & 0xffu) == 0u && k < a1) {
+            const uint32_t i = a.active ? a.active[k] : k;
+            const float phi = fmaf(a.posm[i < a.n ? i : 0u].w, a.inv_eps, sum.w);
+            a.acc[k] = make_float4(a.G * sum.x, a.G * sum.y, a.G * sum.z, a.G * phi);
+        }
+    }
+}
+
+// One group g of system a (Sec. 2.3) by one warp.  The interactions and MAC tests are added to stat[0] and
+// stat[1].  lx: the warp's WARP_SM words of shared memory.
+template <int MAC>
+__device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx, uint2 *q,
+                                           unsigned long long *stat) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t qmask = gt_queue_ring(a.qcap) - 1u;
+    const unsigned FULL = 0xffffffffu;
+    const unsigned lt = lanemask_lt();
+    float4 *mem = (float4 *)(lx + 4 * LIST_CAP) + lane;
+    uint32_t a0, a1;
+    group_range(a, g, ngroups, a0, a1);
+    const bool two = a1 - a0 > 32u;
+    Pseudo ps;
+    if (!group_setup(a, a0, a1 - a0, mem, ps)) {
+        if (lane == 0) gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
+        return;
+    }
+    uint32_t list_n = 0, chunks = 0, tests = 0;  // entries in the list; chunks summed; this lane's MAC tests
+    auto chunk = [&](uint32_t k0, uint32_t k1) {
+        add_force(mem[64], chunk_force(lx, LIST_CAP, mem[0], a.eps2, k0, k1));
+        if (two) add_force(mem[96], chunk_force(lx, LIST_CAP, mem[32], a.eps2, k0, k1));
+    };
+    // every full chunk of the list, then the rest moved to its front
     auto flush = [&]() {
         cp_async_wait_all();
         __syncwarp();
-        // entries are taken four at a time (one 16-byte load per coordinate), as the pairs
-        // (e, e + 1) and (e + 2, e + 3); the list is padded with massless entries to a
-        // multiple of four, which add exactly nothing
-        const int pad = (-list_n) & 3;
-        if (pad) {
-            if (lane < pad) {
-                lx[list_n + lane] = 0.f; ly[list_n + lane] = 0.f; lz[list_n + lane] = 0.f; lw[list_n + lane] = 0.f;
-            }
-            __syncwarp();
-        }
-        const int nquad = (list_n + 3) >> 2;
-        const float4 *px = (const float4 *)lx, *py = (const float4 *)ly, *pz = (const float4 *)lz,
-                     *pw = (const float4 *)lw;
-        // one i-particle against quads k0, k0 + step, ... (its sums carried in and out)
-        auto run = [&](const float4 &p, float &sx_, float &sy_, float &sz_, float &sp_, int k0, int step) {
-            const float2 e2 = make_float2(a.eps2, a.eps2);
-            const float2 nx = make_float2(-p.x, -p.x), ny = make_float2(-p.y, -p.y), nz = make_float2(-p.z, -p.z);
-            float2 sx = make_float2(sx_, 0.f), sy = make_float2(sy_, 0.f), sz = make_float2(sz_, 0.f);
-            float2 sp = make_float2(-sp_, 0.f);
-            for (int k = k0; k < nquad; k += step) {
-                const float4 X = px[k], Y = py[k], Z = pz[k], W = pw[k];
-                interact_pairs(make_float2(X.x, X.y), make_float2(Y.x, Y.y), make_float2(Z.x, Z.y),
-                               make_float2(W.x, W.y), nx, ny, nz, e2, sx, sy, sz, sp);
-                interact_pairs(make_float2(X.z, X.w), make_float2(Y.z, Y.w), make_float2(Z.z, Z.w),
-                               make_float2(W.z, W.w), nx, ny, nz, e2, sx, sy, sz, sp);
-            }
-            sx_ = __fadd_rn(sx.x, sx.y); sy_ = __fadd_rn(sy.x, sy.y); sz_ = __fadd_rn(sz.x, sz.y);
-            sp_ = -__fadd_rn(sp.x, sp.y);
-        };
-        if (two) {  // both members of the lane over every pair, one after the other
-            run(pi, ax, ay, az, ph, 0, 1);
-            run(pi2, bx, by, bz, qh, 0, 1);
-        } else {  // S lanes per i-particle: lane sub takes quads sub, sub + S, ...
-            run(pi, ax, ay, az, ph, sub, S);
-        }
-        n_inter += (unsigned long long)list_n * cnt;
-        list_n = 0;
+        const uint32_t full = list_n / CHUNK;
+        for (uint32_t c = 0; c < full; c++) chunk(c * (CHUNK / 4), (c + 1) * (CHUNK / 4));
+        list_n -= full * CHUNK;
+        chunks += full;
+        if (full) move_rest(lx, LIST_CAP, list_n, full * (CHUNK / 4));
         __syncwarp();
     };
-
-#if GT_DEBUG
-    const uint32_t nnodes = a.ctl->level_start[GT_TREE_LEVELS];
-#endif
     uint32_t head = 0, tail = 1;
-    if (lane == 0) q[0] = 0u;  // the root
+    if (lane == 0) q[0] = make_uint2(0u, 1u);  // the root
     __syncwarp();
     bool overflow = false;
     while (head != tail) {
-        const uint32_t live = tail - head;
-        const uint32_t nb = min(live, 32u);
-#if !GT_DEBUG
-        const bool valid = (uint32_t)lane < nb;
-#endif
         // breadth-first from the head while there is room, depth-first from the tail after
-        uint32_t base;
-        if ((int)live > lifo_at) {
+        const uint32_t nb = min(tail - head, 4u);
+        uint32_t base = head;
+        if (8 * (int)(tail - head) > a.qcap - LIFO_ROOM) {
             tail -= nb;
             base = tail;
         } else {
-            base = head;
             head += nb;
         }
-        float4 jp = make_float4(0.f, 0.f, 0.f, 0.f), wk = make_float4(0.f, 0.f, 0.f, 0.f);
-#if GT_DEBUG
-        bool valid = (uint32_t)lane < nb;
-        if (valid) {
-            const uint32_t node = q[(base + lane) & qmask];
-            if (node >= nnodes) {
-                gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
-                valid = false;
-            } else {
-                jp = a.jpos[node];
-                wk = a.walk[node];
-                const uint32_t c = __float_as_uint(wk.z), f = __float_as_uint(wk.y);
-                const bool lf = (c & GT_LEAF_FLAG) != 0u;
-                if ((unsigned long long)f + (lf ? (c & ~GT_LEAF_FLAG) : c) > (lf ? a.n : nnodes)) {
-                    gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
-                    valid = false;
-                }
-            }
-        }
-#else
-        if (valid) {
-            const uint32_t node = q[(base + lane) & qmask];
-            jp = a.jpos[node];
-            wk = a.walk[node];
-        }
-#endif
-        n_tests += nb;
-        const bool ok = valid && mac_accept(a.mac, a.theta, dacc_amin, a.delta_acc, a.G, cx, cy, cz, bI, jp,
-                                            wk.x, wk.w);
-        const uint32_t l0 = __float_as_uint(wk.y), l1 = __float_as_uint(wk.z);
-        const bool leaf = (l1 & GT_LEAF_FLAG) != 0u;
-        // accepted cells -> list
-        const unsigned am = __ballot_sync(FULL, ok);
-        if (am) {
-            const int nacc = __popc(am);
-            if (list_n + nacc > LIST_CAP) flush();
-            if (ok) {
-                const int e = list_n + __popc(am & lt);
-                lx[e] = jp.x; ly[e] = jp.y; lz[e] = jp.z; lw[e] = jp.w;
-            }
-            list_n += nacc;
-        }
-        // opened cells -> their children into the queue; opened leaves -> their particles
-        // into the list (asynchronous copies).  One warp scan counts both (children in the
-        // low 16 bits, particles in the high 16: they fit while every leaf of the batch holds
-        // fewer than 2048 particles) and one loop writes both: entry e of the batch belongs
-        // to the first lane whose inclusive count exceeds e (a binary search over the lanes
-        // by shuffles); each lane's entries are its cell's children or its leaf's particles.
-        const uint32_t nch = (valid && !ok && !leaf) ? l1 : 0u;
-        const uint32_t lc = (valid && !ok && leaf) ? (l1 & ~GT_LEAF_FLAG) : 0u;
-        if (__all_sync(FULL, lc < 2048u)) {
-            const uint32_t mine = nch | (lc << 16);
-            const uint32_t incl = warp_incl_scan(mine);
-            const uint32_t tot = __shfl_sync(FULL, incl, 31);
-            const uint32_t tc = tot & 0xffffu, tp = tot >> 16;
-            if (tail - head + tc > (uint32_t)a.qcap) {
-                overflow = true;
-                break;
-            }
-            const uint32_t inclm = (incl & 0xffffu) + (incl >> 16);  // entries up to this lane
-            int pbase = list_n;  // list slot of the batch's first particle
-            uint32_t pdone = 0;  // particles written by earlier rounds
-            for (uint32_t r = 0; r < tc + tp; r += 32) {
-                const uint32_t e = r + (uint32_t)lane;
-                int own = 0;
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (__shfl_sync(FULL, inclm, own + step - 1) <= e) own += step;
-                const uint32_t oi = __shfl_sync(FULL, incl, own);
-                const uint32_t om = __shfl_sync(FULL, mine, own);
-                const uint32_t ol = __shfl_sync(FULL, l0, own);
-                const uint32_t ec = (oi & 0xffffu) - (om & 0xffffu), ep = (oi >> 16) - (om >> 16);
-                const bool in = e < tc + tp;
-                const bool isp = in && (om >> 16) != 0u;
-                const uint32_t off = e - ec - ep;
-                const unsigned pm = __ballot_sync(FULL, isp);
-                if (pm && pbase + (int)pdone + __popc(pm) > LIST_CAP) {
-                    list_n = pbase + (int)pdone;
-                    flush();
-                    pbase = -(int)pdone;
-                }
-                if (in && !isp) q[(tail + ec + off) & qmask] = ol + off;
-                if (isp) {
-                    const int slot = pbase + (int)(ep + off);
-                    const float *src = (const float *)&a.posm[ol + off];
-                    cp_async4(&lx[slot], src);
-                    cp_async4(&ly[slot], src + 1);
-                    cp_async4(&lz[slot], src + 2);
-                    cp_async4(&lw[slot], src + 3);
-                }
-                pdone += (uint32_t)__popc(pm);
-            }
-            tail += tc;
-            list_n = pbase + (int)pdone;
-        } else {
-            // a leaf of 2048 or more particles (coincident particles chained to level 21)
-            const uint32_t incl = warp_incl_scan(nch);
-            const uint32_t tot = __shfl_sync(FULL, incl, 31);
-            if (tot) {
-                if (tail - head + tot > (uint32_t)a.qcap) {
+        const Batch t = test_batch<MAC>(a, ps, q, base, nb, qmask, tests);
+        // opened cells: their children join the queue as one entry per cell
+        const unsigned om = __ballot_sync(FULL, t.nch != 0u);
+        if (om) {
+            if (t.nch) q[(tail + __popc(om & lt)) & qmask] = make_uint2(t.l0, t.nch);
+            tail += __popc(om);
+            if (8u * (tail - head) > (uint32_t)a.qcap) {  // more cells than the queue may hold?  count them
+                __syncwarp();
+                uint32_t live = 0;
+                for (uint32_t e = head + lane; e < tail; e += 32) live += q[e & qmask].y;
+                if (__reduce_add_sync(FULL, live) > (uint32_t)a.qcap) {
                     overflow = true;
                     break;
                 }
-                // the warp writes the children together: entry e belongs to the first lane whose
-                // inclusive count exceeds e (a binary search over the lanes by shuffles)
-                const uint32_t cbase = l0 - (incl - nch);
-                for (uint32_t r = 0; r < tot; r += 32) {
-                    const uint32_t e = r + (uint32_t)lane;
-                    int own = 0;
-#pragma unroll
-                    for (int step = 16; step > 0; step >>= 1)
-                        if (__shfl_sync(FULL, incl, own + step - 1) <= e) own += step;
-                    const uint32_t cb = __shfl_sync(FULL, cbase, own);
-                    if (e < tot) q[(tail + e) & qmask] = cb + e;
-                }
-                tail += tot;
-            }
-            // opened leaves -> their particles into the list (asynchronous copies)
-            const uint32_t lincl = warp_incl_scan(lc);
-            const uint32_t ltot = __shfl_sync(FULL, lincl, 31);
-            if (ltot) {
-                if (list_n + (int)ltot > LIST_CAP) flush();
-                if (ltot <= (uint32_t)LIST_CAP) {
-                    const uint32_t pbase = l0 - (lincl - lc);
-                    for (uint32_t r = 0; r < ltot; r += 32) {
-                        const uint32_t e = r + (uint32_t)lane;
-                        int own = 0;
-#pragma unroll
-                        for (int step = 16; step > 0; step >>= 1)
-                            if (__shfl_sync(FULL, lincl, own + step - 1) <= e) own += step;
-                        const uint32_t pb = __shfl_sync(FULL, pbase, own);
-                        if (e < ltot) {
-                            const float *src = (const float *)&a.posm[pb + e];
-                            cp_async4(&lx[list_n + e], src);
-                            cp_async4(&ly[list_n + e], src + 1);
-                            cp_async4(&lz[list_n + e], src + 2);
-                            cp_async4(&lw[list_n + e], src + 3);
-                        }
-                    }
-                    list_n += (int)ltot;
-                } else {  // leaves holding more particles than the list: one at a time, in chunks
-                    unsigned lm = __ballot_sync(FULL, lc != 0u);
-                    while (lm) {
-                        const int src = __ffs(lm) - 1;
-                        lm &= lm - 1;
-                        const uint32_t lf = __shfl_sync(FULL, l0, src);
-                        const uint32_t lcount = __shfl_sync(FULL, lc, src);
-                        uint32_t done = 0;
-                        while (done < lcount) {
-                            if (list_n == LIST_CAP) flush();
-                            const uint32_t take = min(lcount - done, (uint32_t)(LIST_CAP - list_n));
-                            for (uint32_t k = lane; k < take; k += 32) {
-                                const float *src = (const float *)&a.posm[lf + done + k];
-                                cp_async4(&lx[list_n + k], src);
-                                cp_async4(&ly[list_n + k], src + 1);
-                                cp_async4(&lz[list_n + k], src + 2);
-                                cp_async4(&lw[list_n + k], src + 3);
-                            }
-                            list_n += (int)take;
-                            done += take;
-                        }
-                    }
-                }
             }
         }
-        if (list_n >= FLUSH_AT) flush();
+        // accepted cells and opened leaves: entries of the list, in the cells' order
+        const unsigned am = __ballot_sync(FULL, t.ok);
+        const unsigned lm = __ballot_sync(FULL, t.mine != 0u) & ~am;
+        if (!lm && list_n + 32u <= LIST_CAP) {
+            if (t.ok) {
+                float *e = lx + list_n + __popc(am & lt);
+                e[0] = t.jp.x; e[LIST_CAP] = t.jp.y; e[2 * LIST_CAP] = t.jp.z; e[3 * LIST_CAP] = t.jp.w;
+            }
+            list_n += __popc(am);
+        } else {
+            const uint32_t incl = warp_incl_scan(t.mine);
+            const uint32_t tot = __shfl_sync(FULL, incl, 31);
+            // a window of the batch's entries at a time: what the list has room for
+            for (uint32_t w0 = 0; w0 < tot;) {
+                const uint32_t w1 = min(tot, w0 + (LIST_CAP - list_n));
+                write_entries(a, t, incl - t.mine, lm, lx, LIST_CAP, list_n - w0, w0, w1);
+                list_n += w1 - w0;
+                w0 = w1;
+                if (w0 < tot) flush();
+            }
+        }
+        if (list_n >= CHUNK) flush();
         __syncwarp();
     }
-    if (overflow) {
+    if (!overflow) {
+        flush();
+        if (list_n) {  // the last, shorter chunk
+            pad_list(lx, LIST_CAP, list_n);
+            chunk(0, (list_n + 3) >> 2);
+        }
+    } else {
         if (lane == 0) gt_set_error(a.ctl, GT_EOVERFLOW, GTK_WALK);
         cp_async_wait_all();
-        list_n = 0;
-        if (sub == 0 && have) a.acc[kk] = make_float4(NAN, NAN, NAN, NAN);
-        if (have2) a.acc[kk2] = make_float4(NAN, NAN, NAN, NAN);
-        __syncwarp();
-        return;
+        mem[64] = mem[96] = make_float4(NAN, NAN, NAN, NAN);
+        list_n = chunks = 0;
     }
-    flush();
-    for (int o = 1; o < S; o <<= 1) {
-        ax += __shfl_xor_sync(FULL, ax, o);
-        ay += __shfl_xor_sync(FULL, ay, o);
-        az += __shfl_xor_sync(FULL, az, o);
-        ph += __shfl_xor_sync(FULL, ph, o);
+    __syncwarp();
+    // the range is read again: held over the traversal it would cost registers
+    group_range(a, g, ngroups, a0, a1);
+    tests = __reduce_add_sync(FULL, tests);
+    if (lane == 0) {
+        stat[0] += ((unsigned long long)chunks * CHUNK + list_n) * (a1 - a0);
+        stat[1] += tests;
     }
-    if (sub == 0 && have) {
-        const float phi = fmaf(pi.w, a.inv_eps, ph);
-        a.acc[kk] = make_float4(a.G * ax, a.G * ay, a.G * az, a.G * phi);
+    store_group(a, a0, a1, mem);
+    __syncwarp();
+}
+
+// The barrier of a team (a power of two of the block's warps).
+__device__ __forceinline__ void team_sync(uint32_t team, uint32_t T) {
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "r"(T * 32u) : "memory");
+}
+
+// One group by a team of T warps: every round tests up to 4 T queue entries, 4 per warp, and lists what they
+// give in the order that one warp would (the queue is first in, first out, and entries and queue slots follow
+// from scans over the team's warps); the team's warps sum different chunks, and their partial sums are added in
+// the chunks' order.  So the result is the one warp's, bit for bit, whatever T is.  A queue that grows to
+// where one warp may turn depth-first ends the attempt: false, and one warp walks the group.
+// lx: T x WARP_SM words: four arrays of T LIST_CAP entries, the members and sums, T x 64 partial sums.
+template <int MAC>
+__device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx, uint2 *q,
+                                           unsigned long long *stat, uint2 *counts, uint32_t team, uint32_t T) {
+    const uint32_t lane = threadIdx.x & 31u, w = (threadIdx.x >> 5) & (T - 1u);
+    const uint32_t qmask = gt_queue_ring(a.qcap) - 1u, cap = T * LIST_CAP;
+    const unsigned FULL = 0xffffffffu;
+    const unsigned lt = lanemask_lt();
+    float4 *mem = (float4 *)(lx + 4 * cap) + lane;
+    float4 *part = mem + 128;  // of warp v: part[64 v], part[64 v + 32]
+    uint32_t a0, a1;
+    group_range(a, g, ngroups, a0, a1);
+    const bool two = a1 - a0 > 32u;
+    Pseudo ps;
+    {   // every warp finds the same sphere; the first one's members are the team's
+        float4 *own = w == 0 ? mem : part + 64 * (T - 2u) ;
+        if (!group_setup(a, a0, a1 - a0, own, ps)) {
+            if (w == 0 && lane == 0) gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
+            return true;
+        }
     }
-    if (have2) {
-        const float phi = fmaf(pi2.w, a.inv_eps, qh);
-        a.acc[kk2] = make_float4(a.G * bx, a.G * by, a.G * bz, a.G * phi);
+    uint32_t list_n = 0, chunks = 0, tests = 0;
+    // the list's full chunks (at the end: all of it), then the rest moved to its front
+    auto flush = [&](bool last) {
+        cp_async_wait_all();
+        team_sync(team, T);
+        const uint32_t full = list_n / CHUNK, todo = last ? (list_n + CHUNK - 1) / CHUNK : full;
+        if (last && w == 0) pad_list(lx, cap, list_n);
+        if (last) team_sync(team, T);
+        for (uint32_t c0 = 0; c0 < todo; c0 += T) {
+            const uint32_t c = c0 + w;
+            if (c < todo) {
+                const uint32_t k0 = c * (CHUNK / 4), k1 = c < full ? k0 + CHUNK / 4 : (list_n + 3) >> 2;
+                part[64 * w] = chunk_force(lx, cap, mem[0], a.eps2, k0, k1);
+                if (two) part[64 * w + 32] = chunk_force(lx, cap, mem[32], a.eps2, k0, k1);
+            }
+            team_sync(team, T);
+            if (w == 0)
+                for (uint32_t v = 0; v < min(T, todo - c0); v++) {
+                    add_force(mem[64], part[64 * v]);
+                    if (two) add_force(mem[96], part[64 * v + 32]);
+                }
+            if (c0 + T < todo) team_sync(team, T);
+        }
+        chunks += full;
+        list_n -= full * CHUNK;
+        if (!last) {
+            if (full && w == T - 1u) move_rest(lx, cap, list_n, full * (CHUNK / 4));
+            team_sync(team, T);
+        }
+    };
+    uint32_t head = 0, tail = 1;
+    if (w == 0 && lane == 0) q[0] = make_uint2(0u, 1u);
+    team_sync(team, T);
+    while (head != tail) {
+        const uint32_t live = tail - head, nb = min(live, 4u * T), b0 = min(4u * w, nb);
+        const Batch t = test_batch<MAC>(a, ps, q, head + b0, min(nb - b0, 4u), qmask, tests);
+        head += nb;
+        const unsigned om = __ballot_sync(FULL, t.nch != 0u), am = __ballot_sync(FULL, t.ok);
+        const unsigned lm = __ballot_sync(FULL, t.mine != 0u) & ~am;
+        const uint32_t incl = lm ? warp_incl_scan(t.mine) : (uint32_t)__popc(am & (lt | (1u << lane)));
+        if (lane == 31) counts[w] = make_uint2(__popc(om), incl);
+        team_sync(team, T);
+        uint32_t push = 0, pushes = 0, first = 0, tot = 0;
+        for (uint32_t v = 0; v < T; v++) {
+            const uint2 c = counts[v];
+            if (v == w) { push = pushes; first = tot; }
+            pushes += c.x;
+            tot += c.y;
+        }
+        if (8 * (int)(live + pushes) > a.qcap - LIFO_ROOM) {  // the same for every warp
+            cp_async_wait_all();
+            team_sync(team, T);
+            return false;
+        }
+        if (t.nch) q[(tail + push + __popc(om & lt)) & qmask] = make_uint2(t.l0, t.nch);
+        tail += pushes;
+        const uint32_t excl = first + incl - t.mine;
+        for (uint32_t w0 = 0; w0 < tot;) {
+            const uint32_t w1 = min(tot, w0 + (cap - list_n));
+            write_entries(a, t, excl, lm, lx, cap, list_n - w0, w0, w1);
+            list_n += w1 - w0;
+            w0 = w1;
+            if (w0 < tot) flush(false);
+        }
+        if (list_n >= T * CHUNK) flush(false);  // its last barrier ends the round
+        else team_sync(team, T);
     }
+    flush(true);
+    tests = __reduce_add_sync(FULL, tests);
+    group_range(a, g, ngroups, a0, a1);
+    if (lane == 0) {
+        if (w == 0) stat[0] += ((unsigned long long)chunks * CHUNK + list_n) * (a1 - a0);
+        stat[1] += tests;
+    }
+    if (w == 0) store_group(a, a0, a1, mem);
+    return true;
+}
+
+// Groups are taken one after another from a counter, by single warps or, when there are too few of them to
+// keep the grid busy, by teams.  A team of T does a group in ~T / 1.2, T / 1.7, T / 2.7 (T = 2, 4, 8) of one
+// warp's time (barriers, and batches that the first levels of the tree do not fill), so it pays where the
+// longest groups, not their sum, set the time.  Whole calls in us with T = 1, 2, 4, 8 (3648 warps): 476 groups
+// 704, 509, 399, 354; 4600 groups 370, 264, 214, 238; 6080 groups 412, 368, 365, 415; 11333 groups 272, 303,
+// 380, 573; 115000 groups 2620, 3207, 4456, 7118.
+__device__ __forceinline__ uint32_t team_of(uint32_t ngroups, uint32_t warps) {
+    return ngroups > 2u * warps ? 1u : (ngroups > warps ? 2u : (ngroups > warps / 4u ? 4u : 8u));
 }
 
 // groups of one system in a list of the systems' group counts: gprefix[s] is the first
@@ -523,46 +653,75 @@ __device__ __forceinline__ int system_of(const uint32_t *gprefix, int nsys, uint
     return lo;
 }
 
+template <int MAC>
 __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(WalkArgs a) {
-    __shared__ __align__(16) float list_sm[NWARP][4 * LIST_CAP];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *list = list_sm[warp];
-    uint32_t *q = a.queue + (size_t)(blockIdx.x * NWARP + warp) * (size_t)a.qcap;
+    __shared__ __align__(16) float list_sm[NWARP][WARP_SM];
+    __shared__ unsigned long long stat_sm[NWARP][2];
+    __shared__ uint2 counts_sm[NWARP];
+    __shared__ uint32_t g_sm[NWARP];
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     const uint32_t na = a.ctl->n_active;
     const uint32_t gmax = (uint32_t)a.gmax;
     const uint32_t ngroups = a.gstart ? a.ctl->n_groups : (na + gmax - 1) / gmax;
-    unsigned long long n_inter = 0, n_tests = 0;
-    for (;;) {
-        uint32_t g = 0;
-        if (lane == 0) g = atomicAdd(&a.ctl->group_next, 1u);
-        g = __shfl_sync(0xffffffffu, g, 0);
-        if (g >= ngroups) break;
-        walk_group(a, g, ngroups, list, q, n_inter, n_tests);
+    const uint32_t T = team_of(ngroups, gridDim.x * NWARP), team = warp / T, first = team * T;
+    uint2 *q = (uint2 *)a.queue + (size_t)(blockIdx.x * NWARP + first) * gt_queue_ring(a.qcap);
+    unsigned long long *stat = stat_sm[warp];
+    if (lane < 2) stat[lane] = 0;
+    __syncwarp();
+    if (T == 1) {
+        for (;;) {
+            uint32_t g = 0;
+            if (lane == 0) g = atomicAdd(&a.ctl->group_next, 1u);
+            g = __shfl_sync(0xffffffffu, g, 0);
+            if (g >= ngroups) break;
+            walk_group<MAC>(a, g, ngroups, list_sm[warp], q, stat);
+        }
+    } else {
+        for (;;) {
+            if (warp == first && lane == 0) g_sm[team] = atomicAdd(&a.ctl->group_next, 1u);
+            team_sync(team, T);
+            const uint32_t g = g_sm[team];
+            if (g >= ngroups) break;
+            if (!team_group<MAC>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
+                walk_group<MAC>(a, g, ngroups, list_sm[first], q, stat);
+            team_sync(team, T);
+        }
     }
+    __syncwarp();
     if (lane == 0) {
-        if (n_inter) atomicAdd(&a.ctl->interactions, n_inter);
-        if (n_tests) atomicAdd(&a.ctl->mac_tests, n_tests);
+        if (stat[0]) atomicAdd(&a.ctl->interactions, stat[0]);
+        if (stat[1]) atomicAdd(&a.ctl->mac_tests, stat[1]);
     }
 }
 
 // Many systems in one persistent launch: global group numbers run over the systems
-// in order (gprefix), every warp takes the next one from one counter and walks it
+// in order (gprefix), every warp or team takes the next one from one counter and walks it
 // with that system's arguments (copied to shared memory).  mac >= 0 overrides every
 // system's MAC (the opening-angle start-up pass).
-__global__ __launch_bounds__(WT, 3) void k_walk_batch(const WalkArgs *__restrict__ args, int nsys,
-                                                      const uint32_t *__restrict__ gprefix,
-                                                      unsigned int *group_next, uint32_t *queue, int qcap,
-                                                      int mac) {
-    __shared__ __align__(16) float list_sm[NWARP][4 * LIST_CAP];
+template <int MAC>
+__global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs *__restrict__ args, int nsys,
+                                                                 const uint32_t *__restrict__ gprefix,
+                                                                 unsigned int *group_next, uint32_t *queue, int qcap,
+                                                                 int mac) {
+    __shared__ __align__(16) float list_sm[NWARP][WARP_SM];
     __shared__ WalkArgs sargs[NWARP];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *list = list_sm[warp];
-    uint32_t *q = queue + (size_t)(blockIdx.x * NWARP + warp) * (size_t)qcap;
+    __shared__ unsigned long long stat_sm[NWARP][2];
+    __shared__ uint2 counts_sm[NWARP];
+    __shared__ uint32_t g_sm[NWARP];
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     const uint32_t total = gprefix[nsys];
+    const uint32_t T = team_of(total, gridDim.x * NWARP), team = warp / T, first = team * T;
+    uint2 *q = (uint2 *)queue + (size_t)(blockIdx.x * NWARP + first) * gt_queue_ring(qcap);
     for (;;) {
         uint32_t gg = 0;
-        if (lane == 0) gg = atomicAdd(group_next, 1u);
-        gg = __shfl_sync(0xffffffffu, gg, 0);
+        if (T == 1) {
+            if (lane == 0) gg = atomicAdd(group_next, 1u);
+            gg = __shfl_sync(0xffffffffu, gg, 0);
+        } else {
+            if (warp == first && lane == 0) g_sm[team] = atomicAdd(group_next, 1u);
+            team_sync(team, T);
+            gg = g_sm[team];
+        }
         if (gg >= total) break;
         int sys = 0;
         if (lane == 0) sys = system_of(gprefix, nsys, gg);
@@ -571,18 +730,26 @@ __global__ __launch_bounds__(WT, 3) void k_walk_batch(const WalkArgs *__restrict
         const uint32_t *src = (const uint32_t *)&args[sys];
         uint32_t *dst = (uint32_t *)&sargs[warp];
         for (int w = lane; w < (int)(sizeof(WalkArgs) / 4); w += 32) dst[w] = src[w];
+        unsigned long long *stat = stat_sm[warp];
+        if (lane < 2) stat[lane] = 0;
         __syncwarp();
         if (mac >= 0 && lane == 0) sargs[warp].mac = mac;
         __syncwarp();
         const WalkArgs &a = sargs[warp];
         const uint32_t g = gg - gprefix[sys];
         const uint32_t ngroups = gprefix[sys + 1] - gprefix[sys];
-        unsigned long long n_inter = 0, n_tests = 0;
         // the batch queue replaces the system's own
-        walk_group(a, g, ngroups, list, q, n_inter, n_tests);
+        if (T == 1) {
+            walk_group<MAC>(a, g, ngroups, list_sm[warp], q, stat);
+        } else {
+            if (!team_group<MAC>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
+                walk_group<MAC>(a, g, ngroups, list_sm[first], q, stat);
+            team_sync(team, T);
+        }
+        __syncwarp();
         if (lane == 0) {
-            if (n_inter) atomicAdd(&a.ctl->interactions, n_inter);
-            if (n_tests) atomicAdd(&a.ctl->mac_tests, n_tests);
+            if (stat[0]) atomicAdd(&a.ctl->interactions, stat[0]);
+            if (stat[1]) atomicAdd(&a.ctl->mac_tests, stat[1]);
         }
         __syncwarp();
     }
@@ -615,7 +782,7 @@ __global__ void k_batch_prefix(DevCtl *const *__restrict__ ctls, const WalkArgs 
 
 int gt_walk_blocks(int nsm) {
     int per = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk, WT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<MAC_ANY>, WT, 0);
     if (per < 1) per = 1;
     return per * nsm;
 }
@@ -623,13 +790,19 @@ int gt_walk_blocks(int nsm) {
 int gt_walk_warps_per_block() { return NWARP; }
 
 void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st) {
-    { k_walk<<<nblocks, WT, 0, st>>>(a); gt_note_launches(1); }
+    if (a.mac == GT_MAC_ACCELERATION) k_walk<GT_MAC_ACCELERATION><<<nblocks, WT, 0, st>>>(a);
+    else k_walk<MAC_ANY><<<nblocks, WT, 0, st>>>(a);
+    gt_note_launches(1);
 }
 
 void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, uint32_t *gprefix,
-                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, int nblocks,
+                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, int nblocks,
                           cudaStream_t st) {
     if (nsys <= 0) return;
     { k_batch_prefix<<<1, 32, 0, st>>>(ctls, args, nsys, gprefix, group_next); gt_note_launches(1); }
-    { k_walk_batch<<<nblocks, WT, 0, st>>>(args, nsys, gprefix, group_next, queue, qcap, mac); gt_note_launches(1); }
+    if (all_acc && mac < 0)
+        k_walk_batch<GT_MAC_ACCELERATION><<<nblocks, WT, 0, st>>>(args, nsys, gprefix, group_next, queue, qcap, mac);
+    else
+        k_walk_batch<MAC_ANY><<<nblocks, WT, 0, st>>>(args, nsys, gprefix, group_next, queue, qcap, mac);
+    gt_note_launches(1);
 }
