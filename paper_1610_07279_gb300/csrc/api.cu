@@ -393,22 +393,24 @@ double c2_of(const gt_params &p) {
 }
 
 // A6 groups + A7 walk over the active list already in s->active / ctl->n_active
-// (cell grouping needs the prefix s->prefix of that list), or over a caller's list.
-void walk(gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac, cudaStream_t st) {
+// (cell grouping needs the prefix s->prefix of that list), or over a caller's list.  levels: for the
+// integration (the forces choose the particles' levels).
+void walk(gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac, bool levels,
+          cudaStream_t st) {
     if (cell_groups(s->prm))
         gt_launch_groups(s->nd, s->cap, s->prefix, s->gmax_now, s->rcrit_now, s->n, s->marks, s->ctl, s->gstart,
                          s->status, s->nsm, st);
-    const WalkArgs a = gt_sys_walk_args(s, active, aold, acc, mac);
+    const WalkArgs a = gt_sys_walk_args(s, active, aold, acc, mac, levels);
     ph_begin(s, PH_WALK, st);
     gt_launch_walk(a, s->walk_blocks, st);
     ph_end(s, PH_WALK, st);
 }
 
 // every particle active (start-up passes, gt_accel_active with no list)
-void walk_all(gt_system *s, const float *aold, float4 *acc, int mac, cudaStream_t st) {
+void walk_all(gt_system *s, const float *aold, float4 *acc, int mac, bool levels, cudaStream_t st) {
     gt_launch_prepare(s->ctl, 0, st);
     gt_launch_active(s->st[0], s->n, s->prm.levels, 1, s->ctl, s->active, s->prefix, s->status, s->nsm, st);
-    walk(s, nullptr, aold, acc, mac, st);
+    walk(s, nullptr, aold, acc, mac, levels, st);
 }
 
 }  // namespace
@@ -464,7 +466,8 @@ void gt_sys_groups_all(gt_system *s, cudaStream_t st) {
                          s->status, s->nsm, st);
 }
 
-WalkArgs gt_sys_walk_args(const gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac) {
+WalkArgs gt_sys_walk_args(const gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac,
+                          bool levels) {
     WalkArgs a;
     a.gstart = cell_groups(s->prm) ? s->gstart : nullptr;
     a.jpos = s->nd.jpos;
@@ -498,6 +501,7 @@ void gt_sys_step_pre(gt_system *s, cudaStream_t st, bool rebuild, bool predicted
         ph_begin(s, PH_PREDICT, st);
         gt_launch_predict(s->st[0], n, s->ctl, rebuild ? s->posm_tmp : s->posm, st);
         ph_end(s, PH_PREDICT, st);
+    a.inv_c2 = levels ? (float)(1.0 / c2_of(s->prm)) : 0.0f;
     } else if (!rebuild) {
         std::swap(s->posm, s->posm_tmp);  // the prediction enqueued ahead went to posm_tmp
     }
@@ -677,16 +681,16 @@ int gt_accel_active(gt_system *s, const uint32_t *d_active, int64_t n_active, co
     drop_ahead(s, st);
     const float *aold = d_aold ? d_aold : s->st[0].aold;
     if (!d_active) {
-        walk_all(s, aold, (float4 *)d_acc, s->prm.mac, st);
+        walk_all(s, aold, (float4 *)d_acc, s->prm.mac, false, st);
     } else if (cell_groups(s->prm)) {
         gt_launch_prepare(s->ctl, 0, st);
         gt_launch_active_from_list(d_active, n_active, s->n, s->flags, s->ctl, s->active, s->prefix, s->status,
                                    s->nsm, st);
-        walk(s, s->active, aold, (float4 *)d_acc, s->prm.mac, st);
+        walk(s, s->active, aold, (float4 *)d_acc, s->prm.mac, false, st);
     } else {
         gt_launch_prepare(s->ctl, 0, st);
         gt_launch_set_nactive(s->ctl, (unsigned)n_active, st);
-        walk(s, d_active, aold, (float4 *)d_acc, s->prm.mac, st);
+        walk(s, d_active, aold, (float4 *)d_acc, s->prm.mac, false, st);
     }
     return last_cuda();
 }
@@ -703,11 +707,11 @@ int gt_start(gt_system *s, const float *p_aold_boot, gt_stream stream) {
             return GT_ECUDA;
         gt_launch_gather_f(s->aold_tmp, t.id, n, t.aold, st);
     } else {
-        walk_all(s, nullptr, s->acc_out, GT_MAC_OPENING_ANGLE, st);
+        walk_all(s, nullptr, s->acc_out, GT_MAC_OPENING_ANGLE, false, st);
         gt_launch_aold(s->acc_out, n, t.aold, st);
         ph_sync_collect(s, st);
     }
-    walk_all(s, t.aold, s->acc_out, s->prm.mac, st);
+    walk_all(s, t.aold, s->acc_out, s->prm.mac, true, st);
     gt_sys_start_levels(s, st);
     return last_cuda();
 }
@@ -761,7 +765,7 @@ int gt_block_step(gt_system *s, gt_stream stream) {
     s->last_rebuilt = rebuild;
     gt_sys_step_pre(s, st, rebuild, predicted);
     State &t = s->st[0];
-    walk(s, s->active, t.aold, s->acc_out, s->prm.mac, st);
+    walk(s, s->active, t.aold, s->acc_out, s->prm.mac, true, st);
     gt_sys_step_post(s, st);
     // Look-ahead (automatic interval; the tuners wait for every step): the control
     // words the next call reads, then the prediction of every particle to the next

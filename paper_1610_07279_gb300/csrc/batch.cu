@@ -92,7 +92,7 @@ int upload_args(gt_batch *b) {
     if (!b->args_dirty) return GT_OK;
     for (int k = 0; k < b->nsys; k++) {
         gt_system *s = b->sys[k];
-        b->h_args[k] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, s->prm.mac);
+        b->h_args[k] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, s->prm.mac, false);
         b->h_args[k].queue = b->queue;
     }
     if (cudaMemcpy(b->d_args, b->h_args.data(), (size_t)b->nsys * sizeof(WalkArgs), cudaMemcpyHostToDevice) !=
@@ -130,7 +130,7 @@ void enqueue(gt_batch *b, int bootstrap, cudaStream_t st) {
     join(b, st);
     if (bootstrap) {
         gt_launch_walk_batch(b->d_ctls, b->d_args, b->nsys, b->d_gprefix, b->d_next, b->queue, b->qcap,
-                             GT_MAC_OPENING_ANGLE, false, b->walk_blocks, st);
+                             GT_MAC_OPENING_ANGLE, false, false, b->walk_blocks, st);
         fork(b, st);
         for (int k = 0; k < b->nsys; k++)
             if (b->sys[k]->n > 0) gt_sys_aold_from_acc(b->sys[k], b->streams[k % nstreams(b)]);
@@ -139,7 +139,7 @@ void enqueue(gt_batch *b, int bootstrap, cudaStream_t st) {
     bool all_acc = true;
     for (const gt_system *s : b->sys) all_acc = all_acc && s->prm.mac == GT_MAC_ACCELERATION;
     gt_launch_walk_batch(b->d_ctls, b->d_args, b->nsys, b->d_gprefix, b->d_next, b->queue, b->qcap, -1, all_acc,
-                         b->walk_blocks, st);
+                         false, b->walk_blocks, st);
 }
 
 long long launches_now() {

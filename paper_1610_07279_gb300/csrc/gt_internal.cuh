@@ -102,6 +102,15 @@ struct Nodes {
 };
 
 __device__ __forceinline__ void gt_set_error(DevCtl *ctl, int code, int where) {
+// FP32 values as unsigned integers in the same order (for atomic minima and maxima), and back.
+__device__ __forceinline__ unsigned int gt_ordered(float f) {
+    const unsigned int b = __float_as_uint(f);
+    return b >> 31 ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float gt_unordered(unsigned int u) {
+    return __uint_as_float(u >> 31 ? u & 0x7fffffffu : ~u);
+}
+
     if (atomicCAS(&ctl->err, 0, code) == 0) ctl->err_where = where;
 }
 
@@ -341,6 +350,7 @@ struct WalkArgs {
 // newest pairs are taken first, which keeps at most ~700 more, so half as many pairs as cells (and
 // 1024 for the smallest queues) hold every walk that walk_queue admits.
 __host__ __device__ inline uint32_t gt_queue_ring(int qcap) { return qcap >= 2048 ? (uint32_t)qcap / 2u : 1024u; }
+    float inv_c2;            // block steps: 1 / (2 eta eps)^2, the scale of the levels' thresholds; otherwise 0
 __host__ __device__ inline size_t gt_queue_words(int qcap) { return 2 * (size_t)gt_queue_ring(qcap); }
 int gt_walk_blocks(int nsm);
 // tuner.cu
@@ -360,7 +370,7 @@ extern "C" int gt_rebuild_interval(const double *t_walk, int n, double t_make, i
 int gt_walk_warps_per_block();
 void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st);
 // one launch over the groups of nsys systems (args, ctls: device arrays of nsys entries); all_acc: every
-// system uses the acceleration MAC
+// system uses the acceleration MAC; levels: some have inv_c2 > 0
 void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, uint32_t *gprefix,
-                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, int nblocks,
-                          cudaStream_t st);
+                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, bool levels,
+                          int nblocks, cudaStream_t st);

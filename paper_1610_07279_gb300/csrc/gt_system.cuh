@@ -126,8 +126,9 @@ void gt_sys_apply_params(gt_system *s, const gt_params &p);
 void gt_sys_build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src);
 // A6 with every particle active: the active list and, for cell grouping, the groups
 void gt_sys_groups_all(gt_system *s, cudaStream_t st);
-// arguments of one walk over the current active list / groups
-WalkArgs gt_sys_walk_args(const gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac);
+// arguments of one walk over the current active list / groups; levels: its forces choose the particles' levels
+WalkArgs gt_sys_walk_args(const gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac,
+                          bool levels);
 // |a| of the last walk over every particle -> a_old (start-up pass)
 void gt_sys_aold_from_acc(gt_system *s, cudaStream_t st);
 // after the start-up walks: levels and block time of every particle (the system is started)

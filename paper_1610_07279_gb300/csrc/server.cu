@@ -123,7 +123,7 @@ void batched_walk(gt_server *v, const TickList &L) {
     for (int k = 0; k < L.n; k++)
         all_acc = all_acc && L.variant[k] != V_BOOT && v->slots[L.slot[k]].sys->prm.mac == GT_MAC_ACCELERATION;
     gt_launch_walk_batch(v->d_tick_ctls, v->d_tick_args, L.n, v->d_gprefix, v->d_next, v->queue, v->qcap, -1, all_acc,
-                         v->walk_blocks, v->main);
+                         true, v->walk_blocks, v->main);
     v->walk_launches++;
 }
 
@@ -375,9 +375,9 @@ int gt_submit(gt_server *v, const gt_request *req, uint64_t *ticket) {
     }
     // the three walk-argument variants of this slot
     WalkArgs a[NVARIANT];
-    a[V_STEP] = gt_sys_walk_args(s, s->active, s->st[0].aold, s->acc_out, prm.mac);
-    a[V_BOOT] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, GT_MAC_OPENING_ANGLE);
-    a[V_FIRST] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, prm.mac);
+    a[V_STEP] = gt_sys_walk_args(s, s->active, s->st[0].aold, s->acc_out, prm.mac, true);
+    a[V_BOOT] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, GT_MAC_OPENING_ANGLE, false);
+    a[V_FIRST] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, prm.mac, true);
     DevCtl *ctl = s->ctl;
     if (cudaMemcpyAsync(v->d_pool + (size_t)k * NVARIANT, a, sizeof(a), cudaMemcpyHostToDevice, v->admit) ||
         cudaMemcpyAsync(v->d_ctl_pool + k, &ctl, sizeof(ctl), cudaMemcpyHostToDevice, v->admit) ||

@@ -52,6 +52,9 @@ constexpr int NWARP = WT / 32;
 constexpr uint32_t LIST_CAP = 256;  // interaction-list entries per warp
 constexpr uint32_t CHUNK = 128;     // entries whose forces are summed from zero before they join a member's sums
 constexpr uint32_t WARP_SM = 4 * LIST_CAP + 4 * 4 * 32;  // the list, then the lanes' members and sums
+// walk_group_ordered: the whole of a warp's words is the list; a batch that leaves FLUSH_AT entries has it summed
+constexpr uint32_t SEG_CAP = 384, FLUSH_AT = 256;
+static_assert(4 * SEG_CAP <= WARP_SM, "the list of walk_group_ordered");
 // Depth-first reserve of the queue: popping the newest 32 cells and pushing at most
 // 8 children each grows the queue by <= 224 per tree level, <= ~22 x 256 in all.
 constexpr int LIFO_ROOM = 6144;
@@ -215,9 +218,10 @@ struct Pseudo {
     float x, y, z, b, dacc_amin;  // centre and radius of the group's sphere; Delta_acc times its smallest |a_old|
 };
 
-// A group's pseudo i-particle, and the lane's members in shared memory: mem[0], [32] the first and second,
-// negated, with the first quad and the quad step of the lane's share in the fourth word; mem[64], [96] their
-// sums, zero.  False for a malformed group.
+// A group's pseudo i-particle, and the lane's members: mem[0], mem[MS] the first and second, negated, with the
+// first quad and the quad step of the lane's share in the fourth word; mem[2 MS], mem[3 MS] their sums, zero (MS 32:
+// in shared memory; 1: the lane's own).  ORDERED: a second member has one lane.  False for a malformed group.
+template <bool ORDERED, uint32_t MS>
 __device__ __forceinline__ bool group_setup(const WalkArgs &a, uint32_t a0, uint32_t cnt, float4 *mem, Pseudo &ps) {
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
@@ -229,7 +233,7 @@ __device__ __forceinline__ bool group_setup(const WalkArgs &a, uint32_t a0, uint
     const int slot = lane >> logS, sub = lane & (S - 1);
     const bool have = (uint32_t)slot < cnt;
     // lanes of one second member: like S, as many as their count (1 to 32) leaves, so that they don't idle
-    const int logS2 = (two && !a.ij_share) ? 5 - (cnt <= 33u ? 0 : 32 - __clz(cnt - 33u)) : 0;
+    const int logS2 = (!ORDERED && two && !a.ij_share) ? 5 - (cnt <= 33u ? 0 : 32 - __clz(cnt - 33u)) : 0;
     const int slot2 = 32 + (lane >> logS2), sub2 = lane & ((1 << logS2) - 1);
     const bool have2 = two && (uint32_t)slot2 < cnt;
     const uint32_t i = member_of(a, a0 + (have ? (uint32_t)slot : 0u));
@@ -266,8 +270,8 @@ __device__ __forceinline__ bool group_setup(const WalkArgs &a, uint32_t a0, uint
     for (int o = 16; o > 0; o >>= 1) d2 = fmaxf(d2, __shfl_xor_sync(FULL, d2, o));
     ps = Pseudo{cx, cy, cz, __fmul_rn(__fsqrt_rn(d2), GT_RADIUS_MARGIN), __fmul_rn(a.delta_acc, ao)};
     mem[0] = make_float4(-pi.x, -pi.y, -pi.z, __uint_as_float((uint32_t)sub | (1u << logS << 8)));
-    mem[32] = make_float4(-pi2.x, -pi2.y, -pi2.z, __uint_as_float((uint32_t)sub2 | (1u << logS2 << 8)));
-    mem[64] = mem[96] = make_float4(0.f, 0.f, 0.f, 0.f);
+    mem[MS] = make_float4(-pi2.x, -pi2.y, -pi2.z, __uint_as_float((uint32_t)sub2 | (1u << logS2 << 8)));
+    mem[2 * MS] = mem[3 * MS] = make_float4(0.f, 0.f, 0.f, 0.f);
     return true;
 }
 
@@ -390,12 +394,24 @@ __device__ __forceinline__ void write_entries(const WalkArgs &a, const Batch &t,
     }
 }
 
-// The members' sums, reduced over their lanes, to the caller's accelerations.
-__device__ __forceinline__ void store_group(const WalkArgs &a, uint32_t a0, uint32_t a1, const float4 *mem) {
+// Whether a force is so close to the threshold of a block-step level (|a|^2 / c^2 a power of 16) that the order of
+// its sums may decide: within 2^-17, some thirty times the rounding errors of the sums.
+__device__ __forceinline__ bool near_level(float4 f, float inv_c2) {
+    const float x = (f.x * f.x + f.y * f.y + f.z * f.z) * inv_c2;
+    const uint32_t b = __float_as_uint(x), e = b >> 23, m = b & 0x7fffffu;
+    if (e == 0u || e >= 255u) return false;
+    return (m < 64u && ((e - 127u) & 3u) == 0u) || (m >= 0x800000u - 64u && ((e - 126u) & 3u) == 0u);
+}
+
+// The members' sums, reduced over their lanes, to the caller's accelerations.  True (for the warp) if LEVELS, the walk
+// is one that chooses levels (inv_c2 > 0), and one of them is near a level's threshold.
+template <bool LEVELS, uint32_t MS>
+__device__ __forceinline__ bool store_group(const WalkArgs &a, uint32_t a0, uint32_t a1, const float4 *mem) {
     const uint32_t lane = threadIdx.x & 31u;
+    bool near = false;
     for (uint32_t who = 0; who < a1 - a0; who += 32) {
-        const uint32_t share = __float_as_uint(mem[who].w), S = share >> 8;
-        float4 sum = mem[64 + who];
+        const uint32_t share = __float_as_uint(mem[who / 32 * MS].w), S = share >> 8;
+        float4 sum = mem[2 * MS + who / 32 * MS];
         for (uint32_t o = 1; o < S; o <<= 1) {
             sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
             sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
@@ -406,14 +422,268 @@ __device__ __forceinline__ void store_group(const WalkArgs &a, uint32_t a0, uint
         if ((share & 0xffu) == 0u && k < a1) {
             const uint32_t i = a.active ? a.active[k] : k;
             const float phi = fmaf(a.posm[i < a.n ? i : 0u].w, a.inv_eps, sum.w);
-            a.acc[k] = make_float4(a.G * sum.x, a.G * sum.y, a.G * sum.z, a.G * phi);
+            const float4 f = make_float4(a.G * sum.x, a.G * sum.y, a.G * sum.z, a.G * phi);
+            a.acc[k] = f;
+            if (LEVELS) near = near || near_level(f, a.inv_c2);
+        }
+    }
+    return LEVELS && __any_sync(0xffffffffu, near);
+}
+
+// Forces of a list's first nquad quads (arrays of `cap` entries from lx on) on one member of every lane, added to
+// its sums.
+__device__ __forceinline__ void sum_segment(const float *lx, uint32_t cap, float4 *member, float4 *sum, float eps2,
+                                            uint32_t nquad) {
+    const float4 *px = (const float4 *)lx, *py = (const float4 *)(lx + cap), *pz = (const float4 *)(lx + 2 * cap),
+                 *pw = (const float4 *)(lx + 3 * cap);
+    const float4 p = *member, s = *sum;
+    const uint32_t share = __float_as_uint(p.w), step = share >> 8;
+    const float2 e2 = make_float2(eps2, eps2);
+    const float2 nx = make_float2(p.x, p.x), ny = make_float2(p.y, p.y), nz = make_float2(p.z, p.z);
+    float2 sx = make_float2(s.x, 0.f), sy = make_float2(s.y, 0.f), sz = make_float2(s.z, 0.f);
+    float2 sp = make_float2(-s.w, 0.f);
+#pragma unroll 1
+    for (uint32_t k = share & 0xffu; k < nquad; k += step) {
+        const float4 X = px[k], Y = py[k], Z = pz[k], W = pw[k];
+        interact_pairs(make_float2(X.x, X.y), make_float2(Y.x, Y.y), make_float2(Z.x, Z.y), make_float2(W.x, W.y),
+                       nx, ny, nz, e2, sx, sy, sz, sp);
+        interact_pairs(make_float2(X.z, X.w), make_float2(Y.z, Y.w), make_float2(Z.z, Z.w), make_float2(W.z, W.w),
+                       nx, ny, nz, e2, sx, sy, sz, sp);
+    }
+    *sum = make_float4(__fadd_rn(sx.x, sx.y), __fadd_rn(sy.x, sy.y), __fadd_rn(sz.x, sz.y), -__fadd_rn(sp.x, sp.y));
+}
+
+struct Cell {
+    float4 jp;
+    uint32_t l0;      // first child or first particle
+    uint32_t nch, lc; // children of an opened cell, particles of an opened leaf
+    bool ok;          // accepted
+};
+
+// One cell per lane, and what the MAC says.
+template <int MAC>
+__device__ __forceinline__ Cell test_cell(const WalkArgs &a, const Pseudo &ps, uint32_t node, bool valid) {
+#if GT_DEBUG
+    const uint32_t nnodes = a.ctl->level_start[GT_TREE_LEVELS];
+    if (valid && node >= nnodes) {
+        gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
+        valid = false;
+    }
+#endif
+    if (!valid) node = 0u;
+    Cell t;
+    t.jp = a.jpos[node];
+    const float4 wk = a.walk[node];
+    const uint32_t l1 = __float_as_uint(wk.z);
+    const bool leaf = (l1 & GT_LEAF_FLAG) != 0u;
+    t.l0 = __float_as_uint(wk.y);
+#if GT_DEBUG
+    if (valid && (unsigned long long)t.l0 + (l1 & ~GT_LEAF_FLAG) > (leaf ? a.n : nnodes)) {
+        gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
+        valid = false;
+    }
+#endif
+    t.ok = valid && mac_accept<MAC>(a.mac, a.theta, ps.dacc_amin, a.delta_acc, a.G, ps.x, ps.y, ps.z, ps.b, t.jp, wk.x,
+                                    wk.w);
+    const bool opened = valid && !t.ok;
+    t.nch = opened && !leaf ? l1 : 0u;
+    t.lc = opened && leaf ? (l1 & ~GT_LEAF_FLAG) : 0u;
+    return t;
+}
+
+// An accepted cell's entry.
+__device__ __forceinline__ void write_cell(const Cell &t, float *e, uint32_t cap) {
+    e[0] = t.jp.x; e[cap] = t.jp.y; e[2 * cap] = t.jp.z; e[3 * cap] = t.jp.w;
+}
+
+// The particles of a batch's opened leaves with index in [w0, w1) into the list: particle e goes to slot to + e.
+// `incl`: the warp scan of lc; lm: lanes with an opened leaf.  Opened leaves next to each other in the batch that
+// hold one range of particles (siblings) are copied together, asynchronously.
+__device__ __forceinline__ void write_particles(const WalkArgs &a, const Cell &t, uint32_t incl, unsigned lm, float *lx,
+                                                uint32_t cap, uint32_t to, uint32_t w0, uint32_t w1) {
+    const unsigned FULL = 0xffffffffu;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t before = __shfl_up_sync(FULL, t.l0 + t.lc, 1);  // where the lane before ends
+    const bool joins = lane > 0 && t.lc && (lm >> (lane - 1u) & 1u) && before == t.l0;
+    const unsigned starts = lm & ~__ballot_sync(FULL, joins);
+    for (unsigned m = starts; m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        // the run's last lane: before the next lane that is no leaf or starts a run of its own
+        const unsigned stop = (~lm | (starts & ~(1u << src))) & (0xfffffffeu << src);
+        const int end = stop ? __ffs(stop) - 2 : 31;
+        const uint32_t le = __shfl_sync(FULL, incl - t.lc, src);
+        const uint32_t e1 = min(__shfl_sync(FULL, incl, end), w1);
+        const float4 *p = a.posm + __shfl_sync(FULL, t.l0, src);
+        for (uint32_t e = max(le, w0) + lane; e < e1; e += 32) {
+            const float *from = (const float *)&p[e - le];
+            float *d = lx + to + e;
+            cp_async4(d, from);
+            cp_async4(d + cap, from + 1);
+            cp_async4(d + 2 * cap, from + 2);
+            cp_async4(d + 3 * cap, from + 3);
         }
     }
 }
 
+// Particles among the batch's children and particles number 32 r to 32 r + 31 (they are counted together, lane by
+// lane; `first`: the number of the lane's first).  A batch whose particles don't fit behind the list goes on in
+// steps of these 32: a segment ends before the step that would overflow it.
+__device__ __forceinline__ uint32_t particles_of_step(uint32_t first, uint32_t lc, uint32_t r) {
+    const uint32_t lo = max(first, 32u * r), hi = min(first + lc, 32u * r + 32u);
+    return __reduce_add_sync(0xffffffffu, hi > lo ? hi - lo : 0u);
+}
+
+// One group again, in a fixed order of summation: a batch is the queue's next 32 cells, its accepted cells precede
+// the particles of its opened leaves in the list, the list is summed whenever a batch leaves FLUSH_AT entries or
+// would overflow it, every chain of additions runs over the whole walk, and a second member has one lane.  Block
+// steps turn forces into discrete levels, and a particle whose |a| is within a rounding of a level's threshold
+// would get another step from any other order of the same sums (1 particle in 10^7 and step).  The groups of
+// such particles (near_level: 2 groups in 10^4) are walked a second time by this function, so that levels, and
+// with them the trajectories, don't depend on how walk_group arranges its sums.  As the only walk it would take 2.9 ms
+// against walk_group's 2.6 (every particle at 2^22).  lx: the warp's WARP_SM words of shared memory.
+__device__ __noinline__ void walk_group_ordered(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx, uint2 *q) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t qmask = gt_queue_ring(a.qcap) - 1u;
+    const unsigned FULL = 0xffffffffu;
+    const unsigned lt = lanemask_lt();
+    float4 mem[4];
+    uint32_t a0, a1;
+    group_range(a, g, ngroups, a0, a1);
+    const bool two = a1 - a0 > 32u;
+    Pseudo ps;
+    if (!group_setup<true, 1>(a, a0, a1 - a0, mem, ps)) return;
+    uint32_t list_n = 0;
+    auto flush = [&]() {
+        cp_async_wait_all();
+        __syncwarp();
+        pad_list(lx, SEG_CAP, list_n);
+        const uint32_t nquad = (list_n + 3) >> 2;
+        sum_segment(lx, SEG_CAP, &mem[0], &mem[2], a.eps2, nquad);
+        if (two) sum_segment(lx, SEG_CAP, &mem[1], &mem[3], a.eps2, nquad);
+        list_n = 0;
+        __syncwarp();
+    };
+    uint32_t head = 0, tail = 1, off = 0;  // queue entries; children of the head's entry already taken
+    if (lane == 0) q[0] = make_uint2(0u, 1u);  // the root
+    __syncwarp();
+    bool overflow = false;
+    while (head != tail) {
+        // the next 32 cells: breadth-first from the head while there is room, depth-first from the tail after
+        const uint32_t avail = tail - head;
+        uint32_t node, ncell;
+        if (8 * (int)avail <= a.qcap - LIFO_ROOM) {
+            uint2 e = make_uint2(0u, 0u);
+            if (lane < avail) e = q[(head + lane) & qmask];
+            if (lane == 0) {
+                e.x += off;
+                e.y -= off;
+            }
+            if ((__ballot_sync(FULL, e.y == 8u) & 0xfu) == 0xfu) {  // four whole entries of eight
+                node = __shfl_sync(FULL, e.x, lane >> 3) + (lane & 7u);
+                ncell = 32u;
+                head += 4u;
+                off = 0u;
+            } else {
+                const uint32_t incl = warp_incl_scan(e.y), excl = incl - e.y;
+                // bit p: an entry's first cell has lane p; the entries before it are one after another from lane 0
+                const unsigned m = __reduce_or_sync(FULL, e.y && excl < 32u ? 1u << excl : 0u) & (lt | (1u << lane));
+                node = __shfl_sync(FULL, e.x, __popc(m) - 1) + lane - (31u - (uint32_t)__clz(m));
+                ncell = min(__shfl_sync(FULL, incl, 31), 32u);
+                const uint32_t whole = __popc(__ballot_sync(FULL, e.y && incl <= 32u));
+                const uint32_t cut = __shfl_sync(FULL, excl, whole & 31u), left = __shfl_sync(FULL, incl, 31);
+                head += whole;
+                off = left > 32u ? 32u - cut : 0u;
+            }
+        } else {
+            const uint32_t nb = min(avail, 4u), o = lane >> 3;
+            tail -= nb;
+            uint2 e = o < nb ? q[(tail + o) & qmask] : make_uint2(0u, 0u);
+            if (o < nb && tail + o == head) {
+                e.x += off;
+                e.y -= off;
+            }
+            if (tail == head) off = 0u;
+            // the cells side by side in the lanes, as from the head
+            const uint32_t n0 = __shfl_sync(FULL, e.y, 0), n1 = n0 + __shfl_sync(FULL, e.y, 8),
+                           n2 = n1 + __shfl_sync(FULL, e.y, 16), n3 = n2 + __shfl_sync(FULL, e.y, 24);
+            const uint32_t own = (lane >= n0 ? 1u : 0u) + (lane >= n1 ? 1u : 0u) + (lane >= n2 ? 1u : 0u);
+            node = __shfl_sync(FULL, e.x, 8u * own) + lane - (own == 0 ? 0u : own == 1 ? n0 : own == 2 ? n1 : n2);
+            ncell = n3;
+        }
+        const Cell t = test_cell<MAC_ANY>(a, ps, node, lane < ncell);
+        // accepted cells -> list (there is room: fewer than FLUSH_AT entries at a batch's begin)
+        const unsigned am = __ballot_sync(FULL, t.ok);
+        if (t.ok) write_cell(t, lx + list_n + __popc(am & lt), SEG_CAP);
+        list_n += __popc(am);
+        // opened cells: their children join the queue as one entry per cell
+        const unsigned om = __ballot_sync(FULL, t.nch != 0u);
+        if (om) {
+            if (t.nch) q[(tail + __popc(om & lt)) & qmask] = make_uint2(t.l0, t.nch);
+            tail += __popc(om);
+            if (8u * (tail - head) > (uint32_t)a.qcap) {  // more cells than the queue may hold?  count them
+                __syncwarp();
+                uint32_t live = 0;
+                for (uint32_t e = head + lane; e < tail; e += 32) live += q[e & qmask].y;
+                if (__reduce_add_sync(FULL, live) - off > (uint32_t)a.qcap) {
+                    overflow = true;
+                    break;
+                }
+            }
+        }
+        // opened leaves -> their particles
+        const unsigned lm = __ballot_sync(FULL, t.lc != 0u);
+        if (lm) {
+            const uint32_t incl = warp_incl_scan(t.lc), tot = __shfl_sync(FULL, incl, 31);
+            if (list_n + tot <= SEG_CAP) {
+                write_particles(a, t, incl, lm, lx, SEG_CAP, list_n, 0u, tot);
+                list_n += tot;
+            } else if (__all_sync(FULL, t.lc < 2048u)) {  // in steps of 32 children and particles
+                const uint32_t both = warp_incl_scan(t.nch + t.lc), first = both - t.lc;  // a lane has one or the other
+                const uint32_t steps = (__shfl_sync(FULL, both, 31) + 31u) >> 5;
+                uint32_t w0 = 0, w1 = 0;  // particles before this window, and before this step
+                for (uint32_t r = 0; r < steps; r++) {
+                    const uint32_t pm = particles_of_step(first, t.lc, r);
+                    if (pm && list_n + (w1 - w0) + pm > SEG_CAP) {
+                        write_particles(a, t, incl, lm, lx, SEG_CAP, list_n - w0, w0, w1);
+                        list_n += w1 - w0;
+                        flush();
+                        w0 = w1;
+                    }
+                    w1 += pm;
+                }
+                write_particles(a, t, incl, lm, lx, SEG_CAP, list_n - w0, w0, w1);
+                list_n += w1 - w0;
+            } else {  // a leaf of 2048 or more particles (coincident particles chained to level 21)
+                flush();
+                for (uint32_t w0 = 0; w0 < tot;) {
+                    const uint32_t w1 = min(tot, w0 + (SEG_CAP - list_n));
+                    write_particles(a, t, incl, lm, lx, SEG_CAP, list_n - w0, w0, w1);
+                    list_n += w1 - w0;
+                    w0 = w1;
+                    if (list_n == SEG_CAP) flush();
+                }
+            }
+        }
+        if (list_n >= FLUSH_AT) flush();
+        __syncwarp();
+    }
+    if (!overflow) {
+        flush();
+    } else {
+        if (lane == 0) gt_set_error(a.ctl, GT_EOVERFLOW, GTK_WALK);
+        cp_async_wait_all();
+        mem[2] = mem[3] = make_float4(NAN, NAN, NAN, NAN);
+    }
+    __syncwarp();
+    // the range is read again: held over the traversal it would cost registers
+    group_range(a, g, ngroups, a0, a1);
+    (void)store_group<false, 1>(a, a0, a1, mem);
+    __syncwarp();
+}
+
 // One group g of system a (Sec. 2.3) by one warp.  The interactions and MAC tests are added to stat[0] and
 // stat[1].  lx: the warp's WARP_SM words of shared memory.
-template <int MAC>
+template <int MAC, bool LEVELS>
 __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx, uint2 *q,
                                            unsigned long long *stat) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -425,7 +695,7 @@ __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32
     group_range(a, g, ngroups, a0, a1);
     const bool two = a1 - a0 > 32u;
     Pseudo ps;
-    if (!group_setup(a, a0, a1 - a0, mem, ps)) {
+    if (!group_setup<false, 32>(a, a0, a1 - a0, mem, ps)) {
         if (lane == 0) gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
         return;
     }
@@ -519,8 +789,9 @@ __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32
         stat[0] += ((unsigned long long)chunks * CHUNK + list_n) * (a1 - a0);
         stat[1] += tests;
     }
-    store_group(a, a0, a1, mem);
+    const bool again = store_group<LEVELS, 32>(a, a0, a1, mem) && !overflow;
     __syncwarp();
+    if (LEVELS && again) walk_group_ordered(a, g, ngroups, lx, q);
 }
 
 // The barrier of a team (a power of two of the block's warps).
@@ -534,7 +805,7 @@ __device__ __forceinline__ void team_sync(uint32_t team, uint32_t T) {
 // the chunks' order.  So the result is the one warp's, bit for bit, whatever T is.  A queue that grows to
 // where one warp may turn depth-first ends the attempt: false, and one warp walks the group.
 // lx: T x WARP_SM words: four arrays of T LIST_CAP entries, the members and sums, T x 64 partial sums.
-template <int MAC>
+template <int MAC, bool LEVELS>
 __device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx, uint2 *q,
                                            unsigned long long *stat, uint2 *counts, uint32_t team, uint32_t T) {
     const uint32_t lane = threadIdx.x & 31u, w = (threadIdx.x >> 5) & (T - 1u);
@@ -549,7 +820,7 @@ __device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32
     Pseudo ps;
     {   // every warp finds the same sphere; the first one's members are the team's
         float4 *own = w == 0 ? mem : part + 64 * (T - 2u) ;
-        if (!group_setup(a, a0, a1 - a0, own, ps)) {
+        if (!group_setup<false, 32>(a, a0, a1 - a0, own, ps)) {
             if (w == 0 && lane == 0) gt_set_error(a.ctl, GT_EINVAL, GTK_WALK);
             return true;
         }
@@ -628,7 +899,10 @@ __device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32
         if (w == 0) stat[0] += ((unsigned long long)chunks * CHUNK + list_n) * (a1 - a0);
         stat[1] += tests;
     }
-    if (w == 0) store_group(a, a0, a1, mem);
+    if (w == 0 && store_group<LEVELS, 32>(a, a0, a1, mem)) {
+        __syncwarp();
+        if (LEVELS) walk_group_ordered(a, g, ngroups, lx, q);
+    }
     return true;
 }
 
@@ -653,8 +927,8 @@ __device__ __forceinline__ int system_of(const uint32_t *gprefix, int nsys, uint
     return lo;
 }
 
-template <int MAC>
-__global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(WalkArgs a) {
+template <int MAC, bool LEVELS>
+__global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant__ WalkArgs a) {
     __shared__ __align__(16) float list_sm[NWARP][WARP_SM];
     __shared__ unsigned long long stat_sm[NWARP][2];
     __shared__ uint2 counts_sm[NWARP];
@@ -674,7 +948,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(WalkArgs a) {
             if (lane == 0) g = atomicAdd(&a.ctl->group_next, 1u);
             g = __shfl_sync(0xffffffffu, g, 0);
             if (g >= ngroups) break;
-            walk_group<MAC>(a, g, ngroups, list_sm[warp], q, stat);
+            walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[warp], q, stat);
         }
     } else {
         for (;;) {
@@ -682,8 +956,8 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(WalkArgs a) {
             team_sync(team, T);
             const uint32_t g = g_sm[team];
             if (g >= ngroups) break;
-            if (!team_group<MAC>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
-                walk_group<MAC>(a, g, ngroups, list_sm[first], q, stat);
+            if (!team_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
+                walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat);
             team_sync(team, T);
         }
     }
@@ -698,7 +972,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(WalkArgs a) {
 // in order (gprefix), every warp or team takes the next one from one counter and walks it
 // with that system's arguments (copied to shared memory).  mac >= 0 overrides every
 // system's MAC (the opening-angle start-up pass).
-template <int MAC>
+template <int MAC, bool LEVELS>
 __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs *__restrict__ args, int nsys,
                                                                  const uint32_t *__restrict__ gprefix,
                                                                  unsigned int *group_next, uint32_t *queue, int qcap,
@@ -740,10 +1014,10 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
         const uint32_t ngroups = gprefix[sys + 1] - gprefix[sys];
         // the batch queue replaces the system's own
         if (T == 1) {
-            walk_group<MAC>(a, g, ngroups, list_sm[warp], q, stat);
+            walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[warp], q, stat);
         } else {
-            if (!team_group<MAC>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
-                walk_group<MAC>(a, g, ngroups, list_sm[first], q, stat);
+            if (!team_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
+                walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat);
             team_sync(team, T);
         }
         __syncwarp();
@@ -782,7 +1056,7 @@ __global__ void k_batch_prefix(DevCtl *const *__restrict__ ctls, const WalkArgs 
 
 int gt_walk_blocks(int nsm) {
     int per = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<MAC_ANY>, WT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<MAC_ANY, true>, WT, 0);
     if (per < 1) per = 1;
     return per * nsm;
 }
@@ -790,19 +1064,23 @@ int gt_walk_blocks(int nsm) {
 int gt_walk_warps_per_block() { return NWARP; }
 
 void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st) {
-    if (a.mac == GT_MAC_ACCELERATION) k_walk<GT_MAC_ACCELERATION><<<nblocks, WT, 0, st>>>(a);
-    else k_walk<MAC_ANY><<<nblocks, WT, 0, st>>>(a);
+    constexpr int ACC = GT_MAC_ACCELERATION;
+    const bool acc = a.mac == ACC, levels = a.inv_c2 > 0.0f;
+    auto launch = [&](auto kernel) { kernel<<<nblocks, WT, 0, st>>>(a); };
+    if (levels) launch(acc ? k_walk<ACC, true> : k_walk<MAC_ANY, true>);
+    else launch(acc ? k_walk<ACC, false> : k_walk<MAC_ANY, false>);
     gt_note_launches(1);
 }
 
 void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, uint32_t *gprefix,
-                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, int nblocks,
-                          cudaStream_t st) {
+                          unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, bool levels,
+                          int nblocks, cudaStream_t st) {
     if (nsys <= 0) return;
     { k_batch_prefix<<<1, 32, 0, st>>>(ctls, args, nsys, gprefix, group_next); gt_note_launches(1); }
-    if (all_acc && mac < 0)
-        k_walk_batch<GT_MAC_ACCELERATION><<<nblocks, WT, 0, st>>>(args, nsys, gprefix, group_next, queue, qcap, mac);
-    else
-        k_walk_batch<MAC_ANY><<<nblocks, WT, 0, st>>>(args, nsys, gprefix, group_next, queue, qcap, mac);
+    constexpr int ACC = GT_MAC_ACCELERATION;
+    const bool acc = all_acc && mac < 0;
+    auto launch = [&](auto kernel) { kernel<<<nblocks, WT, 0, st>>>(args, nsys, gprefix, group_next, queue, qcap, mac); };
+    if (levels) launch(acc ? k_walk_batch<ACC, true> : k_walk_batch<MAC_ANY, true>);
+    else launch(acc ? k_walk_batch<ACC, false> : k_walk_batch<MAC_ANY, false>);
     gt_note_launches(1);
 }
