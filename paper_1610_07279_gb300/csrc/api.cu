@@ -117,9 +117,9 @@ size_t carve(gt_system *s, char *base, int64_t n, const gt_params *p, int nsm, i
         s->sb.key[b] = L.take<uint64_t>(base, N);
         s->sb.val[b] = L.take<uint32_t>(base, N);
     }
-    s->sb.status = (uint32_t *)L.take<char>(base, gt_sort_scratch_bytes(n));
-    s->sb.hist = L.take<uint32_t>(base, 8 * 256);
-    s->sb.digit_base = L.take<uint32_t>(base, 8 * 256);
+    s->sb.hist = (uint32_t *)L.take<char>(base, gt_sort_scratch_bytes(n));
+    s->sb.status = s->sb.hist ? s->sb.hist + GT_SORT_PASSES * GT_SORT_DIGITS : nullptr;
+    s->sb.digit_base = L.take<uint32_t>(base, GT_SORT_PASSES * GT_SORT_DIGITS);
     const int64_t cap = node_capacity(n, p);
     s->cap = cap;
     s->nd.first = L.take<uint32_t>(base, cap);
@@ -142,8 +142,6 @@ size_t carve(gt_system *s, char *base, int64_t n, const gt_params *p, int nsm, i
     s->aold_tmp = L.take<float>(base, N);
     s->scratch3 = L.take<double>(base, 3 * N + 8);  // also stages 13 B per particle on resume
     s->bscratch = L.take<uint8_t>(base, gt_build_scratch_bytes(n));
-    s->bbox_blocks = nsm * 4;
-    s->bbox_partial = L.take<float>(base, 6 * (size_t)s->bbox_blocks);
     s->walk_blocks = walk_blocks;
     s->walk_warps = walk_blocks * gt_walk_warps_per_block();
     s->queue_entries = own_queue ? (int64_t)(s->walk_warps * gt_queue_words(p->walk_queue)) : 0;
@@ -357,9 +355,9 @@ void build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src) {
     const int64_t n = s->n;
     gt_launch_prepare(s->ctl, 0, st);
     ph_begin(s, PH_SORT, st);
-    gt_launch_bbox(posm_src, n, s->bbox_partial, s->bbox_blocks, s->ctl, st);
-    gt_launch_keys(posm_src, n, s->ctl, s->prm.key_curve, s->sb.key[0], s->sb.val[0], st);
-    gt_launch_sort(s->sb, n, s->ctl, st);
+    gt_launch_bbox(posm_src, n, s->nsm * 4, s->ctl, st);
+    gt_launch_keys(posm_src, n, s->prm.key_curve, s->ctl, s->sb, s->nsm, st);
+    gt_launch_sort(s->sb, n, s->ctl, true, st);
     ph_end(s, PH_SORT, st);
     ph_begin(s, PH_PERMUTE, st);
     if (!s->fixed_buffers) {
@@ -442,7 +440,7 @@ int gt_sys_init(gt_system *s, int64_t n, const gt_params *p, void *ws, size_t ws
     const size_t st_bytes = (size_t)((s->cap + 511) / 512 + (n + 4095) / 4096 + 64) * 8;
     if (cudaMemsetAsync(s->ctl, 0, sizeof(DevCtl), st) != cudaSuccess ||
         cudaMemsetAsync(s->status, 0, st_bytes, st) != cudaSuccess ||
-        cudaMemsetAsync(s->sb.status, 0, gt_sort_scratch_bytes(n), st) != cudaSuccess ||
+        cudaMemsetAsync(s->sb.hist, 0, gt_sort_scratch_bytes(n), st) != cudaSuccess ||
         (st ? cudaStreamSynchronize(st) : cudaDeviceSynchronize()) != cudaSuccess)
         return GT_ECUDA;
     return GT_OK;

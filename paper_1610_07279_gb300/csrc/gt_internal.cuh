@@ -54,12 +54,9 @@ struct DevCtl {
     double dt_max;                    // longest block step (a power of two)
     int M;                            // log2(dt_max)
     int levels_m1;                    // L - 1 (finest level)
-    float bbox_min[3];
-    float pad1;
-    double side;                      // side of the bounding cube (FP64)
-    double scale;                     // 2^21 / side
+    unsigned int bbox[6];             // extrema of the positions (gt_ordered): minima, then maxima
+    unsigned int digits_done;         // blocks that have added their digit counts (the sort)
     unsigned int spin_limit;          // bound on every spin-wait of this system; 0: GT_SPIN_LIMIT
-    unsigned int pad2;
 };
 
 // The bound of a spin-wait: the control block's own, or the default.
@@ -252,23 +249,29 @@ __device__ __forceinline__ unsigned int lookback_warp(unsigned long long *status
 // Every helper reports the kernels it launched (counted for gt_kernel_launches).
 void gt_note_launches(int k);
 
+#define GT_SORT_BITS 8
+#define GT_SORT_DIGITS 256
+#define GT_SORT_PASSES 8             // 64 / 8 (bit 63 is always 0)
+
 struct SortBufs {
     uint64_t *key[2];
     uint32_t *val[2];
-    uint32_t *status;            // look-back status of the 8 passes, 8 x tiles x RADIX
-    uint32_t *hist;              // digit histograms of the 8 passes, 8 x RADIX
-    uint32_t *digit_base;        // digit starts of the 8 passes, 8 x RADIX
+    uint32_t *hist;              // digit counts of the 8 passes, 8 x 256, and behind them
+    uint32_t *status;            // look-back status of the 8 passes, 8 x tiles x 256 (cleared together)
+    uint32_t *digit_base;        // digit starts of the 8 passes, 8 x 256
 };
 
 // keys.cu
-void gt_launch_bbox(const float4 *posm, int64_t n, float *partial, int nblk, DevCtl *ctl,
-                    cudaStream_t st);
-void gt_launch_keys(const float4 *posm, int64_t n, const DevCtl *ctl, int curve, uint64_t *key, uint32_t *idx,
-                    cudaStream_t st);
-// sort.cu: sorts (key, val) in buffers 0; result in buffers 0 (even passes).
+// extrema into ctl->bbox (reset by gt_launch_prepare); keys into b.key[0] and their digit counts (so
+// that gt_launch_sort need not count them)
+void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, cudaStream_t st);
+void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st);
+// sort.cu: sorts (key, val) in buffers 0; result in buffers 0 (even passes).  counted: the digits are counted, and
+// the values are the keys' positions (b.val[0] is not read).
 int gt_sort_tiles(int64_t n);
 size_t gt_sort_scratch_bytes(int64_t n);
-void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st);
+void gt_sort_clear(SortBufs &b, int64_t n, cudaStream_t st);  // the digit counts and the look-back words
+void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, bool counted, cudaStream_t st);
 void gt_sort_init();
 // tree.cu
 // scratch: gt_build_scratch_bytes(n) bytes (per-particle marks and per-tile counts)

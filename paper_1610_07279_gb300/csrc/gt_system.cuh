@@ -90,8 +90,6 @@ struct gt_system {
     float *aold_tmp = nullptr;
     double *scratch3 = nullptr;
     uint8_t *bscratch = nullptr;  // tree build marks and counts
-    float *bbox_partial = nullptr;
-    int bbox_blocks = 0;
     uint32_t *queue = nullptr;    // the walk queue (a batch's shared queue for batch members)
     int64_t queue_entries = 0;
     DevCtl *ctl = nullptr;

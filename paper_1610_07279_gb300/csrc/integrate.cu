@@ -19,6 +19,8 @@
 // (no root, no division: FP64 throughput is low on this GPU).  A shorter step is taken
 // at once; a longer one only by one level and only when T is a multiple of it.  Every
 // FP64 operation carries an explicit rounding, so results are reproducible bit for bit.
+#include <float.h>
+
 #include "gt_internal.cuh"
 
 namespace {
@@ -27,6 +29,7 @@ __global__ void k_prepare(DevCtl *ctl, int begin_step) {
     ctl->epoch += 1u;
     for (int l = 0; l < GT_TREE_LEVELS + 4; l++) ctl->tile_ticket[l] = 0;
     ctl->group_next = 0;
+    for (int a = 0; a < 6; a++) ctl->bbox[a] = gt_ordered(a < 3 ? FLT_MAX : -FLT_MAX);
     if (begin_step) {
         ctl->tnext = ctl->tnext_acc;
         ctl->tnext_acc = ~0ull;

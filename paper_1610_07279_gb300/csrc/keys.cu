@@ -1,21 +1,24 @@
 // Step A1: bounding cube and 63-bit Morton keys (Sec. 2.1; Morton key layout of
 // Appendix A: every 3-bit digit is (x, y, z) with x the most significant bit).
 //
-// The bounding box reads 16 B per particle, the key pass reads 16 B and writes 12 B
-// (key + index); the key pass is bound by the exact quantisation's integer work, split
-// with the FP64 pipe (one axis there, two on the integer pipe).
+// The bounding box reads 16 B per particle and folds every block's extrema into the control
+// block; the key pass reads 16 B and writes 8 B (the index of the first sort pass's input is its
+// position), counts the digits of the sort's eight passes on the way, and its last block turns the
+// counts into the digits' starts.
 #include <float.h>
 
 #include "gt_internal.cuh"
 #include "keys_quant.cuh"
+#include "sort_digits.cuh"
 
 namespace {
 
 constexpr int BBOX_THREADS = 256;
+#ifndef GT_KEYS_BLOCKS
+#define GT_KEYS_BLOCKS 8  // blocks per SM of the key pass
+#endif
 
-__global__ __launch_bounds__(BBOX_THREADS) void k_bbox_partial(const float4 *__restrict__ posm,
-                                                               long long n,
-                                                               float *__restrict__ partial) {
+__global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict__ posm, long long n, DevCtl *ctl) {
     float mn0 = FLT_MAX, mn1 = FLT_MAX, mn2 = FLT_MAX;
     float mx0 = -FLT_MAX, mx1 = -FLT_MAX, mx2 = -FLT_MAX;
     for (long long i = blockIdx.x * (long long)BBOX_THREADS + threadIdx.x; i < n;
@@ -45,72 +48,37 @@ __global__ __launch_bounds__(BBOX_THREADS) void k_bbox_partial(const float4 *__r
         float v = s[0][threadIdx.x];
         for (int k = 1; k < BBOX_THREADS / 32; k++)
             v = threadIdx.x < 3 ? fminf(v, s[k][threadIdx.x]) : fmaxf(v, s[k][threadIdx.x]);
-        partial[blockIdx.x * 6 + threadIdx.x] = v;
+        if (threadIdx.x < 3) atomicMin(&ctl->bbox[threadIdx.x], gt_ordered(v));
+        else atomicMax(&ctl->bbox[threadIdx.x], gt_ordered(v));
     }
 }
 
-__global__ void k_bbox_final(const float *__restrict__ partial, int nblk, long long n, DevCtl *ctl) {
-    // one warp: reduce the per-block extrema, then the cube of Sec. 2.1's keys
-    float v[6];
-    for (int a = 0; a < 6; a++) v[a] = a < 3 ? FLT_MAX : -FLT_MAX;
-    for (int b = lane_id(); b < nblk; b += 32)
-        for (int a = 0; a < 6; a++)
-            v[a] = a < 3 ? fminf(v[a], partial[b * 6 + a]) : fmaxf(v[a], partial[b * 6 + a]);
-    for (int o = 16; o > 0; o >>= 1)
-        for (int a = 0; a < 6; a++) {
-            const float t = __shfl_xor_sync(0xffffffffu, v[a], o);
-            v[a] = a < 3 ? fminf(v[a], t) : fmaxf(v[a], t);
-        }
-    if (lane_id() == 0) {
-        double side = 0.0;
-        if (n > 0)
-            for (int a = 0; a < 3; a++) {
-                const double ext = __dsub_rn((double)v[a + 3], (double)v[a]);
-                if (ext > side) side = ext;
-            }
-        for (int a = 0; a < 3; a++) ctl->bbox_min[a] = n > 0 ? v[a] : 0.0f;
-        ctl->side = side;
-        ctl->scale = side > 0.0 ? __ddiv_rn((double)(1u << GT_KEY_LEVELS), side) : 0.0;
-    }
+// Spread the low 11 bits of v so that bit b lands on bit 3b.
+__device__ __forceinline__ uint32_t spread3(uint32_t v) {
+    v = (v | (v << 16)) & 0x070000ffu;
+    v = (v | (v << 8)) & 0x0700f00fu;
+    v = (v | (v << 4)) & 0x430c30c3u;
+    return (v | (v << 2)) & 0x49249249u;
 }
 
-// Spread the low 21 bits of v so that bit b lands on bit 3b.
-__device__ __forceinline__ unsigned long long spread3(unsigned long long v) {
-    v &= 0x1fffffull;
-    v = (v | (v << 32)) & 0x001f00000000ffffull;
-    v = (v | (v << 16)) & 0x001f0000ff0000ffull;
-    v = (v | (v << 8)) & 0x100f00f00f00f00full;
-    v = (v | (v << 4)) & 0x10c30c30c30c30c3ull;
-    v = (v | (v << 2)) & 0x1249249249249249ull;
-    return v;
+// The bits of three 21-bit integers interleaved, x the most significant of every triplet.
+__device__ __forceinline__ unsigned long long interleave(uint32_t x, uint32_t y, uint32_t z) {
+    const uint32_t xl = spread3(x & 0x7ffu);
+    const uint32_t lo = (xl << 2) | (spread3(y & 0x7ffu) << 1) | spread3(z & 0x7ffu);
+    const uint32_t hi = (spread3(x >> 11) << 2) | (spread3(y >> 11) << 1) | spread3(z >> 11);
+    return ((unsigned long long)((hi << 1) | (xl >> 30)) << 32) | lo;
 }
 
 constexpr unsigned long long QMAX = (1ull << GT_KEY_LEVELS) - 1ull;
 
-__device__ __forceinline__ unsigned long long quantise(float x, float xmin, double scale) {
-    // floor((x - xmin) * 2^21/side) with FP64 roundings (RN difference, RN product, then
-    // the floor), clamped to 2^21 - 1: in integer arithmetic (keys_quant.cuh), or for the
-    // rare operands it does not take, on the FP64 pipe -- x widened exactly on the
-    // integer pipe, the floor the round-down conversion (the product is >= 0).
+// floor((x - xmin) * 2^21/side) with FP64 roundings (RN difference, RN product, then the floor), clamped to
+// 2^21 - 1: in integer arithmetic (keys_quant.cuh), or for the operands it does not take, on the FP64 pipe -- x
+// widened exactly on the integer pipe, the floor the round-down conversion (the product is >= 0).
+__device__ __noinline__ uint32_t quantise_slow(float x, float xmin, double scale) {
     unsigned long long q;
-    if (quantise_exact(x, xmin, (unsigned long long)__double_as_longlong(scale), QMAX, &q)) return q;
+    if (quantise_exact(x, xmin, (unsigned long long)__double_as_longlong(scale), QMAX, &q)) return (uint32_t)q;
     q = __double2ull_rd(__dmul_rn(__dsub_rn(f2d(x), f2d(xmin)), scale));
-    return q < QMAX ? q : QMAX;
-}
-
-// The same quantisation with the two roundings on the FP64 pipe (x and xmin widened
-// exactly on the integer pipe; the floor of the non-negative product taken from its
-// bits).  k_keys runs one axis this way and two through quantise(): the FP64 pipe is
-// narrow on this GPU, the integer pipe bounds the pass, so the two share the work.
-__device__ __forceinline__ unsigned long long quantise_fp64(float x, float xmin, double scale) {
-    const double p = __dmul_rn(__dsub_rn(f2d(x), f2d(xmin)), scale);
-    const unsigned long long b = (unsigned long long)__double_as_longlong(p);
-    if (b >> 63) return 0ull;                    // negative (x below xmin: not produced by the bounding box)
-    const int e = (int)(b >> 52) - 1023;         // p = 1.f 2^e
-    if (e < 0) return 0ull;                      // p < 1, zero included
-    if (e >= GT_KEY_LEVELS) return QMAX;         // p >= 2^21 (and inf, nan)
-    const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
-    return m >> (52 - e);
+    return (uint32_t)(q < QMAX ? q : QMAX);
 }
 
 // Peano-Hilbert order (Sec. 2.1, App. A), Skilling's transpose method on the three
@@ -136,41 +104,62 @@ __device__ __forceinline__ void hilbert_transpose(uint32_t &x0, uint32_t &x1, ui
     x2 ^= t;
 }
 
-__global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, long long n,
-                                              const DevCtl *__restrict__ ctl, int curve,
-                                              unsigned long long *__restrict__ key,
-                                              uint32_t *__restrict__ idx) {
-    const long long i = blockIdx.x * 256ll + threadIdx.x;
-    if (i >= n) return;
-    const double side = ctl->side, scale = ctl->scale;
-    unsigned long long k = 0;
-    if (side > 0.0) {
-        const float4 p = posm[i];
-        const unsigned long long qx = quantise_fp64(p.x, ctl->bbox_min[0], scale);
-        const unsigned long long qy = quantise(p.y, ctl->bbox_min[1], scale);
-        const unsigned long long qz = quantise(p.z, ctl->bbox_min[2], scale);
-        if (curve == GT_KEY_HILBERT) {
-            uint32_t x0 = (uint32_t)qx, x1 = (uint32_t)qy, x2 = (uint32_t)qz;
-            hilbert_transpose(x0, x1, x2);
-            k = (spread3(x0) << 2) | (spread3(x1) << 1) | spread3(x2);
-        } else {
-            k = (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
+// Bound by issue: ~100 instructions per key of quantisation and interleaving on the FP32 and integer pipes and
+// ~50 of digit counting, against 24 B of HBM.
+__global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, long long n, int curve, DevCtl *ctl,
+                                              unsigned long long *__restrict__ key, uint32_t *__restrict__ hist,
+                                              uint32_t *__restrict__ base) {
+    __shared__ uint32_t h[GT_SORT_PASSES][GT_SORT_DIGITS];
+    __shared__ double scale_sh;
+    __shared__ float min_sh[3];
+    for (int p = 0; p < GT_SORT_PASSES; p++) h[p][threadIdx.x] = 0;
+    if (threadIdx.x == 0) {  // the cube of Sec. 2.1's keys, from the extrema
+        double side = 0.0;
+        for (int a = 0; a < 3; a++) {
+            const float lo = gt_unordered(ctl->bbox[a]);
+            const double ext = __dsub_rn((double)gt_unordered(ctl->bbox[a + 3]), (double)lo);
+            if (ext > side) side = ext;
+            min_sh[a] = lo;
         }
+        scale_sh = side > 0.0 ? __ddiv_rn((double)(1u << GT_KEY_LEVELS), side) : 0.0;
     }
-    key[i] = k;
-    idx[i] = (uint32_t)i;
+    __syncthreads();
+    const double scale = scale_sh;
+    const float x0 = min_sh[0], y0 = min_sh[1], z0 = min_sh[2];
+    float sh, sl;
+    const bool fp32 = gtq_fp32_scale(scale, &sh, &sl), sized = scale > 0.0;
+    for (long long i0 = (long long)blockIdx.x * 256; i0 < n; i0 += (long long)gridDim.x * 256) {
+        const long long i = i0 + threadIdx.x;
+        const bool ok = i < n;
+        unsigned long long k = 0;
+        if (ok && sized) {
+            const float4 p = posm[i];
+            uint32_t x = 0, y = 0, z = 0;
+            if (!fp32 || !quantise_fp32(p.x, x0, sh, sl, &x)) x = quantise_slow(p.x, x0, scale);
+            if (!fp32 || !quantise_fp32(p.y, y0, sh, sl, &y)) y = quantise_slow(p.y, y0, scale);
+            if (!fp32 || !quantise_fp32(p.z, z0, sh, sl, &z)) z = quantise_slow(p.z, z0, scale);
+            if (curve == GT_KEY_HILBERT) hilbert_transpose(x, y, z);
+            k = interleave(x, y, z);
+        }
+        if (ok) key[i] = k;
+        gt_count_digits(k, ok, h);
+    }
+    gt_finish_digits(h, hist, base, ctl);
 }
 
 }  // namespace
 
-void gt_launch_bbox(const float4 *posm, int64_t n, float *partial, int nblk, DevCtl *ctl,
-                    cudaStream_t st) {
-    { k_bbox_partial<<<nblk, BBOX_THREADS, 0, st>>>(posm, n, partial); gt_note_launches(1); }
-    { k_bbox_final<<<1, 32, 0, st>>>(partial, nblk, n, ctl); gt_note_launches(1); }
+void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, cudaStream_t st) {
+    if (n <= 0) return;
+    const int64_t need = (n + BBOX_THREADS - 1) / BBOX_THREADS;
+    { k_bbox<<<(unsigned)(need < nblk ? need : nblk), BBOX_THREADS, 0, st>>>(posm, n, ctl); gt_note_launches(1); }
 }
 
-void gt_launch_keys(const float4 *posm, int64_t n, const DevCtl *ctl, int curve, uint64_t *key, uint32_t *idx,
-                    cudaStream_t st) {
+void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st) {
     if (n <= 0) return;
-    { k_keys<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(posm, n, ctl, curve, (unsigned long long *)key, idx); gt_note_launches(1); }
+    gt_sort_clear(b, n, st);
+    const int64_t need = (n + 255) / 256, most = (int64_t)nsm * GT_KEYS_BLOCKS;
+    k_keys<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(posm, n, curve, ctl, (unsigned long long *)b.key[0],
+                                                                  b.hist, b.digit_base);
+    gt_note_launches(1);
 }

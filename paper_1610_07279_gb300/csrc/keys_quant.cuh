@@ -8,6 +8,7 @@
 // the handled range (see quantise_exact).
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -99,4 +100,51 @@ __host__ __device__ __forceinline__ bool quantise_exact(float x, float xmin, uns
         v = -e >= 64 ? 0ull : (m >> -e);
     *q = v < qmax ? v : qmax;
     return true;
+}
+
+// The same quantisation on the FP32 pipe, for nearly every operand: x - xmin as an unevaluated sum of two floats
+// (Knuth's two-sum, exact), times scale as sh + sl with the products' errors kept (fused multiply-adds), so that
+// the product is p + t with an error below 2^-22 for p < 2^22.  *q = floor and true where p + t is further than
+// 2^-19 from an integer, so that neither that error nor the two FP64 roundings (2^-31 together) can move the
+// floor; false otherwise (1 operand in 2^18, and the few on the cube's lower faces), also for infinities, NaN and
+// an overflowing difference.  sh, sl: scale rounded to FP32 and the rest, with sh in [2^-60, 2^100] (subnormal
+// rests would lose bits; the caller asks gtq_fp32_scale).
+__host__ __device__ __forceinline__ float gtq_fma(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(a, b, c);
+#else
+    return fmaf(a, b, c);
+#endif
+}
+__host__ __device__ __forceinline__ float gtq_add(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+__host__ __device__ __forceinline__ float gtq_mul(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+
+__host__ __device__ __forceinline__ bool gtq_fp32_scale(double scale, float *sh, float *sl) {
+    const bool ok = scale >= 0x1p-60 && scale <= 0x1p100;
+    *sh = ok ? (float)scale : 0.0f;
+    *sl = ok ? (float)(scale - (double)*sh) : 0.0f;
+    return ok;
+}
+
+__host__ __device__ __forceinline__ bool quantise_fp32(float x, float xmin, float sh, float sl, uint32_t *q) {
+    const float s = gtq_add(x, -xmin), bb = gtq_add(s, -x);
+    const float err = gtq_add(gtq_add(x, -gtq_add(s, -bb)), gtq_add(-xmin, -bb));  // x - xmin = s + err
+    const float p = gtq_mul(s, sh);
+    const float t = gtq_fma(s, sl, gtq_fma(err, sh, gtq_fma(s, sh, -p)));
+    const float m = gtq_add(p, 0x1p23f);  // p rounded to an integer, in the low bits
+    const float r = gtq_add(gtq_add(p, -gtq_add(m, -0x1p23f)), t);
+    *q = gtq_bits(m) - 0x4b000000u - (r < 0.0f ? 1u : 0u);
+    return p < 0x1p22f && (r > 0x1p-19f || r < -0x1p-19f);
 }

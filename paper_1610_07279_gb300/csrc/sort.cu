@@ -1,9 +1,9 @@
 // Step A2: stable LSD radix sort of (63-bit key, 32-bit index) pairs (Sec. 2.1: the
 // particles are sorted by their space-filling key with a library radix sort).
 //
-// Eight passes of 8-bit digits, one kernel per pass after one histogram pass:
-//   k_hist_all     all eight digit histograms in one read of the keys   (reads 8 B/key)
-//   k_digit_bases  exclusive scans of the histograms -> where every digit starts
+// Eight passes of 8-bit digits, one kernel per pass; the digits of all passes are counted by the kernel that
+// makes the keys (keys.cu), or for a caller's pairs by
+//   k_hist_all     all eight digit counts in one read of the keys, and their starts   (reads 8 B/key)
 //   k_onesweep     per 4096-key tile (512 threads) taken in ticket order: a stable rank of
 //                  every key inside the tile (warp-striped; a key's peers with the same
 //                  digit from nine ballots, its rank by popc), the tile's per-digit counts
@@ -18,6 +18,7 @@
 #include <mutex>
 
 #include "gt_internal.cuh"
+#include "sort_digits.cuh"
 
 namespace {
 
@@ -33,14 +34,14 @@ namespace {
 #ifndef GT_SORT_LB
 #define GT_SORT_LB 8               // earlier tiles read per look-back step
 #endif
-constexpr int RB = 8;              // digit bits
+constexpr int RB = GT_SORT_BITS;   // digit bits
 constexpr int R = 1 << RB;         // digits
-constexpr int HT = R;              // threads of the histogram and digit-base kernels
+constexpr int HT = R;              // threads of the histogram kernel
 constexpr int ST = GT_SORT_ST;     // threads per tile (the first R of them also own one digit each)
 constexpr int IPT = GT_SORT_IPT;   // keys per thread
 constexpr int TILE = ST * IPT;     // keys per tile
 constexpr int NW = ST / 32;
-constexpr int PASSES = 8;          // 64 / RB (bit 63 is always 0; the last pass is cheap)
+constexpr int PASSES = GT_SORT_PASSES;
 constexpr uint32_t ST_AGG = 1u << 30;   // status word: the tile's own count of the digit
 constexpr uint32_t ST_PRE = 2u << 30;   // status word: the inclusive count over tiles 0..t
 constexpr uint32_t ST_VAL = ST_AGG - 1u;
@@ -49,44 +50,16 @@ constexpr size_t SCATTER_SMEM = TILE * sizeof(unsigned long long) + TILE * sizeo
 static_assert(ST >= R && ST % 32 == 0, "one thread per digit in the per-tile scans");
 
 __global__ __launch_bounds__(HT) void k_hist_all(long long n, const unsigned long long *__restrict__ key,
-                                                 uint32_t *__restrict__ hist /* PASSES x R */) {
+                                                 uint32_t *__restrict__ hist /* PASSES x R */,
+                                                 uint32_t *__restrict__ base, DevCtl *ctl) {
     __shared__ uint32_t h[PASSES][R];
     for (int p = 0; p < PASSES; p++) h[p][threadIdx.x] = 0;
     __syncthreads();
-    // the keys of a tree rebuild arrive nearly sorted (the particles are still in the
-    // previous key order), so a warp's 32 neighbouring keys often share their high digits:
-    // such a digit is counted once for the whole warp, the others by one atomic per lane
     for (long long i0 = (long long)blockIdx.x * HT; i0 < n; i0 += (long long)gridDim.x * HT) {
         const long long i = i0 + threadIdx.x;
-        const bool ok = i < n;
-        const unsigned long long k = ok ? key[i] : 0ull;
-        const bool full = __all_sync(0xffffffffu, ok);
-#pragma unroll
-        for (int p = 0; p < PASSES; p++) {
-            const unsigned int d = (unsigned int)((k >> (p * RB)) & (R - 1));
-            const unsigned int d0 = __shfl_sync(0xffffffffu, d, 0);
-            if (full && __all_sync(0xffffffffu, d == d0)) {
-                if ((threadIdx.x & 31) == 0) atomicAdd(&h[p][d], 32u);
-            } else if (ok) {
-                atomicAdd(&h[p][d], 1u);
-            }
-        }
+        gt_count_digits(i < n ? key[i] : 0ull, i < n, h);
     }
-    __syncthreads();
-    for (int p = 0; p < PASSES; p++)
-        if (h[p][threadIdx.x]) atomicAdd(&hist[p * R + threadIdx.x], h[p][threadIdx.x]);
-}
-
-// one block: digit starts of every pass; also resets the tile tickets
-__global__ __launch_bounds__(HT) void k_digit_bases(const uint32_t *__restrict__ hist,
-                                                    uint32_t *__restrict__ base, DevCtl *ctl) {
-    __shared__ uint32_t tmp[HT / 32 + 1];
-    for (int p = 0; p < PASSES; p++) {
-        uint32_t tot;
-        const uint32_t b = block_excl_scan<HT>(hist[p * R + threadIdx.x], &tot, tmp);
-        base[p * R + threadIdx.x] = b;
-    }
-    if (threadIdx.x < PASSES) ctl->sort_ticket[threadIdx.x] = 0;
+    gt_finish_digits(h, hist, base, ctl);
 }
 
 // Look-back of one digit: the count of digit d in all tiles before `tile`.  The status
@@ -132,6 +105,8 @@ __device__ __forceinline__ uint32_t lookback_digit(const uint32_t *status, int t
     return excl;
 }
 
+// INDEX: the values are the keys' positions (vin is not read)
+template <bool INDEX>
 __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int pass,
                                                  const unsigned long long *__restrict__ kin,
                                                  const uint32_t *__restrict__ vin,
@@ -165,7 +140,7 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
     for (int j = 0; j < IPT; j++) {
         const long long i = base + j * 32 + lane;
         k[j] = i < n ? kin[i] : 0ull;
-        v[j] = i < n ? vin[i] : 0u;
+        v[j] = INDEX ? (uint32_t)i : (i < n ? vin[i] : 0u);
     }
     const unsigned int lt = lanemask_lt();
 #pragma unroll
@@ -241,38 +216,51 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
 int gt_sort_tiles(int64_t n) { return (int)((n + TILE - 1) / TILE); }
 
 size_t gt_sort_scratch_bytes(int64_t n) {
-    // look-back status of every pass (PASSES x tiles x R x 4 B)
-    return (size_t)PASSES * R * (size_t)(gt_sort_tiles(n) > 0 ? gt_sort_tiles(n) : 1) * sizeof(uint32_t);
+    // digit counts, and look-back status of every pass (PASSES x tiles x R x 4 B)
+    return (size_t)PASSES * R * (size_t)(1 + (gt_sort_tiles(n) > 0 ? gt_sort_tiles(n) : 1)) * sizeof(uint32_t);
 }
 
 void gt_sort_init() {
-    cudaFuncSetAttribute(k_onesweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+    cudaFuncSetAttribute(k_onesweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+    cudaFuncSetAttribute(k_onesweep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
 }
 
-void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st) {
-    if (n <= 1) return;
+void gt_sort_clear(SortBufs &b, int64_t n, cudaStream_t st) {
+    cudaMemsetAsync(b.hist, 0, (size_t)PASSES * R * (1 + (size_t)gt_sort_tiles(n)) * sizeof(uint32_t), st);
+}
+
+void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, bool counted, cudaStream_t st) {
+    if (n <= 0 || (n == 1 && !counted)) return;
     const int ntiles = gt_sort_tiles(n);
-    cudaMemsetAsync(b.hist, 0, PASSES * R * sizeof(uint32_t), st);
-    cudaMemsetAsync(b.status, 0, (size_t)PASSES * R * ntiles * sizeof(uint32_t), st);
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const long long blocks = (n + HT - 1) / HT;
-    { k_hist_all<<<(unsigned)(blocks < nsm * 8 ? blocks : nsm * 8), HT, 0, st>>>(n, (const unsigned long long *)b.key[0], b.hist); gt_note_launches(1); }
-    { k_digit_bases<<<1, HT, 0, st>>>(b.hist, b.digit_base, ctl); gt_note_launches(1); }
+    if (!counted) {
+        gt_sort_clear(b, n, st);
+        int dev = 0, nsm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        const long long blocks = (n + HT - 1) / HT;
+        k_hist_all<<<(unsigned)(blocks < nsm * 8 ? blocks : nsm * 8), HT, 0, st>>>(n, (const unsigned long long *)b.key[0],
+                                                                                   b.hist, b.digit_base, ctl);
+        gt_note_launches(1);
+    }
     for (int p = 0; p < PASSES; p++) {
         const int src = p & 1, dst = src ^ 1;
-        { k_onesweep<<<ntiles, ST, SCATTER_SMEM, st>>>(n, p, (const unsigned long long *)b.key[src], b.val[src],
-                                                       (unsigned long long *)b.key[dst], b.val[dst], b.digit_base,
-                                                       b.status + (size_t)p * R * ntiles, ntiles, ctl);
-          gt_note_launches(1); }
+        const unsigned long long *kin = (const unsigned long long *)b.key[src];
+        unsigned long long *kout = (unsigned long long *)b.key[dst];
+        uint32_t *status = b.status + (size_t)p * R * ntiles;
+        if (p == 0 && counted)
+            k_onesweep<true><<<ntiles, ST, SCATTER_SMEM, st>>>(n, p, kin, nullptr, kout, b.val[dst], b.digit_base, status,
+                                                               ntiles, ctl);
+        else
+            k_onesweep<false><<<ntiles, ST, SCATTER_SMEM, st>>>(n, p, kin, b.val[src], kout, b.val[dst], b.digit_base,
+                                                                status, ntiles, ctl);
+        gt_note_launches(1);
     }
 }
 
 // ---- sort without allocation (gt_sort_pairs_noalloc) -----------------------------
 // All scratch of one sort of up to GT_NOALLOC_SORT_MAX pairs lives in this array:
-// [control block | alternate keys | alternate values | look-back status | digit
-// histograms | digit bases].  Host code must not use the symbol as an address: the device
+// [control block | alternate keys | alternate values | digit counts | look-back status |
+// digit bases].  Host code must not use the symbol as an address: the device
 // address is looked up once per device below.
 namespace {
 
@@ -281,9 +269,9 @@ constexpr size_t na_up(size_t b) { return (b + NA_ALIGN - 1) / NA_ALIGN * NA_ALI
 constexpr size_t NA_TILES = (GT_NOALLOC_SORT_MAX + TILE - 1) / TILE;
 constexpr size_t NA_OFF_KEY = na_up(sizeof(DevCtl));
 constexpr size_t NA_OFF_VAL = NA_OFF_KEY + na_up((size_t)GT_NOALLOC_SORT_MAX * sizeof(unsigned long long));
-constexpr size_t NA_OFF_STATUS = NA_OFF_VAL + na_up((size_t)GT_NOALLOC_SORT_MAX * sizeof(uint32_t));
-constexpr size_t NA_OFF_HIST = NA_OFF_STATUS + na_up(PASSES * R * NA_TILES * sizeof(uint32_t));
-constexpr size_t NA_OFF_BASE = NA_OFF_HIST + na_up(PASSES * R * sizeof(uint32_t));
+constexpr size_t NA_OFF_HIST = NA_OFF_VAL + na_up((size_t)GT_NOALLOC_SORT_MAX * sizeof(uint32_t));
+constexpr size_t NA_OFF_STATUS = NA_OFF_HIST + PASSES * R * sizeof(uint32_t);
+constexpr size_t NA_OFF_BASE = NA_OFF_STATUS + na_up(PASSES * R * NA_TILES * sizeof(uint32_t));
 constexpr size_t NA_BYTES = NA_OFF_BASE + na_up(PASSES * R * sizeof(uint32_t));
 
 __device__ __align__(256) unsigned char g_noalloc_sort_scratch[NA_BYTES];
@@ -336,7 +324,7 @@ extern "C" int gt_sort_pairs_noalloc(uint64_t *d_keys, uint32_t *d_vals, int64_t
     b.status = (uint32_t *)(base + NA_OFF_STATUS);
     b.hist = (uint32_t *)(base + NA_OFF_HIST);
     b.digit_base = (uint32_t *)(base + NA_OFF_BASE);
-    gt_launch_sort(b, n, ctl, st);  // an even number of passes leaves the result in d_keys/d_vals
+    gt_launch_sort(b, n, ctl, false, st);  // an even number of passes leaves the result in d_keys/d_vals
     return cudaGetLastError() == cudaSuccess ? GT_OK : GT_ECUDA;
 }
 
