@@ -347,6 +347,20 @@ void ph_sync_collect(gt_system *s, cudaStream_t st) {
 
 cudaStream_t S(gt_stream s) { return (cudaStream_t)s; }
 
+// Whether a caller's array can be read or written by a kernel in place of a copy into the system's scratch: memory
+// of this device (or managed), aligned for its elements.  Anything else is copied, as host memory is.
+bool in_place(const void *p, size_t align) {
+    if (!p || (uintptr_t)p % align) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    int dev = -1;
+    return a.type == cudaMemoryTypeManaged ||
+           (a.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && a.device == dev);
+}
+
 // A1-A5 on FP32 positions posm_src (s->posm or the predicted s->posm_tmp): keys, sort,
 // then every particle array gathered into key order.  Buffer roles never change
 // (state 0 and posm always hold the current data), so the launches can be captured
@@ -650,12 +664,16 @@ int gt_set_state(gt_system *s, const double *p_pos, const double *p_vel, const f
     const int64_t n = s->n;
     State &t = s->st[0];
     if (n > 0) {
-        if (cudaMemcpyAsync(s->scratch3, p_pos, (size_t)n * 24, cudaMemcpyDefault, st) != cudaSuccess) return GT_ECUDA;
-        gt_launch_deinterleave3(s->scratch3, n, t.rx, t.ry, t.rz, st);
-        if (cudaMemcpyAsync(s->scratch3, p_vel, (size_t)n * 24, cudaMemcpyDefault, st) != cudaSuccess) return GT_ECUDA;
-        gt_launch_deinterleave3(s->scratch3, n, t.vx, t.vy, t.vz, st);
-        if (cudaMemcpyAsync(t.mass, p_mass, (size_t)n * 4, cudaMemcpyDefault, st) != cudaSuccess) return GT_ECUDA;
-        gt_launch_load(t, s->posm, n, st);
+        if (in_place(p_pos, 8) && in_place(p_vel, 8) && in_place(p_mass, 4)) {
+            gt_launch_load_from(t, s->posm, n, p_pos, p_vel, p_mass, st);
+        } else {
+            if (cudaMemcpyAsync(s->scratch3, p_pos, (size_t)n * 24, cudaMemcpyDefault, st) != cudaSuccess) return GT_ECUDA;
+            gt_launch_deinterleave3(s->scratch3, n, t.rx, t.ry, t.rz, st);
+            if (cudaMemcpyAsync(s->scratch3, p_vel, (size_t)n * 24, cudaMemcpyDefault, st) != cudaSuccess) return GT_ECUDA;
+            gt_launch_deinterleave3(s->scratch3, n, t.vx, t.vy, t.vz, st);
+            if (cudaMemcpyAsync(t.mass, p_mass, (size_t)n * 4, cudaMemcpyDefault, st) != cudaSuccess) return GT_ECUDA;
+            gt_launch_load(t, s->posm, n, st);
+        }
     }
     s->started = false;
     s->have_tree = false;
@@ -798,17 +816,21 @@ int gt_set_integrator_state(gt_system *s, const uint8_t *p_level, const int64_t 
     const int L = s->prm.levels;
     State &t = s->st[0];
     if (n > 0) {
-        // stage the caller-order arrays in scratch (24 B per particle is enough for 1+8+4 B)
-        char *base = (char *)s->scratch3;
-        uint8_t *lv = (uint8_t *)base;
-        long long *t0 = (long long *)(base + ((n + 15) / 16) * 16);
-        float *ao = (float *)(t0 + n);
-        if (cudaMemcpyAsync(lv, p_level, (size_t)n, cudaMemcpyDefault, st) ||
-            cudaMemcpyAsync(t0, p_t0, (size_t)n * 8, cudaMemcpyDefault, st) ||
-            cudaMemcpyAsync(ao, p_aold, (size_t)n * 4, cudaMemcpyDefault, st))
-            return GT_ECUDA;
-        if (p_acc && cudaMemcpyAsync(s->acc_out, p_acc, (size_t)n * 16, cudaMemcpyDefault, st)) return GT_ECUDA;
-        gt_launch_gather_resume(lv, t0, ao, p_acc ? s->acc_out : nullptr, t, n, st);
+        if (in_place(p_level, 1) && in_place(p_t0, 8) && in_place(p_aold, 4) && (!p_acc || in_place(p_acc, 16))) {
+            gt_launch_gather_resume(p_level, (const long long *)p_t0, p_aold, (const float4 *)p_acc, t, n, st);
+        } else {
+            // stage the caller-order arrays in scratch (24 B per particle is enough for 1+8+4 B)
+            char *base = (char *)s->scratch3;
+            uint8_t *lv = (uint8_t *)base;
+            long long *t0 = (long long *)(base + ((n + 15) / 16) * 16);
+            float *ao = (float *)(t0 + n);
+            if (cudaMemcpyAsync(lv, p_level, (size_t)n, cudaMemcpyDefault, st) ||
+                cudaMemcpyAsync(t0, p_t0, (size_t)n * 8, cudaMemcpyDefault, st) ||
+                cudaMemcpyAsync(ao, p_aold, (size_t)n * 4, cudaMemcpyDefault, st))
+                return GT_ECUDA;
+            if (p_acc && cudaMemcpyAsync(s->acc_out, p_acc, (size_t)n * 16, cudaMemcpyDefault, st)) return GT_ECUDA;
+            gt_launch_gather_resume(lv, t0, ao, p_acc ? s->acc_out : nullptr, t, n, st);
+        }
     }
     gt_launch_set_clock(s->ctl, e - 1, L, T, st);
     gt_launch_tnext_all(t, n, L, s->ctl, s->nsm, st);
@@ -913,13 +935,13 @@ int gt_get_state(gt_system *s, double *p_pos, double *p_vel, float *p_mass, floa
     const int64_t n = s->n;
     if (n == 0) return GT_OK;
     const State &t = s->st[0];
-    if (p_pos) {
-        gt_launch_interleave3(t.rx, t.ry, t.rz, n, s->scratch3, st);
-        if (cudaMemcpyAsync(p_pos, s->scratch3, (size_t)n * 24, cudaMemcpyDefault, st)) return GT_ECUDA;
-    }
-    if (p_vel) {
-        gt_launch_interleave3(t.vx, t.vy, t.vz, n, s->scratch3, st);
-        if (cudaMemcpyAsync(p_vel, s->scratch3, (size_t)n * 24, cudaMemcpyDefault, st)) return GT_ECUDA;
+    const double *from[2][3] = {{t.rx, t.ry, t.rz}, {t.vx, t.vy, t.vz}};
+    double *to[2] = {p_pos, p_vel};
+    for (int k = 0; k < 2; k++) {
+        if (!to[k]) continue;
+        const bool direct = in_place(to[k], 8);
+        gt_launch_interleave3(from[k][0], from[k][1], from[k][2], n, direct ? to[k] : s->scratch3, st);
+        if (!direct && cudaMemcpyAsync(to[k], s->scratch3, (size_t)n * 24, cudaMemcpyDefault, st)) return GT_ECUDA;
     }
     if (p_mass && cudaMemcpyAsync(p_mass, t.mass, (size_t)n * 4, cudaMemcpyDefault, st)) return GT_ECUDA;
     if (p_acc && cudaMemcpyAsync(p_acc, t.acc, (size_t)n * 16, cudaMemcpyDefault, st)) return GT_ECUDA;

@@ -298,6 +298,9 @@ struct StepMirror {
 };
 void gt_launch_mirror(const DevCtl *ctl, StepMirror *dst, cudaStream_t st);
 void gt_launch_load(const State &s, float4 *posm, int64_t n, cudaStream_t st);
+// the same from the caller's n x 3 positions and velocities and n masses in device memory
+void gt_launch_load_from(const State &s, float4 *posm, int64_t n, const double *pos, const double *vel,
+                         const float *mass, cudaStream_t st);
 void gt_launch_permute(const State &src, const State &dst, const float4 *posm_in, float4 *posm_out,
                        const uint32_t *perm, int64_t n, cudaStream_t st);
 void gt_launch_copy_state(const State &src, const State &dst, const float4 *posm_in, float4 *posm_out,
