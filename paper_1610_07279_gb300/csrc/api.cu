@@ -501,6 +501,7 @@ WalkArgs gt_sys_walk_args(const gt_system *s, const uint32_t *active, const floa
     a.eps2 = s->prm.eps * s->prm.eps;
     a.G = s->prm.G;
     a.inv_eps = 1.0f / s->prm.eps;
+    a.inv_c2 = levels ? (float)(1.0 / c2_of(s->prm)) : 0.0f;
     return a;
 }
 
@@ -513,7 +514,6 @@ void gt_sys_step_pre(gt_system *s, cudaStream_t st, bool rebuild, bool predicted
         ph_begin(s, PH_PREDICT, st);
         gt_launch_predict(s->st[0], n, s->ctl, rebuild ? s->posm_tmp : s->posm, st);
         ph_end(s, PH_PREDICT, st);
-    a.inv_c2 = levels ? (float)(1.0 / c2_of(s->prm)) : 0.0f;
     } else if (!rebuild) {
         std::swap(s->posm, s->posm_tmp);  // the prediction enqueued ahead went to posm_tmp
     }

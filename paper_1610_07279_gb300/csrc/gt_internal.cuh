@@ -99,6 +99,9 @@ struct Nodes {
 };
 
 __device__ __forceinline__ void gt_set_error(DevCtl *ctl, int code, int where) {
+    if (atomicCAS(&ctl->err, 0, code) == 0) ctl->err_where = where;
+}
+
 // FP32 values as unsigned integers in the same order (for atomic minima and maxima), and back.
 __device__ __forceinline__ unsigned int gt_ordered(float f) {
     const unsigned int b = __float_as_uint(f);
@@ -106,9 +109,6 @@ __device__ __forceinline__ unsigned int gt_ordered(float f) {
 }
 __device__ __forceinline__ float gt_unordered(unsigned int u) {
     return __uint_as_float(u >> 31 ? u & 0x7fffffffu : ~u);
-}
-
-    if (atomicCAS(&ctl->err, 0, code) == 0) ctl->err_where = where;
 }
 
 __device__ __forceinline__ unsigned int lane_id() { return threadIdx.x & 31u; }
@@ -350,13 +350,13 @@ struct WalkArgs {
     int ij_share;            // lanes per i-particle; 0: 32 / (members rounded up to a power of two)
     int sphere;              // pseudo i-particle: 0 GEO centre, 1 Ritter's efficient bounding sphere
     float theta, delta_acc, eps2, G, inv_eps;
+    float inv_c2;            // block steps: 1 / (2 eta eps)^2, the scale of the levels' thresholds; otherwise 0
 };
 // A warp's cell queue: a ring of (first child, number of children) pairs, one for every opened cell.
 // walk_queue bounds the cells in it; from 8 x pairs > walk_queue - (the depth-first reserve) on the
 // newest pairs are taken first, which keeps at most ~700 more, so half as many pairs as cells (and
 // 1024 for the smallest queues) hold every walk that walk_queue admits.
 __host__ __device__ inline uint32_t gt_queue_ring(int qcap) { return qcap >= 2048 ? (uint32_t)qcap / 2u : 1024u; }
-    float inv_c2;            // block steps: 1 / (2 eta eps)^2, the scale of the levels' thresholds; otherwise 0
 __host__ __device__ inline size_t gt_queue_words(int qcap) { return 2 * (size_t)gt_queue_ring(qcap); }
 int gt_walk_blocks(int nsm);
 // tuner.cu
