@@ -56,6 +56,7 @@ struct DevCtl {
     int levels_m1;                    // L - 1 (finest level)
     unsigned int bbox[6];             // extrema of the positions (gt_ordered): minima, then maxima
     unsigned int digits_done;         // blocks that have added their digit counts (the sort)
+    unsigned int scan_done, cells_done;  // the same for the octree's tile scan and the cell list's counts
     unsigned int spin_limit;          // bound on every spin-wait of this system; 0: GT_SPIN_LIMIT
 };
 

@@ -25,11 +25,16 @@
 
 namespace {
 
-__global__ void k_prepare(DevCtl *ctl, int begin_step) {
+__global__ void k_prepare(DevCtl *ctl, int begin_step) {  // one warp
+    static_assert(GT_TREE_LEVELS + 4 <= 32, "a lane per ticket");
+    const int l = threadIdx.x;
+    if (l < GT_TREE_LEVELS + 4) ctl->tile_ticket[l] = 0;
+    if (l < GT_TREE_LEVELS) ctl->pl_done[l] = 0;
+    if (l < 6) ctl->bbox[l] = gt_ordered(l < 3 ? FLT_MAX : -FLT_MAX);
+    if (l != 0) return;
     ctl->epoch += 1u;
-    for (int l = 0; l < GT_TREE_LEVELS + 4; l++) ctl->tile_ticket[l] = 0;
     ctl->group_next = 0;
-    for (int a = 0; a < 6; a++) ctl->bbox[a] = gt_ordered(a < 3 ? FLT_MAX : -FLT_MAX);
+    ctl->pl_ticket = 0;
     if (begin_step) {
         ctl->tnext = ctl->tnext_acc;
         ctl->tnext_acc = ~0ull;
@@ -530,7 +535,7 @@ inline unsigned nblk(long long n) { return (unsigned)((n + 255) / 256); }
 }  // namespace
 
 void gt_launch_prepare(DevCtl *ctl, int begin_step, cudaStream_t st) {
-    { k_prepare<<<1, 1, 0, st>>>(ctl, begin_step); gt_note_launches(1); }
+    { k_prepare<<<1, 32, 0, st>>>(ctl, begin_step); gt_note_launches(1); }
 }
 
 void gt_launch_set_nactive(DevCtl *ctl, unsigned int n_active, cudaStream_t st) {

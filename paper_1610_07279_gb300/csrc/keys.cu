@@ -14,9 +14,9 @@
 namespace {
 
 constexpr int BBOX_THREADS = 256;
-#ifndef GT_KEYS_BLOCKS
-#define GT_KEYS_BLOCKS 8  // blocks per SM of the key pass
-#endif
+// Blocks per SM of the key pass: every block adds up to 2048 counts to the global ones, which below ~2^22 keys costs
+// more than the warps hide (2^20: 407 us the whole build at 4, 413 at 8; 2^24: 3009 and 3001).
+constexpr int64_t KEYS_MANY = 1 << 22;
 
 __global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict__ posm, long long n, DevCtl *ctl) {
     float mn0 = FLT_MAX, mn1 = FLT_MAX, mn2 = FLT_MAX;
@@ -158,7 +158,7 @@ void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, cudaSt
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st) {
     if (n <= 0) return;
     gt_sort_clear(b, n, st);
-    const int64_t need = (n + 255) / 256, most = (int64_t)nsm * GT_KEYS_BLOCKS;
+    const int64_t need = (n + 255) / 256, most = (int64_t)nsm * (n < KEYS_MANY ? 4 : 8);
     k_keys<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(posm, n, curve, ctl, (unsigned long long *)b.key[0],
                                                                   b.hist, b.digit_base);
     gt_note_launches(1);

@@ -8,12 +8,16 @@
 // still in the previous key order), so a warp's 32 neighbouring keys often share their high digits: such a digit
 // is counted once for the whole warp, the others by one atomic per lane.
 __device__ __forceinline__ void gt_count_digits(unsigned long long k, bool ok, uint32_t (*h)[GT_SORT_DIGITS]) {
-    const bool full = __all_sync(0xffffffffu, ok);
+    const uint32_t lo = (uint32_t)k, hi = (uint32_t)(k >> 32);
+    // bits in which some lane's key differs from the first one's (a lane without a key: all)
+    const uint32_t lo0 = __shfl_sync(0xffffffffu, lo, 0), hi0 = __shfl_sync(0xffffffffu, hi, 0);
+    const uint32_t dlo = __reduce_or_sync(0xffffffffu, ok ? lo ^ lo0 : ~0u);
+    const uint32_t dhi = __reduce_or_sync(0xffffffffu, ok ? hi ^ hi0 : ~0u);
+    static_assert(GT_SORT_BITS == 8 && GT_SORT_PASSES == 8, "a byte per digit");
 #pragma unroll
     for (int p = 0; p < GT_SORT_PASSES; p++) {
-        const unsigned int d = (unsigned int)(k >> (p * GT_SORT_BITS)) & (GT_SORT_DIGITS - 1);
-        const unsigned int d0 = __shfl_sync(0xffffffffu, d, 0);
-        if (full && __all_sync(0xffffffffu, d == d0)) {
+        const uint32_t word = p < 4 ? lo : hi, d = (word >> (8 * (p & 3))) & 0xffu;
+        if ((((p < 4 ? dlo : dhi) >> (8 * (p & 3))) & 0xffu) == 0u) {
             if ((threadIdx.x & 31) == 0) atomicAdd(&h[p][d], 32u);
         } else if (ok) {
             atomicAdd(&h[p][d], 1u);

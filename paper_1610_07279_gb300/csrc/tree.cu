@@ -30,6 +30,8 @@ constexpr int NPT = 1;          // cells per thread
 constexpr int BTILE = BT * NPT; // cells per tile
 
 __global__ void k_build_init(long long n, Nodes nd, DevCtl *ctl) {
+    for (int b = threadIdx.x; b < GT_CELL_BUCKETS; b += blockDim.x) ctl->cell_bucket[b] = 0;
+    if (threadIdx.x != 0) return;
     // root = level 0, all particles; level_start[0..1]
     ctl->level_start[0] = 0;
     ctl->level_start[1] = n > 0 ? 1u : 0u;
@@ -159,8 +161,13 @@ __global__ __launch_bounds__(BT) void k_build_level(int lvl, const unsigned long
 // first particle.  A node's first child starts at its own first particle; the others
 // are the next nodes of the child level that start before its end.
 constexpr int FLAT_LWIN = 64;              // the largest leaf_max of this build
-constexpr int FT = 2048;                   // particles per tile
 constexpr int FB = 256;                    // threads per block
+// Particles per tile: a block takes its tile's rounds of FB particles one after another, so that small systems,
+// which fill few blocks, get short tiles (8192 particles: k_flat_scatter 15.6 us with 8 rounds).
+#ifndef GT_FLAT_SMALL
+#define GT_FLAT_SMALL (1 << 21)            // systems up to this size take tiles of two rounds, larger ones of eight
+#endif
+int flat_rounds(int64_t n) { return n <= GT_FLAT_SMALL ? 2 : 8; }
 constexpr int NREC = 2 * GT_TREE_LEVELS;   // start and end counters per level
 
 __device__ __forceinline__ int key_diff_digit(unsigned long long a, unsigned long long b) {
@@ -193,11 +200,11 @@ __device__ __forceinline__ int leaf_level_of(const int8_t *ds, int j) {
 // d and the leaf level of every particle (packed (d + 1) | leaf << 8), and every tile's
 // start and end counts per level (column-major: counter k of tile t at cnt[k * ntiles + t]).
 // MT > 0: leaf_max == MT; MT == 0: any leaf_max up to FLAT_LWIN (running minima in shared memory).
-template <int MT>
+template <int MT, int ROUNDS>
 __global__ __launch_bounds__(FB) void k_flat_marks(const unsigned long long *__restrict__ skey, long long n,
                                                    int M, uint16_t *__restrict__ dl,
                                                    uint32_t *__restrict__ cnt, int ntiles) {
-    constexpr int W = FLAT_LWIN;
+    constexpr int W = FLAT_LWIN, FT = ROUNDS * FB;
     constexpr int MW = MT > 0 ? 1 : W;
     __shared__ int8_t ds[FT + 2 * W + 1];      // d of positions base - W .. base + FT + W
     __shared__ uint8_t mr[MW][FB];             // generic: 1 + smallest d over (i, i + b]
@@ -209,7 +216,7 @@ __global__ __launch_bounds__(FB) void k_flat_marks(const unsigned long long *__r
     }
     for (int j = threadIdx.x; j < NREC; j += FB) c[j] = 0;
     __syncthreads();
-    for (int r = 0; r < FT / FB; r++) {
+    for (int r = 0; r < ROUNDS; r++) {
         const int t = r * FB + threadIdx.x;
         const long long i = base + t;
         if (i >= n) break;
@@ -239,9 +246,25 @@ __global__ __launch_bounds__(FB) void k_flat_marks(const unsigned long long *__r
     for (int k = threadIdx.x; k < NREC; k += FB) cnt[(size_t)k * ntiles + blockIdx.x] = c[k];
 }
 
-// one block per counter: exclusive scan over the tiles, the column total into tot[k]
-__global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, int ntiles,
-                                                    uint32_t *__restrict__ tot) {
+// The last block of a kernel to come here gets true (its threads see what the others wrote before); *done starts at
+// zero and is left at zero.
+__device__ __forceinline__ bool last_block(unsigned int *done) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(done, 1u) == gridDim.x - 1u;
+        if (last) *done = 0u;
+    }
+    __syncthreads();
+    __threadfence();
+    return last;
+}
+
+// one block per counter: exclusive scan over the tiles, the column total into tot[k]; the last block then sets the
+// level starts from the per-level node counts (clamped to the node capacity) and clears the cell list's counters
+__global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, int ntiles, uint32_t *__restrict__ tot,
+                                                    long long cap, DevCtl *ctl) {
     __shared__ unsigned int tmp[1024 / 32 + 1];
     uint32_t *col = cnt + (size_t)blockIdx.x * ntiles;
     unsigned int carry = 0;
@@ -254,28 +277,29 @@ __global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, 
         carry += total;
     }
     if (threadIdx.x == 0) tot[blockIdx.x] = carry;
-}
-
-// level starts from the per-level node counts (clamped to the node capacity)
-__global__ void k_flat_levels(const uint32_t *__restrict__ tot, long long cap, DevCtl *ctl) {
-    unsigned long long s = 0;
-    for (int l = 0; l < GT_TREE_LEVELS; l++) {
-        ctl->level_start[l] = (uint32_t)(s < (unsigned long long)cap ? s : (unsigned long long)cap);
-        s += tot[l];
+    if (!last_block(&ctl->scan_done)) return;
+    for (int b = threadIdx.x; b < GT_CELL_BUCKETS; b += 1024) ctl->cell_bucket[b] = 0;
+    if (threadIdx.x >= 32) return;
+    const int l = threadIdx.x;
+    unsigned long long sum = l < GT_TREE_LEVELS ? __ldcg(&tot[l]) : 0ull;
+    const unsigned long long own = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(0xffffffffu, sum, o);
+        if (l >= o) sum += t;
     }
-    if (s > (unsigned long long)cap) {
-        gt_set_error(ctl, GT_EOVERFLOW, GTK_BUILD);
-        s = (unsigned long long)cap;
-    }
-    ctl->level_start[GT_TREE_LEVELS] = (uint32_t)s;
-    ctl->level_start[GT_TREE_LEVELS + 1] = (uint32_t)s;
+    const unsigned long long most = (unsigned long long)cap, before = l < GT_TREE_LEVELS ? sum - own : sum;
+    if (l < GT_TREE_LEVELS + 2) ctl->level_start[l] = (uint32_t)(before < most ? before : most);
+    if (l == GT_TREE_LEVELS && sum > most) gt_set_error(ctl, GT_EOVERFLOW, GTK_BUILD);
 }
 
 // every start and end to its node: first, the first child and the parent along a
 // particle's own chain of starts, leaves; an end goes to count (as the end position)
+template <int ROUNDS>
 __global__ __launch_bounds__(FB) void k_flat_scatter(const uint16_t *__restrict__ dl, long long n,
                                                      const uint32_t *__restrict__ cnt, int ntiles,
                                                      long long cap, Nodes nd, const DevCtl *__restrict__ ctl) {
+    constexpr int FT = ROUNDS * FB;
     __shared__ uint32_t lb[GT_TREE_LEVELS];
     __shared__ uint32_t run[NREC];
     __shared__ uint32_t wc[FB / 32][NREC];
@@ -287,7 +311,7 @@ __global__ __launch_bounds__(FB) void k_flat_scatter(const uint16_t *__restrict_
     __syncthreads();
     const int w = threadIdx.x >> 5;
     const unsigned int lt = lanemask_lt();
-    for (int r = 0; r < FT / FB; r++) {
+    for (int r = 0; r < ROUNDS; r++) {
         const int t = r * FB + threadIdx.x;
         const long long i = base + t;
         const bool valid = i < n;
@@ -416,29 +440,35 @@ __global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, Dev
     __syncthreads();
     for (int i = threadIdx.x; i < GT_CELL_BUCKETS; i += 256)
         if (h[i]) atomicAdd(&ctl->cell_bucket[i], h[i]);
-}
-
-// one block: bucket sizes -> fill cursors, and where every level's leaves and cells
-// with children start
-__global__ __launch_bounds__(1024) void k_cell_scan(DevCtl *ctl) {
-    static_assert(GT_CELL_BUCKETS <= 1024, "one thread per bucket");
-    __shared__ unsigned int tmp[1024 / 32 + 1];
-    const int b = threadIdx.x;
-    const uint32_t v = b < GT_CELL_BUCKETS ? ctl->cell_bucket[b] : 0u;
-    uint32_t total;
-    const uint32_t start = block_excl_scan<1024>(v, &total, tmp);
-    if (b < GT_CELL_BUCKETS) {
-        ctl->cell_bucket[b] = start;
-        const int q = b % GT_LEVEL_BUCKETS;
-        if (q == 0) ctl->seg[2 * (b / GT_LEVEL_BUCKETS)] = start;
-        if (q == GT_LEAF_BUCKETS) ctl->seg[2 * (b / GT_LEVEL_BUCKETS) + 1] = start;
+    if (!last_block(&ctl->cells_done)) return;
+    // bucket sizes -> fill cursors, and where every level's leaves and cells with children start
+    constexpr int PER = (GT_CELL_BUCKETS + 255) / 256;  // neighbouring buckets of a thread
+    __shared__ unsigned int tmp[256 / 32 + 1];
+    uint32_t v[PER], sum = 0, total;
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+        const int b = PER * (int)threadIdx.x + j;
+        v[j] = b < GT_CELL_BUCKETS ? __ldcg(&ctl->cell_bucket[b]) : 0u;
+        sum += v[j];
     }
-    if (b == 0) ctl->seg[2 * GT_TREE_LEVELS] = total;
+    uint32_t start = block_excl_scan<256>(sum, &total, tmp);
+#pragma unroll
+    for (int j = 0; j < PER; j++) {
+        const int b = PER * (int)threadIdx.x + j;
+        if (b < GT_CELL_BUCKETS) {
+            ctl->cell_bucket[b] = start;
+            const int q = b % GT_LEVEL_BUCKETS;
+            if (q == 0) ctl->seg[2 * (b / GT_LEVEL_BUCKETS)] = start;
+            if (q == GT_LEAF_BUCKETS) ctl->seg[2 * (b / GT_LEVEL_BUCKETS) + 1] = start;
+        }
+        start += v[j];
+    }
+    if (threadIdx.x == 0) ctl->seg[2 * GT_TREE_LEVELS] = total;
 }
 
 // A block takes a contiguous range of nodes, counts them per bucket in shared memory,
 // reserves its room in every bucket with one global atomic each, and fills it.
-constexpr int CF_NODES = 4096;  // nodes per fill block
+constexpr int CF_NODES = 4096;  // most nodes of such a range; small trees take shorter ones, so that every block has one
 
 __global__ __launch_bounds__(256) void k_cell_fill(Nodes nd, long long cap, DevCtl *ctl) {
     __shared__ uint32_t ls[GT_TREE_LEVELS + 1];
@@ -446,11 +476,13 @@ __global__ __launch_bounds__(256) void k_cell_fill(Nodes nd, long long cap, DevC
     for (int i = threadIdx.x; i <= GT_TREE_LEVELS; i += 256) ls[i] = ctl->level_start[i];
     long long nn = ctl->level_start[GT_TREE_LEVELS];
     if (nn > cap) nn = cap;
-    for (long long b0 = (long long)blockIdx.x * CF_NODES; b0 < nn; b0 += (long long)gridDim.x * CF_NODES) {
+    const long long share = ((nn + gridDim.x - 1) / gridDim.x + 255) / 256 * 256;
+    const long long chunk = share < CF_NODES ? share : CF_NODES;
+    for (long long b0 = (long long)blockIdx.x * chunk; b0 < nn; b0 += (long long)gridDim.x * chunk) {
         __syncthreads();
         for (int i = threadIdx.x; i < GT_CELL_BUCKETS; i += 256) h[i] = 0;
         __syncthreads();
-        const long long b1 = b0 + CF_NODES < nn ? b0 + CF_NODES : nn;
+        const long long b1 = b0 + chunk < nn ? b0 + chunk : nn;
         for (long long p = b0 + threadIdx.x; p < b1; p += 256)
             atomicAdd(&h[cell_bucket_of(nd, (uint32_t)p, ls)], 1u);
         __syncthreads();
@@ -543,15 +575,27 @@ __device__ __forceinline__ void pseudo_leaf(const Nodes &nd, const float4 *__res
                              __uint_as_float(k | GT_LEAF_FLAG), b2);
 }
 
+// What a cell's lane reads of the cell itself, before it waits for the level below.
+struct CellInfo {
+    uint32_t p, nch;
+    int32_t ch0;
+    double m;  // the stored mass (WITH_MASS: 0, it is summed)
+};
+
+template <bool WITH_MASS>
+__device__ __forceinline__ CellInfo cell_info(const Nodes &nd, uint32_t p) {
+    return CellInfo{p, nd.nchild[p], nd.child[p], WITH_MASS ? 0.0 : nd.sum[p].m};
+}
+
 // Cell p with children: its children's FP64 sums added in child order.  The children
 // were written by other blocks of this launch: they are read through L2 (__ldcg), an
 // SM's L1 may hold a line of them from before they were written.  Loads go out four
 // children at a time, so a level costs few L2 round trips.
 template <bool WITH_MASS>
-__device__ __forceinline__ void pseudo_cell(const Nodes &nd, uint32_t p) {
-    const int32_t ch0 = nd.child[p];
-    const uint32_t nch = nd.nchild[p];
-    double m = WITH_MASS ? 0.0 : nd.sum[p].m, sx = 0.0, sy = 0.0, sz = 0.0;
+__device__ __forceinline__ void pseudo_cell(const Nodes &nd, const CellInfo &ci) {
+    const uint32_t p = ci.p, nch = ci.nch;
+    const int32_t ch0 = ci.ch0;
+    double m = ci.m, sx = 0.0, sy = 0.0, sz = 0.0;
     for (uint32_t q0 = 0; q0 < nch; q0 += CU) {
         double2 s0[CU], s1[CU];  // (m, x), (y, z)
 #pragma unroll
@@ -600,17 +644,17 @@ __device__ __forceinline__ void pseudo_cell(const Nodes &nd, uint32_t p) {
 
 // The same cell with eight lanes, one child each (lanes 8g .. 8g + 7 of the warp hold cell
 // g of four): the children's records arrive in one round of loads instead of one per
-// pair of children.  Every lane of the group forms the FP64 sums and the B_2 sum itself,
-// in child order, from its neighbours' values (shuffles), so the operations and their
+// pair of children.  The FP64 sums and the B_2 sum are formed in child order from the lanes'
+// values (shuffles), so the operations and their
 // order are those of pseudo_cell; the radius is a maximum, taken across the lanes.  For
 // the levels near the root, whose few cells each wait for the level below.  Every lane
 // of the warp must call it; `valid` marks groups that own a cell.
 template <bool WITH_MASS>
-__device__ __forceinline__ void pseudo_cell_coop(const Nodes &nd, uint32_t p, bool valid) {
+__device__ __forceinline__ void pseudo_cell_coop(const Nodes &nd, const CellInfo &ci, bool valid) {
+    const uint32_t p = ci.p, nch = ci.nch;
+    const int32_t ch0 = ci.ch0;
     const unsigned FULL = 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31u, j = lane & 7u, g0 = lane & ~7u;
-    const int32_t ch0 = valid ? nd.child[p] : 0;
-    const uint32_t nch = valid ? nd.nchild[p] : 0u;
     const bool has = j < nch;
     double2 s0 = make_double2(0.0, 0.0), s1 = make_double2(0.0, 0.0);  // (m, x), (y, z)
     float4 cj = make_float4(0.f, 0.f, 0.f, 0.f), cw = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -621,22 +665,22 @@ __device__ __forceinline__ void pseudo_cell_coop(const Nodes &nd, uint32_t p, bo
         cj = __ldcg(&nd.jpos[ch0 + j]);
         cw = __ldcg(&nd.walk[ch0 + j]);
     }
-    double m = (WITH_MASS || !valid) ? 0.0 : nd.sum[p].m, sx = 0.0, sy = 0.0, sz = 0.0;
+    // lanes 0 to 3 of the group sum a component each (the FP64 unit takes 16 cycles per warp instruction, so that the
+    // four sums on every lane were half of a level's time)
+    double acc = j == 0 ? ci.m : 0.0;
 #pragma unroll
     for (uint32_t q = 0; q < 8; q++) {
         const double cm = __shfl_sync(FULL, s0.x, g0 + q), cx = __shfl_sync(FULL, s0.y, g0 + q);
         const double cy = __shfl_sync(FULL, s1.x, g0 + q), cz = __shfl_sync(FULL, s1.y, g0 + q);
-        if (q < nch) {
-            if (WITH_MASS) m = __dadd_rn(m, cm);
-            sx = __dadd_rn(sx, cx);
-            sy = __dadd_rn(sy, cy);
-            sz = __dadd_rn(sz, cz);
-        }
+        const double c = j == 0 ? cm : (j == 1 ? cx : (j == 2 ? cy : cz));
+        if (q < nch && (WITH_MASS || j != 0)) acc = __dadd_rn(acc, c);
     }
-    const float mf = d2f(m);
-    const float jx = __fdiv_rn(d2f(sx), mf);
-    const float jy = __fdiv_rn(d2f(sy), mf);
-    const float jz = __fdiv_rn(d2f(sz), mf);
+    const float af = d2f(acc), mf = __shfl_sync(FULL, af, g0);
+    const float jf = __fdiv_rn(af, mf);
+    const float jx = __shfl_sync(FULL, jf, g0 + 1), jy = __shfl_sync(FULL, jf, g0 + 2),
+                jz = __shfl_sync(FULL, jf, g0 + 3);
+    const double m = __shfl_sync(FULL, acc, g0), sx = __shfl_sync(FULL, acc, g0 + 1),
+                 sy = __shfl_sync(FULL, acc, g0 + 2), sz = __shfl_sync(FULL, acc, g0 + 3);
     const float d2 = sq3f(__fsub_rn(cj.x, jx), __fsub_rn(cj.y, jy), __fsub_rn(cj.z, jz));
     float b = 0.0f;
     if (has) {
@@ -700,33 +744,23 @@ __global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const f
     __syncthreads();
     const uint32_t total = ocum[NSEG];
     for (;;) {
-        if (threadIdx.x == 0) {
-            const unsigned int t = atomicAdd(&ctl->pl_ticket, 1u);
-            int o = 0;
-            if (t < total)
-                while (ocum[o + 1] <= t) o++;
-            t_sh = t;
-            o_sh = o;
-            if (t < total && ocell[o] == 1 && olvl[o] + 1 < GT_TREE_LEVELS) {
-                const int l1 = olvl[o] + 1;  // every chunk of that level first
-                const unsigned int need = nchunk[2 * l1] + nchunk[2 * l1 + 1];
-                unsigned int spins = 0;
-                const unsigned int limit = gt_spin_limit(ctl);
-                while (*((volatile unsigned int *)&ctl->pl_done[l1]) < need) {
-                    if (++spins > limit) {
-                        gt_set_error(ctl, GT_ETIMEOUT, GTK_PSEUDO);
-                        bad_sh = 1;
-                        break;
-                    }
-                    __nanosleep(64);
-                }
-                __threadfence();
+        if (threadIdx.x < 32) {
+            unsigned int t = 0;
+            if (threadIdx.x == 0) t = atomicAdd(&ctl->pl_ticket, 1u);
+            t = __shfl_sync(0xffffffffu, t, 0);
+            // the last entry that begins at or before t
+            static_assert(NSEG <= 64, "two entries per lane");
+            int o = __popc(__ballot_sync(0xffffffffu, ocum[threadIdx.x + 1] <= t));
+            o += __popc(__ballot_sync(0xffffffffu, threadIdx.x + 33 <= NSEG && ocum[min(threadIdx.x + 33u, (uint32_t)NSEG)] <= t));
+            if (threadIdx.x == 0) {
+                t_sh = t;
+                o_sh = o < NSEG ? o : NSEG - 1;
             }
         }
         __syncthreads();
         const unsigned int t = t_sh;
         const int o = o_sh;
-        if (t >= total || bad_sh) break;
+        if (t >= total) break;
         const int lvl = olvl[o], kind = ocell[o], sg = 2 * lvl + kind;
 #if GT_DEBUG
         {   // every node of the chunk: its particle or child range inside the tree
@@ -749,20 +783,40 @@ __global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const f
             }
         }
 #endif
-        if (coop[sg]) {  // the whole block: PL / 8 cells, eight lanes each
-            const long long idx = (long long)seg[sg] + (long long)(t - ocum[o]) * (PL / 8) + (threadIdx.x >> 3);
-            const bool valid = idx < (long long)seg[sg + 1];
-            pseudo_cell_coop<WITH_MASS>(nd, valid ? nd.cells[idx] : 0u, valid);
+        const uint32_t per = coop[sg] ? PL / 8 : PL;  // coop: eight lanes each
+        const long long idx = (long long)seg[sg] + (long long)(t - ocum[o]) * per + (coop[sg] ? threadIdx.x >> 3 : threadIdx.x);
+        const bool valid = idx < (long long)seg[sg + 1];
+        const uint32_t node = valid ? nd.cells[idx] : 0u;
+        if (kind == 0) {
+            if (valid) pseudo_leaf<WITH_MASS>(nd, posm, node);
         } else {
-            const long long idx = (long long)seg[sg] + (long long)(t - ocum[o]) * PL + threadIdx.x;
-            if (idx < (long long)seg[sg + 1]) {
-                if (kind == 0) pseudo_leaf<WITH_MASS>(nd, posm, nd.cells[idx]);
-                else pseudo_cell<WITH_MASS>(nd, nd.cells[idx]);
+            CellInfo ci{0u, 0u, 0, 0.0};
+            if (valid) ci = cell_info<WITH_MASS>(nd, node);
+            if (threadIdx.x == 0 && lvl + 1 < GT_TREE_LEVELS) {
+                const int l1 = lvl + 1;  // every chunk of that level first
+                const unsigned int need = nchunk[2 * l1] + nchunk[2 * l1 + 1];
+                unsigned int spins = 0;
+                const unsigned int limit = gt_spin_limit(ctl);
+                while (*((volatile unsigned int *)&ctl->pl_done[l1]) < need) {
+                    if (++spins > limit) {
+                        gt_set_error(ctl, GT_ETIMEOUT, GTK_PSEUDO);
+                        bad_sh = 1;
+                        break;
+                    }
+                    __nanosleep(20);
+                }
+                __threadfence();
             }
+            __syncthreads();
+            if (bad_sh) break;
+            if (coop[sg]) pseudo_cell_coop<WITH_MASS>(nd, ci, valid);
+            else if (valid) pseudo_cell<WITH_MASS>(nd, ci);
         }
-        __threadfence();  // every thread's node is visible device-wide before the chunk counts as done
         __syncthreads();
-        if (threadIdx.x == 0) atomicAdd(&ctl->pl_done[lvl], 1u);
+        if (threadIdx.x == 0) {  // the block's nodes are visible device-wide before the chunk counts as done
+            __threadfence();
+            atomicAdd(&ctl->pl_done[lvl], 1u);
+        }
     }
 }
 
@@ -770,56 +824,64 @@ __global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const f
 
 size_t gt_build_scratch_bytes(int64_t n) {
     const size_t N = (size_t)(n > 0 ? n : 1);
-    const size_t tiles = (N + FT - 1) / FT;
+    const size_t FT = (size_t)flat_rounds(n) * FB, tiles = (N + FT - 1) / FT;
     return (2 * N + 15) / 16 * 16 + 4 * (size_t)NREC * (tiles + 1);
 }
+
+namespace {
+
+template <int ROUNDS>
+void launch_flat(const unsigned long long *k, int64_t n, int leaf_max, Nodes nd, int64_t cap, uint8_t *scratch,
+                 DevCtl *ctl, int nsm, cudaStream_t st) {
+    constexpr int FT = ROUNDS * FB;
+    const int ntiles = (int)((n + FT - 1) / FT);
+    uint16_t *dl = (uint16_t *)scratch;
+    uint32_t *cnt = (uint32_t *)(scratch + (2 * (size_t)(n > 0 ? n : 1) + 15) / 16 * 16);
+    uint32_t *tot = cnt + (size_t)NREC * ntiles;
+    if (ntiles > 0) {
+        auto marks = k_flat_marks<0, ROUNDS>;
+        switch (leaf_max) {
+        case 4: marks = k_flat_marks<4, ROUNDS>; break;
+        case 8: marks = k_flat_marks<8, ROUNDS>; break;
+        case 16: marks = k_flat_marks<16, ROUNDS>; break;
+        case 24: marks = k_flat_marks<24, ROUNDS>; break;
+        case 32: marks = k_flat_marks<32, ROUNDS>; break;
+        }
+        marks<<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles);
+        gt_note_launches(1);
+    }
+    { k_flat_scan<<<NREC, 1024, 0, st>>>(cnt, ntiles, tot, cap, ctl); gt_note_launches(1); }
+    if (ntiles > 0) {
+        k_flat_scatter<ROUNDS><<<ntiles, FB, 0, st>>>(dl, n, cnt, ntiles, cap, nd, ctl);
+        { k_flat_link<<<nsm * 8, 256, 0, st>>>(nd, cap, ctl); }
+        gt_note_launches(2);
+    }
+}
+
+}  // namespace
 
 void gt_launch_build(const uint64_t *skey, int64_t n, int leaf_max, Nodes nd, int64_t cap,
                      unsigned long long *status, uint8_t *scratch, DevCtl *ctl, int nsm, cudaStream_t st) {
     if (leaf_max <= FLAT_LWIN) {
-        const int ntiles = (int)((n + FT - 1) / FT);
-        uint16_t *dl = (uint16_t *)scratch;
-        uint32_t *cnt = (uint32_t *)(scratch + (2 * (size_t)(n > 0 ? n : 1) + 15) / 16 * 16);
-        uint32_t *tot = cnt + (size_t)NREC * ntiles;
-        if (ntiles > 0) {
-            const unsigned long long *k = (const unsigned long long *)skey;
-            switch (leaf_max) {
-            case 4: k_flat_marks<4><<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles); break;
-            case 8: k_flat_marks<8><<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles); break;
-            case 16: k_flat_marks<16><<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles); break;
-            case 24: k_flat_marks<24><<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles); break;
-            case 32: k_flat_marks<32><<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles); break;
-            default: k_flat_marks<0><<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles); break;
-            }
-            gt_note_launches(1);
-        }
-        { k_flat_scan<<<NREC, 1024, 0, st>>>(cnt, ntiles, tot); gt_note_launches(1); }
-        { k_flat_levels<<<1, 1, 0, st>>>(tot, cap, ctl); gt_note_launches(1); }
-        if (ntiles > 0) {
-            k_flat_scatter<<<ntiles, FB, 0, st>>>(dl, n, cnt, ntiles, cap, nd, ctl);
-            { k_flat_link<<<nsm * 8, 256, 0, st>>>(nd, cap, ctl); }
-            gt_note_launches(2);
-        }
+        const unsigned long long *k = (const unsigned long long *)skey;
+        if (flat_rounds(n) == 2) launch_flat<2>(k, n, leaf_max, nd, cap, scratch, ctl, nsm, st);
+        else launch_flat<8>(k, n, leaf_max, nd, cap, scratch, ctl, nsm, st);
         return;
     }
-    { k_build_init<<<1, 1, 0, st>>>(n, nd, ctl); gt_note_launches(1); }
+    { k_build_init<<<1, 256, 0, st>>>(n, nd, ctl); gt_note_launches(1); }
     for (int l = 0; l < GT_TREE_LEVELS; l++)
         { k_build_level<<<nsm * 4, BT, 0, st>>>(l, (const unsigned long long *)skey, leaf_max, nd, cap,
                                               status, ctl); gt_note_launches(1); }
 }
 
 void gt_launch_cell_lists(Nodes nd, int64_t cap, DevCtl *ctl, int nsm, cudaStream_t st) {
-    cudaMemsetAsync(ctl->cell_bucket, 0, sizeof(ctl->cell_bucket), st);
     { k_cell_count<<<nsm * 4, 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
-    { k_cell_scan<<<1, 1024, 0, st>>>(ctl); gt_note_launches(1); }
     { k_cell_fill<<<nsm * 2, 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
 }
 
 void gt_launch_pseudo(Nodes nd, int64_t cap, const float4 *posm, DevCtl *ctl, int nsm, bool with_mass,
                       cudaStream_t st) {
-    (void)cap;
-    // the ticket and the per-level counters start at zero
-    cudaMemsetAsync(&ctl->pl_ticket, 0, sizeof(ctl->pl_ticket) + sizeof(ctl->pl_done), st);
+    (void)cap;  // the ticket and the per-level counters were cleared by gt_launch_prepare
     if (with_mass) { k_pseudo<true><<<nsm * GT_PSEUDO_MINB, PL, 0, st>>>(nd, posm, ctl); }
     else { k_pseudo<false><<<nsm * GT_PSEUDO_MINB, PL, 0, st>>>(nd, posm, ctl); }
     gt_note_launches(1);
