@@ -371,7 +371,7 @@ void build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src) {
     ph_begin(s, PH_SORT, st);
     gt_launch_bbox(posm_src, n, s->nsm * 4, s->ctl, st);
     gt_launch_keys(posm_src, n, s->prm.key_curve, s->ctl, s->sb, s->nsm, st);
-    gt_launch_sort(s->sb, n, s->ctl, true, st);
+    gt_launch_sort_tree(s->sb, n, s->ctl, s->nsm, st);
     ph_end(s, PH_SORT, st);
     ph_begin(s, PH_PERMUTE, st);
     if (!s->fixed_buffers) {

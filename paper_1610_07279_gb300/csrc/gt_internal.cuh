@@ -56,6 +56,8 @@ struct DevCtl {
     int levels_m1;                    // L - 1 (finest level)
     unsigned int bbox[6];             // extrema of the positions (gt_ordered): minima, then maxima
     unsigned int digits_done;         // blocks that have added their digit counts (the sort)
+    unsigned int run_count;           // runs of equal sorted bits listed for k_fix_long_runs
+    unsigned int sort_whole;          // the tree's keys are sorted by all of their bits in whole passes
     unsigned int scan_done, cells_done;  // the same for the octree's tile scan and the cell list's counts
     unsigned int spin_limit;          // bound on every spin-wait of this system; 0: GT_SPIN_LIMIT
 };
@@ -263,16 +265,16 @@ struct SortBufs {
 };
 
 // keys.cu
-// extrema into ctl->bbox (reset by gt_launch_prepare); keys into b.key[0] and their digit counts (so
-// that gt_launch_sort need not count them)
+// extrema into ctl->bbox (reset by gt_launch_prepare); keys and their digit counts for gt_launch_sort_tree
 void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, cudaStream_t st);
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st);
-// sort.cu: sorts (key, val) in buffers 0; result in buffers 0 (even passes).  counted: the digits are counted, and
-// the values are the keys' positions (b.val[0] is not read).
+// sort.cu: gt_launch_sort sorts (key, val) in buffers 0; gt_launch_sort_tree the keys that gt_launch_keys made, with
+// their positions as values, into buffers 0
 int gt_sort_tiles(int64_t n);
 size_t gt_sort_scratch_bytes(int64_t n);
 void gt_sort_clear(SortBufs &b, int64_t n, cudaStream_t st);  // the digit counts and the look-back words
-void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, bool counted, cudaStream_t st);
+void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st);
+void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStream_t st);
 void gt_sort_init();
 // tree.cu
 // scratch: gt_build_scratch_bytes(n) bytes (per-particle marks and per-tile counts)

@@ -142,9 +142,9 @@ __global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, l
             k = interleave(x, y, z);
         }
         if (ok) key[i] = k;
-        gt_count_digits(k, ok, h);
+        gt_count_digits<true>(k, ok, h);
     }
-    gt_finish_digits(h, hist, base, ctl);
+    gt_finish_digits(h, n, hist, base, ctl);
 }
 
 }  // namespace

@@ -1,8 +1,9 @@
 // Step A2: stable LSD radix sort of (63-bit key, 32-bit index) pairs (Sec. 2.1: the
 // particles are sorted by their space-filling key with a library radix sort).
 //
-// Eight passes of 8-bit digits, one kernel per pass; the digits of all passes are counted by the kernel that
-// makes the keys (keys.cu), or for a caller's pairs by
+// Passes of 8-bit digits, one kernel per pass: eight for a caller's pairs, six over the highest 48 bits for
+// the tree's keys, whose ties in those bits are then put in order (k_fix_runs); the digits of all passes are
+// counted by the kernel that makes the keys (keys.cu), or for a caller's pairs by
 //   k_hist_all     all eight digit counts in one read of the keys, and their starts   (reads 8 B/key)
 //   k_onesweep     per 4096-key tile (512 threads) taken in ticket order: a stable rank of
 //                  every key inside the tile (warp-striped; a key's peers with the same
@@ -57,9 +58,9 @@ __global__ __launch_bounds__(HT) void k_hist_all(long long n, const unsigned lon
     __syncthreads();
     for (long long i0 = (long long)blockIdx.x * HT; i0 < n; i0 += (long long)gridDim.x * HT) {
         const long long i = i0 + threadIdx.x;
-        gt_count_digits(i < n ? key[i] : 0ull, i < n, h);
+        gt_count_digits<false>(i < n ? key[i] : 0ull, i < n, h);
     }
-    gt_finish_digits(h, hist, base, ctl);
+    gt_finish_digits(h, n, hist, base, ctl);
 }
 
 // Look-back of one digit: the count of digit d in all tiles before `tile`.  The status
@@ -105,9 +106,40 @@ __device__ __forceinline__ uint32_t lookback_digit(const uint32_t *status, int t
     return excl;
 }
 
-// INDEX: the values are the keys' positions (vin is not read)
-template <bool INDEX>
-__global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int pass,
+// Stable ranks of a warp's keys among its keys with the same digit, item j of lane l being key 32 j + l of m; cnt (R
+// counts, zero before) receives the warp's digit counts.  FULL: m == 32 IPT.
+template <bool FULL>
+__device__ __forceinline__ void rank_keys(const unsigned long long (&k)[IPT], int shift, int m, uint32_t *cnt,
+                                          uint32_t (&loc)[IPT]) {
+    const unsigned int lt = lanemask_lt();
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < IPT; j++) {
+        const bool ok = FULL || 32 * j + lane < m;
+        const unsigned int d = ok ? (unsigned int)((k[j] >> shift) & (R - 1)) : (unsigned int)R;
+        unsigned int peers = 0xffffffffu;  // lanes with the same digit (bit 8: past the end)
+#pragma unroll
+        for (int b = 0; b < (FULL ? RB : RB + 1); b++) {
+            const unsigned int bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+            peers &= ((d >> b) & 1u) ? bal : ~bal;
+        }
+        const unsigned int rank = __popc(peers & lt);
+        unsigned int prev = 0;
+        if (ok) prev = cnt[d];
+        __syncwarp();
+        if (ok && rank == 0) cnt[d] = prev + __popc(peers);
+        __syncwarp();
+        loc[j] = prev + rank;
+    }
+}
+
+// What a pass over the tree's keys does that another doesn't: the first of the low passes makes the values (the keys'
+// positions), both of them run only if the whole keys are sorted by passes (ctl->sort_whole), and the first of the
+// others makes the values if not.
+enum { PASS_PLAIN = 0, PASS_LOW_FIRST, PASS_LOW, PASS_HIGH_FIRST };
+
+template <int MODE>
+__global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int pass, int shift,
                                                  const unsigned long long *__restrict__ kin,
                                                  const uint32_t *__restrict__ vin,
                                                  unsigned long long *__restrict__ kout,
@@ -123,7 +155,8 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
     uint32_t *gbase = dstart + R;     // R: global slot of every digit's first key in this tile
     uint32_t *scantmp = gbase + R;    // NW + 1
     __shared__ uint32_t tile_sh;
-    const int shift = pass * RB;
+    if ((MODE == PASS_LOW_FIRST || MODE == PASS_LOW) && !ctl->sort_whole) return;
+    const bool index = MODE == PASS_LOW_FIRST || (MODE == PASS_HIGH_FIRST && !ctl->sort_whole);
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) tile_sh = atomicAdd(&ctl->sort_ticket[pass], 1u);
     for (int k = threadIdx.x; k < NW * R; k += ST) wcnt[k] = 0;
@@ -140,27 +173,14 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
     for (int j = 0; j < IPT; j++) {
         const long long i = base + j * 32 + lane;
         k[j] = i < n ? kin[i] : 0ull;
-        v[j] = INDEX ? (uint32_t)i : (i < n ? vin[i] : 0u);
+        v[j] = MODE == PASS_LOW_FIRST ? (uint32_t)i : (i < n ? vin[i] : 0u);
     }
-    const unsigned int lt = lanemask_lt();
+    if (MODE == PASS_HIGH_FIRST && index) {
 #pragma unroll
-    for (int j = 0; j < IPT; j++) {
-        const bool ok = base + j * 32 + lane < n;
-        const unsigned int d = ok ? (unsigned int)((k[j] >> shift) & (R - 1)) : (unsigned int)R;
-        unsigned int peers = 0xffffffffu;  // lanes with the same digit (bit 8: past the end)
-#pragma unroll
-        for (int b = 0; b <= RB; b++) {
-            const unsigned int bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-            peers &= ((d >> b) & 1u) ? bal : ~bal;
-        }
-        const unsigned int rank = __popc(peers & lt);
-        unsigned int prev = 0;
-        if (ok) prev = wcnt[w * R + d];
-        __syncwarp();
-        if (ok && rank == 0) wcnt[w * R + d] = prev + __popc(peers);
-        __syncwarp();
-        loc[j] = prev + rank;
+        for (int j = 0; j < IPT; j++) v[j] = (uint32_t)(base + j * 32 + lane);
     }
+    if ((long long)(tile + 1) * TILE <= n) rank_keys<true>(k, shift, 32 * IPT, wcnt + w * R, loc);
+    else rank_keys<false>(k, shift, (int)(n - base < 0 ? 0 : (n - base < 32 * IPT ? n - base : 32 * IPT)), wcnt + w * R, loc);
     __syncthreads();
     // thread d < R: exclusive offsets of the warps for digit d, the tile's count of digit d
     const int d = threadIdx.x;
@@ -211,6 +231,181 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
     }
 }
 
+// ---- keys that agree in the sorted bits --------------------------------------------
+// The tree's keys are spread over the bounding cube by construction, so few of them agree in their highest 16 levels
+// (48 bits): six passes over those bits leave short runs of keys that differ only below, and these are put in order
+// here -- two passes fewer over all keys (2^24: 322 us of 1290) for one read of them (25 us).  The passes and all three
+// ways below are stable, so the result is that of a stable sort by the whole key.  Where the particles fill only a
+// small part of the cube (one far particle is enough), the digit of levels 11 to 13 takes few values: once one of them
+// holds a sixteenth of the keys (smooth models: a few hundredths of that share) the two low passes run as well.
+constexpr uint32_t RUN_SHORT = 16;  // keys that one thread puts in order by insertion
+constexpr int RUN_SMEM = TILE;      // keys that a block puts in order in shared memory
+
+__device__ __forceinline__ bool same_run(unsigned long long a, unsigned long long b, int shift) {
+    return ((a ^ b) >> shift) == 0ull;
+}
+
+// One thread per key: the first key of a run of two or more has it put in order, or listed if it is longer and not in
+// order already as far as looked.
+__global__ __launch_bounds__(256) void k_fix_runs(long long n, int shift, unsigned long long *key, uint32_t *val,
+                                                  uint32_t *list, DevCtl *ctl) {
+    if (ctl->sort_whole) return;
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
+        const unsigned long long k0 = key[i];
+        if (i + 1 >= n || !same_run(k0, key[i + 1], shift)) continue;
+        if (i > 0 && same_run(key[i - 1], k0, shift)) continue;
+        uint32_t len = 2;
+        while (len <= RUN_SHORT && i + len < n && same_run(k0, key[i + len], shift)) len++;
+        if (len > RUN_SHORT) {
+            list[atomicAdd(&ctl->run_count, 1u)] = (uint32_t)i;
+            continue;
+        }
+        for (uint32_t j = 1; j < len; j++) {
+            const unsigned long long k = key[i + j];
+            const uint32_t v = val[i + j];
+            uint32_t p = j;
+            for (; p > 0 && key[i + p - 1] > k; p--) {
+                key[i + p] = key[i + p - 1];
+                val[i + p] = val[i + p - 1];
+            }
+            if (p != j) {
+                key[i + p] = k;
+                val[i + p] = v;
+            }
+        }
+    }
+}
+
+// The listed runs, a block each: by digits in shared memory, or, beyond RUN_SMEM keys, tile by tile through the
+// other buffers.  Runs that are in order (equal keys, most of all) are left alone.
+__global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, unsigned long long *key0, uint32_t *val0,
+                                                      unsigned long long *key1, uint32_t *val1,
+                                                      const uint32_t *__restrict__ list, DevCtl *ctl) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    unsigned long long *skey = (unsigned long long *)smraw;
+    uint32_t *sval = (uint32_t *)(skey + TILE);
+    uint32_t *wcnt = sval + TILE;      // NW x R
+    uint32_t *dstart = wcnt + NW * R;  // R: where the next key of every digit goes
+    uint32_t *scantmp = dstart + 2 * R;
+    __shared__ int sorted_sh;
+    __shared__ unsigned long long len_sh;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t runs = ctl->run_count;  // 0 if the whole keys were sorted
+    for (uint32_t r = blockIdx.x; r < runs; r += gridDim.x) {
+        const long long first = list[r];
+        const unsigned long long k0 = key0[first];
+        if (threadIdx.x == 0) {
+            sorted_sh = 1;
+            len_sh = ~0ull;
+        }
+        __syncthreads();
+        for (long long at = first;; at += ST) {  // the run's end, and whether its keys are in order
+            const long long i = at + threadIdx.x;
+            const bool in = i < n && same_run(k0, key0[i], shift);
+            if (!in) atomicMin(&len_sh, (unsigned long long)(i - first));
+            else if (i > first && key0[i - 1] > key0[i]) sorted_sh = 0;
+            __syncthreads();
+            const bool end = len_sh != ~0ull;
+            __syncthreads();
+            if (end) break;
+        }
+        const long long len = (long long)len_sh;
+        const bool sorted = sorted_sh != 0;
+        __syncthreads();
+        if (sorted) continue;
+        unsigned long long *ka = key0 + first, *kb = key1 + first;
+        uint32_t *va = val0 + first, *vb = val1 + first;
+        const bool once = len <= RUN_SMEM;
+        for (int s0 = 0; s0 < shift; s0 += RB) {  // (digits above the run's own bits agree: the last one may hold some)
+            if (!once) {  // where every digit starts
+                if (threadIdx.x < R) wcnt[threadIdx.x] = 0;
+                __syncthreads();
+                for (long long i = threadIdx.x; i < len; i += ST) atomicAdd(&wcnt[(ka[i] >> s0) & (R - 1)], 1u);
+                __syncthreads();
+                uint32_t total;
+                const uint32_t c = threadIdx.x < R ? wcnt[threadIdx.x] : 0u;
+                const uint32_t e = block_excl_scan<ST>(c, &total, scantmp);
+                if (threadIdx.x < R) dstart[threadIdx.x] = e;
+                __syncthreads();
+            }
+            for (long long t0 = 0; t0 < len; t0 += TILE) {
+                for (int i = threadIdx.x; i < NW * R; i += ST) wcnt[i] = 0;
+                __syncthreads();
+                const long long base = t0 + w * (32 * IPT);
+                const int m = (int)(len - base < 0 ? 0 : (len - base < 32 * IPT ? len - base : 32 * IPT));
+                unsigned long long k[IPT];
+                uint32_t v[IPT], loc[IPT];
+#pragma unroll
+                for (int j = 0; j < IPT; j++) {
+                    const int i = 32 * j + lane;
+                    k[j] = 0ull;
+                    v[j] = 0u;
+                    if (i < m) {
+                        if (once && s0 > 0) {
+                            k[j] = skey[base + i];
+                            v[j] = sval[base + i];
+                        } else {
+                            k[j] = ka[base + i];
+                            v[j] = va[base + i];
+                        }
+                    }
+                }
+                rank_keys<false>(k, s0, m, wcnt + w * R, loc);
+                __syncthreads();
+                uint32_t cnt = 0;
+                if (threadIdx.x < R)
+                    for (int ww = 0; ww < NW; ww++) {
+                        const uint32_t t = wcnt[ww * R + threadIdx.x];
+                        wcnt[ww * R + threadIdx.x] = cnt;
+                        cnt += t;
+                    }
+                if (once) {
+                    uint32_t total;
+                    const uint32_t e = block_excl_scan<ST>(cnt, &total, scantmp);
+                    if (threadIdx.x < R) dstart[threadIdx.x] = e;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int j = 0; j < IPT; j++) {
+                    if (32 * j + lane >= m) continue;
+                    const uint32_t d = (uint32_t)(k[j] >> s0) & (R - 1);
+                    const uint32_t pos = dstart[d] + wcnt[w * R + d] + loc[j];
+                    if (once) {
+                        skey[pos] = k[j];
+                        sval[pos] = v[j];
+                    } else {
+                        kb[pos] = k[j];
+                        vb[pos] = v[j];
+                    }
+                }
+                __syncthreads();
+                if (!once && threadIdx.x < R) dstart[threadIdx.x] += cnt;
+                __syncthreads();
+            }
+            if (!once) {
+                unsigned long long *kt = ka;
+                ka = kb;
+                kb = kt;
+                uint32_t *vt = va;
+                va = vb;
+                vb = vt;
+            }
+        }
+        if (once) {
+            for (long long i = threadIdx.x; i < len; i += ST) {
+                key0[first + i] = skey[i];
+                val0[first + i] = sval[i];
+            }
+        } else if (ka != key0 + first) {
+            for (long long i = threadIdx.x; i < len; i += ST) {
+                key0[first + i] = ka[i];
+                val0[first + i] = va[i];
+            }
+        }
+        __syncthreads();
+    }
+}
+
 }  // namespace
 
 int gt_sort_tiles(int64_t n) { return (int)((n + TILE - 1) / TILE); }
@@ -221,40 +416,57 @@ size_t gt_sort_scratch_bytes(int64_t n) {
 }
 
 void gt_sort_init() {
-    cudaFuncSetAttribute(k_onesweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
-    cudaFuncSetAttribute(k_onesweep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+    for (auto kernel : {k_onesweep<PASS_PLAIN>, k_onesweep<PASS_LOW_FIRST>, k_onesweep<PASS_LOW>,
+                        k_onesweep<PASS_HIGH_FIRST>})
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+    cudaFuncSetAttribute(k_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
 }
 
 void gt_sort_clear(SortBufs &b, int64_t n, cudaStream_t st) {
     cudaMemsetAsync(b.hist, 0, (size_t)PASSES * R * (1 + (size_t)gt_sort_tiles(n)) * sizeof(uint32_t), st);
 }
 
-void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, bool counted, cudaStream_t st) {
-    if (n <= 0 || (n == 1 && !counted)) return;
-    const int ntiles = gt_sort_tiles(n);
-    if (!counted) {
-        gt_sort_clear(b, n, st);
-        int dev = 0, nsm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        const long long blocks = (n + HT - 1) / HT;
-        k_hist_all<<<(unsigned)(blocks < nsm * 8 ? blocks : nsm * 8), HT, 0, st>>>(n, (const unsigned long long *)b.key[0],
-                                                                                   b.hist, b.digit_base, ctl);
-        gt_note_launches(1);
-    }
-    for (int p = 0; p < PASSES; p++) {
-        const int src = p & 1, dst = src ^ 1;
-        const unsigned long long *kin = (const unsigned long long *)b.key[src];
-        unsigned long long *kout = (unsigned long long *)b.key[dst];
-        uint32_t *status = b.status + (size_t)p * R * ntiles;
-        if (p == 0 && counted)
-            k_onesweep<true><<<ntiles, ST, SCATTER_SMEM, st>>>(n, p, kin, nullptr, kout, b.val[dst], b.digit_base, status,
-                                                               ntiles, ctl);
-        else
-            k_onesweep<false><<<ntiles, ST, SCATTER_SMEM, st>>>(n, p, kin, b.val[src], kout, b.val[dst], b.digit_base,
-                                                                status, ntiles, ctl);
-        gt_note_launches(1);
-    }
+namespace {
+
+// pass p reads buffers p & 1 and writes the others
+template <int MODE>
+void onesweep(SortBufs &b, int64_t n, DevCtl *ctl, int pass, int shift, cudaStream_t st) {
+    const int ntiles = gt_sort_tiles(n), src = pass & 1;
+    k_onesweep<MODE><<<ntiles, ST, SCATTER_SMEM, st>>>(n, pass, shift, (const unsigned long long *)b.key[src], b.val[src],
+                                                       (unsigned long long *)b.key[src ^ 1], b.val[src ^ 1], b.digit_base,
+                                                       b.status + (size_t)pass * R * ntiles, ntiles, ctl);
+    gt_note_launches(1);
+}
+
+}  // namespace
+
+void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStream_t st) {
+    if (n <= 0) return;
+    onesweep<PASS_LOW_FIRST>(b, n, ctl, 0, gt_tree_digit_shift(0), st);
+    onesweep<PASS_LOW>(b, n, ctl, 1, gt_tree_digit_shift(1), st);
+    onesweep<PASS_HIGH_FIRST>(b, n, ctl, 2, gt_tree_digit_shift(2), st);
+    for (int p = 3; p < PASSES; p++) onesweep<PASS_PLAIN>(b, n, ctl, p, gt_tree_digit_shift(p), st);
+    const int shift = gt_tree_digit_shift(2);
+    uint32_t *list = b.status;  // the look-backs are over
+    const int64_t need = (n + 255) / 256, most = (int64_t)nsm * 16;
+    k_fix_runs<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
+                                                                      list, ctl);
+    k_fix_long_runs<<<nsm, ST, SCATTER_SMEM, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
+                                                   (unsigned long long *)b.key[1], b.val[1], list, ctl);
+    gt_note_launches(2);
+}
+
+void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st) {
+    if (n <= 1) return;
+    gt_sort_clear(b, n, st);
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const long long blocks = (n + HT - 1) / HT;
+    k_hist_all<<<(unsigned)(blocks < nsm * 8 ? blocks : nsm * 8), HT, 0, st>>>(n, (const unsigned long long *)b.key[0],
+                                                                               b.hist, b.digit_base, ctl);
+    gt_note_launches(1);
+    for (int p = 0; p < PASSES; p++) onesweep<PASS_PLAIN>(b, n, ctl, p, RB * p, st);
 }
 
 // ---- sort without allocation (gt_sort_pairs_noalloc) -----------------------------
@@ -324,7 +536,7 @@ extern "C" int gt_sort_pairs_noalloc(uint64_t *d_keys, uint32_t *d_vals, int64_t
     b.status = (uint32_t *)(base + NA_OFF_STATUS);
     b.hist = (uint32_t *)(base + NA_OFF_HIST);
     b.digit_base = (uint32_t *)(base + NA_OFF_BASE);
-    gt_launch_sort(b, n, ctl, false, st);  // an even number of passes leaves the result in d_keys/d_vals
+    gt_launch_sort(b, n, ctl, st);  // an even number of passes leaves the result in d_keys/d_vals
     return cudaGetLastError() == cudaSuccess ? GT_OK : GT_ECUDA;
 }
 

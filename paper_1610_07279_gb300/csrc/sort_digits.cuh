@@ -4,20 +4,30 @@
 
 #include "gt_internal.cuh"
 
+// Where the digits of the tree's keys begin: two for the lowest 15 bits (the second reaches one bit into the next,
+// which changes nothing), six for the 48 above (16 levels of the tree).
+__host__ __device__ constexpr int gt_tree_digit_shift(int p) { return p < 2 ? 8 * p : 8 * p - 1; }
+
 // One key per lane into the block's counts.  The keys of a tree rebuild arrive nearly sorted (the particles are
 // still in the previous key order), so a warp's 32 neighbouring keys often share their high digits: such a digit
-// is counted once for the whole warp, the others by one atomic per lane.
+// is counted once for the whole warp, the others by one atomic per lane.  TREE: the digits of the tree's keys.
+template <bool TREE>
 __device__ __forceinline__ void gt_count_digits(unsigned long long k, bool ok, uint32_t (*h)[GT_SORT_DIGITS]) {
-    const uint32_t lo = (uint32_t)k, hi = (uint32_t)(k >> 32);
+    static_assert(GT_SORT_BITS == 8 && GT_SORT_PASSES == 8, "a byte per digit");
+    const unsigned long long high = TREE ? k << 1 : k;  // digits 2 to 7 (of the tree's keys) are bytes of this
+    const uint32_t lo = (uint32_t)high, hi = (uint32_t)(high >> 32);
     // bits in which some lane's key differs from the first one's (a lane without a key: all)
     const uint32_t lo0 = __shfl_sync(0xffffffffu, lo, 0), hi0 = __shfl_sync(0xffffffffu, hi, 0);
     const uint32_t dlo = __reduce_or_sync(0xffffffffu, ok ? lo ^ lo0 : ~0u);
     const uint32_t dhi = __reduce_or_sync(0xffffffffu, ok ? hi ^ hi0 : ~0u);
-    static_assert(GT_SORT_BITS == 8 && GT_SORT_PASSES == 8, "a byte per digit");
 #pragma unroll
     for (int p = 0; p < GT_SORT_PASSES; p++) {
-        const uint32_t word = p < 4 ? lo : hi, d = (word >> (8 * (p & 3))) & 0xffu;
-        if ((((p < 4 ? dlo : dhi) >> (8 * (p & 3))) & 0xffu) == 0u) {
+        const uint32_t word = p < 4 ? lo : hi;
+        const uint32_t d = TREE && p < 2 ? (uint32_t)(k >> (8 * p)) & 0xffu : (word >> (8 * (p & 3))) & 0xffu;
+        // (a low digit of the tree's keys lies in the bits 1 to 16 of lo)
+        const uint32_t differ = TREE && p < 2 ? (dlo >> (8 * p + 1)) & 0xffu
+                                              : ((p < 4 ? dlo : dhi) >> (8 * (p & 3))) & 0xffu;
+        if (differ == 0u) {
             if ((threadIdx.x & 31) == 0) atomicAdd(&h[p][d], 32u);
         } else if (ok) {
             atomicAdd(&h[p][d], 1u);
@@ -26,9 +36,11 @@ __device__ __forceinline__ void gt_count_digits(unsigned long long k, bool ok, u
 }
 
 // The block's counts into the global ones; the last block to come turns them into every pass's digit starts (a
-// launch of its own for that took 7 to 8 us) and resets the passes' tile tickets.
-__device__ __forceinline__ void gt_finish_digits(const uint32_t (*h)[GT_SORT_DIGITS], uint32_t *hist, uint32_t *base,
-                                                 DevCtl *ctl) {
+// launch of its own for that took 7 to 8 us), resets the passes' tile tickets, and says whether the tree's keys crowd
+// into so small a part of the cube that they are sorted by all of their bits (n: the number of keys).
+constexpr int GT_CROWD_PASS = 3;  // the digit of levels 11 to 13
+__device__ __forceinline__ void gt_finish_digits(const uint32_t (*h)[GT_SORT_DIGITS], long long n, uint32_t *hist,
+                                                 uint32_t *base, DevCtl *ctl) {
     __shared__ bool last;
     __syncthreads();
     for (int p = 0; p < GT_SORT_PASSES; p++)
@@ -41,12 +53,15 @@ __device__ __forceinline__ void gt_finish_digits(const uint32_t (*h)[GT_SORT_DIG
     __threadfence();
     static_assert(GT_SORT_DIGITS == 32 * GT_SORT_PASSES, "a warp per pass, eight digits per lane");
     const uint32_t p = threadIdx.x >> 5, lane = threadIdx.x & 31u;
-    uint32_t v[8], sum = 0;
+    uint32_t v[8], sum = 0, most = 0;
 #pragma unroll
     for (int j = 0; j < 8; j++) {
         v[j] = __ldcg(&hist[p * GT_SORT_DIGITS + 8 * lane + j]);
         sum += v[j];
+        most = max(most, v[j]);
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (p == GT_CROWD_PASS && lane == 0) ctl->sort_whole = (long long)most * 16 >= n ? 1u : 0u;
     uint32_t at = warp_incl_scan(sum) - sum;
 #pragma unroll
     for (int j = 0; j < 8; j++) {
@@ -54,5 +69,5 @@ __device__ __forceinline__ void gt_finish_digits(const uint32_t (*h)[GT_SORT_DIG
         at += v[j];
     }
     if (threadIdx.x < GT_SORT_PASSES) ctl->sort_ticket[threadIdx.x] = 0;
-    if (threadIdx.x == 0) ctl->digits_done = 0;
+    if (threadIdx.x == 0) ctl->digits_done = ctl->run_count = 0;
 }
