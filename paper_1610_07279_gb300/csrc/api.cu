@@ -369,9 +369,13 @@ void build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src) {
     const int64_t n = s->n;
     gt_launch_prepare(s->ctl, 0, st);
     ph_begin(s, PH_SORT, st);
-    gt_launch_bbox(posm_src, n, s->nsm * 4, s->ctl, st);
-    gt_launch_keys(posm_src, n, s->prm.key_curve, s->ctl, s->sb, s->nsm, st);
-    gt_launch_sort_tree(s->sb, n, s->ctl, s->nsm, st);
+    if (n <= GT_SMALL_SORT) {
+        gt_launch_small_sort(posm_src, n, s->prm.key_curve, s->sb, st);
+    } else {
+        gt_launch_bbox(posm_src, n, s->nsm * 4, s->ctl, st);
+        gt_launch_keys(posm_src, n, s->prm.key_curve, s->ctl, s->sb, s->nsm, st);
+        gt_launch_sort_tree(s->sb, n, s->ctl, s->nsm, st);
+    }
     ph_end(s, PH_SORT, st);
     ph_begin(s, PH_PERMUTE, st);
     if (!s->fixed_buffers) {

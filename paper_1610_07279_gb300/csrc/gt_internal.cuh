@@ -252,6 +252,7 @@ __device__ __forceinline__ unsigned int lookback_warp(unsigned long long *status
 // Every helper reports the kernels it launched (counted for gt_kernel_launches).
 void gt_note_launches(int k);
 
+#define GT_SMALL_SORT 8192           // systems whose keys one block makes and sorts
 #define GT_SORT_BITS 8
 #define GT_SORT_DIGITS 256
 #define GT_SORT_PASSES 8             // 64 / 8 (bit 63 is always 0)
@@ -268,6 +269,9 @@ struct SortBufs {
 // extrema into ctl->bbox (reset by gt_launch_prepare); keys and their digit counts for gt_launch_sort_tree
 void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, cudaStream_t st);
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st);
+// box, keys and sort of at most GT_SMALL_SORT particles in one launch
+void gt_keys_init();
+void gt_launch_small_sort(const float4 *posm, int64_t n, int curve, SortBufs &b, cudaStream_t st);
 // sort.cu: gt_launch_sort sorts (key, val) in buffers 0; gt_launch_sort_tree the keys that gt_launch_keys made, with
 // their positions as values, into buffers 0
 int gt_sort_tiles(int64_t n);

@@ -104,6 +104,31 @@ __device__ __forceinline__ void hilbert_transpose(uint32_t &x0, uint32_t &x1, ui
     x2 ^= t;
 }
 
+// The grid of a set of positions: the cube's lower corner and scale, and the scale on the FP32 pipe.
+struct KeyGrid {
+    float x0, y0, z0, sh, sl;
+    double scale;
+    bool fp32;
+    __device__ __forceinline__ unsigned long long key(const float4 &p, int curve) const {
+        uint32_t x = 0, y = 0, z = 0;
+        if (!fp32 || !quantise_fp32(p.x, x0, sh, sl, &x)) x = quantise_slow(p.x, x0, scale);
+        if (!fp32 || !quantise_fp32(p.y, y0, sh, sl, &y)) y = quantise_slow(p.y, y0, scale);
+        if (!fp32 || !quantise_fp32(p.z, z0, sh, sl, &z)) z = quantise_slow(p.z, z0, scale);
+        if (curve == GT_KEY_HILBERT) hilbert_transpose(x, y, z);
+        return interleave(x, y, z);
+    }
+};
+
+// 2^21 / the cube's side, 0 for a side of 0, from the extrema (minima, then maxima).
+__device__ __forceinline__ double cube_scale(const float *ext) {
+    double side = 0.0;
+    for (int a = 0; a < 3; a++) {
+        const double e = __dsub_rn((double)ext[a + 3], (double)ext[a]);
+        if (e > side) side = e;
+    }
+    return side > 0.0 ? __ddiv_rn((double)(1u << GT_KEY_LEVELS), side) : 0.0;
+}
+
 // Bound by issue: ~100 instructions per key of quantisation and interleaving on the FP32 and integer pipes and
 // ~50 of digit counting, against 24 B of HBM.
 __global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, long long n, int curve, DevCtl *ctl,
@@ -111,40 +136,176 @@ __global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, l
                                               uint32_t *__restrict__ base) {
     __shared__ uint32_t h[GT_SORT_PASSES][GT_SORT_DIGITS];
     __shared__ double scale_sh;
-    __shared__ float min_sh[3];
+    __shared__ float ext[6];
     for (int p = 0; p < GT_SORT_PASSES; p++) h[p][threadIdx.x] = 0;
-    if (threadIdx.x == 0) {  // the cube of Sec. 2.1's keys, from the extrema
-        double side = 0.0;
-        for (int a = 0; a < 3; a++) {
-            const float lo = gt_unordered(ctl->bbox[a]);
-            const double ext = __dsub_rn((double)gt_unordered(ctl->bbox[a + 3]), (double)lo);
-            if (ext > side) side = ext;
-            min_sh[a] = lo;
-        }
-        scale_sh = side > 0.0 ? __ddiv_rn((double)(1u << GT_KEY_LEVELS), side) : 0.0;
-    }
+    if (threadIdx.x < 6) ext[threadIdx.x] = gt_unordered(ctl->bbox[threadIdx.x]);
     __syncthreads();
-    const double scale = scale_sh;
-    const float x0 = min_sh[0], y0 = min_sh[1], z0 = min_sh[2];
-    float sh, sl;
-    const bool fp32 = gtq_fp32_scale(scale, &sh, &sl), sized = scale > 0.0;
+    if (threadIdx.x == 0) scale_sh = cube_scale(ext);
+    __syncthreads();
+    KeyGrid grid{ext[0], ext[1], ext[2], 0.f, 0.f, scale_sh, false};
+    grid.fp32 = gtq_fp32_scale(grid.scale, &grid.sh, &grid.sl);
+    const bool sized = grid.scale > 0.0;
     for (long long i0 = (long long)blockIdx.x * 256; i0 < n; i0 += (long long)gridDim.x * 256) {
         const long long i = i0 + threadIdx.x;
         const bool ok = i < n;
         unsigned long long k = 0;
-        if (ok && sized) {
-            const float4 p = posm[i];
-            uint32_t x = 0, y = 0, z = 0;
-            if (!fp32 || !quantise_fp32(p.x, x0, sh, sl, &x)) x = quantise_slow(p.x, x0, scale);
-            if (!fp32 || !quantise_fp32(p.y, y0, sh, sl, &y)) y = quantise_slow(p.y, y0, scale);
-            if (!fp32 || !quantise_fp32(p.z, z0, sh, sl, &z)) z = quantise_slow(p.z, z0, scale);
-            if (curve == GT_KEY_HILBERT) hilbert_transpose(x, y, z);
-            k = interleave(x, y, z);
-        }
+        if (ok && sized) k = grid.key(posm[i], curve);
         if (ok) key[i] = k;
         gt_count_digits<true>(k, ok, h);
     }
     gt_finish_digits(h, n, hist, base, ctl);
+}
+
+// Small systems: the bounding box, the keys and the whole sort in one block, in shared memory (through the kernels
+// above: thirteen launches, of which every sort pass takes 10 us for the latency of its chain; 8192 particles ~90 us).
+// The passes move 16-bit positions only and look the digits up in the keys, which stay: the wavefronts of one SM's
+// shared memory and its ballots bound it (7 us a pass; 48 us in all, 70 with keys that move too and eight passes).  Five passes over the
+// highest 40 bits, then the short runs that agree there; a longer run that is out of order takes all eight passes.
+constexpr int SMALL_THREADS = 1024, SMALL_WARPS = SMALL_THREADS / 32, SMALL_IPT = 8;
+static_assert(SMALL_THREADS * SMALL_IPT == GT_SMALL_SORT && SMALL_THREADS == 4 * GT_SORT_DIGITS, "one block's keys");
+constexpr size_t SMALL_SMEM = GT_SMALL_SORT * (sizeof(unsigned long long) + sizeof(uint16_t)) +
+                              SMALL_WARPS * GT_SORT_DIGITS * sizeof(uint32_t);
+constexpr int SMALL_SHIFT = 23, SMALL_RUN = 32;  // bits left to the runs; the longest one that a thread puts in order
+
+__global__ __launch_bounds__(SMALL_THREADS) void k_small_sort(const float4 *__restrict__ posm, int n, int curve,
+                                                              unsigned long long *__restrict__ key,
+                                                              uint32_t *__restrict__ val) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    unsigned long long *skey = (unsigned long long *)smraw;
+    uint32_t *wcnt = (uint32_t *)(skey + GT_SMALL_SORT);  // a count per warp and digit
+    uint16_t *sid = (uint16_t *)(wcnt + SMALL_WARPS * GT_SORT_DIGITS);
+    __shared__ float part_ext[SMALL_WARPS][6], ext[6];
+    __shared__ uint32_t part[4][GT_SORT_DIGITS], tmp[SMALL_THREADS / 32 + 1];
+    __shared__ double scale_sh;
+    __shared__ int redo_sh;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, base = w * 32 * SMALL_IPT;
+    const int m = n - base < 0 ? 0 : (n - base < 32 * SMALL_IPT ? n - base : 32 * SMALL_IPT);  // this warp's keys
+    float v[6];
+    for (int a = 0; a < 6; a++) v[a] = a < 3 ? FLT_MAX : -FLT_MAX;
+    for (int i = lane; i < m; i += 32) {
+        const float4 p = posm[base + i];
+        v[0] = fminf(v[0], p.x); v[1] = fminf(v[1], p.y); v[2] = fminf(v[2], p.z);
+        v[3] = fmaxf(v[3], p.x); v[4] = fmaxf(v[4], p.y); v[5] = fmaxf(v[5], p.z);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        for (int a = 0; a < 6; a++) {
+            const float t = __shfl_xor_sync(0xffffffffu, v[a], o);
+            v[a] = a < 3 ? fminf(v[a], t) : fmaxf(v[a], t);
+        }
+    if (lane == 0)
+        for (int a = 0; a < 6; a++) part_ext[w][a] = v[a];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        float t = part_ext[0][threadIdx.x];
+        for (int k = 1; k < SMALL_WARPS; k++)
+            t = threadIdx.x < 3 ? fminf(t, part_ext[k][threadIdx.x]) : fmaxf(t, part_ext[k][threadIdx.x]);
+        ext[threadIdx.x] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        scale_sh = cube_scale(ext);
+        redo_sh = 0;
+    }
+    __syncthreads();
+    KeyGrid grid{ext[0], ext[1], ext[2], 0.f, 0.f, scale_sh, false};
+    grid.fp32 = gtq_fp32_scale(grid.scale, &grid.sh, &grid.sl);
+    const bool sized = grid.scale > 0.0;
+    uint32_t id[SMALL_IPT];
+#pragma unroll
+    for (int j = 0; j < SMALL_IPT; j++) {
+        const int i = 32 * j + lane;
+        id[j] = (uint32_t)(base + i);
+        if (i < m) skey[base + i] = sized ? grid.key(posm[base + i], curve) : 0ull;
+    }
+    const unsigned char *bytes = (const unsigned char *)skey;
+    const int d = threadIdx.x & (GT_SORT_DIGITS - 1), q = threadIdx.x / GT_SORT_DIGITS;  // a digit, and eight warps
+    // one pass over the digit at `shift`: the positions in sid, and in the order's items again in id
+    auto pass = [&](int shift) {
+        for (int i = threadIdx.x; i < SMALL_WARPS * GT_SORT_DIGITS; i += SMALL_THREADS) wcnt[i] = 0;
+        __syncthreads();
+        uint32_t dig[SMALL_IPT], loc[SMALL_IPT];
+#pragma unroll
+        for (int j = 0; j < SMALL_IPT; j++) {
+            dig[j] = GT_SORT_DIGITS;
+            if (32 * j + lane < m) {
+                if ((shift & 7) == 0) dig[j] = bytes[8 * id[j] + shift / 8];
+                else dig[j] = (uint32_t)(skey[id[j]] >> shift) & (GT_SORT_DIGITS - 1);
+            }
+        }
+        uint32_t *own = wcnt + w * GT_SORT_DIGITS;
+#pragma unroll
+        for (int j = 0; j < SMALL_IPT; j++)
+            loc[j] = m == 32 * SMALL_IPT ? gt_rank_digit<true>(dig[j], own) : gt_rank_digit<false>(dig[j], own);
+        __syncthreads();
+        uint32_t cnt = 0;
+#pragma unroll
+        for (int ww = 0; ww < SMALL_WARPS / 4; ww++) {
+            uint32_t *c = &wcnt[(q * (SMALL_WARPS / 4) + ww) * GT_SORT_DIGITS + d];
+            const uint32_t t = *c;
+            *c = cnt;
+            cnt += t;
+        }
+        part[q][d] = cnt;
+        __syncthreads();
+        uint32_t sum = 0, total;
+        if (q == 0)
+            for (int r = 0; r < 4; r++) sum += part[r][d];
+        uint32_t at = block_excl_scan<SMALL_THREADS>(sum, &total, tmp);
+        if (q == 0)
+            for (int r = 0; r < 4; r++) {
+                const uint32_t c = part[r][d];
+                part[r][d] = at;
+                at += c;
+            }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < SMALL_IPT; j++)
+            if (32 * j + lane < m) sid[part[w / (SMALL_WARPS / 4)][dig[j]] + own[dig[j]] + loc[j]] = (uint16_t)id[j];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < SMALL_IPT; j++)
+            if (32 * j + lane < m) id[j] = sid[base + 32 * j + lane];
+    };
+    for (int shift = SMALL_SHIFT; shift < 63; shift += GT_SORT_BITS) pass(shift);
+    auto same = [&](int i, int j) { return ((skey[sid[i]] ^ skey[sid[j]]) >> SMALL_SHIFT) == 0ull; };
+    for (int i = threadIdx.x; i + 1 < n; i += SMALL_THREADS) {  // runs that begin at i
+        if (!same(i, i + 1) || (i > 0 && same(i - 1, i))) continue;
+        int len = 2;
+        bool sorted = skey[sid[i]] <= skey[sid[i + 1]];
+        for (; i + len < n && same(i, i + len); len++) {
+            sorted = sorted && skey[sid[i + len - 1]] <= skey[sid[i + len]];
+            if (len > SMALL_RUN && !sorted) break;
+        }
+        if (sorted) continue;
+        if (len > SMALL_RUN) {
+            redo_sh = 1;
+            continue;
+        }
+        for (int j = 1; j < len; j++) {
+            const uint16_t v = sid[i + j];
+            const unsigned long long kv = skey[v];
+            int p = j;
+            for (; p > 0 && skey[sid[i + p - 1]] > kv; p--) sid[i + p] = sid[i + p - 1];
+            sid[i + p] = v;
+        }
+    }
+    __syncthreads();
+    const bool redo = redo_sh != 0;
+#pragma unroll
+    for (int j = 0; j < SMALL_IPT; j++)
+        if (32 * j + lane < m) id[j] = sid[base + 32 * j + lane];
+    __syncthreads();
+    if (redo)  // (the order so far is stable, so sorting it by the whole key is too)
+        for (int shift = 0; shift < 63; shift += GT_SORT_BITS) pass(shift);
+#pragma unroll
+    for (int j = 0; j < SMALL_IPT; j++) {
+        const int i = 32 * j + lane;
+        if (i < m) {
+            key[base + i] = skey[id[j]];
+            val[base + i] = id[j];
+        }
+    }
 }
 
 }  // namespace
@@ -161,5 +322,15 @@ void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortB
     const int64_t need = (n + 255) / 256, most = (int64_t)nsm * (n < KEYS_MANY ? 4 : 8);
     k_keys<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(posm, n, curve, ctl, (unsigned long long *)b.key[0],
                                                                   b.hist, b.digit_base);
+    gt_note_launches(1);
+}
+
+void gt_keys_init() {
+    cudaFuncSetAttribute(k_small_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM);
+}
+
+void gt_launch_small_sort(const float4 *posm, int64_t n, int curve, SortBufs &b, cudaStream_t st) {
+    if (n <= 0) return;
+    k_small_sort<<<1, SMALL_THREADS, SMALL_SMEM, st>>>(posm, (int)n, curve, (unsigned long long *)b.key[0], b.val[0]);
     gt_note_launches(1);
 }

@@ -106,33 +106,6 @@ __device__ __forceinline__ uint32_t lookback_digit(const uint32_t *status, int t
     return excl;
 }
 
-// Stable ranks of a warp's keys among its keys with the same digit, item j of lane l being key 32 j + l of m; cnt (R
-// counts, zero before) receives the warp's digit counts.  FULL: m == 32 IPT.
-template <bool FULL>
-__device__ __forceinline__ void rank_keys(const unsigned long long (&k)[IPT], int shift, int m, uint32_t *cnt,
-                                          uint32_t (&loc)[IPT]) {
-    const unsigned int lt = lanemask_lt();
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int j = 0; j < IPT; j++) {
-        const bool ok = FULL || 32 * j + lane < m;
-        const unsigned int d = ok ? (unsigned int)((k[j] >> shift) & (R - 1)) : (unsigned int)R;
-        unsigned int peers = 0xffffffffu;  // lanes with the same digit (bit 8: past the end)
-#pragma unroll
-        for (int b = 0; b < (FULL ? RB : RB + 1); b++) {
-            const unsigned int bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-            peers &= ((d >> b) & 1u) ? bal : ~bal;
-        }
-        const unsigned int rank = __popc(peers & lt);
-        unsigned int prev = 0;
-        if (ok) prev = cnt[d];
-        __syncwarp();
-        if (ok && rank == 0) cnt[d] = prev + __popc(peers);
-        __syncwarp();
-        loc[j] = prev + rank;
-    }
-}
-
 // What a pass over the tree's keys does that another doesn't: the first of the low passes makes the values (the keys'
 // positions), both of them run only if the whole keys are sorted by passes (ctl->sort_whole), and the first of the
 // others makes the values if not.
@@ -179,8 +152,8 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
 #pragma unroll
         for (int j = 0; j < IPT; j++) v[j] = (uint32_t)(base + j * 32 + lane);
     }
-    if ((long long)(tile + 1) * TILE <= n) rank_keys<true>(k, shift, 32 * IPT, wcnt + w * R, loc);
-    else rank_keys<false>(k, shift, (int)(n - base < 0 ? 0 : (n - base < 32 * IPT ? n - base : 32 * IPT)), wcnt + w * R, loc);
+    if ((long long)(tile + 1) * TILE <= n) gt_rank_keys<true, IPT>(k, shift, 32 * IPT, wcnt + w * R, loc);
+    else gt_rank_keys<false, IPT>(k, shift, (int)(n - base < 0 ? 0 : (n - base < 32 * IPT ? n - base : 32 * IPT)), wcnt + w * R, loc);
     __syncthreads();
     // thread d < R: exclusive offsets of the warps for digit d, the tile's count of digit d
     const int d = threadIdx.x;
@@ -350,7 +323,7 @@ __global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, un
                         }
                     }
                 }
-                rank_keys<false>(k, s0, m, wcnt + w * R, loc);
+                gt_rank_keys<false, IPT>(k, s0, m, wcnt + w * R, loc);
                 __syncthreads();
                 uint32_t cnt = 0;
                 if (threadIdx.x < R)
@@ -416,6 +389,7 @@ size_t gt_sort_scratch_bytes(int64_t n) {
 }
 
 void gt_sort_init() {
+    gt_keys_init();
     for (auto kernel : {k_onesweep<PASS_PLAIN>, k_onesweep<PASS_LOW_FIRST>, k_onesweep<PASS_LOW>,
                         k_onesweep<PASS_HIGH_FIRST>})
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);

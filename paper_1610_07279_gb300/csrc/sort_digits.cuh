@@ -1,5 +1,5 @@
 // Digit counts of the radix sort's passes, gathered by the kernel that reads or makes the keys (blocks of
-// GT_SORT_DIGITS threads).
+// GT_SORT_DIGITS threads), and the ranking of keys by a digit.
 #pragma once
 
 #include "gt_internal.cuh"
@@ -70,4 +70,36 @@ __device__ __forceinline__ void gt_finish_digits(const uint32_t (*h)[GT_SORT_DIG
     }
     if (threadIdx.x < GT_SORT_PASSES) ctl->sort_ticket[threadIdx.x] = 0;
     if (threadIdx.x == 0) ctl->digits_done = ctl->run_count = 0;
+}
+
+// Stable rank of a lane's digit among those that the warp has counted into cnt (a count per digit) and its lower
+// lanes; the warp's digits are then counted too.  FULL: every lane has one; otherwise one without has GT_SORT_DIGITS.
+template <bool FULL>
+__device__ __forceinline__ uint32_t gt_rank_digit(uint32_t d, uint32_t *cnt) {
+    const bool ok = FULL || d < GT_SORT_DIGITS;
+    unsigned int peers = 0xffffffffu;  // lanes with the same digit (bit 8: none)
+#pragma unroll
+    for (int b = 0; b < (FULL ? GT_SORT_BITS : GT_SORT_BITS + 1); b++) {
+        const unsigned int bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        peers &= ((d >> b) & 1u) ? bal : ~bal;
+    }
+    const unsigned int rank = __popc(peers & lanemask_lt());
+    unsigned int prev = 0;
+    if (ok) prev = cnt[d];
+    __syncwarp();
+    if (ok && rank == 0) cnt[d] = prev + __popc(peers);
+    __syncwarp();
+    return prev + rank;
+}
+
+// The same for a warp's keys, item j of lane l being key 32 j + l of m.  FULL: m == 32 IPT.
+template <bool FULL, int IPT>
+__device__ __forceinline__ void gt_rank_keys(const unsigned long long (&k)[IPT], int shift, int m, uint32_t *cnt,
+                                             uint32_t (&loc)[IPT]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < IPT; j++) {
+        const bool ok = FULL || 32 * j + lane < m;
+        loc[j] = gt_rank_digit<FULL>(ok ? (uint32_t)(k[j] >> shift) & (GT_SORT_DIGITS - 1) : GT_SORT_DIGITS, cnt);
+    }
 }

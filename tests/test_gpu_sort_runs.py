@@ -32,6 +32,9 @@ def _clumps(sizes, n_field, radius, seed, far=None):
     ((), 30000, 0.0, (40000.0, 0.0, 0.0)),                      # all but one in a corner: crowded
     ((64,), 5000, 4e-6, (0.5, 3000.0, 0.5)),                    # near the crowding threshold
     ((), 1, 0.0, None), ((2,), 1, 0.0, None),
+    # one block's sort (at most 8192 particles): runs around its limit of 32, a run that takes all passes
+    ((2, 5, 31, 32, 33, 34), 8000, 4e-6, None), ((33,), 8160, 4e-6, None), ((3000,), 5192, 1e-5, None),
+    ((5000,), 300, 1e-9, None), ((), 8192, 0.0, (40000.0, 0.0, 0.0)), ((), 8193, 0.0, None), ((), 255, 0.0, None),
 ])
 def test_runs_of_equal_sorted_bits(env, sizes, n_field, radius, far):  # noqa: F811
     torch, g, O = env
