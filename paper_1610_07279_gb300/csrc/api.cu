@@ -394,10 +394,10 @@ void build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src) {
     ph_end(s, PH_PERMUTE, st);
     ph_begin(s, PH_BUILD, st);
     gt_launch_build(s->sb.key[0], n, s->prm.leaf_max, s->nd, s->cap, s->status, s->bscratch, s->ctl, s->nsm, st);
-    gt_launch_cell_lists(s->nd, s->cap, s->ctl, s->nsm, st);
+    gt_launch_cell_lists(s->nd, n, s->cap, s->ctl, s->nsm, st);
     ph_end(s, PH_BUILD, st);
     ph_begin(s, PH_PSEUDO, st);
-    gt_launch_pseudo(s->nd, s->cap, s->posm, s->ctl, s->nsm, true, st);
+    gt_launch_pseudo(s->nd, n, s->posm, s->ctl, s->nsm, true, st);
     ph_end(s, PH_PSEUDO, st);
     s->have_tree = true;
     s->rebuilds++;
@@ -525,7 +525,7 @@ void gt_sys_step_pre(gt_system *s, cudaStream_t st, bool rebuild, bool predicted
         build_tree(s, st, s->posm_tmp);
     } else {
         ph_begin(s, PH_PSEUDO, st);
-        gt_launch_pseudo(s->nd, s->cap, s->posm, s->ctl, s->nsm, false, st);  // masses as at the build
+        gt_launch_pseudo(s->nd, n, s->posm, s->ctl, s->nsm, false, st);  // masses as at the build
         ph_end(s, PH_PSEUDO, st);
     }
     ph_begin(s, PH_ACTIVE, st);

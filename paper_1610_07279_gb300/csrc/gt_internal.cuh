@@ -252,6 +252,14 @@ __device__ __forceinline__ unsigned int lookback_warp(unsigned long long *status
 // Every helper reports the kernels it launched (counted for gt_kernel_launches).
 void gt_note_launches(int k);
 
+// Blocks of a kernel that loops over its work: one for every `per` particles, at most `most`.  (The cells of a tree
+// are fewer than its particles but for chains, so `per` bounds the blocks with work; a full grid for each of many
+// small systems keeps the device busy with blocks that have none.)
+inline unsigned gt_grid(int64_t n, int64_t per, int64_t most) {
+    const int64_t b = (n + per - 1) / per;
+    return (unsigned)(b < 1 ? 1 : (b < most ? b : most));
+}
+
 #define GT_SMALL_SORT 8192           // systems whose keys one block makes and sorts
 #define GT_SORT_BITS 8
 #define GT_SORT_DIGITS 256
@@ -285,9 +293,9 @@ void gt_sort_init();
 size_t gt_build_scratch_bytes(int64_t n);
 void gt_launch_build(const uint64_t *skey, int64_t n, int leaf_max, Nodes nd, int64_t cap,
                      unsigned long long *status, uint8_t *scratch, DevCtl *ctl, int nsm, cudaStream_t st);
-void gt_launch_cell_lists(Nodes nd, int64_t cap, DevCtl *ctl, int nsm, cudaStream_t st);
+void gt_launch_cell_lists(Nodes nd, int64_t n, int64_t cap, DevCtl *ctl, int nsm, cudaStream_t st);
 // with_mass: form the FP64 mass sums (after a build); otherwise reuse the stored ones
-void gt_launch_pseudo(Nodes nd, int64_t cap, const float4 *posm, DevCtl *ctl, int nsm, bool with_mass,
+void gt_launch_pseudo(Nodes nd, int64_t n, const float4 *posm, DevCtl *ctl, int nsm, bool with_mass,
                       cudaStream_t st);
 // integrate.cu
 void gt_launch_prepare(DevCtl *ctl, int begin_step, cudaStream_t st);

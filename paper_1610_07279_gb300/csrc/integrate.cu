@@ -594,7 +594,7 @@ void gt_launch_gather_f(const float *in, const uint32_t *id, int64_t n, float *o
 
 void gt_launch_active(const State &s, int64_t n, int L, int all, DevCtl *ctl, uint32_t *active,
                       uint32_t *prefix, unsigned long long *status, int nsm, cudaStream_t st) {
-    { k_compact<<<nsm * 4, AT, 0, st>>>(n, nullptr, all ? CM_ALL : CM_TIME, s.t0, s.level, L, nullptr, ctl,
+    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(n, nullptr, all ? CM_ALL : CM_TIME, s.t0, s.level, L, nullptr, ctl,
                                         GT_TREE_LEVELS, 30u, active, prefix, &ctl->n_active, status);
       gt_note_launches(1); }
 }
@@ -604,7 +604,7 @@ void gt_launch_active_from_list(const uint32_t *list, int64_t n_list, int64_t n,
                                 cudaStream_t st) {
     if (n > 0) cudaMemsetAsync(flags, 0, (size_t)n, st);
     if (n_list > 0) { k_scatter_flags<<<nblk(n_list), 256, 0, st>>>(list, n_list, n, flags, ctl); gt_note_launches(1); }
-    { k_compact<<<nsm * 4, AT, 0, st>>>(n, nullptr, CM_FLAGS, nullptr, nullptr, 0, flags, ctl, GT_TREE_LEVELS,
+    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(n, nullptr, CM_FLAGS, nullptr, nullptr, 0, flags, ctl, GT_TREE_LEVELS,
                                         30u, active, prefix, &ctl->n_active, status);
       gt_note_launches(1); }
 }
@@ -613,15 +613,15 @@ void gt_launch_groups(Nodes nd, int64_t cap, const uint32_t *prefix, int gmax, f
                       uint8_t *marks, DevCtl *ctl, uint32_t *gstart, unsigned long long *status, int nsm,
                       cudaStream_t st) {
     if (n > 0) cudaMemsetAsync(marks, 0, (size_t)n, st);
-    { k_group_cells<<<nsm * 8, 256, 0, st>>>(nd, cap, prefix, gmax, r_crit, marks, ctl); gt_note_launches(1); }
-    { k_compact<<<nsm * 4, AT, 0, st>>>(0, &ctl->n_active, CM_FLAGS, nullptr, nullptr, 0, marks, ctl,
+    { k_group_cells<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(nd, cap, prefix, gmax, r_crit, marks, ctl); gt_note_launches(1); }
+    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(0, &ctl->n_active, CM_FLAGS, nullptr, nullptr, 0, marks, ctl,
                                         GT_TREE_LEVELS + 1, 31u, gstart, nullptr, &ctl->n_groups, status);
       gt_note_launches(1); }
 }
 
 void gt_launch_correct(const State &s, const uint32_t *active, const float4 *acc, DevCtl *ctl,
                        int64_t n, int L, double c2, int nsm, cudaStream_t st) {
-    if (n > 0) { k_correct<<<nsm * 8, 256, 0, st>>>(s, active, acc, ctl, n, L, c2); gt_note_launches(1); }
+    if (n > 0) { k_correct<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(s, active, acc, ctl, n, L, c2); gt_note_launches(1); }
 }
 
 void gt_launch_aold(const float4 *acc, int64_t n, float *aold, cudaStream_t st) {
@@ -641,7 +641,7 @@ void gt_launch_set_u32(unsigned int *dst, unsigned int v, cudaStream_t st) {
 }
 
 void gt_launch_tnext_all(const State &s, int64_t n, int L, DevCtl *ctl, int nsm, cudaStream_t st) {
-    if (n > 0) { k_tnext_all<<<nsm * 4, 256, 0, st>>>(s.t0, s.level, n, L, ctl); gt_note_launches(1); }
+    if (n > 0) { k_tnext_all<<<gt_grid(n, 256, nsm * 4), 256, 0, st>>>(s.t0, s.level, n, L, ctl); gt_note_launches(1); }
 }
 
 void gt_launch_gather_resume(const uint8_t *lv, const long long *t0, const float *ao, const float4 *acc,
@@ -652,6 +652,6 @@ void gt_launch_gather_resume(const uint8_t *lv, const long long *t0, const float
 void gt_launch_init_levels(const State &s, const float4 *acc, int64_t n, int L, double c2, int M_given,
                            int have_M, DevCtl *ctl, int nsm, cudaStream_t st) {
     { k_reset_start<<<1, 1, 0, st>>>(ctl); gt_note_launches(1); }
-    if (!have_M && n > 0) { k_min_a2<<<nsm * 4, 256, 0, st>>>(acc, n, ctl); gt_note_launches(1); }
-    { k_init_levels<<<nsm * 8, 256, 0, st>>>(s, acc, n, L, c2, M_given, have_M, ctl); gt_note_launches(1); }
+    if (!have_M && n > 0) { k_min_a2<<<gt_grid(n, 256, nsm * 4), 256, 0, st>>>(acc, n, ctl); gt_note_launches(1); }
+    { k_init_levels<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(s, acc, n, L, c2, M_given, have_M, ctl); gt_note_launches(1); }
 }

@@ -425,7 +425,7 @@ void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStrea
     const int64_t need = (n + 255) / 256, most = (int64_t)nsm * 16;
     k_fix_runs<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
                                                                       list, ctl);
-    k_fix_long_runs<<<nsm, ST, SCATTER_SMEM, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
+    k_fix_long_runs<<<gt_grid(n, 4 * TILE, nsm), ST, SCATTER_SMEM, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
                                                    (unsigned long long *)b.key[1], b.val[1], list, ctl);
     gt_note_launches(2);
 }

@@ -516,7 +516,6 @@ __global__ __launch_bounds__(256) void k_cell_fill(Nodes nd, long long cap, DevC
 #endif
 constexpr int PL = 128;  // nodes per chunk, one per thread
 constexpr uint32_t PU = GT_PSEUDO_PU, CU = GT_PSEUDO_CU;
-constexpr int PSEUDO_LAG = 1;  // levels of leaves between a level's cells and the level below
 constexpr int NSEG = 2 * GT_TREE_LEVELS;
 
 // Leaf c: one lane sums its particles in FP64 (mass, m x, m y, m z) in particle order.
@@ -718,28 +717,27 @@ __global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const f
     __shared__ int o_sh, bad_sh;
     for (int i = threadIdx.x; i <= NSEG; i += PL) seg[i] = ctl->seg[i];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < NSEG; k++) {
-            const uint32_t cnt = seg[k + 1] - seg[k];
-            coop[k] = (k & 1) && cnt <= (uint32_t)GT_PSEUDO_COOP;
-            const uint32_t per = coop[k] ? PL / 8 : PL;
-            nchunk[k] = (cnt + per - 1) / per;
-        }
-        int o = 0;  // level l's cells go right after the leaves of level l - PSEUDO_LAG
-        for (int s = 0; s < GT_TREE_LEVELS + PSEUDO_LAG; s++) {
-            const int ll = GT_TREE_LEVELS - 1 - s, lc = GT_TREE_LEVELS - 1 + PSEUDO_LAG - s;
-            if (ll >= 0) { olvl[o] = (uint8_t)ll; ocell[o] = 0; o++; }
-            if (lc >= 0 && lc < GT_TREE_LEVELS - 1) { olvl[o] = (uint8_t)lc; ocell[o] = 1; o++; }
-        }
-        // o == NSEG - 1 (level 21 has no cells with children): the last entry is empty
-        olvl[o] = 0; ocell[o] = 2;
-        uint32_t c = 0;
-        for (int k = 0; k < NSEG; k++) {
-            ocum[k] = c;
-            if (ocell[k] < 2) c += nchunk[2 * olvl[k] + ocell[k]];
-        }
-        ocum[NSEG] = c;
-        bad_sh = 0;
+    for (int k = threadIdx.x; k < NSEG; k += PL) {
+        const uint32_t cnt = seg[k + 1] - seg[k];
+        coop[k] = (k & 1) && cnt <= (uint32_t)GT_PSEUDO_COOP;
+        const uint32_t per = coop[k] ? PL / 8 : PL;
+        nchunk[k] = (cnt + per - 1) / per;
+        // the order of entries: the leaves of levels 21 and 20; then for l = 19 .. 0 the leaves of level l and the cells
+        // with children of level l + 1; those of level 0; an empty entry (level 21 has no cells with children)
+        const int kind = k < 2 ? 0 : (k < NSEG - 2 ? (k & 1) : k - (NSEG - 3));
+        const int lvl = k < 2 ? GT_TREE_LEVELS - 1 - k : (k < NSEG - 2 ? GT_TREE_LEVELS - 2 + (k & 1) - k / 2 : 0);
+        olvl[k] = (uint8_t)lvl;
+        ocell[k] = (uint8_t)kind;
+    }
+    if (threadIdx.x == 0) bad_sh = 0;
+    __syncthreads();
+    if (threadIdx.x < 32) {  // first tickets: entries l and l + 32 of lane l
+        const uint32_t l = threadIdx.x;
+        auto chunks = [&](uint32_t k) { return k < NSEG && ocell[k] < 2 ? nchunk[2 * olvl[k] + ocell[k]] : 0u; };
+        const uint32_t c0 = chunks(l), c1 = chunks(l + 32);
+        const uint32_t i0 = warp_incl_scan(c0), half = __shfl_sync(0xffffffffu, i0, 31), i1 = half + warp_incl_scan(c1);
+        ocum[l] = i0 - c0;
+        if (l + 32 <= NSEG) ocum[l + 32] = i1 - c1;
     }
     __syncthreads();
     const uint32_t total = ocum[NSEG];
@@ -853,7 +851,7 @@ void launch_flat(const unsigned long long *k, int64_t n, int leaf_max, Nodes nd,
     { k_flat_scan<<<NREC, 1024, 0, st>>>(cnt, ntiles, tot, cap, ctl); gt_note_launches(1); }
     if (ntiles > 0) {
         k_flat_scatter<ROUNDS><<<ntiles, FB, 0, st>>>(dl, n, cnt, ntiles, cap, nd, ctl);
-        { k_flat_link<<<nsm * 8, 256, 0, st>>>(nd, cap, ctl); }
+        { k_flat_link<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(nd, cap, ctl); }
         gt_note_launches(2);
     }
 }
@@ -874,15 +872,16 @@ void gt_launch_build(const uint64_t *skey, int64_t n, int leaf_max, Nodes nd, in
                                               status, ctl); gt_note_launches(1); }
 }
 
-void gt_launch_cell_lists(Nodes nd, int64_t cap, DevCtl *ctl, int nsm, cudaStream_t st) {
-    { k_cell_count<<<nsm * 4, 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
-    { k_cell_fill<<<nsm * 2, 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
+void gt_launch_cell_lists(Nodes nd, int64_t n, int64_t cap, DevCtl *ctl, int nsm, cudaStream_t st) {
+    { k_cell_count<<<gt_grid(n, 512, nsm * 4), 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
+    { k_cell_fill<<<gt_grid(n, 1024, nsm * 2), 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
 }
 
-void gt_launch_pseudo(Nodes nd, int64_t cap, const float4 *posm, DevCtl *ctl, int nsm, bool with_mass,
+void gt_launch_pseudo(Nodes nd, int64_t n, const float4 *posm, DevCtl *ctl, int nsm, bool with_mass,
                       cudaStream_t st) {
-    (void)cap;  // the ticket and the per-level counters were cleared by gt_launch_prepare
-    if (with_mass) { k_pseudo<true><<<nsm * GT_PSEUDO_MINB, PL, 0, st>>>(nd, posm, ctl); }
-    else { k_pseudo<false><<<nsm * GT_PSEUDO_MINB, PL, 0, st>>>(nd, posm, ctl); }
+    // the ticket and the per-level counters were cleared by gt_launch_prepare
+    const unsigned grid = gt_grid(n, 64, nsm * GT_PSEUDO_MINB);
+    if (with_mass) { k_pseudo<true><<<grid, PL, 0, st>>>(nd, posm, ctl); }
+    else { k_pseudo<false><<<grid, PL, 0, st>>>(nd, posm, ctl); }
     gt_note_launches(1);
 }
