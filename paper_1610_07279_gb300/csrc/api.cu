@@ -134,9 +134,9 @@ size_t carve(gt_system *s, char *base, int64_t n, const gt_params *p, int nsm, i
     const int64_t st_tiles = (cap + 511) / 512 + (n + 4095) / 4096 + 64;
     s->status = L.take<unsigned long long>(base, st_tiles);
     s->active = L.take<uint32_t>(base, N);
-    s->prefix = L.take<uint32_t>(base, N + 1);
-    s->flags = L.take<uint8_t>(base, N);
-    s->marks = L.take<uint8_t>(base, N);
+    s->flags = L.take<uint32_t>(base, N / 32 + 1);
+    s->marks = L.take<uint32_t>(base, N / 32 + 1);
+    s->rank = L.take<uint2>(base, N / 32 + 2);
     s->gstart = L.take<uint32_t>(base, N);
     s->acc_out = L.take<float4>(base, N);
     s->aold_tmp = L.take<float>(base, N);
@@ -365,14 +365,15 @@ bool in_place(const void *p, size_t align) {
 // then every particle array gathered into key order.  Buffer roles never change
 // (state 0 and posm always hold the current data), so the launches can be captured
 // in a CUDA graph and replayed.
-void build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src) {
+// prepared: gt_launch_prepare has just run.
+void build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src, bool prepared = false) {
     const int64_t n = s->n;
-    gt_launch_prepare(s->ctl, 0, st);
+    if (!prepared) gt_launch_prepare(s->ctl, 0, st);
     ph_begin(s, PH_SORT, st);
     if (n <= GT_SMALL_SORT) {
         gt_launch_small_sort(posm_src, n, s->prm.key_curve, s->sb, st);
     } else {
-        gt_launch_bbox(posm_src, n, s->nsm * 4, s->ctl, st);
+        gt_launch_bbox(posm_src, n, s->nsm * 4, s->ctl, s->sb, st);
         gt_launch_keys(posm_src, n, s->prm.key_curve, s->ctl, s->sb, s->nsm, st);
         gt_launch_sort_tree(s->sb, n, s->ctl, s->nsm, st);
     }
@@ -408,30 +409,38 @@ double c2_of(const gt_params &p) {
     return c * c;
 }
 
-// A6 groups + A7 walk over the active list already in s->active / ctl->n_active
-// (cell grouping needs the prefix s->prefix of that list), or over a caller's list.  levels: for the
-// integration (the forces choose the particles' levels).
+// A6: the groups of the active set in s->active / s->rank, or of every particle
+void groups(gt_system *s, bool all, cudaStream_t st) {
+    if (cell_groups(s->prm))
+        gt_launch_groups(s->nd, s->cap, all ? nullptr : s->rank, s->gmax_now, s->rcrit_now, s->n, s->marks, s->ctl,
+                         s->gstart, s->status, s->nsm, st);
+    else if (all)
+        gt_launch_set_nactive(s->ctl, (unsigned)s->n, st);
+}
+
+// A7 over the groups (or runs) of the active list.  levels: for the integration (the forces choose the particles'
+// levels).
 void walk(gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac, bool levels,
           cudaStream_t st) {
-    if (cell_groups(s->prm))
-        gt_launch_groups(s->nd, s->cap, s->prefix, s->gmax_now, s->rcrit_now, s->n, s->marks, s->ctl, s->gstart,
-                         s->status, s->nsm, st);
     const WalkArgs a = gt_sys_walk_args(s, active, aold, acc, mac, levels);
     ph_begin(s, PH_WALK, st);
     gt_launch_walk(a, s->walk_blocks, st);
     ph_end(s, PH_WALK, st);
 }
 
-// every particle active (start-up passes, gt_accel_active with no list)
-void walk_all(gt_system *s, const float *aold, float4 *acc, int mac, bool levels, cudaStream_t st) {
-    gt_launch_prepare(s->ctl, 0, st);
-    gt_launch_active(s->st[0], s->n, s->prm.levels, 1, s->ctl, s->active, s->prefix, s->status, s->nsm, st);
+// every particle active (start-up passes, gt_accel_active with no list); prepared: gt_launch_prepare has run, and
+// only a build since
+void walk_all(gt_system *s, const float *aold, float4 *acc, int mac, bool levels, bool prepared, cudaStream_t st) {
+    if (!prepared) gt_launch_prepare(s->ctl, 0, st);
+    groups(s, true, st);
     walk(s, nullptr, aold, acc, mac, levels, st);
 }
 
 }  // namespace
 
 // ---- helpers shared with the batch and the server ------------------------------
+bool gt_in_place(const void *p, size_t align) { return in_place(p, align); }
+
 int gt_sys_check_params(const gt_params *p) { return check_params(p); }
 
 int gt_sys_device_sms(int *dev, int *nsm) { return device_sms(dev, nsm); }
@@ -458,6 +467,8 @@ int gt_sys_init(gt_system *s, int64_t n, const gt_params *p, void *ws, size_t ws
     const size_t st_bytes = (size_t)((s->cap + 511) / 512 + (n + 4095) / 4096 + 64) * 8;
     if (cudaMemsetAsync(s->ctl, 0, sizeof(DevCtl), st) != cudaSuccess ||
         cudaMemsetAsync(s->status, 0, st_bytes, st) != cudaSuccess ||
+        // active, flags and marks
+        cudaMemsetAsync(s->active, 0, (size_t)((char *)s->rank - (char *)s->active), st) != cudaSuccess ||
         cudaMemsetAsync(s->sb.hist, 0, gt_sort_scratch_bytes(n), st) != cudaSuccess ||
         (st ? cudaStreamSynchronize(st) : cudaDeviceSynchronize()) != cudaSuccess)
         return GT_ECUDA;
@@ -474,13 +485,7 @@ void gt_sys_apply_params(gt_system *s, const gt_params &p) {
 
 void gt_sys_build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src) { build_tree(s, st, posm_src); }
 
-void gt_sys_groups_all(gt_system *s, cudaStream_t st) {
-    gt_launch_prepare(s->ctl, 0, st);
-    gt_launch_active(s->st[0], s->n, s->prm.levels, 1, s->ctl, s->active, s->prefix, s->status, s->nsm, st);
-    if (cell_groups(s->prm))
-        gt_launch_groups(s->nd, s->cap, s->prefix, s->gmax_now, s->rcrit_now, s->n, s->marks, s->ctl, s->gstart,
-                         s->status, s->nsm, st);
-}
+void gt_sys_groups_all(gt_system *s, cudaStream_t st) { groups(s, true, st); }
 
 WalkArgs gt_sys_walk_args(const gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac,
                           bool levels) {
@@ -522,22 +527,18 @@ void gt_sys_step_pre(gt_system *s, cudaStream_t st, bool rebuild, bool predicted
         std::swap(s->posm, s->posm_tmp);  // the prediction enqueued ahead went to posm_tmp
     }
     if (rebuild) {
-        build_tree(s, st, s->posm_tmp);
+        build_tree(s, st, s->posm_tmp, true);
     } else {
         ph_begin(s, PH_PSEUDO, st);
         gt_launch_pseudo(s->nd, n, s->posm, s->ctl, s->nsm, false, st);  // masses as at the build
         ph_end(s, PH_PSEUDO, st);
     }
     ph_begin(s, PH_ACTIVE, st);
-    gt_launch_active(s->st[0], n, s->prm.levels, 0, s->ctl, s->active, s->prefix, s->status, s->nsm, st);
+    gt_launch_active(s->st[0], n, s->prm.levels, s->ctl, s->active, s->rank, s->status, s->nsm, st);
     ph_end(s, PH_ACTIVE, st);
 }
 
-void gt_sys_step_groups(gt_system *s, cudaStream_t st) {
-    if (cell_groups(s->prm))
-        gt_launch_groups(s->nd, s->cap, s->prefix, s->gmax_now, s->rcrit_now, s->n, s->marks, s->ctl, s->gstart,
-                         s->status, s->nsm, st);
-}
+void gt_sys_step_groups(gt_system *s, cudaStream_t st) { groups(s, false, st); }
 
 void gt_sys_step_post(gt_system *s, cudaStream_t st) {
     ph_begin(s, PH_CORRECT, st);
@@ -701,11 +702,12 @@ int gt_accel_active(gt_system *s, const uint32_t *d_active, int64_t n_active, co
     drop_ahead(s, st);
     const float *aold = d_aold ? d_aold : s->st[0].aold;
     if (!d_active) {
-        walk_all(s, aold, (float4 *)d_acc, s->prm.mac, false, st);
+        walk_all(s, aold, (float4 *)d_acc, s->prm.mac, false, false, st);
     } else if (cell_groups(s->prm)) {
         gt_launch_prepare(s->ctl, 0, st);
-        gt_launch_active_from_list(d_active, n_active, s->n, s->flags, s->ctl, s->active, s->prefix, s->status,
+        gt_launch_active_from_list(d_active, n_active, s->n, s->flags, s->ctl, s->active, s->rank, s->status,
                                    s->nsm, st);
+        groups(s, false, st);
         walk(s, s->active, aold, (float4 *)d_acc, s->prm.mac, false, st);
     } else {
         gt_launch_prepare(s->ctl, 0, st);
@@ -727,11 +729,11 @@ int gt_start(gt_system *s, const float *p_aold_boot, gt_stream stream) {
             return GT_ECUDA;
         gt_launch_gather_f(s->aold_tmp, t.id, n, t.aold, st);
     } else {
-        walk_all(s, nullptr, s->acc_out, GT_MAC_OPENING_ANGLE, false, st);
+        walk_all(s, nullptr, s->acc_out, GT_MAC_OPENING_ANGLE, false, true, st);
         gt_launch_aold(s->acc_out, n, t.aold, st);
         ph_sync_collect(s, st);
     }
-    walk_all(s, t.aold, s->acc_out, s->prm.mac, true, st);
+    walk_all(s, t.aold, s->acc_out, s->prm.mac, true, p_aold_boot != nullptr, st);
     gt_sys_start_levels(s, st);
     return last_cuda();
 }
@@ -785,6 +787,7 @@ int gt_block_step(gt_system *s, gt_stream stream) {
     s->last_rebuilt = rebuild;
     gt_sys_step_pre(s, st, rebuild, predicted);
     State &t = s->st[0];
+    groups(s, false, st);
     walk(s, s->active, t.aold, s->acc_out, s->prm.mac, true, st);
     gt_sys_step_post(s, st);
     // Look-ahead (automatic interval; the tuners wait for every step): the control
@@ -1001,6 +1004,7 @@ int gt_get_active(gt_system *s, uint32_t *p_active, int64_t *n_inout, gt_stream 
     *n_inout = na;
     if (!p_active) return GT_OK;
     if ((int64_t)na > cap) return GT_EOVERFLOW;
+    if ((int64_t)na == s->n) gt_launch_iota(s->active, s->n, st);  // walks over every particle don't write the list
     if (na && cudaMemcpyAsync(p_active, s->active, (size_t)na * 4, cudaMemcpyDefault, st)) return GT_ECUDA;
     return cudaStreamSynchronize(st) ? GT_ECUDA : GT_OK;
 }

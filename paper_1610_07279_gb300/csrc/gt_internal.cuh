@@ -274,8 +274,8 @@ struct SortBufs {
 };
 
 // keys.cu
-// extrema into ctl->bbox (reset by gt_launch_prepare); keys and their digit counts for gt_launch_sort_tree
-void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, cudaStream_t st);
+// extrema into ctl->bbox (reset by gt_launch_prepare), and the sort's counts and look-back words cleared; keys and their digit counts for gt_launch_sort_tree
+void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, SortBufs &b, cudaStream_t st);
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st);
 // box, keys and sort of at most GT_SMALL_SORT particles in one launch
 void gt_keys_init();
@@ -284,7 +284,6 @@ void gt_launch_small_sort(const float4 *posm, int64_t n, int curve, SortBufs &b,
 // their positions as values, into buffers 0
 int gt_sort_tiles(int64_t n);
 size_t gt_sort_scratch_bytes(int64_t n);
-void gt_sort_clear(SortBufs &b, int64_t n, cudaStream_t st);  // the digit counts and the look-back words
 void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st);
 void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStream_t st);
 void gt_sort_init();
@@ -326,14 +325,19 @@ void gt_launch_interleave3(const double *x, const double *y, const double *z, in
                            cudaStream_t st);
 void gt_launch_state_out(const State &t, int64_t n, double *pos, double *vel, cudaStream_t st);
 void gt_launch_gather_f(const float *in, const uint32_t *id, int64_t n, float *out, cudaStream_t st);
-void gt_launch_active(const State &s, int64_t n, int L, int all, DevCtl *ctl, uint32_t *active,
-                      uint32_t *prefix, unsigned long long *status, int nsm, cudaStream_t st);
-void gt_launch_active_from_list(const uint32_t *list, int64_t n_list, int64_t n, uint8_t *flags, DevCtl *ctl,
-                                uint32_t *active, uint32_t *prefix, unsigned long long *status, int nsm,
-                                cudaStream_t st);
-void gt_launch_groups(Nodes nd, int64_t cap, const uint32_t *prefix, int gmax, float r_crit, int64_t n,
-                      uint8_t *marks, DevCtl *ctl, uint32_t *gstart, unsigned long long *status, int nsm,
-                      cudaStream_t st);
+// The active set at the block time, or a caller's list: the indices in order and the rank words (32 particles' mask
+// and the number of actives before them; n / 32 + 1 words).  flags: a bit per particle, zero between calls.
+void gt_launch_active(const State &s, int64_t n, int L, DevCtl *ctl, uint32_t *active, uint2 *rank,
+                      unsigned long long *status, int nsm, cudaStream_t st);
+void gt_launch_active_from_list(const uint32_t *list, int64_t n_list, int64_t n, uint32_t *flags, DevCtl *ctl,
+                                uint32_t *active, uint2 *rank, unsigned long long *status, int nsm, cudaStream_t st);
+void gt_launch_iota(uint32_t *out, int64_t n, cudaStream_t st);
+void gt_launch_acc_out(const float4 *acc, const uint32_t *id, int64_t n, float4 *acc_out, uint32_t *id_out,
+                       cudaStream_t st);
+// Groups of the active set with these rank words, or (rank null) of every particle, whose number it then makes the
+// number of actives.  marks: a bit per active, zero between calls.
+void gt_launch_groups(Nodes nd, int64_t cap, const uint2 *rank, int gmax, float r_crit, int64_t n, uint32_t *marks,
+                      DevCtl *ctl, uint32_t *gstart, unsigned long long *status, int nsm, cudaStream_t st);
 void gt_launch_correct(const State &s, const uint32_t *active, const float4 *acc, DevCtl *ctl,
                        int64_t n, int L, double c2, int nsm, cudaStream_t st);
 void gt_launch_aold(const float4 *acc, int64_t n, float *aold, cudaStream_t st);

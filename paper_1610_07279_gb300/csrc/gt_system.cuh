@@ -81,10 +81,10 @@ struct gt_system {
     SortBufs sb{};
     Nodes nd{};
     unsigned long long *status = nullptr;
-    uint32_t *active = nullptr;
-    uint32_t *prefix = nullptr;   // P[i] = actives below internal index i (n + 1 entries)
-    uint8_t *flags = nullptr;     // a caller's active list as flags
-    uint8_t *marks = nullptr;     // first active position of every group
+    uint32_t *active = nullptr;   // not written by walks over every particle
+    uint2 *rank = nullptr;        // per 32 particles: their mask of actives, and the number of actives before
+    uint32_t *flags = nullptr;    // a caller's active list, a bit per particle
+    uint32_t *marks = nullptr;    // first active position of every group, a bit per active
     uint32_t *gstart = nullptr;   // group starts (cell grouping)
     float4 *acc_out = nullptr;
     float *aold_tmp = nullptr;
@@ -108,6 +108,8 @@ struct gt_system {
 constexpr size_t GT_WS_ALIGN = 256;
 
 int gt_sys_check_params(const gt_params *p);
+// whether a kernel may take a caller's array in place (memory of this device, aligned)
+bool gt_in_place(const void *p, size_t align);
 int gt_sys_device_sms(int *dev, int *nsm);
 // Carve every buffer of a system out of base (or only measure when base == nullptr);
 // own_queue == false leaves the walk queue to the caller (a batch).
@@ -122,7 +124,7 @@ int gt_sys_init(gt_system *s, int64_t n, const gt_params *p, void *ws, size_t ws
 void gt_sys_apply_params(gt_system *s, const gt_params &p);
 // A1-A5 on FP32 positions posm_src
 void gt_sys_build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src);
-// A6 with every particle active: the active list and, for cell grouping, the groups
+// A6 with every particle active, right after a build: for cell grouping, the groups
 void gt_sys_groups_all(gt_system *s, cudaStream_t st);
 // arguments of one walk over the current active list / groups; levels: its forces choose the particles' levels
 WalkArgs gt_sys_walk_args(const gt_system *s, const uint32_t *active, const float *aold, float4 *acc, int mac,

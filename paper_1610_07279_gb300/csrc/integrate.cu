@@ -5,9 +5,11 @@
 //                  rounded to FP32 for the tree                    (HBM: 60 B read, 16 B written)
 //   k_permute      A3: gather every particle array into key order  (HBM: ~100 B each way)
 //   k_compact      A6: order-preserving compaction with a block scan and a bounded decoupled
-//                  look-back; selects by block time (t0 + ticks(level) == T), by a flag array,
-//                  or all, and writes the active prefix P[i] = #actives below i
-//                  (HBM: 9 B read + 4 B prefix per particle, 4 B per active)
+//                  look-back; selects by block time (t0 + ticks(level) == T) and writes the actives
+//                  and, per 32 particles, their mask and the number of actives before (from
+//                  which rank_at has the number below any i: 1/16 of the 4 B per particle of a prefix)
+//                  (HBM: 9 B read per particle, 4 B per active)
+//   k_compact_bits A6: the same for a bit mask (a caller's list, group starts), which it clears
 //   k_group_cells  A6: groups bounded by tree cells (Sec. 2.4): the actives of every maximal
 //                  cell with at most group_max of them (or of a leaf, cut into runs)
 //   k_correct      A9: Eq. (17), the new level, the next half kick; the active particles'
@@ -208,18 +210,18 @@ __global__ __launch_bounds__(256) void k_gather_f(const float *__restrict__ in, 
     if (i < n) out[i] = in[id[i]];
 }
 
-// flags[active[k]] = 1 for a caller's list; a list that is not strictly increasing or
+// bit active[k] set for a caller's list; a list that is not strictly increasing or
 // holds an index >= n latches GT_EINVAL (the cell grouping needs key order)
 __global__ __launch_bounds__(256) void k_scatter_flags(const uint32_t *__restrict__ active, long long na,
-                                                       long long n, uint8_t *__restrict__ flags, DevCtl *ctl) {
+                                                       long long n, uint32_t *__restrict__ bits, DevCtl *ctl) {
     const long long k = blockIdx.x * 256ll + threadIdx.x;
-    if (k >= na) return;
-    const uint32_t i = active[k];
-    if ((long long)i >= n || (k > 0 && active[k - 1] >= i)) {
-        gt_set_error(ctl, GT_EINVAL, GTK_ACTIVE);
-        return;
-    }
-    flags[i] = 1;
+    const uint32_t i = k < na ? active[k] : 0u;
+    const bool bad = k < na && ((long long)i >= n || (k > 0 && active[k - 1] >= i)), on = k < na && !bad;
+    if (bad) gt_set_error(ctl, GT_EINVAL, GTK_ACTIVE);
+    // one atomic per word of the warp's entries (a tenth of 10^6 active: 2.9 us, one per entry 6.1 us)
+    const unsigned int peers = __match_any_sync(0xffffffffu, on ? i >> 5 : ~0u);
+    const uint32_t mask = __reduce_or_sync(peers, on ? 1u << (i & 31u) : 0u);
+    if (on && __ffs(peers) - 1 == lane_id()) atomicOr(&bits[i >> 5], mask);
 }
 
 constexpr int AT = 256, AIPT = 16, ATILE = AT * AIPT;
@@ -233,30 +235,22 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
     return v;
 }
 
-enum { CM_TIME = 0, CM_ALL = 1, CM_FLAGS = 2 };
-
-// Order-preserving compaction of [0, n) (n from n_dev if given).  Writes the selected
-// indices to out, the prefix P[i] = #selected below i (i = 0..n) if prefix != null,
-// and the count to *count_out.  CM_TIME also folds the unselected particles' step
-// ends into the next block time.
-__global__ __launch_bounds__(AT) void k_compact(long long n_host, const unsigned int *n_dev, int mode,
-                                                const long long *__restrict__ t0,
-                                                const uint8_t *__restrict__ level, int L,
-                                                const uint8_t *__restrict__ flags, DevCtl *ctl,
-                                                int ticket, uint32_t tag_slot, uint32_t *__restrict__ out,
-                                                uint32_t *__restrict__ prefix, unsigned int *count_out,
-                                                unsigned long long *status) {
+// Order-preserving compaction of the particles whose step ends at the block time.  Writes their indices to out, the
+// rank words (rank[n / 32] too), the count to ctl->n_active, and folds the others' step ends into the next block time.
+__global__ __launch_bounds__(AT) void k_compact(long long n, const long long *__restrict__ t0,
+                                                const uint8_t *__restrict__ level, int L, DevCtl *ctl, int ticket,
+                                                uint32_t tag_slot, uint32_t *__restrict__ out,
+                                                uint2 *__restrict__ rank, unsigned long long *status) {
     __shared__ uint32_t tmp[AT / 32 + 1];
     __shared__ uint32_t tile_sh, excl_sh;
-    const long long n = n_dev ? (long long)*n_dev : n_host;
     const unsigned long long T = ctl->tnext;
     const uint32_t tag = ctl->epoch * 32u + tag_slot;
     const uint32_t ntiles = (uint32_t)((n + ATILE - 1) / ATILE);
     unsigned long long tmin = ~0ull;
     if (n == 0) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
-            *count_out = 0;
-            if (prefix) prefix[0] = 0;
+            ctl->n_active = 0;
+            rank[0] = make_uint2(0u, 0u);
         }
         return;
     }
@@ -278,16 +272,9 @@ __global__ __launch_bounds__(AT) void k_compact(long long n_host, const unsigned
             const long long i = wbase + 32 * q + lane;
             bool on = false;
             if (i < n) {
-                if (mode == CM_ALL) {
-                    on = true;
-                } else if (mode == CM_FLAGS) {
-                    on = flags[i] != 0;
-                } else {
-                    const unsigned long long tend =
-                        (unsigned long long)t0[i] + (1ull << (L - 1 - (int)level[i]));
-                    on = tend == T;
-                    if (!on) tmin = tend < tmin ? tend : tmin;
-                }
+                const unsigned long long tend = (unsigned long long)t0[i] + (1ull << (L - 1 - (int)level[i]));
+                on = tend == T;
+                if (!on) tmin = tend < tmin ? tend : tmin;
             }
             bal[q] = __ballot_sync(0xffffffffu, on);
             wsel += (uint32_t)__popc(bal[q]);
@@ -303,23 +290,87 @@ __global__ __launch_bounds__(AT) void k_compact(long long n_host, const unsigned
         __syncthreads();
         uint32_t pos = excl_sh + wstart;
         const unsigned int lt = lanemask_lt();
+        uint2 mine = make_uint2(0u, 0u);  // lane q keeps row q's rank word
 #pragma unroll
         for (int q = 0; q < AIPT; q++) {
             const long long i = wbase + 32 * q + lane;
-            const uint32_t at = pos + (uint32_t)__popc(bal[q] & lt);
-            if (i < n && prefix) prefix[i] = at;
-            if ((bal[q] >> lane) & 1u) out[at] = (uint32_t)i;
+            if (lane == q) mine = make_uint2(bal[q], pos);
+            if ((bal[q] >> lane) & 1u) out[pos + (uint32_t)__popc(bal[q] & lt)] = (uint32_t)i;
             pos += (uint32_t)__popc(bal[q]);
+        }
+        if (lane < AIPT && wbase + 32 * lane < n) rank[(wbase >> 5) + lane] = mine;
+        if (tile == ntiles - 1 && threadIdx.x == AT - 1) {
+            ctl->n_active = excl_sh + total;
+            if (n % 32 == 0) rank[n >> 5] = make_uint2(0u, excl_sh + total);
+        }
+    }
+    tmin = warp_min_u64(tmin);
+    if (lane_id() == 0 && tmin != ~0ull) atomicMin(&ctl->tnext_acc, tmin);
+}
+
+// Order-preserving compaction of the bits of [0, n) (n from n_dev if given), which are cleared on the way (masks
+// start at zero, so that no launch has to clear them).  Writes the indices to out, the rank words if rank != null
+// (rank[n / 32] too), and the count to *count_out.  A lane takes a word of 32 items, 8192 items to a
+// tile: at 2^24 items the masks are 2 MB, in L2, where a byte each was 16 MB to clear, write and read.  100 000 of 2^24
+// active, the whole walk: 282 us with bytes, 236 with four words per lane (too few blocks), 225.
+constexpr int BTILE = AT;  // words per tile, a word per lane
+
+__global__ __launch_bounds__(AT) void k_compact_bits(long long n_host, const unsigned int *n_dev,
+                                                     uint32_t *__restrict__ bits, DevCtl *ctl, int ticket,
+                                                     uint32_t tag_slot, uint32_t *__restrict__ out,
+                                                     uint2 *__restrict__ rank, unsigned int *count_out,
+                                                     unsigned long long *status) {
+    __shared__ uint32_t tmp[AT / 32 + 1];
+    __shared__ uint32_t tile_sh, excl_sh;
+    const long long n = n_dev ? (long long)*n_dev : n_host;
+    const uint32_t tag = ctl->epoch * 32u + tag_slot;
+    const long long nwords = (n + 31) / 32;
+    const uint32_t ntiles = (uint32_t)((nwords + BTILE - 1) / BTILE);
+    if (n == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            *count_out = 0;
+            if (rank) rank[0] = make_uint2(0u, 0u);
+        }
+        return;
+    }
+    for (;;) {
+        if (threadIdx.x == 0) tile_sh = atomicAdd(&ctl->tile_ticket[ticket], 1u);
+        __syncthreads();
+        const uint32_t tile = tile_sh;
+        __syncthreads();
+        if (tile >= ntiles) break;
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const long long wbase = (long long)tile * BTILE + 32 * w, i = wbase + lane;  // the warp's first word, the lane's
+        const uint32_t word = i < nwords ? bits[i] : 0u;
+        if (word) bits[i] = 0u;
+        const uint32_t incl = warp_incl_scan((uint32_t)__popc(word));
+        uint32_t total;
+        const uint32_t wexcl = block_excl_scan<AT>(lane == 31 ? incl : 0u, &total, tmp);
+        const uint32_t wstart = __shfl_sync(0xffffffffu, wexcl, 31);
+        if (threadIdx.x < 32) {
+            const uint32_t e = lookback_warp(status, tile, total, tag, ctl, GTK_ACTIVE);
+            if (threadIdx.x == 0) excl_sh = e;
+        }
+        __syncthreads();
+        const uint32_t start = excl_sh + wstart + incl - (uint32_t)__popc(word);
+        if (rank && i < nwords) rank[i] = make_uint2(word, start);
+        const unsigned int lt = lanemask_lt();
+        for (unsigned int m = __ballot_sync(0xffffffffu, word != 0u); m; m &= m - 1) {  // a word at a time
+            const int src = __ffs(m) - 1;
+            const uint32_t b = __shfl_sync(0xffffffffu, word, src), at = __shfl_sync(0xffffffffu, start, src);
+            if ((b >> lane) & 1u) out[at + (uint32_t)__popc(b & lt)] = (uint32_t)(32 * (wbase + src) + lane);
         }
         if (tile == ntiles - 1 && threadIdx.x == AT - 1) {
             *count_out = excl_sh + total;
-            if (prefix) prefix[n] = excl_sh + total;
+            if (rank && n % 32 == 0) rank[n >> 5] = make_uint2(0u, excl_sh + total);
         }
     }
-    if (mode == CM_TIME) {
-        tmin = warp_min_u64(tmin);
-        if (lane_id() == 0 && tmin != ~0ull) atomicMin(&ctl->tnext_acc, tmin);
-    }
+}
+
+// The number of actives below i.
+__device__ __forceinline__ uint32_t rank_at(const uint2 *__restrict__ rank, uint32_t i) {
+    const uint2 r = rank[i >> 5];
+    return r.y + (uint32_t)__popc(r.x & ((1u << (i & 31u)) - 1u));
 }
 
 // Mark the first active position of every group (Sec. 2.4 reading: groups never
@@ -328,27 +379,45 @@ __global__ __launch_bounds__(AT) void k_compact(long long n_host, const unsigned
 // and radii only shrink from a cell to its children, so a group cell is a qualifying
 // cell whose parent does not qualify (or the root), or a leaf under no qualifying cell;
 // its actives are cut into runs of gmax.
-__device__ __forceinline__ bool group_cell_ok(const Nodes &nd, const uint32_t *P, uint32_t c, int gmax,
-                                              float r_crit) {
-    const uint32_t f = nd.first[c];
-    if (P[f + nd.count[c]] - P[f] > (uint32_t)gmax) return false;
+// ALL: every particle is active (the number below i is i).
+template <bool ALL>
+__device__ __forceinline__ bool group_cell_ok(const Nodes &nd, const uint2 *R, uint32_t c, int gmax, float r_crit) {
+    const uint32_t f = nd.first[c], k = nd.count[c];
+    if ((ALL ? k : rank_at(R, f + k) - rank_at(R, f)) > (uint32_t)gmax) return false;
     return nd.child[c] < 0 || r_crit <= 0.0f || nd.walk[c].x <= r_crit;
 }
 
-__global__ __launch_bounds__(256) void k_group_cells(Nodes nd, long long cap, const uint32_t *__restrict__ P,
-                                                     int gmax, float r_crit, uint8_t *__restrict__ marks,
-                                                     const DevCtl *ctl) {
+template <bool ALL>
+__global__ __launch_bounds__(256) void k_group_cells(Nodes nd, long long n, long long cap, const uint2 *__restrict__ R,
+                                                     int gmax, float r_crit, uint32_t *__restrict__ marks,
+                                                     DevCtl *ctl) {
     long long nn = ctl->level_start[GT_TREE_LEVELS];
     if (nn > cap) nn = cap;
+    if (ALL && blockIdx.x == 0 && threadIdx.x == 0) ctl->n_active = (unsigned int)n;
     for (long long c = blockIdx.x * 256ll + threadIdx.x; c < nn; c += (long long)gridDim.x * 256) {
-        const uint32_t f = nd.first[c];
-        const uint32_t a0 = P[f], A = P[f + nd.count[c]] - a0;
+        const uint32_t f = nd.first[c], k = nd.count[c];
+        const uint32_t a0 = ALL ? f : rank_at(R, f), A = ALL ? k : rank_at(R, f + k) - a0;
         if (A == 0) continue;
         const int32_t p = nd.parent[c];
-        if (p >= 0 && group_cell_ok(nd, P, (uint32_t)p, gmax, r_crit)) continue;  // inside a group cell
-        if (nd.child[c] >= 0 && !group_cell_ok(nd, P, (uint32_t)c, gmax, r_crit)) continue;  // children decide
-        for (uint32_t s = a0; s < a0 + A; s += (uint32_t)gmax) marks[s] = 1;
+        if (p >= 0 && group_cell_ok<ALL>(nd, R, (uint32_t)p, gmax, r_crit)) continue;  // inside a group cell
+        if (nd.child[c] >= 0 && !group_cell_ok<ALL>(nd, R, (uint32_t)c, gmax, r_crit)) continue;  // children decide
+        for (uint32_t s = a0; s < a0 + A; s += (uint32_t)gmax) atomicOr(&marks[s >> 5], 1u << (s & 31u));
     }
+}
+
+// a batch member's accelerations and ids to the caller
+__global__ __launch_bounds__(256) void k_acc_out(const float4 *__restrict__ acc, const uint32_t *__restrict__ id,
+                                                 long long n, float4 *__restrict__ acc_out,
+                                                 uint32_t *__restrict__ id_out) {
+    const long long i = blockIdx.x * 256ll + threadIdx.x;
+    if (i >= n) return;
+    if (acc_out) acc_out[i] = acc[i];
+    if (id_out) id_out[i] = id[i];
+}
+
+__global__ __launch_bounds__(256) void k_iota(uint32_t *__restrict__ out, long long n) {
+    const long long i = blockIdx.x * 256ll + threadIdx.x;
+    if (i < n) out[i] = (uint32_t)i;
 }
 
 __device__ __forceinline__ double a2_of(float4 a) {
@@ -592,31 +661,38 @@ void gt_launch_gather_f(const float *in, const uint32_t *id, int64_t n, float *o
     if (n > 0) { k_gather_f<<<nblk(n), 256, 0, st>>>(in, id, n, out); gt_note_launches(1); }
 }
 
-void gt_launch_active(const State &s, int64_t n, int L, int all, DevCtl *ctl, uint32_t *active,
-                      uint32_t *prefix, unsigned long long *status, int nsm, cudaStream_t st) {
-    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(n, nullptr, all ? CM_ALL : CM_TIME, s.t0, s.level, L, nullptr, ctl,
-                                        GT_TREE_LEVELS, 30u, active, prefix, &ctl->n_active, status);
+void gt_launch_active(const State &s, int64_t n, int L, DevCtl *ctl, uint32_t *active, uint2 *rank,
+                      unsigned long long *status, int nsm, cudaStream_t st) {
+    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(n, s.t0, s.level, L, ctl, GT_TREE_LEVELS, 30u, active, rank,
+                                                           status);
       gt_note_launches(1); }
 }
 
-void gt_launch_active_from_list(const uint32_t *list, int64_t n_list, int64_t n, uint8_t *flags, DevCtl *ctl,
-                                uint32_t *active, uint32_t *prefix, unsigned long long *status, int nsm,
-                                cudaStream_t st) {
-    if (n > 0) cudaMemsetAsync(flags, 0, (size_t)n, st);
+void gt_launch_active_from_list(const uint32_t *list, int64_t n_list, int64_t n, uint32_t *flags, DevCtl *ctl,
+                                uint32_t *active, uint2 *rank, unsigned long long *status, int nsm, cudaStream_t st) {
     if (n_list > 0) { k_scatter_flags<<<nblk(n_list), 256, 0, st>>>(list, n_list, n, flags, ctl); gt_note_launches(1); }
-    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(n, nullptr, CM_FLAGS, nullptr, nullptr, 0, flags, ctl, GT_TREE_LEVELS,
-                                        30u, active, prefix, &ctl->n_active, status);
+    { k_compact_bits<<<gt_grid(n, 32 * BTILE, nsm * 4), AT, 0, st>>>(n, nullptr, flags, ctl, GT_TREE_LEVELS, 30u, active,
+                                                                     rank, &ctl->n_active, status);
       gt_note_launches(1); }
 }
 
-void gt_launch_groups(Nodes nd, int64_t cap, const uint32_t *prefix, int gmax, float r_crit, int64_t n,
-                      uint8_t *marks, DevCtl *ctl, uint32_t *gstart, unsigned long long *status, int nsm,
-                      cudaStream_t st) {
-    if (n > 0) cudaMemsetAsync(marks, 0, (size_t)n, st);
-    { k_group_cells<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(nd, cap, prefix, gmax, r_crit, marks, ctl); gt_note_launches(1); }
-    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(0, &ctl->n_active, CM_FLAGS, nullptr, nullptr, 0, marks, ctl,
-                                        GT_TREE_LEVELS + 1, 31u, gstart, nullptr, &ctl->n_groups, status);
-      gt_note_launches(1); }
+void gt_launch_acc_out(const float4 *acc, const uint32_t *id, int64_t n, float4 *acc_out, uint32_t *id_out,
+                       cudaStream_t st) {
+    if (n > 0) { k_acc_out<<<nblk(n), 256, 0, st>>>(acc, id, n, acc_out, id_out); gt_note_launches(1); }
+}
+
+void gt_launch_iota(uint32_t *out, int64_t n, cudaStream_t st) {
+    if (n > 0) { k_iota<<<nblk(n), 256, 0, st>>>(out, n); gt_note_launches(1); }
+}
+
+void gt_launch_groups(Nodes nd, int64_t cap, const uint2 *rank, int gmax, float r_crit, int64_t n, uint32_t *marks,
+                      DevCtl *ctl, uint32_t *gstart, unsigned long long *status, int nsm, cudaStream_t st) {
+    const unsigned grid = gt_grid(n, 256, nsm * 8);
+    if (rank) k_group_cells<false><<<grid, 256, 0, st>>>(nd, n, cap, rank, gmax, r_crit, marks, ctl);
+    else k_group_cells<true><<<grid, 256, 0, st>>>(nd, n, cap, rank, gmax, r_crit, marks, ctl);
+    k_compact_bits<<<gt_grid(n, 32 * BTILE, nsm * 4), AT, 0, st>>>(0, &ctl->n_active, marks, ctl, GT_TREE_LEVELS + 1, 31u,
+                                                                   gstart, nullptr, &ctl->n_groups, status);
+    gt_note_launches(2);
 }
 
 void gt_launch_correct(const State &s, const uint32_t *active, const float4 *acc, DevCtl *ctl,

@@ -18,7 +18,12 @@ constexpr int BBOX_THREADS = 256;
 // more than the warps hide (2^20: 407 us the whole build at 4, 413 at 8; 2^24: 3009 and 3001).
 constexpr int64_t KEYS_MANY = 1 << 22;
 
-__global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict__ posm, long long n, DevCtl *ctl) {
+__global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict__ posm, long long n, DevCtl *ctl,
+                                                       uint4 *__restrict__ clear, long long nclear) {
+    // the sort's counts and look-back words, which the next launch wants at zero
+    for (long long i = blockIdx.x * (long long)BBOX_THREADS + threadIdx.x; i < nclear;
+         i += (long long)gridDim.x * BBOX_THREADS)
+        clear[i] = make_uint4(0u, 0u, 0u, 0u);
     float mn0 = FLT_MAX, mn1 = FLT_MAX, mn2 = FLT_MAX;
     float mx0 = -FLT_MAX, mx1 = -FLT_MAX, mx2 = -FLT_MAX;
     for (long long i = blockIdx.x * (long long)BBOX_THREADS + threadIdx.x; i < n;
@@ -310,15 +315,16 @@ __global__ __launch_bounds__(SMALL_THREADS) void k_small_sort(const float4 *__re
 
 }  // namespace
 
-void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, cudaStream_t st) {
+void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, SortBufs &b, cudaStream_t st) {
     if (n <= 0) return;
-    const int64_t need = (n + BBOX_THREADS - 1) / BBOX_THREADS;
-    { k_bbox<<<(unsigned)(need < nblk ? need : nblk), BBOX_THREADS, 0, st>>>(posm, n, ctl); gt_note_launches(1); }
+    static_assert(GT_SORT_DIGITS * 4 % 16 == 0, "cleared 16 bytes at a time");
+    k_bbox<<<gt_grid(n, BBOX_THREADS, nblk), BBOX_THREADS, 0, st>>>(posm, n, ctl, (uint4 *)b.hist,
+                                                                    (long long)(gt_sort_scratch_bytes(n) / 16));
+    gt_note_launches(1);
 }
 
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st) {
     if (n <= 0) return;
-    gt_sort_clear(b, n, st);
     const int64_t need = (n + 255) / 256, most = (int64_t)nsm * (n < KEYS_MANY ? 4 : 8);
     k_keys<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(posm, n, curve, ctl, (unsigned long long *)b.key[0],
                                                                   b.hist, b.digit_base);

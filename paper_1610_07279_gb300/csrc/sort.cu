@@ -396,10 +396,6 @@ void gt_sort_init() {
     cudaFuncSetAttribute(k_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
 }
 
-void gt_sort_clear(SortBufs &b, int64_t n, cudaStream_t st) {
-    cudaMemsetAsync(b.hist, 0, (size_t)PASSES * R * (1 + (size_t)gt_sort_tiles(n)) * sizeof(uint32_t), st);
-}
-
 namespace {
 
 // pass p reads buffers p & 1 and writes the others
@@ -432,7 +428,7 @@ void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStrea
 
 void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st) {
     if (n <= 1) return;
-    gt_sort_clear(b, n, st);
+    cudaMemsetAsync(b.hist, 0, gt_sort_scratch_bytes(n), st);
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
