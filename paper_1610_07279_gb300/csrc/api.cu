@@ -400,8 +400,7 @@ void build_tree(gt_system *s, cudaStream_t st, const float4 *posm_src, bool prep
     ph_begin(s, PH_PSEUDO, st);
     gt_launch_pseudo(s->nd, n, s->posm, s->ctl, s->nsm, true, st);
     ph_end(s, PH_PSEUDO, st);
-    s->have_tree = true;
-    s->rebuilds++;
+    gt_sys_note_build(s);
 }
 
 double c2_of(const gt_params &p) {
@@ -547,18 +546,81 @@ void gt_sys_step_post(gt_system *s, cudaStream_t st) {
     s->steps++;
 }
 
+namespace {
+
+// the exponent of the given dt_max, if one is given
+bool given_M(const gt_params &p, int *M) {
+    *M = 0;
+    if (!(p.dt_max > 0.0)) return false;
+    int e;
+    frexp(p.dt_max, &e);
+    *M = e - 1;
+    return true;
+}
+
+}  // namespace
+
 void gt_sys_start_levels(gt_system *s, cudaStream_t st) {
-    int M = 0, have_M = 0;
-    if (s->prm.dt_max > 0.0) {
-        int e;
-        frexp(s->prm.dt_max, &e);
-        M = e - 1;
-        have_M = 1;
-    }
+    int M;
+    const int have_M = given_M(s->prm, &M);
     gt_launch_init_levels(s->st[0], s->acc_out, s->n, s->prm.levels, c2_of(s->prm), M, have_M, s->ctl, s->nsm, st);
+    gt_sys_note_start(s);
+}
+
+bool gt_sys_groupable(const gt_system *s) {
+    return s->n > 0 && s->n <= GT_GROUPED_MOST && s->prm.leaf_max <= GT_FLAT_LEAF_MAX && s->fixed_buffers && !s->prof.on;
+}
+
+GroupedSys gt_sys_entry(const gt_system *s, unsigned flags) {
+    GroupedSys g;
+    memset(&g, 0, sizeof(g));  // entries are compared byte by byte
+    g.n = s->n;
+    g.cap = s->cap;
+    g.posm = s->posm;
+    g.posm_tmp = s->posm_tmp;
+    g.st0 = s->st[0];
+    g.st1 = s->st[1];
+    g.sb = s->sb;
+    g.nd = s->nd;
+    g.bscratch = s->bscratch;
+    g.ctl = s->ctl;
+    g.status = s->status;
+    g.active = s->active;
+    g.marks = s->marks;
+    g.gstart = s->gstart;
+    g.rank = s->rank;
+    g.acc = s->acc_out;
+    g.c2 = c2_of(s->prm);
+    g.curve = s->prm.key_curve;
+    g.leaf_max = s->prm.leaf_max;
+    g.gmax = s->gmax_now;
+    g.cells = cell_groups(s->prm) ? 1 : 0;
+    g.levels = s->prm.levels;
+    g.have_M = given_M(s->prm, &g.M);
+    g.r_crit = s->rcrit_now;
+    g.flags = flags;
+    return g;
+}
+
+void gt_sys_note_build(gt_system *s) {
+    s->have_tree = true;
+    s->rebuilds++;
+}
+
+void gt_sys_note_start(gt_system *s) {
     s->started = true;
     s->steps = 0;
     s->tune = RebuildTuner();
+}
+
+void gt_grouped_before_walk(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
+    gt_grouped_prepare(t, p, nsm, st);
+    gt_grouped_predict(t, p, nsm, st);
+    gt_grouped_sort(t, p, nsm, st);
+    gt_grouped_gather(t, p, nsm, st);
+    gt_grouped_build(t, p, nsm, st);
+    gt_grouped_pseudo(t, p, nsm, st);
+    gt_grouped_groups(t, p, nsm, st);
 }
 
 extern "C" {

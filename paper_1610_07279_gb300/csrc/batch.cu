@@ -1,6 +1,6 @@
 // Batches of independent systems (Sec. 2.3, 2.5 applied across systems): the members'
-// tree builds and group setup run on forked streams, so that the many small kernels of
-// small systems overlap; then one persistent walk launch covers the groups of every
+// tree builds and group setup run through one launch per kernel (many small systems) or
+// on forked streams, so that their many small kernels overlap; then one persistent walk launch covers the groups of every
 // member.  The whole evaluation can be captured into a CUDA graph and replayed, and an
 // autotuner picks the walk's leaf size, group size and queue depth by timing replays.
 #include <math.h>
@@ -21,6 +21,9 @@ struct gt_batch {
     DevCtl **d_ctls = nullptr;
     uint32_t *d_gprefix = nullptr;
     unsigned int *d_next = nullptr;
+    // entries of the members built together: for the captured graph, and for evaluations that are not captured
+    GroupedSys *d_tab[2] = {};
+    std::vector<GroupedSys> h_tab[2];
     uint32_t *queue = nullptr;
     std::vector<cudaStream_t> streams;
     std::vector<cudaEvent_t> ev_join;
@@ -56,6 +59,7 @@ size_t plan(int nsys, const int64_t *n, const gt_params *prm, int n_prm, int nsm
     off = align_up(off + (size_t)nsys * sizeof(DevCtl *));
     off = align_up(off + (size_t)(nsys + 1) * sizeof(uint32_t));
     off = align_up(off + sizeof(unsigned int));
+    off = align_up(off + 2 * (size_t)nsys * sizeof(GroupedSys));
     off = align_up(off + warps * gt_queue_words(qcap) * sizeof(uint32_t));
     if (member_bytes) member_bytes->clear();
     for (int k = 0; k < nsys; k++) {
@@ -116,18 +120,55 @@ void join(gt_batch *b, cudaStream_t st) {
     }
 }
 
-// The evaluation itself (enqueued or captured): builds and groups on the forked
-// streams, then the batch walk(s) on st.
-void enqueue(gt_batch *b, int bootstrap, cudaStream_t st) {
-    fork(b, st);
+// Members are built together from eight on: the same time as on streams of their own once captured (16 of 16384 241 us
+// and 242; two of 65536 190 and 188, four of 262144 476 and 461), and less for the host if not (16 of 16384 303 us and
+// 699; four of 262144 536 and 515).
+constexpr int TOGETHER_LEAST = 8;
+bool together(const gt_batch *b) {
+    int k = 0;
+    for (const gt_system *s : b->sys) k += gt_sys_groupable(s) ? 1 : 0;
+    return k >= TOGETHER_LEAST;
+}
+
+// The members that are built together, into table j (written only if it changed).
+int upload_table(gt_batch *b, int j) {
+    std::vector<GroupedSys> tab;
+    for (gt_system *s : b->sys)
+        if (gt_sys_groupable(s)) tab.push_back(gt_sys_entry(s, GT_SYS_BUILD));
+    const size_t bytes = tab.size() * sizeof(GroupedSys);
+    if (tab.size() == b->h_tab[j].size() && (!bytes || !memcmp(tab.data(), b->h_tab[j].data(), bytes))) return GT_OK;
+    // (earlier evaluations may still read it)
+    if (cudaDeviceSynchronize() != cudaSuccess ||
+        cudaMemcpy(b->d_tab[j], tab.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess)
+        return GT_ECUDA;
+    b->h_tab[j] = tab;
+    return GT_OK;
+}
+
+// The evaluation itself (enqueued or captured): builds and groups, of the members in table j together, of the others
+// (or, j < 0, of all) on the forked streams; then the batch walk(s) on st.
+void enqueue(gt_batch *b, int bootstrap, int j, cudaStream_t st) {
+    GroupedPlan plan;
+    bool others = false;
+    for (gt_system *s : b->sys) {
+        if (s->n == 0) continue;
+        if (j >= 0 && gt_sys_groupable(s)) plan.add(s->n, GT_SYS_BUILD, s->prm.leaf_max);
+        else others = true;
+    }
+    if (others) fork(b, st);
     for (int k = 0; k < b->nsys; k++) {
         gt_system *s = b->sys[k];
         cudaStream_t sk = b->streams[k % nstreams(b)];
         if (s->n == 0) continue;
+        if (j >= 0 && gt_sys_groupable(s)) {
+            gt_sys_note_build(s);
+            continue;
+        }
         gt_sys_build_tree(s, sk, s->posm);
         gt_sys_groups_all(s, sk);
     }
-    join(b, st);
+    if (plan.count > 0) gt_grouped_before_walk(b->d_tab[j], plan, b->nsm, st);
+    if (others) join(b, st);
     if (bootstrap) {
         gt_launch_walk_batch(b->d_ctls, b->d_args, b->nsys, b->d_gprefix, b->d_next, b->queue, b->qcap,
                              GT_MAC_OPENING_ANGLE, false, false, b->walk_blocks, st);
@@ -187,6 +228,8 @@ int gt_batch_create(gt_batch **out, int nsys, const int64_t *n, const gt_params 
     off = align_up(off + (size_t)(nsys + 1) * sizeof(uint32_t));
     b->d_next = (unsigned int *)(base + off);
     off = align_up(off + sizeof(unsigned int));
+    for (int j = 0; j < 2; j++) b->d_tab[j] = (GroupedSys *)(base + off) + (size_t)j * nsys;
+    off = align_up(off + 2 * (size_t)nsys * sizeof(GroupedSys));
     const size_t warps = (size_t)b->walk_blocks * (size_t)gt_walk_warps_per_block();
     b->queue = (uint32_t *)(base + off);
     off = align_up(off + warps * gt_queue_words(b->qcap) * sizeof(uint32_t));
@@ -271,7 +314,12 @@ int gt_batch_accel(gt_batch *b, int bootstrap, gt_stream stream) {
     if (!b) return GT_EINVAL;
     int rc = upload_args(b);
     if (rc) return rc;
-    enqueue(b, bootstrap, (cudaStream_t)stream);
+    // (no table is written while a caller captures)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing((cudaStream_t)stream, &capture) != cudaSuccess) return GT_ECUDA;
+    const int table = capture == cudaStreamCaptureStatusNone && together(b) ? 1 : -1;
+    if (table >= 0 && (rc = upload_table(b, table))) return rc;
+    enqueue(b, bootstrap, table, (cudaStream_t)stream);
     return cudaGetLastError() == cudaSuccess ? GT_OK : GT_ECUDA;
 }
 
@@ -280,10 +328,12 @@ int gt_batch_capture(gt_batch *b, int bootstrap, gt_stream stream) {
     int rc = upload_args(b);
     if (rc) return rc;
     drop_graph(b);
+    const int table = together(b) ? 0 : -1;
+    if (table >= 0 && (rc = upload_table(b, table))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const long long before = launches_now();
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return GT_ECUDA;
-    enqueue(b, bootstrap, st);
+    enqueue(b, bootstrap, table, st);
     cudaGraph_t g = nullptr;
     if (cudaStreamEndCapture(st, &g) != cudaSuccess || !g) {
         cudaGetLastError();

@@ -255,15 +255,31 @@ void gt_note_launches(int k);
 // Blocks of a kernel that loops over its work: one for every `per` particles, at most `most`.  (The cells of a tree
 // are fewer than its particles but for chains, so `per` bounds the blocks with work; a full grid for each of many
 // small systems keeps the device busy with blocks that have none.)
-inline unsigned gt_grid(int64_t n, int64_t per, int64_t most) {
+__host__ __device__ inline unsigned gt_grid(int64_t n, int64_t per, int64_t most) {
     const int64_t b = (n + per - 1) / per;
     return (unsigned)(b < 1 ? 1 : (b < most ? b : most));
 }
 
+#define GT_FLAT_LEAF_MAX 64         // largest leaves of the builds without a launch per level
 #define GT_SMALL_SORT 8192           // systems whose keys one block makes and sorts
 #define GT_SORT_BITS 8
 #define GT_SORT_DIGITS 256
 #define GT_SORT_PASSES 8             // 64 / 8 (bit 63 is always 0)
+
+#ifndef GT_SORT_ST
+#define GT_SORT_ST 512
+#endif
+#ifndef GT_SORT_IPT
+#define GT_SORT_IPT 8
+#endif
+// tiles of a pass, and the bytes of digit counts and of look-back status of every pass (passes x tiles x digits x 4 B)
+__host__ __device__ inline int gt_sort_tiles(long long n) {
+    return (int)((n + GT_SORT_ST * GT_SORT_IPT - 1) / (GT_SORT_ST * GT_SORT_IPT));
+}
+__host__ __device__ inline size_t gt_sort_scratch_bytes(long long n) {
+    const int tiles = gt_sort_tiles(n);
+    return (size_t)GT_SORT_PASSES * GT_SORT_DIGITS * (size_t)(1 + (tiles > 0 ? tiles : 1)) * sizeof(uint32_t);
+}
 
 struct SortBufs {
     uint64_t *key[2];
@@ -272,6 +288,63 @@ struct SortBufs {
     uint32_t *status;            // look-back status of the 8 passes, 8 x tiles x 256 (cleared together)
     uint32_t *digit_base;        // digit starts of the 8 passes, 8 x 256
 };
+
+// ---- many small systems at once ------------------------------------------------------
+// The kernels around the walk for a table of systems, one launch each: block (k, b) is block b of system k, which ends
+// at once if the kernel isn't for that system or its grid (gt_grid of its own size) has fewer blocks.  A launch costs
+// ~2 us of the host's time however small its system, and a build takes twenty: 16 builds of 16384 particles 303 us, by
+// one system after another on streams of their own 699.  Systems above GT_GROUPED_MOST fill the device by themselves
+// (two of 2^20 814 us together, 755 apart; limits of 2^17, 2^18 and 2^20 for 64 systems of 2^12 to 2^18 8.04, 7.95 and
+// 7.96 ms, none together 8.03; for a server's requests of 2^12 to 2^17 11.1, 11.0 and 11.1, none 13.2).
+#ifndef GT_GROUPED_MOST
+#define GT_GROUPED_MOST (1 << 18)
+#endif
+enum { GT_SYS_BUILD = 1, GT_SYS_PREDICTED = 2, GT_SYS_STEP = 4, GT_SYS_START = 8 };  // what a launch is to do for it
+struct GroupedSys {
+    long long n, cap;
+    float4 *posm, *posm_tmp;
+    State st0, st1;
+    SortBufs sb;
+    Nodes nd;
+    uint8_t *bscratch;
+    DevCtl *ctl;
+    unsigned long long *status;
+    uint32_t *active, *marks, *gstart;
+    uint2 *rank;
+    float4 *acc;
+    double c2;
+    int curve, leaf_max, gmax, cells, levels, M, have_M;
+    float r_crit;
+    unsigned flags;   // GT_SYS_*
+};
+// What the launches over a table have to know of it.
+struct GroupedPlan {
+    int count = 0;
+    int64_t n_all = 0, n_build = 0, n_step = 0, n_start = 0;  // largest sizes
+    int leaf_max = -1;  // of every build; 0: different ones
+    void add(int64_t n, unsigned flags, int leaf) {
+        auto most = [n](int64_t &m) { m = m > n ? m : n; };
+        count++;
+        most(n_all);
+        if (flags & GT_SYS_BUILD) {
+            most(n_build);
+            leaf_max = leaf_max < 0 || leaf_max == leaf ? leaf : 0;
+        }
+        if (flags & GT_SYS_STEP) most(n_step);
+        if (flags & GT_SYS_START) most(n_start);
+    }
+};
+void gt_grouped_prepare(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);
+void gt_grouped_predict(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);
+void gt_grouped_sort(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);  // keys and sort
+void gt_grouped_small_sort(const GroupedSys *t, const GroupedPlan &p, cudaStream_t st);     // keys.cu's parts of it
+void gt_grouped_keys(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);
+void gt_grouped_gather(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);
+void gt_grouped_build(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);
+void gt_grouped_pseudo(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);
+void gt_grouped_groups(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);  // active sets and groups
+void gt_grouped_aold(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);
+void gt_grouped_correct(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);  // and the starts' levels
 
 // keys.cu
 // extrema into ctl->bbox (reset by gt_launch_prepare), and the sort's counts and look-back words cleared; keys and their digit counts for gt_launch_sort_tree
@@ -282,8 +355,6 @@ void gt_keys_init();
 void gt_launch_small_sort(const float4 *posm, int64_t n, int curve, SortBufs &b, cudaStream_t st);
 // sort.cu: gt_launch_sort sorts (key, val) in buffers 0; gt_launch_sort_tree the keys that gt_launch_keys made, with
 // their positions as values, into buffers 0
-int gt_sort_tiles(int64_t n);
-size_t gt_sort_scratch_bytes(int64_t n);
 void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st);
 void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStream_t st);
 void gt_sort_init();

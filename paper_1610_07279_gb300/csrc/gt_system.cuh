@@ -139,3 +139,13 @@ void gt_sys_start_levels(gt_system *s, cudaStream_t st);
 void gt_sys_step_pre(gt_system *s, cudaStream_t st, bool rebuild, bool predicted = false);
 void gt_sys_step_groups(gt_system *s, cudaStream_t st);
 void gt_sys_step_post(gt_system *s, cudaStream_t st);
+
+// Members of a batch or a server in one launch per kernel (GroupedSys): whether a system may take part, its entry, and
+// what the single-system functions note on the host.
+bool gt_sys_groupable(const gt_system *s);
+GroupedSys gt_sys_entry(const gt_system *s, unsigned flags);
+void gt_sys_note_build(gt_system *s);
+void gt_sys_note_start(gt_system *s);
+// everything before the walk, of every system of the table: gt_sys_build_tree and gt_sys_groups_all, or gt_sys_step_pre
+// and gt_sys_step_groups
+void gt_grouped_before_walk(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);

@@ -27,7 +27,7 @@
 
 namespace {
 
-__global__ void k_prepare(DevCtl *ctl, int begin_step) {  // one warp
+__device__ __forceinline__ void prepare_body(const unsigned bid, const unsigned nb, DevCtl *ctl, int begin_step) {  // one warp
     static_assert(GT_TREE_LEVELS + 4 <= 32, "a lane per ticket");
     const int l = threadIdx.x;
     if (l < GT_TREE_LEVELS + 4) ctl->tile_ticket[l] = 0;
@@ -43,6 +43,10 @@ __global__ void k_prepare(DevCtl *ctl, int begin_step) {  // one warp
     }
 }
 
+__global__ void k_prepare(DevCtl *ctl, int begin_step) {
+    prepare_body(blockIdx.x, gridDim.x, ctl, begin_step);
+}
+
 __global__ void k_set_nactive(DevCtl *ctl, unsigned int n_active) { ctl->n_active = n_active; }
 
 __global__ void k_mirror(const DevCtl *ctl, StepMirror *dst) {
@@ -55,9 +59,9 @@ __global__ void k_mirror(const DevCtl *ctl, StepMirror *dst) {
 
 // Two particles per thread with 16-byte loads (n even, so that every array of the state,
 // and the second and third coordinate arrays inside its block, start 16-byte aligned).
-__global__ __launch_bounds__(256) void k_predict2(State s, long long n, const DevCtl *__restrict__ ctl,
-                                                  float4 *__restrict__ posm, int ahead) {
-    const long long i = 2 * (blockIdx.x * 256ll + threadIdx.x);
+__device__ __forceinline__ void predict2_body(const unsigned bid, const unsigned nb, State s, long long n,
+        const DevCtl *__restrict__ ctl, float4 *__restrict__ posm, int ahead) {
+    const long long i = 2 * (bid * 256ll + threadIdx.x);
     if (i >= n) return;
     const long long T = (long long)(ahead ? ctl->tnext_acc : ctl->tnext);
     const int k = (int)((__double_as_longlong(ctl->dt_max) >> 52) & 0x7ff) - 1023 - ctl->levels_m1;
@@ -73,9 +77,14 @@ __global__ __launch_bounds__(256) void k_predict2(State s, long long n, const De
                               d2f(__fma_rn(dt1, vz.y, rz.y)), m.y);
 }
 
-__global__ __launch_bounds__(256) void k_predict(State s, long long n, const DevCtl *__restrict__ ctl,
-                                                 float4 *__restrict__ posm, int ahead) {
-    const long long i = blockIdx.x * 256ll + threadIdx.x;
+__global__ __launch_bounds__(256) void k_predict2(State s, long long n, const DevCtl *__restrict__ ctl,
+        float4 *__restrict__ posm, int ahead) {
+    predict2_body(blockIdx.x, gridDim.x, s, n, ctl, posm, ahead);
+}
+
+__device__ __forceinline__ void predict_body(const unsigned bid, const unsigned nb, State s, long long n,
+        const DevCtl *__restrict__ ctl, float4 *__restrict__ posm, int ahead) {
+    const long long i = bid * 256ll + threadIdx.x;
     if (i >= n) return;
     const long long T = (long long)(ahead ? ctl->tnext_acc : ctl->tnext);
     // dt = (T - t0) dt_min with dt_min = dt_max 2^-(L-1) a power of two: exact, so it is
@@ -86,6 +95,11 @@ __global__ __launch_bounds__(256) void k_predict(State s, long long n, const Dev
     const float y = d2f(__fma_rn(dt, s.vy[i], s.ry[i]));
     const float z = d2f(__fma_rn(dt, s.vz[i], s.rz[i]));
     posm[i] = make_float4(x, y, z, s.mass[i]);
+}
+
+__global__ __launch_bounds__(256) void k_predict(State s, long long n, const DevCtl *__restrict__ ctl,
+        float4 *__restrict__ posm, int ahead) {
+    predict_body(blockIdx.x, gridDim.x, s, n, ctl, posm, ahead);
 }
 
 __global__ __launch_bounds__(256) void k_load(State s, long long n, float4 *__restrict__ posm) {
@@ -123,10 +137,9 @@ __global__ __launch_bounds__(256) void k_load_from(State s, long long n, const d
     s.acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ __launch_bounds__(256) void k_permute(State src, State dst, const float4 *__restrict__ pin,
-                                                 float4 *__restrict__ pout,
-                                                 const uint32_t *__restrict__ perm, long long n) {
-    const long long i = blockIdx.x * 256ll + threadIdx.x;
+__device__ __forceinline__ void permute_body(const unsigned bid, const unsigned nb, State src, State dst,
+        const float4 *__restrict__ pin, float4 *__restrict__ pout, const uint32_t *__restrict__ perm, long long n) {
+    const long long i = bid * 256ll + threadIdx.x;
     if (i >= n) return;
     const uint32_t k = perm[i];
     dst.rx[i] = src.rx[k];
@@ -145,10 +158,15 @@ __global__ __launch_bounds__(256) void k_permute(State src, State dst, const flo
     pout[i] = p;
 }
 
+__global__ __launch_bounds__(256) void k_permute(State src, State dst, const float4 *__restrict__ pin,
+        float4 *__restrict__ pout, const uint32_t *__restrict__ perm, long long n) {
+    permute_body(blockIdx.x, gridDim.x, src, dst, pin, pout, perm, n);
+}
+
 // copy the permuted state back, so that buffer 0 always holds the current state
-__global__ __launch_bounds__(256) void k_copy_state(State src, State dst, const float4 *__restrict__ pin,
-                                                    float4 *__restrict__ pout, long long n) {
-    const long long i = blockIdx.x * 256ll + threadIdx.x;
+__device__ __forceinline__ void copy_state_body(const unsigned bid, const unsigned nb, State src, State dst,
+        const float4 *__restrict__ pin, float4 *__restrict__ pout, long long n) {
+    const long long i = bid * 256ll + threadIdx.x;
     if (i >= n) return;
     dst.rx[i] = src.rx[i];
     dst.ry[i] = src.ry[i];
@@ -163,6 +181,11 @@ __global__ __launch_bounds__(256) void k_copy_state(State src, State dst, const 
     dst.id[i] = src.id[i];
     dst.mass[i] = src.mass[i];
     if (pin) pout[i] = pin[i];
+}
+
+__global__ __launch_bounds__(256) void k_copy_state(State src, State dst, const float4 *__restrict__ pin,
+        float4 *__restrict__ pout, long long n) {
+    copy_state_body(blockIdx.x, gridDim.x, src, dst, pin, pout, n);
 }
 
 // n x 3 row-major <-> three arrays
@@ -237,10 +260,9 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
 
 // Order-preserving compaction of the particles whose step ends at the block time.  Writes their indices to out, the
 // rank words (rank[n / 32] too), the count to ctl->n_active, and folds the others' step ends into the next block time.
-__global__ __launch_bounds__(AT) void k_compact(long long n, const long long *__restrict__ t0,
-                                                const uint8_t *__restrict__ level, int L, DevCtl *ctl, int ticket,
-                                                uint32_t tag_slot, uint32_t *__restrict__ out,
-                                                uint2 *__restrict__ rank, unsigned long long *status) {
+__device__ __forceinline__ void compact_body(const unsigned bid, const unsigned nb, long long n,
+        const long long *__restrict__ t0, const uint8_t *__restrict__ level, int L, DevCtl *ctl, int ticket,
+        uint32_t tag_slot, uint32_t *__restrict__ out, uint2 *__restrict__ rank, unsigned long long *status) {
     __shared__ uint32_t tmp[AT / 32 + 1];
     __shared__ uint32_t tile_sh, excl_sh;
     const unsigned long long T = ctl->tnext;
@@ -248,7 +270,7 @@ __global__ __launch_bounds__(AT) void k_compact(long long n, const long long *__
     const uint32_t ntiles = (uint32_t)((n + ATILE - 1) / ATILE);
     unsigned long long tmin = ~0ull;
     if (n == 0) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (bid == 0 && threadIdx.x == 0) {
             ctl->n_active = 0;
             rank[0] = make_uint2(0u, 0u);
         }
@@ -308,6 +330,12 @@ __global__ __launch_bounds__(AT) void k_compact(long long n, const long long *__
     if (lane_id() == 0 && tmin != ~0ull) atomicMin(&ctl->tnext_acc, tmin);
 }
 
+__global__ __launch_bounds__(AT) void k_compact(long long n, const long long *__restrict__ t0,
+        const uint8_t *__restrict__ level, int L, DevCtl *ctl, int ticket, uint32_t tag_slot,
+        uint32_t *__restrict__ out, uint2 *__restrict__ rank, unsigned long long *status) {
+    compact_body(blockIdx.x, gridDim.x, n, t0, level, L, ctl, ticket, tag_slot, out, rank, status);
+}
+
 // Order-preserving compaction of the bits of [0, n) (n from n_dev if given), which are cleared on the way (masks
 // start at zero, so that no launch has to clear them).  Writes the indices to out, the rank words if rank != null
 // (rank[n / 32] too), and the count to *count_out.  A lane takes a word of 32 items, 8192 items to a
@@ -315,11 +343,9 @@ __global__ __launch_bounds__(AT) void k_compact(long long n, const long long *__
 // active, the whole walk: 282 us with bytes, 236 with four words per lane (too few blocks), 225.
 constexpr int BTILE = AT;  // words per tile, a word per lane
 
-__global__ __launch_bounds__(AT) void k_compact_bits(long long n_host, const unsigned int *n_dev,
-                                                     uint32_t *__restrict__ bits, DevCtl *ctl, int ticket,
-                                                     uint32_t tag_slot, uint32_t *__restrict__ out,
-                                                     uint2 *__restrict__ rank, unsigned int *count_out,
-                                                     unsigned long long *status) {
+__device__ __forceinline__ void compact_bits_body(const unsigned bid, const unsigned nb, long long n_host,
+        const unsigned int *n_dev, uint32_t *__restrict__ bits, DevCtl *ctl, int ticket, uint32_t tag_slot,
+        uint32_t *__restrict__ out, uint2 *__restrict__ rank, unsigned int *count_out, unsigned long long *status) {
     __shared__ uint32_t tmp[AT / 32 + 1];
     __shared__ uint32_t tile_sh, excl_sh;
     const long long n = n_dev ? (long long)*n_dev : n_host;
@@ -327,7 +353,7 @@ __global__ __launch_bounds__(AT) void k_compact_bits(long long n_host, const uns
     const long long nwords = (n + 31) / 32;
     const uint32_t ntiles = (uint32_t)((nwords + BTILE - 1) / BTILE);
     if (n == 0) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (bid == 0 && threadIdx.x == 0) {
             *count_out = 0;
             if (rank) rank[0] = make_uint2(0u, 0u);
         }
@@ -367,6 +393,12 @@ __global__ __launch_bounds__(AT) void k_compact_bits(long long n_host, const uns
     }
 }
 
+__global__ __launch_bounds__(AT) void k_compact_bits(long long n_host, const unsigned int *n_dev,
+        uint32_t *__restrict__ bits, DevCtl *ctl, int ticket, uint32_t tag_slot, uint32_t *__restrict__ out,
+        uint2 *__restrict__ rank, unsigned int *count_out, unsigned long long *status) {
+    compact_bits_body(blockIdx.x, gridDim.x, n_host, n_dev, bits, ctl, ticket, tag_slot, out, rank, count_out, status);
+}
+
 // The number of actives below i.
 __device__ __forceinline__ uint32_t rank_at(const uint2 *__restrict__ rank, uint32_t i) {
     const uint2 r = rank[i >> 5];
@@ -388,13 +420,12 @@ __device__ __forceinline__ bool group_cell_ok(const Nodes &nd, const uint2 *R, u
 }
 
 template <bool ALL>
-__global__ __launch_bounds__(256) void k_group_cells(Nodes nd, long long n, long long cap, const uint2 *__restrict__ R,
-                                                     int gmax, float r_crit, uint32_t *__restrict__ marks,
-                                                     DevCtl *ctl) {
+__device__ __forceinline__ void group_cells_body(const unsigned bid, const unsigned nb, Nodes nd, long long n,
+        long long cap, const uint2 *__restrict__ R, int gmax, float r_crit, uint32_t *__restrict__ marks, DevCtl *ctl) {
     long long nn = ctl->level_start[GT_TREE_LEVELS];
     if (nn > cap) nn = cap;
-    if (ALL && blockIdx.x == 0 && threadIdx.x == 0) ctl->n_active = (unsigned int)n;
-    for (long long c = blockIdx.x * 256ll + threadIdx.x; c < nn; c += (long long)gridDim.x * 256) {
+    if (ALL && bid == 0 && threadIdx.x == 0) ctl->n_active = (unsigned int)n;
+    for (long long c = bid * 256ll + threadIdx.x; c < nn; c += (long long)nb * 256) {
         const uint32_t f = nd.first[c], k = nd.count[c];
         const uint32_t a0 = ALL ? f : rank_at(R, f), A = ALL ? k : rank_at(R, f + k) - a0;
         if (A == 0) continue;
@@ -403,6 +434,12 @@ __global__ __launch_bounds__(256) void k_group_cells(Nodes nd, long long n, long
         if (nd.child[c] >= 0 && !group_cell_ok<ALL>(nd, R, (uint32_t)c, gmax, r_crit)) continue;  // children decide
         for (uint32_t s = a0; s < a0 + A; s += (uint32_t)gmax) atomicOr(&marks[s >> 5], 1u << (s & 31u));
     }
+}
+
+template <bool ALL>
+__global__ __launch_bounds__(256) void k_group_cells(Nodes nd, long long n, long long cap,
+        const uint2 *__restrict__ R, int gmax, float r_crit, uint32_t *__restrict__ marks, DevCtl *ctl) {
+    group_cells_body<ALL>(blockIdx.x, gridDim.x, nd, n, cap, R, gmax, r_crit, marks, ctl);
 }
 
 // a batch member's accelerations and ids to the caller
@@ -441,9 +478,9 @@ __device__ __forceinline__ int level_from_a2(double a2, double c2, int M, int L)
     return (int)k;
 }
 
-__global__ __launch_bounds__(256) void k_correct(State s, const uint32_t *__restrict__ active,
-                                                 const float4 *__restrict__ acc, DevCtl *ctl, long long n,
-                                                 int L, double c2) {
+__device__ __forceinline__ void correct_body(const unsigned bid, const unsigned nb, State s,
+        const uint32_t *__restrict__ active, const float4 *__restrict__ acc, DevCtl *ctl, long long n, int L,
+        double c2) {
     const uint32_t na = ctl->n_active;
     const long long T = (long long)ctl->tnext;
     const int M = ctl->M;  // dt_max = 2^M
@@ -453,7 +490,7 @@ __global__ __launch_bounds__(256) void k_correct(State s, const uint32_t *__rest
         return (e > -1023 && e < 1024) ? __longlong_as_double((long long)(e + 1023) << 52) : ldexp(1.0, e);
     };
     unsigned long long tmin = ~0ull;
-    for (uint32_t k = blockIdx.x * 256u + threadIdx.x; k < na; k += gridDim.x * 256u) {
+    for (uint32_t k = bid * 256u + threadIdx.x; k < na; k += nb * 256u) {
         const uint32_t i = active[k];
         if ((long long)i >= n) {  // an index outside the system: report it and skip
             gt_set_error(ctl, GT_EINVAL, GTK_CORRECT);
@@ -495,16 +532,26 @@ __global__ __launch_bounds__(256) void k_correct(State s, const uint32_t *__rest
     if (lane_id() == 0 && tmin != ~0ull) atomicMin(&ctl->tnext_acc, tmin);
 }
 
-__global__ __launch_bounds__(256) void k_aold(const float4 *__restrict__ acc, long long n,
-                                              float *__restrict__ aold) {
-    const long long i = blockIdx.x * 256ll + threadIdx.x;
+__global__ __launch_bounds__(256) void k_correct(State s, const uint32_t *__restrict__ active,
+        const float4 *__restrict__ acc, DevCtl *ctl, long long n, int L, double c2) {
+    correct_body(blockIdx.x, gridDim.x, s, active, acc, ctl, n, L, c2);
+}
+
+__device__ __forceinline__ void aold_body(const unsigned bid, const unsigned nb, const float4 *__restrict__ acc,
+        long long n, float *__restrict__ aold) {
+    const long long i = bid * 256ll + threadIdx.x;
     if (i < n) aold[i] = __fsqrt_rn(__double2float_rn(a2_of(acc[i])));
 }
 
+__global__ __launch_bounds__(256) void k_aold(const float4 *__restrict__ acc, long long n, float *__restrict__ aold) {
+    aold_body(blockIdx.x, gridDim.x, acc, n, aold);
+}
+
 // start, phase 1: the smallest positive A2 (bit pattern of a positive double)
-__global__ __launch_bounds__(256) void k_min_a2(const float4 *__restrict__ acc, long long n, DevCtl *ctl) {
+__device__ __forceinline__ void min_a2_body(const unsigned bid, const unsigned nb, const float4 *__restrict__ acc,
+        long long n, DevCtl *ctl) {
     unsigned long long best = ~0ull;
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
+    for (long long i = bid * 256ll + threadIdx.x; i < n; i += (long long)nb * 256) {
         const double a2 = a2_of(acc[i]);
         if (!(a2 > 0.0) || !isfinite(a2)) continue;
         const unsigned long long b = (unsigned long long)__double_as_longlong(a2);
@@ -514,10 +561,14 @@ __global__ __launch_bounds__(256) void k_min_a2(const float4 *__restrict__ acc, 
     if (lane_id() == 0 && best != ~0ull) atomicMin(&ctl->max_dt_bits, best);
 }
 
+__global__ __launch_bounds__(256) void k_min_a2(const float4 *__restrict__ acc, long long n, DevCtl *ctl) {
+    min_a2_body(blockIdx.x, gridDim.x, acc, n, ctl);
+}
+
 // start, phase 2: dt_max (the largest 2^M with 2^(4M) A2min <= c2), levels, t0 = 0,
 // first half kick v^{1/2} = fma(dt/2, a, v)
-__global__ __launch_bounds__(256) void k_init_levels(State s, const float4 *__restrict__ acc, long long n,
-                                                     int L, double c2, int M_given, int have_M, DevCtl *ctl) {
+__device__ __forceinline__ void init_levels_body(const unsigned bid, const unsigned nb, State s,
+        const float4 *__restrict__ acc, long long n, int L, double c2, int M_given, int have_M, DevCtl *ctl) {
     int M = M_given;
     if (!have_M) {
         M = 0;
@@ -531,13 +582,13 @@ __global__ __launch_bounds__(256) void k_init_levels(State s, const float4 *__re
         }
     }
     const double dt_max = ldexp(1.0, M);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (bid == 0 && threadIdx.x == 0) {
         ctl->M = M;
         ctl->dt_max = dt_max;
         ctl->levels_m1 = L - 1;
     }
     unsigned long long tmin = ~0ull;
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
+    for (long long i = bid * 256ll + threadIdx.x; i < n; i += (long long)nb * 256) {
         const float4 a = acc[i];
         const double a2 = a2_of(a);
         const int k = level_from_a2(a2, c2, M, L);
@@ -554,6 +605,11 @@ __global__ __launch_bounds__(256) void k_init_levels(State s, const float4 *__re
     }
     tmin = warp_min_u64(tmin);
     if (lane_id() == 0 && tmin != ~0ull) atomicMin(&ctl->tnext_acc, tmin);
+}
+
+__global__ __launch_bounds__(256) void k_init_levels(State s, const float4 *__restrict__ acc, long long n, int L,
+        double c2, int M_given, int have_M, DevCtl *ctl) {
+    init_levels_body(blockIdx.x, gridDim.x, s, acc, n, L, c2, M_given, have_M, ctl);
 }
 
 // resume: scalars of the integration and the next block time over all particles
@@ -597,6 +653,95 @@ __global__ void k_reset_start(DevCtl *ctl) {
     ctl->max_dt_bits = ~0ull;
     ctl->tnext_acc = ~0ull;
     ctl->tnext = 0;
+}
+
+// ---- a table of systems ----
+__global__ void kg_prepare(const GroupedSys *__restrict__ t) {  // a warp each
+    const GroupedSys &s = t[blockIdx.x];
+    prepare_body(0, 1, s.ctl, (s.flags & GT_SYS_STEP) ? 1 : 0);
+    if ((s.flags & GT_SYS_START) && threadIdx.x == 0) {
+        s.ctl->max_dt_bits = ~0ull;
+        s.ctl->tnext_acc = ~0ull;
+        s.ctl->tnext = 0;
+    }
+}
+
+__global__ __launch_bounds__(256) void kg_predict(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    if (!(s.flags & GT_SYS_STEP)) return;
+    float4 *dst = (s.flags & GT_SYS_BUILD) ? s.posm_tmp : s.posm;
+    // (a system's arrays start 256-byte aligned, so an even number of particles keeps the pairs aligned)
+    if (s.n % 2 == 0) predict2_body(blockIdx.y, gridDim.y, s.st0, s.n, s.ctl, dst, 0);
+    else predict_body(blockIdx.y, gridDim.y, s.st0, s.n, s.ctl, dst, 0);
+}
+
+__global__ __launch_bounds__(256) void kg_permute(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    if (!(s.flags & GT_SYS_BUILD)) return;
+    const bool tmp = (s.flags & GT_SYS_PREDICTED) != 0;
+    permute_body(blockIdx.y, gridDim.y, s.st0, s.st1, tmp ? s.posm_tmp : s.posm, tmp ? s.posm : s.posm_tmp, s.sb.val[0],
+                 s.n);
+}
+
+__global__ __launch_bounds__(256) void kg_copy_state(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    if (!(s.flags & GT_SYS_BUILD)) return;
+    const bool tmp = (s.flags & GT_SYS_PREDICTED) != 0;
+    copy_state_body(blockIdx.y, gridDim.y, s.st1, s.st0, tmp ? nullptr : s.posm_tmp, tmp ? nullptr : s.posm, s.n);
+}
+
+__global__ __launch_bounds__(AT) void kg_compact(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, ATILE, nsm * 4);
+    if (!(s.flags & GT_SYS_STEP) || blockIdx.y >= nb) return;
+    compact_body(blockIdx.y, nb, s.n, s.st0.t0, s.st0.level, s.levels, s.ctl, GT_TREE_LEVELS, 30u, s.active, s.rank,
+                 s.status);
+}
+
+__global__ __launch_bounds__(256) void kg_group_cells(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 256, nsm * 8);
+    if (blockIdx.y >= nb) return;
+    if (!s.cells) {
+        if (!(s.flags & GT_SYS_STEP) && blockIdx.y == 0 && threadIdx.x == 0) s.ctl->n_active = (unsigned int)s.n;
+    } else if (s.flags & GT_SYS_STEP) {
+        group_cells_body<false>(blockIdx.y, nb, s.nd, s.n, s.cap, s.rank, s.gmax, s.r_crit, s.marks, s.ctl);
+    } else {
+        group_cells_body<true>(blockIdx.y, nb, s.nd, s.n, s.cap, nullptr, s.gmax, s.r_crit, s.marks, s.ctl);
+    }
+}
+
+__global__ __launch_bounds__(AT) void kg_groups(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 32 * BTILE, nsm * 4);
+    if (!s.cells || blockIdx.y >= nb) return;
+    compact_bits_body(blockIdx.y, nb, 0, &s.ctl->n_active, s.marks, s.ctl, GT_TREE_LEVELS + 1, 31u, s.gstart, nullptr,
+                      &s.ctl->n_groups, s.status);
+}
+
+__global__ __launch_bounds__(256) void kg_aold(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    if (s.flags & GT_SYS_START) aold_body(blockIdx.y, gridDim.y, s.acc, s.n, s.st0.aold);
+}
+
+__global__ __launch_bounds__(256) void kg_min_a2(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 256, nsm * 4);
+    if ((s.flags & GT_SYS_START) && !s.have_M && blockIdx.y < nb) min_a2_body(blockIdx.y, nb, s.acc, s.n, s.ctl);
+}
+
+__global__ __launch_bounds__(256) void kg_init_levels(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 256, nsm * 8);
+    if ((s.flags & GT_SYS_START) && blockIdx.y < nb)
+        init_levels_body(blockIdx.y, nb, s.st0, s.acc, s.n, s.levels, s.c2, s.M, s.have_M, s.ctl);
+}
+
+__global__ __launch_bounds__(256) void kg_correct(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 256, nsm * 8);
+    if ((s.flags & GT_SYS_STEP) && blockIdx.y < nb)
+        correct_body(blockIdx.y, nb, s.st0, s.active, s.acc, s.ctl, s.n, s.levels, s.c2);
 }
 
 inline unsigned nblk(long long n) { return (unsigned)((n + 255) / 256); }
@@ -730,4 +875,51 @@ void gt_launch_init_levels(const State &s, const float4 *acc, int64_t n, int L, 
     { k_reset_start<<<1, 1, 0, st>>>(ctl); gt_note_launches(1); }
     if (!have_M && n > 0) { k_min_a2<<<gt_grid(n, 256, nsm * 4), 256, 0, st>>>(acc, n, ctl); gt_note_launches(1); }
     { k_init_levels<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(s, acc, n, L, c2, M_given, have_M, ctl); gt_note_launches(1); }
+}
+
+// ---- a table of systems ----
+void gt_grouped_prepare(const GroupedSys *t, const GroupedPlan &p, int, cudaStream_t st) {
+    kg_prepare<<<p.count, 32, 0, st>>>(t);
+    gt_note_launches(1);
+}
+
+void gt_grouped_predict(const GroupedSys *t, const GroupedPlan &p, int, cudaStream_t st) {
+    if (p.n_step <= 0) return;
+    kg_predict<<<dim3(p.count, nblk(p.n_step)), 256, 0, st>>>(t);
+    gt_note_launches(1);
+}
+
+void gt_grouped_gather(const GroupedSys *t, const GroupedPlan &p, int, cudaStream_t st) {
+    if (p.n_build <= 0) return;
+    kg_permute<<<dim3(p.count, nblk(p.n_build)), 256, 0, st>>>(t);
+    kg_copy_state<<<dim3(p.count, nblk(p.n_build)), 256, 0, st>>>(t);
+    gt_note_launches(2);
+}
+
+void gt_grouped_groups(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
+    if (p.n_step > 0) {
+        kg_compact<<<dim3(p.count, gt_grid(p.n_step, ATILE, nsm * 4)), AT, 0, st>>>(t, nsm);
+        gt_note_launches(1);
+    }
+    kg_group_cells<<<dim3(p.count, gt_grid(p.n_all, 256, nsm * 8)), 256, 0, st>>>(t, nsm);
+    kg_groups<<<dim3(p.count, gt_grid(p.n_all, 32 * BTILE, nsm * 4)), AT, 0, st>>>(t, nsm);
+    gt_note_launches(2);
+}
+
+void gt_grouped_aold(const GroupedSys *t, const GroupedPlan &p, int, cudaStream_t st) {
+    if (p.n_start <= 0) return;
+    kg_aold<<<dim3(p.count, nblk(p.n_start)), 256, 0, st>>>(t);
+    gt_note_launches(1);
+}
+
+void gt_grouped_correct(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
+    if (p.n_start > 0) {
+        kg_min_a2<<<dim3(p.count, gt_grid(p.n_start, 256, nsm * 4)), 256, 0, st>>>(t, nsm);
+        kg_init_levels<<<dim3(p.count, gt_grid(p.n_start, 256, nsm * 8)), 256, 0, st>>>(t, nsm);
+        gt_note_launches(2);
+    }
+    if (p.n_step > 0) {
+        kg_correct<<<dim3(p.count, gt_grid(p.n_step, 256, nsm * 8)), 256, 0, st>>>(t, nsm);
+        gt_note_launches(1);
+    }
 }

@@ -18,16 +18,16 @@ constexpr int BBOX_THREADS = 256;
 // more than the warps hide (2^20: 407 us the whole build at 4, 413 at 8; 2^24: 3009 and 3001).
 constexpr int64_t KEYS_MANY = 1 << 22;
 
-__global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict__ posm, long long n, DevCtl *ctl,
-                                                       uint4 *__restrict__ clear, long long nclear) {
+__device__ __forceinline__ void bbox_body(const unsigned bid, const unsigned nb, const float4 *__restrict__ posm,
+        long long n, DevCtl *ctl, uint4 *__restrict__ clear, long long nclear) {
     // the sort's counts and look-back words, which the next launch wants at zero
-    for (long long i = blockIdx.x * (long long)BBOX_THREADS + threadIdx.x; i < nclear;
-         i += (long long)gridDim.x * BBOX_THREADS)
+    for (long long i = bid * (long long)BBOX_THREADS + threadIdx.x; i < nclear;
+         i += (long long)nb * BBOX_THREADS)
         clear[i] = make_uint4(0u, 0u, 0u, 0u);
     float mn0 = FLT_MAX, mn1 = FLT_MAX, mn2 = FLT_MAX;
     float mx0 = -FLT_MAX, mx1 = -FLT_MAX, mx2 = -FLT_MAX;
-    for (long long i = blockIdx.x * (long long)BBOX_THREADS + threadIdx.x; i < n;
-         i += (long long)gridDim.x * BBOX_THREADS) {
+    for (long long i = bid * (long long)BBOX_THREADS + threadIdx.x; i < n;
+         i += (long long)nb * BBOX_THREADS) {
         const float4 p = posm[i];
         mn0 = fminf(mn0, p.x); mx0 = fmaxf(mx0, p.x);
         mn1 = fminf(mn1, p.y); mx1 = fmaxf(mx1, p.y);
@@ -56,6 +56,11 @@ __global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict_
         if (threadIdx.x < 3) atomicMin(&ctl->bbox[threadIdx.x], gt_ordered(v));
         else atomicMax(&ctl->bbox[threadIdx.x], gt_ordered(v));
     }
+}
+
+__global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict__ posm, long long n, DevCtl *ctl,
+        uint4 *__restrict__ clear, long long nclear) {
+    bbox_body(blockIdx.x, gridDim.x, posm, n, ctl, clear, nclear);
 }
 
 // Spread the low 11 bits of v so that bit b lands on bit 3b.
@@ -136,9 +141,9 @@ __device__ __forceinline__ double cube_scale(const float *ext) {
 
 // Bound by issue: ~100 instructions per key of quantisation and interleaving on the FP32 and integer pipes and
 // ~50 of digit counting, against 24 B of HBM.
-__global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, long long n, int curve, DevCtl *ctl,
-                                              unsigned long long *__restrict__ key, uint32_t *__restrict__ hist,
-                                              uint32_t *__restrict__ base) {
+__device__ __forceinline__ void keys_body(const unsigned bid, const unsigned nb, const float4 *__restrict__ posm,
+        long long n, int curve, DevCtl *ctl, unsigned long long *__restrict__ key, uint32_t *__restrict__ hist,
+        uint32_t *__restrict__ base) {
     __shared__ uint32_t h[GT_SORT_PASSES][GT_SORT_DIGITS];
     __shared__ double scale_sh;
     __shared__ float ext[6];
@@ -150,7 +155,7 @@ __global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, l
     KeyGrid grid{ext[0], ext[1], ext[2], 0.f, 0.f, scale_sh, false};
     grid.fp32 = gtq_fp32_scale(grid.scale, &grid.sh, &grid.sl);
     const bool sized = grid.scale > 0.0;
-    for (long long i0 = (long long)blockIdx.x * 256; i0 < n; i0 += (long long)gridDim.x * 256) {
+    for (long long i0 = (long long)bid * 256; i0 < n; i0 += (long long)nb * 256) {
         const long long i = i0 + threadIdx.x;
         const bool ok = i < n;
         unsigned long long k = 0;
@@ -158,7 +163,12 @@ __global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, l
         if (ok) key[i] = k;
         gt_count_digits<true>(k, ok, h);
     }
-    gt_finish_digits(h, n, hist, base, ctl);
+    gt_finish_digits(nb, h, n, hist, base, ctl);
+}
+
+__global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, long long n, int curve, DevCtl *ctl,
+        unsigned long long *__restrict__ key, uint32_t *__restrict__ hist, uint32_t *__restrict__ base) {
+    keys_body(blockIdx.x, gridDim.x, posm, n, curve, ctl, key, hist, base);
 }
 
 // Small systems: the bounding box, the keys and the whole sort in one block, in shared memory (through the kernels
@@ -172,9 +182,9 @@ constexpr size_t SMALL_SMEM = GT_SMALL_SORT * (sizeof(unsigned long long) + size
                               SMALL_WARPS * GT_SORT_DIGITS * sizeof(uint32_t);
 constexpr int SMALL_SHIFT = 23, SMALL_RUN = 32;  // bits left to the runs; the longest one that a thread puts in order
 
-__global__ __launch_bounds__(SMALL_THREADS) void k_small_sort(const float4 *__restrict__ posm, int n, int curve,
-                                                              unsigned long long *__restrict__ key,
-                                                              uint32_t *__restrict__ val) {
+__device__ __forceinline__ void small_sort_body(const unsigned bid, const unsigned nb,
+        const float4 *__restrict__ posm, int n, int curve, unsigned long long *__restrict__ key,
+        uint32_t *__restrict__ val) {
     extern __shared__ __align__(16) unsigned char smraw[];
     unsigned long long *skey = (unsigned long long *)smraw;
     uint32_t *wcnt = (uint32_t *)(skey + GT_SMALL_SORT);  // a count per warp and digit
@@ -313,6 +323,41 @@ __global__ __launch_bounds__(SMALL_THREADS) void k_small_sort(const float4 *__re
     }
 }
 
+__global__ __launch_bounds__(SMALL_THREADS) void k_small_sort(const float4 *__restrict__ posm, int n, int curve,
+        unsigned long long *__restrict__ key, uint32_t *__restrict__ val) {
+    small_sort_body(blockIdx.x, gridDim.x, posm, n, curve, key, val);
+}
+
+// ---- a table of systems ----
+__device__ __forceinline__ const float4 *keyed(const GroupedSys &s) {
+    return (s.flags & GT_SYS_PREDICTED) ? s.posm_tmp : s.posm;
+}
+
+__host__ __device__ inline unsigned keys_blocks(long long n, int nsm) {
+    return gt_grid(n, 256, (long long)nsm * (n < KEYS_MANY ? 4 : 8));
+}
+
+__global__ __launch_bounds__(BBOX_THREADS) void kg_bbox(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, BBOX_THREADS, nsm * 4);
+    if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
+        bbox_body(blockIdx.y, nb, keyed(s), s.n, s.ctl, (uint4 *)s.sb.hist, (long long)(gt_sort_scratch_bytes(s.n) / 16));
+}
+
+__global__ __launch_bounds__(256) void kg_keys(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = keys_blocks(s.n, nsm);
+    if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
+        keys_body(blockIdx.y, nb, keyed(s), s.n, s.curve, s.ctl, (unsigned long long *)s.sb.key[0], s.sb.hist,
+                  s.sb.digit_base);
+}
+
+__global__ __launch_bounds__(SMALL_THREADS) void kg_small_sort(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    if (s.flags & GT_SYS_BUILD)
+        small_sort_body(0, 1, keyed(s), (int)s.n, s.curve, (unsigned long long *)s.sb.key[0], s.sb.val[0]);
+}
+
 }  // namespace
 
 void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, SortBufs &b, cudaStream_t st) {
@@ -325,18 +370,29 @@ void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, SortBu
 
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st) {
     if (n <= 0) return;
-    const int64_t need = (n + 255) / 256, most = (int64_t)nsm * (n < KEYS_MANY ? 4 : 8);
-    k_keys<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(posm, n, curve, ctl, (unsigned long long *)b.key[0],
-                                                                  b.hist, b.digit_base);
+    k_keys<<<keys_blocks(n, nsm), 256, 0, st>>>(posm, n, curve, ctl, (unsigned long long *)b.key[0], b.hist,
+                                                b.digit_base);
     gt_note_launches(1);
 }
 
 void gt_keys_init() {
     cudaFuncSetAttribute(k_small_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM);
+    cudaFuncSetAttribute(kg_small_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM);
 }
 
 void gt_launch_small_sort(const float4 *posm, int64_t n, int curve, SortBufs &b, cudaStream_t st) {
     if (n <= 0) return;
     k_small_sort<<<1, SMALL_THREADS, SMALL_SMEM, st>>>(posm, (int)n, curve, (unsigned long long *)b.key[0], b.val[0]);
     gt_note_launches(1);
+}
+
+void gt_grouped_small_sort(const GroupedSys *t, const GroupedPlan &p, cudaStream_t st) {
+    kg_small_sort<<<p.count, SMALL_THREADS, SMALL_SMEM, st>>>(t);
+    gt_note_launches(1);
+}
+
+void gt_grouped_keys(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
+    kg_bbox<<<dim3(p.count, gt_grid(p.n_build, BBOX_THREADS, nsm * 4)), BBOX_THREADS, 0, st>>>(t, nsm);
+    kg_keys<<<dim3(p.count, keys_blocks(p.n_build, nsm)), 256, 0, st>>>(t, nsm);
+    gt_note_launches(2);
 }

@@ -2,8 +2,8 @@
 //
 // Every tick advances each resident request by one unit of work -- the start-up for a
 // new request (tree, opening-angle pass, a_old, first force with the request's MAC,
-// levels), one block step for a running one -- with the per-request parts on forked
-// streams and the tree walks of all requests of the tick in one persistent launch over
+// levels), one block step for a running one -- with every kernel of the small requests in one
+// launch (large ones have their own on forked streams) and the tree walks of all requests of the tick in one persistent launch over
 // their groups (the walk-argument table of a tick is gathered on the device from a
 // list passed by value, so no host buffer has to outlive a launch).  Requests join and
 // leave between ticks; the host never waits for the device except to admit a request
@@ -40,6 +40,21 @@ __global__ void k_select_args(TickList L, const WalkArgs *__restrict__ pool, Dev
     }
 }
 
+struct GroupList {
+    uint16_t slot[GT_SERVER_MAX_SLOTS];
+    uint8_t flags[GT_SERVER_MAX_SLOTS];
+};
+
+// the tick's table: a block per entry
+__global__ void k_select_entries(GroupList L, const GroupedSys *__restrict__ pool, GroupedSys *__restrict__ out) {
+    static_assert(sizeof(GroupedSys) % 8 == 0, "copied as words");
+    const unsigned long long *src = (const unsigned long long *)&pool[L.slot[blockIdx.x]];
+    unsigned long long *dst = (unsigned long long *)&out[blockIdx.x];
+    for (int w = threadIdx.x; w < (int)(sizeof(GroupedSys) / 8); w += blockDim.x) dst[w] = src[w];
+    __syncthreads();
+    if (threadIdx.x == 0) out[blockIdx.x].flags = L.flags[blockIdx.x];
+}
+
 struct Slot {
     bool used = false;
     uint64_t ticket = 0;
@@ -73,6 +88,8 @@ struct gt_server {
     DevCtl **d_ctl_pool = nullptr;
     WalkArgs *d_tick_args = nullptr;
     DevCtl **d_tick_ctls = nullptr;
+    GroupedSys *d_entries = nullptr;  // of every slot, and of the requests of a tick
+    GroupedSys *d_tick_entries = nullptr;
     uint32_t *d_gprefix = nullptr;
     unsigned int *d_next = nullptr;
     uint32_t *queue = nullptr;
@@ -94,6 +111,7 @@ cudaStream_t slot_stream(gt_server *v, int slot) { return v->streams[slot % (int
 
 // fork the streams of the given slots off the main stream / join them back
 void fork(gt_server *v, const std::vector<int> &use) {
+    if (use.empty()) return;
     cudaEventRecord(v->ev_fork, v->main);
     for (int j : use) cudaStreamWaitEvent(v->streams[j], v->ev_fork, 0);
 }
@@ -127,9 +145,24 @@ void batched_walk(gt_server *v, const TickList &L) {
     v->walk_launches++;
 }
 
-// One tick; false when no resident request has work left to enqueue.
+// One tick; false when no resident request has work left to enqueue.  The requests that gt_sys_groupable admits go
+// through one launch per kernel, the others through their own on forked streams: the host enqueues a tick of a dozen
+// requests in ~0.1 ms, with a launch per kernel and request it took ~0.4 ms, which was most of the time of a burst of
+// short ones (12 of 2^12 to 2^17 particles, 6 steps each: 12.1 ms, now 10.2).
 bool enqueue_tick(gt_server *v) {
-    std::vector<int> starts, runs;
+    std::vector<int> starts, runs;       // every request of the tick
+    std::vector<int> own_starts, own_runs;  // those with launches of their own
+    GroupList G;
+    GroupedPlan plan;
+    auto join_group = [&](int k, unsigned flags) {
+        gt_system *s = v->slots[k].sys;
+        if (!gt_sys_groupable(s)) return false;
+        G.slot[plan.count] = (uint16_t)k;
+        G.flags[plan.count] = (uint8_t)flags;
+        plan.add(s->n, flags, s->prm.leaf_max);
+        if (flags & GT_SYS_BUILD) gt_sys_note_build(s);
+        return true;
+    };
     for (int k = 0; k < v->max_slots; k++) {
         const Slot &s = v->slots[k];
         if (!s.used) continue;
@@ -138,14 +171,26 @@ bool enqueue_tick(gt_server *v) {
     }
     if (starts.empty() && runs.empty()) return false;
     const long long id = ++v->ticks;
-    const std::vector<int> all = streams_of(v, starts, runs), boot = streams_of(v, starts, {});
+    for (int k : starts)
+        if (!join_group(k, GT_SYS_BUILD | GT_SYS_START)) own_starts.push_back(k);
+    for (int k : runs) {
+        const Slot &sl = v->slots[k];
+        const bool rebuild = sl.sys->steps % sl.rebuild_every == 0;
+        if (!join_group(k, rebuild ? GT_SYS_STEP | GT_SYS_BUILD | GT_SYS_PREDICTED : GT_SYS_STEP)) own_runs.push_back(k);
+    }
+    const std::vector<int> all = streams_of(v, own_starts, own_runs), boot = streams_of(v, own_starts, {});
     fork(v, all);
-    for (int k : starts) {
+    if (plan.count > 0) {
+        k_select_entries<<<plan.count, 64, 0, v->main>>>(G, v->d_entries, v->d_tick_entries);
+        gt_note_launches(1);
+        gt_grouped_before_walk(v->d_tick_entries, plan, v->nsm, v->main);
+    }
+    for (int k : own_starts) {
         gt_system *s = v->slots[k].sys;
         gt_sys_build_tree(s, slot_stream(v, k), s->posm);
         gt_sys_groups_all(s, slot_stream(v, k));
     }
-    for (int k : runs) {
+    for (int k : own_runs) {
         Slot &sl = v->slots[k];
         const bool rebuild = sl.sys->steps % sl.rebuild_every == 0;
         gt_sys_step_pre(sl.sys, slot_stream(v, k), rebuild);
@@ -159,22 +204,28 @@ bool enqueue_tick(gt_server *v) {
     batched_walk(v, L);
     if (!starts.empty()) {
         fork(v, boot);
-        for (int k : starts) gt_sys_aold_from_acc(v->slots[k].sys, slot_stream(v, k));
+        gt_grouped_aold(v->d_tick_entries, plan, v->nsm, v->main);
+        for (int k : own_starts) gt_sys_aold_from_acc(v->slots[k].sys, slot_stream(v, k));
         join(v, boot);
         L.n = 0;
         for (int k : starts) { L.slot[L.n] = (uint16_t)k; L.variant[L.n++] = V_FIRST; }
         batched_walk(v, L);
     }
     fork(v, all);
+    gt_grouped_correct(v->d_tick_entries, plan, v->nsm, v->main);
+    for (int k : own_starts) gt_sys_start_levels(v->slots[k].sys, slot_stream(v, k));
+    for (int k : own_runs) gt_sys_step_post(v->slots[k].sys, slot_stream(v, k));
+    for (int j = 0; j < plan.count; j++) {
+        if (G.flags[j] & GT_SYS_START) gt_sys_note_start(v->slots[G.slot[j]].sys);
+        else v->slots[G.slot[j]].sys->steps++;
+    }
     for (int k : starts) {
         Slot &sl = v->slots[k];
-        gt_sys_start_levels(sl.sys, slot_stream(v, k));
         sl.phase = sl.nsteps > 0 ? PH_RUN : PH_FINISHING;
         if (sl.phase == PH_FINISHING) sl.done_tick = id;
     }
     for (int k : runs) {
         Slot &sl = v->slots[k];
-        gt_sys_step_post(sl.sys, slot_stream(v, k));
         if (++sl.steps_enq == sl.nsteps) {
             sl.phase = PH_FINISHING;
             sl.done_tick = id;
@@ -274,6 +325,7 @@ int gt_server_create(gt_server **out, size_t hbm_cap, int max_slots, int walk_qu
     const size_t o_ctlp = off; off = align_up(off + (size_t)max_slots * sizeof(DevCtl *));
     const size_t o_targ = off; off = align_up(off + (size_t)max_slots * sizeof(WalkArgs));
     const size_t o_tctl = off; off = align_up(off + (size_t)max_slots * sizeof(DevCtl *));
+    const size_t o_ent = off; off = align_up(off + 2 * (size_t)max_slots * sizeof(GroupedSys));
     const size_t o_gpre = off; off = align_up(off + (size_t)(max_slots + 1) * sizeof(uint32_t));
     const size_t o_next = off; off = align_up(off + sizeof(unsigned int));
     const size_t o_queue = off; off = align_up(off + warps * gt_queue_words(walk_queue) * sizeof(uint32_t));
@@ -291,6 +343,8 @@ int gt_server_create(gt_server **out, size_t hbm_cap, int max_slots, int walk_qu
     v->d_ctl_pool = (DevCtl **)(b + o_ctlp);
     v->d_tick_args = (WalkArgs *)(b + o_targ);
     v->d_tick_ctls = (DevCtl **)(b + o_tctl);
+    v->d_entries = (GroupedSys *)(b + o_ent);
+    v->d_tick_entries = v->d_entries + max_slots;
     v->d_gprefix = (uint32_t *)(b + o_gpre);
     v->d_next = (unsigned int *)(b + o_next);
     v->queue = (uint32_t *)(b + o_queue);
@@ -379,7 +433,9 @@ int gt_submit(gt_server *v, const gt_request *req, uint64_t *ticket) {
     a[V_BOOT] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, GT_MAC_OPENING_ANGLE, false);
     a[V_FIRST] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, prm.mac, true);
     DevCtl *ctl = s->ctl;
-    if (cudaMemcpyAsync(v->d_pool + (size_t)k * NVARIANT, a, sizeof(a), cudaMemcpyHostToDevice, v->admit) ||
+    const GroupedSys entry = gt_sys_entry(s, 0);
+    if (cudaMemcpyAsync(v->d_entries + k, &entry, sizeof(entry), cudaMemcpyHostToDevice, v->admit) ||
+        cudaMemcpyAsync(v->d_pool + (size_t)k * NVARIANT, a, sizeof(a), cudaMemcpyHostToDevice, v->admit) ||
         cudaMemcpyAsync(v->d_ctl_pool + k, &ctl, sizeof(ctl), cudaMemcpyHostToDevice, v->admit) ||
         cudaStreamSynchronize(v->admit)) {
         release(v, k);

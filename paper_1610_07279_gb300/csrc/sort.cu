@@ -23,12 +23,6 @@
 
 namespace {
 
-#ifndef GT_SORT_ST
-#define GT_SORT_ST 512
-#endif
-#ifndef GT_SORT_IPT
-#define GT_SORT_IPT 8
-#endif
 #ifndef GT_SORT_MINB
 #define GT_SORT_MINB 3
 #endif
@@ -60,7 +54,7 @@ __global__ __launch_bounds__(HT) void k_hist_all(long long n, const unsigned lon
         const long long i = i0 + threadIdx.x;
         gt_count_digits<false>(i < n ? key[i] : 0ull, i < n, h);
     }
-    gt_finish_digits(h, n, hist, base, ctl);
+    gt_finish_digits(gridDim.x, h, n, hist, base, ctl);
 }
 
 // Look-back of one digit: the count of digit d in all tiles before `tile`.  The status
@@ -112,14 +106,10 @@ __device__ __forceinline__ uint32_t lookback_digit(const uint32_t *status, int t
 enum { PASS_PLAIN = 0, PASS_LOW_FIRST, PASS_LOW, PASS_HIGH_FIRST };
 
 template <int MODE>
-__global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int pass, int shift,
-                                                 const unsigned long long *__restrict__ kin,
-                                                 const uint32_t *__restrict__ vin,
-                                                 unsigned long long *__restrict__ kout,
-                                                 uint32_t *__restrict__ vout,
-                                                 const uint32_t *__restrict__ digit_base,
-                                                 uint32_t *status /* this pass: ntiles x R */, int ntiles,
-                                                 DevCtl *ctl) {
+__device__ __forceinline__ void onesweep_body(const unsigned bid, const unsigned nb, long long n, int pass, int shift,
+        const unsigned long long *__restrict__ kin, const uint32_t *__restrict__ vin,
+        unsigned long long *__restrict__ kout, uint32_t *__restrict__ vout, const uint32_t *__restrict__ digit_base,
+        uint32_t *status, int ntiles, DevCtl *ctl) {
     extern __shared__ __align__(16) unsigned char smraw[];
     unsigned long long *skey = (unsigned long long *)smraw;
     uint32_t *sval = (uint32_t *)(skey + TILE);
@@ -204,6 +194,14 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
     }
 }
 
+template <int MODE>
+__global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int pass, int shift,
+        const unsigned long long *__restrict__ kin, const uint32_t *__restrict__ vin,
+        unsigned long long *__restrict__ kout, uint32_t *__restrict__ vout, const uint32_t *__restrict__ digit_base,
+        uint32_t *status, int ntiles, DevCtl *ctl) {
+    onesweep_body<MODE>(blockIdx.x, gridDim.x, n, pass, shift, kin, vin, kout, vout, digit_base, status, ntiles, ctl);
+}
+
 // ---- keys that agree in the sorted bits --------------------------------------------
 // The tree's keys are spread over the bounding cube by construction, so few of them agree in their highest 16 levels
 // (48 bits): six passes over those bits leave short runs of keys that differ only below, and these are put in order
@@ -220,10 +218,10 @@ __device__ __forceinline__ bool same_run(unsigned long long a, unsigned long lon
 
 // One thread per key: the first key of a run of two or more has it put in order, or listed if it is longer and not in
 // order already as far as looked.
-__global__ __launch_bounds__(256) void k_fix_runs(long long n, int shift, unsigned long long *key, uint32_t *val,
-                                                  uint32_t *list, DevCtl *ctl) {
+__device__ __forceinline__ void fix_runs_body(const unsigned bid, const unsigned nb, long long n, int shift,
+        unsigned long long *key, uint32_t *val, uint32_t *list, DevCtl *ctl) {
     if (ctl->sort_whole) return;
-    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
+    for (long long i = bid * 256ll + threadIdx.x; i < n; i += (long long)nb * 256) {
         const unsigned long long k0 = key[i];
         if (i + 1 >= n || !same_run(k0, key[i + 1], shift)) continue;
         if (i > 0 && same_run(key[i - 1], k0, shift)) continue;
@@ -249,11 +247,16 @@ __global__ __launch_bounds__(256) void k_fix_runs(long long n, int shift, unsign
     }
 }
 
+__global__ __launch_bounds__(256) void k_fix_runs(long long n, int shift, unsigned long long *key, uint32_t *val,
+        uint32_t *list, DevCtl *ctl) {
+    fix_runs_body(blockIdx.x, gridDim.x, n, shift, key, val, list, ctl);
+}
+
 // The listed runs, a block each: by digits in shared memory, or, beyond RUN_SMEM keys, tile by tile through the
 // other buffers.  Runs that are in order (equal keys, most of all) are left alone.
-__global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, unsigned long long *key0, uint32_t *val0,
-                                                      unsigned long long *key1, uint32_t *val1,
-                                                      const uint32_t *__restrict__ list, DevCtl *ctl) {
+__device__ __forceinline__ void fix_long_runs_body(const unsigned bid, const unsigned nb, long long n, int shift,
+        unsigned long long *key0, uint32_t *val0, unsigned long long *key1, uint32_t *val1,
+        const uint32_t *__restrict__ list, DevCtl *ctl) {
     extern __shared__ __align__(16) unsigned char smraw[];
     unsigned long long *skey = (unsigned long long *)smraw;
     uint32_t *sval = (uint32_t *)(skey + TILE);
@@ -264,7 +267,7 @@ __global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, un
     __shared__ unsigned long long len_sh;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t runs = ctl->run_count;  // 0 if the whole keys were sorted
-    for (uint32_t r = blockIdx.x; r < runs; r += gridDim.x) {
+    for (uint32_t r = bid; r < runs; r += nb) {
         const long long first = list[r];
         const unsigned long long k0 = key0[first];
         if (threadIdx.x == 0) {
@@ -379,20 +382,51 @@ __global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, un
     }
 }
 
-}  // namespace
-
-int gt_sort_tiles(int64_t n) { return (int)((n + TILE - 1) / TILE); }
-
-size_t gt_sort_scratch_bytes(int64_t n) {
-    // digit counts, and look-back status of every pass (PASSES x tiles x R x 4 B)
-    return (size_t)PASSES * R * (size_t)(1 + (gt_sort_tiles(n) > 0 ? gt_sort_tiles(n) : 1)) * sizeof(uint32_t);
+__global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, unsigned long long *key0,
+        uint32_t *val0, unsigned long long *key1, uint32_t *val1, const uint32_t *__restrict__ list, DevCtl *ctl) {
+    fix_long_runs_body(blockIdx.x, gridDim.x, n, shift, key0, val0, key1, val1, list, ctl);
 }
+
+// ---- a table of systems ----
+template <int MODE>
+__global__ __launch_bounds__(ST, GT_SORT_MINB) void kg_onesweep(const GroupedSys *__restrict__ t, int pass, int shift) {
+    const GroupedSys &s = t[blockIdx.x];
+    const int ntiles = gt_sort_tiles(s.n), src = pass & 1;
+    if (!(s.flags & GT_SYS_BUILD) || (int)blockIdx.y >= ntiles) return;
+    onesweep_body<MODE>(blockIdx.y, (unsigned)ntiles, s.n, pass, shift, (const unsigned long long *)s.sb.key[src],
+                        s.sb.val[src], (unsigned long long *)s.sb.key[src ^ 1], s.sb.val[src ^ 1], s.sb.digit_base,
+                        s.sb.status + (size_t)pass * R * ntiles, ntiles, s.ctl);
+}
+
+__host__ __device__ inline unsigned fix_blocks(long long n, int nsm) { return gt_grid(n, 256, nsm * 16); }
+__host__ __device__ inline unsigned fix_long_blocks(long long n, int nsm) { return gt_grid(n, 4 * TILE, nsm); }
+
+__global__ __launch_bounds__(256) void kg_fix_runs(const GroupedSys *__restrict__ t, int shift, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = fix_blocks(s.n, nsm);
+    if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
+        fix_runs_body(blockIdx.y, nb, s.n, shift, (unsigned long long *)s.sb.key[0], s.sb.val[0], s.sb.status, s.ctl);
+}
+
+__global__ __launch_bounds__(ST) void kg_fix_long_runs(const GroupedSys *__restrict__ t, int shift, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = fix_long_blocks(s.n, nsm);
+    if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
+        fix_long_runs_body(blockIdx.y, nb, s.n, shift, (unsigned long long *)s.sb.key[0], s.sb.val[0],
+                           (unsigned long long *)s.sb.key[1], s.sb.val[1], s.sb.status, s.ctl);
+}
+
+}  // namespace
 
 void gt_sort_init() {
     gt_keys_init();
     for (auto kernel : {k_onesweep<PASS_PLAIN>, k_onesweep<PASS_LOW_FIRST>, k_onesweep<PASS_LOW>,
                         k_onesweep<PASS_HIGH_FIRST>})
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+    for (auto kernel : {kg_onesweep<PASS_PLAIN>, kg_onesweep<PASS_LOW_FIRST>, kg_onesweep<PASS_LOW>,
+                        kg_onesweep<PASS_HIGH_FIRST>})
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+    cudaFuncSetAttribute(kg_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
     cudaFuncSetAttribute(k_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
 }
 
@@ -418,10 +452,8 @@ void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStrea
     for (int p = 3; p < PASSES; p++) onesweep<PASS_PLAIN>(b, n, ctl, p, gt_tree_digit_shift(p), st);
     const int shift = gt_tree_digit_shift(2);
     uint32_t *list = b.status;  // the look-backs are over
-    const int64_t need = (n + 255) / 256, most = (int64_t)nsm * 16;
-    k_fix_runs<<<(unsigned)(need < most ? need : most), 256, 0, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
-                                                                      list, ctl);
-    k_fix_long_runs<<<gt_grid(n, 4 * TILE, nsm), ST, SCATTER_SMEM, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
+    k_fix_runs<<<fix_blocks(n, nsm), 256, 0, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0], list, ctl);
+    k_fix_long_runs<<<fix_long_blocks(n, nsm), ST, SCATTER_SMEM, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
                                                    (unsigned long long *)b.key[1], b.val[1], list, ctl);
     gt_note_launches(2);
 }
@@ -531,4 +563,23 @@ extern "C" int gt_sort_noalloc_status(gt_stream stream) {
                 cudaStreamSynchronize(st) != cudaSuccess))
         return GT_ECUDA;
     return err;
+}
+
+void gt_grouped_sort(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
+    if (p.n_build <= 0) return;
+    if (p.n_build <= GT_SMALL_SORT) {  // (a small system among larger ones costs their launches nothing)
+        gt_grouped_small_sort(t, p, st);
+        return;
+    }
+    gt_grouped_keys(t, p, nsm, st);
+    const dim3 grid(p.count, gt_sort_tiles(p.n_build));
+    kg_onesweep<PASS_LOW_FIRST><<<grid, ST, SCATTER_SMEM, st>>>(t, 0, gt_tree_digit_shift(0));
+    kg_onesweep<PASS_LOW><<<grid, ST, SCATTER_SMEM, st>>>(t, 1, gt_tree_digit_shift(1));
+    kg_onesweep<PASS_HIGH_FIRST><<<grid, ST, SCATTER_SMEM, st>>>(t, 2, gt_tree_digit_shift(2));
+    for (int q = 3; q < PASSES; q++)
+        kg_onesweep<PASS_PLAIN><<<grid, ST, SCATTER_SMEM, st>>>(t, q, gt_tree_digit_shift(q));
+    const int shift = gt_tree_digit_shift(2);
+    kg_fix_runs<<<dim3(p.count, fix_blocks(p.n_build, nsm)), 256, 0, st>>>(t, shift, nsm);
+    kg_fix_long_runs<<<dim3(p.count, fix_long_blocks(p.n_build, nsm)), ST, SCATTER_SMEM, st>>>(t, shift, nsm);
+    gt_note_launches(PASSES + 2);
 }

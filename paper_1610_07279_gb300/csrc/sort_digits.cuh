@@ -39,15 +39,15 @@ __device__ __forceinline__ void gt_count_digits(unsigned long long k, bool ok, u
 // launch of its own for that took 7 to 8 us), resets the passes' tile tickets, and says whether the tree's keys crowd
 // into so small a part of the cube that they are sorted by all of their bits (n: the number of keys).
 constexpr int GT_CROWD_PASS = 3;  // the digit of levels 11 to 13
-__device__ __forceinline__ void gt_finish_digits(const uint32_t (*h)[GT_SORT_DIGITS], long long n, uint32_t *hist,
-                                                 uint32_t *base, DevCtl *ctl) {
+__device__ __forceinline__ void gt_finish_digits(unsigned nb, const uint32_t (*h)[GT_SORT_DIGITS], long long n,
+                                                 uint32_t *hist, uint32_t *base, DevCtl *ctl) {
     __shared__ bool last;
     __syncthreads();
     for (int p = 0; p < GT_SORT_PASSES; p++)
         if (h[p][threadIdx.x]) atomicAdd(&hist[p * GT_SORT_DIGITS + threadIdx.x], h[p][threadIdx.x]);
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&ctl->digits_done, 1u) == gridDim.x - 1u;
+    if (threadIdx.x == 0) last = atomicAdd(&ctl->digits_done, 1u) == nb - 1u;
     __syncthreads();
     if (!last) return;
     __threadfence();

@@ -160,7 +160,7 @@ __global__ __launch_bounds__(BT) void k_build_level(int lvl, const unsigned long
 // the same numbering as the level-by-level split: level by level, and inside a level by
 // first particle.  A node's first child starts at its own first particle; the others
 // are the next nodes of the child level that start before its end.
-constexpr int FLAT_LWIN = 64;              // the largest leaf_max of this build
+constexpr int FLAT_LWIN = GT_FLAT_LEAF_MAX;              // the largest leaf_max of this build
 constexpr int FB = 256;                    // threads per block
 // Particles per tile: a block takes its tile's rounds of FB particles one after another, so that small systems,
 // which fill few blocks, get short tiles (8192 particles: k_flat_scatter 15.6 us with 8 rounds).
@@ -201,15 +201,15 @@ __device__ __forceinline__ int leaf_level_of(const int8_t *ds, int j) {
 // start and end counts per level (column-major: counter k of tile t at cnt[k * ntiles + t]).
 // MT > 0: leaf_max == MT; MT == 0: any leaf_max up to FLAT_LWIN (running minima in shared memory).
 template <int MT, int ROUNDS>
-__global__ __launch_bounds__(FB) void k_flat_marks(const unsigned long long *__restrict__ skey, long long n,
-                                                   int M, uint16_t *__restrict__ dl,
-                                                   uint32_t *__restrict__ cnt, int ntiles) {
+__device__ __forceinline__ void flat_marks_body(const unsigned bid, const unsigned nb,
+        const unsigned long long *__restrict__ skey, long long n, int M, uint16_t *__restrict__ dl,
+        uint32_t *__restrict__ cnt, int ntiles) {
     constexpr int W = FLAT_LWIN, FT = ROUNDS * FB;
     constexpr int MW = MT > 0 ? 1 : W;
     __shared__ int8_t ds[FT + 2 * W + 1];      // d of positions base - W .. base + FT + W
     __shared__ uint8_t mr[MW][FB];             // generic: 1 + smallest d over (i, i + b]
     __shared__ unsigned int c[NREC];
-    const long long base = (long long)blockIdx.x * FT;
+    const long long base = (long long)bid * FT;
     for (int j = threadIdx.x; j < FT + 2 * W + 1; j += FB) {
         const long long p = base - W + j;
         ds[j] = (int8_t)((p > 0 && p < n) ? key_diff_digit(skey[p - 1], skey[p]) : -1);
@@ -243,17 +243,23 @@ __global__ __launch_bounds__(FB) void k_flat_marks(const unsigned long long *__r
         for (int l = d1 + 1; l <= leaf; l++) atomicAdd(&c[GT_TREE_LEVELS + l], 1u);
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < NREC; k += FB) cnt[(size_t)k * ntiles + blockIdx.x] = c[k];
+    for (int k = threadIdx.x; k < NREC; k += FB) cnt[(size_t)k * ntiles + bid] = c[k];
+}
+
+template <int MT, int ROUNDS>
+__global__ __launch_bounds__(FB) void k_flat_marks(const unsigned long long *__restrict__ skey, long long n, int M,
+        uint16_t *__restrict__ dl, uint32_t *__restrict__ cnt, int ntiles) {
+    flat_marks_body<MT, ROUNDS>(blockIdx.x, gridDim.x, skey, n, M, dl, cnt, ntiles);
 }
 
 // The last block of a kernel to come here gets true (its threads see what the others wrote before); *done starts at
 // zero and is left at zero.
-__device__ __forceinline__ bool last_block(unsigned int *done) {
+__device__ __forceinline__ bool last_block(unsigned nb, unsigned int *done) {
     __shared__ bool last;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        last = atomicAdd(done, 1u) == gridDim.x - 1u;
+        last = atomicAdd(done, 1u) == nb - 1u;
         if (last) *done = 0u;
     }
     __syncthreads();
@@ -263,10 +269,10 @@ __device__ __forceinline__ bool last_block(unsigned int *done) {
 
 // one block per counter: exclusive scan over the tiles, the column total into tot[k]; the last block then sets the
 // level starts from the per-level node counts (clamped to the node capacity) and clears the cell list's counters
-__global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, int ntiles, uint32_t *__restrict__ tot,
-                                                    long long cap, DevCtl *ctl) {
+__device__ __forceinline__ void flat_scan_body(const unsigned bid, const unsigned nb, uint32_t *__restrict__ cnt,
+        int ntiles, uint32_t *__restrict__ tot, long long cap, DevCtl *ctl) {
     __shared__ unsigned int tmp[1024 / 32 + 1];
-    uint32_t *col = cnt + (size_t)blockIdx.x * ntiles;
+    uint32_t *col = cnt + (size_t)bid * ntiles;
     unsigned int carry = 0;
     for (int b0 = 0; b0 < ntiles; b0 += 1024) {
         const int t = b0 + (int)threadIdx.x;
@@ -276,8 +282,8 @@ __global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, 
         if (t < ntiles) col[t] = carry + e;
         carry += total;
     }
-    if (threadIdx.x == 0) tot[blockIdx.x] = carry;
-    if (!last_block(&ctl->scan_done)) return;
+    if (threadIdx.x == 0) tot[bid] = carry;
+    if (!last_block(nb, &ctl->scan_done)) return;
     for (int b = threadIdx.x; b < GT_CELL_BUCKETS; b += 1024) ctl->cell_bucket[b] = 0;
     if (threadIdx.x >= 32) return;
     const int l = threadIdx.x;
@@ -293,20 +299,25 @@ __global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, 
     if (l == GT_TREE_LEVELS && sum > most) gt_set_error(ctl, GT_EOVERFLOW, GTK_BUILD);
 }
 
+__global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, int ntiles,
+        uint32_t *__restrict__ tot, long long cap, DevCtl *ctl) {
+    flat_scan_body(blockIdx.x, gridDim.x, cnt, ntiles, tot, cap, ctl);
+}
+
 // every start and end to its node: first, the first child and the parent along a
 // particle's own chain of starts, leaves; an end goes to count (as the end position)
 template <int ROUNDS>
-__global__ __launch_bounds__(FB) void k_flat_scatter(const uint16_t *__restrict__ dl, long long n,
-                                                     const uint32_t *__restrict__ cnt, int ntiles,
-                                                     long long cap, Nodes nd, const DevCtl *__restrict__ ctl) {
+__device__ __forceinline__ void flat_scatter_body(const unsigned bid, const unsigned nb,
+        const uint16_t *__restrict__ dl, long long n, const uint32_t *__restrict__ cnt, int ntiles, long long cap,
+        Nodes nd, const DevCtl *__restrict__ ctl) {
     constexpr int FT = ROUNDS * FB;
     __shared__ uint32_t lb[GT_TREE_LEVELS];
     __shared__ uint32_t run[NREC];
     __shared__ uint32_t wc[FB / 32][NREC];
     __shared__ uint16_t dls[FT + 1];
-    const long long base = (long long)blockIdx.x * FT;
+    const long long base = (long long)bid * FT;
     for (int k = threadIdx.x; k < GT_TREE_LEVELS; k += FB) lb[k] = ctl->level_start[k];
-    for (int k = threadIdx.x; k < NREC; k += FB) run[k] = cnt[(size_t)k * ntiles + blockIdx.x];
+    for (int k = threadIdx.x; k < NREC; k += FB) run[k] = cnt[(size_t)k * ntiles + bid];
     for (int j = threadIdx.x; j <= FT; j += FB) dls[j] = base + j < n ? dl[base + j] : (uint16_t)0;  // d(n) = -1
     __syncthreads();
     const int w = threadIdx.x >> 5;
@@ -374,14 +385,21 @@ __global__ __launch_bounds__(FB) void k_flat_scatter(const uint16_t *__restrict_
     }
 }
 
+template <int ROUNDS>
+__global__ __launch_bounds__(FB) void k_flat_scatter(const uint16_t *__restrict__ dl, long long n,
+        const uint32_t *__restrict__ cnt, int ntiles, long long cap, Nodes nd, const DevCtl *__restrict__ ctl) {
+    flat_scatter_body<ROUNDS>(blockIdx.x, gridDim.x, dl, n, cnt, ntiles, cap, nd, ctl);
+}
+
 // per node: count = end - first; a node with children counts them (the nodes of the
 // next level from its first child on that start before its end) and is their parent
-__global__ __launch_bounds__(256) void k_flat_link(Nodes nd, long long cap, const DevCtl *__restrict__ ctl) {
+__device__ __forceinline__ void flat_link_body(const unsigned bid, const unsigned nb, Nodes nd, long long cap,
+        const DevCtl *__restrict__ ctl) {
     __shared__ uint32_t ls[GT_TREE_LEVELS + 2];
     for (int i = threadIdx.x; i < GT_TREE_LEVELS + 2; i += 256) ls[i] = ctl->level_start[i];
     __syncthreads();
     const long long nn = ls[GT_TREE_LEVELS];
-    for (long long p = blockIdx.x * 256ll + threadIdx.x; p < nn; p += (long long)gridDim.x * 256) {
+    for (long long p = bid * 256ll + threadIdx.x; p < nn; p += (long long)nb * 256) {
         const uint32_t f = nd.first[p], e = nd.count[p];
         nd.count[p] = e - f;
         const int32_t c0 = nd.child[p];
@@ -401,6 +419,10 @@ __global__ __launch_bounds__(256) void k_flat_link(Nodes nd, long long cap, cons
         }
         nd.nchild[p] = nch;
     }
+}
+
+__global__ __launch_bounds__(256) void k_flat_link(Nodes nd, long long cap, const DevCtl *__restrict__ ctl) {
+    flat_link_body(blockIdx.x, gridDim.x, nd, cap, ctl);
 }
 
 __device__ __forceinline__ float sq3f(float dx, float dy, float dz) {
@@ -427,7 +449,8 @@ __device__ __forceinline__ int cell_bucket_of(const Nodes &nd, uint32_t p, const
     return lvl * GT_LEVEL_BUCKETS + GT_LEAF_BUCKETS + (int)nd.nchild[p] - 1;
 }
 
-__global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, DevCtl *ctl) {
+__device__ __forceinline__ void cell_count_body(const unsigned bid, const unsigned nb, Nodes nd, long long cap,
+        DevCtl *ctl) {
     __shared__ uint32_t ls[GT_TREE_LEVELS + 1];
     __shared__ uint32_t h[GT_CELL_BUCKETS];
     for (int i = threadIdx.x; i <= GT_TREE_LEVELS; i += 256) ls[i] = ctl->level_start[i];
@@ -435,12 +458,12 @@ __global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, Dev
     __syncthreads();
     long long nn = ls[GT_TREE_LEVELS];
     if (nn > cap) nn = cap;
-    for (long long p = blockIdx.x * 256ll + threadIdx.x; p < nn; p += (long long)gridDim.x * 256)
+    for (long long p = bid * 256ll + threadIdx.x; p < nn; p += (long long)nb * 256)
         atomicAdd(&h[cell_bucket_of(nd, (uint32_t)p, ls)], 1u);
     __syncthreads();
     for (int i = threadIdx.x; i < GT_CELL_BUCKETS; i += 256)
         if (h[i]) atomicAdd(&ctl->cell_bucket[i], h[i]);
-    if (!last_block(&ctl->cells_done)) return;
+    if (!last_block(nb, &ctl->cells_done)) return;
     // bucket sizes -> fill cursors, and where every level's leaves and cells with children start
     constexpr int PER = (GT_CELL_BUCKETS + 255) / 256;  // neighbouring buckets of a thread
     __shared__ unsigned int tmp[256 / 32 + 1];
@@ -466,19 +489,24 @@ __global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, Dev
     if (threadIdx.x == 0) ctl->seg[2 * GT_TREE_LEVELS] = total;
 }
 
+__global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, DevCtl *ctl) {
+    cell_count_body(blockIdx.x, gridDim.x, nd, cap, ctl);
+}
+
 // A block takes a contiguous range of nodes, counts them per bucket in shared memory,
 // reserves its room in every bucket with one global atomic each, and fills it.
 constexpr int CF_NODES = 4096;  // most nodes of such a range; small trees take shorter ones, so that every block has one
 
-__global__ __launch_bounds__(256) void k_cell_fill(Nodes nd, long long cap, DevCtl *ctl) {
+__device__ __forceinline__ void cell_fill_body(const unsigned bid, const unsigned nb, Nodes nd, long long cap,
+        DevCtl *ctl) {
     __shared__ uint32_t ls[GT_TREE_LEVELS + 1];
     __shared__ uint32_t h[GT_CELL_BUCKETS];
     for (int i = threadIdx.x; i <= GT_TREE_LEVELS; i += 256) ls[i] = ctl->level_start[i];
     long long nn = ctl->level_start[GT_TREE_LEVELS];
     if (nn > cap) nn = cap;
-    const long long share = ((nn + gridDim.x - 1) / gridDim.x + 255) / 256 * 256;
+    const long long share = ((nn + nb - 1) / nb + 255) / 256 * 256;
     const long long chunk = share < CF_NODES ? share : CF_NODES;
-    for (long long b0 = (long long)blockIdx.x * chunk; b0 < nn; b0 += (long long)gridDim.x * chunk) {
+    for (long long b0 = (long long)bid * chunk; b0 < nn; b0 += (long long)nb * chunk) {
         __syncthreads();
         for (int i = threadIdx.x; i < GT_CELL_BUCKETS; i += 256) h[i] = 0;
         __syncthreads();
@@ -492,6 +520,10 @@ __global__ __launch_bounds__(256) void k_cell_fill(Nodes nd, long long cap, DevC
         for (long long p = b0 + threadIdx.x; p < b1; p += 256)
             nd.cells[atomicAdd(&h[cell_bucket_of(nd, (uint32_t)p, ls)], 1u)] = (uint32_t)p;
     }
+}
+
+__global__ __launch_bounds__(256) void k_cell_fill(Nodes nd, long long cap, DevCtl *ctl) {
+    cell_fill_body(blockIdx.x, gridDim.x, nd, cap, ctl);
 }
 
 // ---- A5: pseudo j-particles, every node in one launch ------------------------------
@@ -707,7 +739,8 @@ __device__ __forceinline__ void pseudo_cell_coop(const Nodes &nd, const CellInfo
 }
 
 template <bool WITH_MASS>
-__global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const float4 *__restrict__ posm, DevCtl *ctl) {
+__device__ __forceinline__ void pseudo_body(const unsigned bid, const unsigned nb, Nodes nd,
+        const float4 *__restrict__ posm, DevCtl *ctl) {
     __shared__ uint32_t seg[NSEG + 1];
     __shared__ uint8_t olvl[NSEG], ocell[NSEG];      // ticket order: segment level and kind
     __shared__ uint32_t ocum[NSEG + 1];              // first ticket of every entry
@@ -818,6 +851,71 @@ __global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const f
     }
 }
 
+template <bool WITH_MASS>
+__global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const float4 *__restrict__ posm, DevCtl *ctl) {
+    pseudo_body<WITH_MASS>(blockIdx.x, gridDim.x, nd, posm, ctl);
+}
+
+// ---- a table of systems (two rounds of marks each: GT_GROUPED_MOST is below GT_FLAT_SMALL) ----
+struct FlatScratch {
+    uint16_t *dl;
+    uint32_t *cnt, *tot;
+    int ntiles;
+    __host__ __device__ FlatScratch(uint8_t *scratch, long long n, int rounds) {
+        ntiles = (int)((n + rounds * FB - 1) / (rounds * FB));
+        dl = (uint16_t *)scratch;
+        cnt = (uint32_t *)(scratch + (2 * (size_t)(n > 0 ? n : 1) + 15) / 16 * 16);
+        tot = cnt + (size_t)NREC * ntiles;
+    }
+};
+
+template <int MT>
+__global__ __launch_bounds__(FB) void kg_flat_marks(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    const FlatScratch f(s.bscratch, s.n, 2);
+    if ((s.flags & GT_SYS_BUILD) && (int)blockIdx.y < f.ntiles)
+        flat_marks_body<MT, 2>(blockIdx.y, (unsigned)f.ntiles, (const unsigned long long *)s.sb.key[0], s.n, s.leaf_max,
+                               f.dl, f.cnt, f.ntiles);
+}
+
+__global__ __launch_bounds__(1024) void kg_flat_scan(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    const FlatScratch f(s.bscratch, s.n, 2);
+    if (s.flags & GT_SYS_BUILD) flat_scan_body(blockIdx.y, NREC, f.cnt, f.ntiles, f.tot, s.cap, s.ctl);
+}
+
+__global__ __launch_bounds__(FB) void kg_flat_scatter(const GroupedSys *__restrict__ t) {
+    const GroupedSys &s = t[blockIdx.x];
+    const FlatScratch f(s.bscratch, s.n, 2);
+    if ((s.flags & GT_SYS_BUILD) && (int)blockIdx.y < f.ntiles)
+        flat_scatter_body<2>(blockIdx.y, (unsigned)f.ntiles, f.dl, s.n, f.cnt, f.ntiles, s.cap, s.nd, s.ctl);
+}
+
+__global__ __launch_bounds__(256) void kg_flat_link(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 256, nsm * 8);
+    if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb) flat_link_body(blockIdx.y, nb, s.nd, s.cap, s.ctl);
+}
+
+__global__ __launch_bounds__(256) void kg_cell_count(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 512, nsm * 4);
+    if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb) cell_count_body(blockIdx.y, nb, s.nd, s.cap, s.ctl);
+}
+
+__global__ __launch_bounds__(256) void kg_cell_fill(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    const unsigned nb = gt_grid(s.n, 1024, nsm * 2);
+    if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb) cell_fill_body(blockIdx.y, nb, s.nd, s.cap, s.ctl);
+}
+
+__global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void kg_pseudo(const GroupedSys *__restrict__ t, int nsm) {
+    const GroupedSys &s = t[blockIdx.x];
+    if (blockIdx.y >= gt_grid(s.n, 64, nsm * GT_PSEUDO_MINB)) return;
+    if (s.flags & GT_SYS_BUILD) pseudo_body<true>(blockIdx.y, gridDim.y, s.nd, s.posm, s.ctl);
+    else pseudo_body<false>(blockIdx.y, gridDim.y, s.nd, s.posm, s.ctl);
+}
+
 }  // namespace
 
 size_t gt_build_scratch_bytes(int64_t n) {
@@ -831,12 +929,8 @@ namespace {
 template <int ROUNDS>
 void launch_flat(const unsigned long long *k, int64_t n, int leaf_max, Nodes nd, int64_t cap, uint8_t *scratch,
                  DevCtl *ctl, int nsm, cudaStream_t st) {
-    constexpr int FT = ROUNDS * FB;
-    const int ntiles = (int)((n + FT - 1) / FT);
-    uint16_t *dl = (uint16_t *)scratch;
-    uint32_t *cnt = (uint32_t *)(scratch + (2 * (size_t)(n > 0 ? n : 1) + 15) / 16 * 16);
-    uint32_t *tot = cnt + (size_t)NREC * ntiles;
-    if (ntiles > 0) {
+    const FlatScratch f(scratch, n, ROUNDS);
+    if (f.ntiles > 0) {
         auto marks = k_flat_marks<0, ROUNDS>;
         switch (leaf_max) {
         case 4: marks = k_flat_marks<4, ROUNDS>; break;
@@ -845,12 +939,12 @@ void launch_flat(const unsigned long long *k, int64_t n, int leaf_max, Nodes nd,
         case 24: marks = k_flat_marks<24, ROUNDS>; break;
         case 32: marks = k_flat_marks<32, ROUNDS>; break;
         }
-        marks<<<ntiles, FB, 0, st>>>(k, n, leaf_max, dl, cnt, ntiles);
+        marks<<<f.ntiles, FB, 0, st>>>(k, n, leaf_max, f.dl, f.cnt, f.ntiles);
         gt_note_launches(1);
     }
-    { k_flat_scan<<<NREC, 1024, 0, st>>>(cnt, ntiles, tot, cap, ctl); gt_note_launches(1); }
-    if (ntiles > 0) {
-        k_flat_scatter<ROUNDS><<<ntiles, FB, 0, st>>>(dl, n, cnt, ntiles, cap, nd, ctl);
+    { k_flat_scan<<<NREC, 1024, 0, st>>>(f.cnt, f.ntiles, f.tot, cap, ctl); gt_note_launches(1); }
+    if (f.ntiles > 0) {
+        k_flat_scatter<ROUNDS><<<f.ntiles, FB, 0, st>>>(f.dl, n, f.cnt, f.ntiles, cap, nd, ctl);
         { k_flat_link<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(nd, cap, ctl); }
         gt_note_launches(2);
     }
@@ -883,5 +977,35 @@ void gt_launch_pseudo(Nodes nd, int64_t n, const float4 *posm, DevCtl *ctl, int 
     const unsigned grid = gt_grid(n, 64, nsm * GT_PSEUDO_MINB);
     if (with_mass) { k_pseudo<true><<<grid, PL, 0, st>>>(nd, posm, ctl); }
     else { k_pseudo<false><<<grid, PL, 0, st>>>(nd, posm, ctl); }
+    gt_note_launches(1);
+}
+
+void gt_grouped_build(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
+    static_assert(GT_GROUPED_MOST <= GT_FLAT_SMALL, "two rounds");
+    const int64_t n = p.n_build;
+    if (n <= 0) return;
+    auto marks = kg_flat_marks<0>;
+    switch (p.leaf_max) {
+    case 4: marks = kg_flat_marks<4>; break;
+    case 8: marks = kg_flat_marks<8>; break;
+    case 16: marks = kg_flat_marks<16>; break;
+    case 24: marks = kg_flat_marks<24>; break;
+    case 32: marks = kg_flat_marks<32>; break;
+    }
+    const unsigned tiles = (unsigned)((n + 2 * FB - 1) / (2 * FB));
+    marks<<<dim3(p.count, tiles), FB, 0, st>>>(t);
+    kg_flat_scan<<<dim3(p.count, NREC), 1024, 0, st>>>(t);
+    kg_flat_scatter<<<dim3(p.count, tiles), FB, 0, st>>>(t);
+    kg_flat_link<<<dim3(p.count, gt_grid(n, 256, nsm * 8)), 256, 0, st>>>(t, nsm);
+    kg_cell_count<<<dim3(p.count, gt_grid(n, 512, nsm * 4)), 256, 0, st>>>(t, nsm);
+    kg_cell_fill<<<dim3(p.count, gt_grid(n, 1024, nsm * 2)), 256, 0, st>>>(t, nsm);
+    gt_note_launches(6);
+}
+
+void gt_grouped_pseudo(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
+    // A block of a system waits for that system's blocks only, so all systems should have some at once: the systems
+    // vary fastest, and four grids' worth of blocks let those of finished systems make room for the others'.
+    const int most = nsm * GT_PSEUDO_MINB, share = (4 * most + p.count - 1) / p.count;
+    kg_pseudo<<<dim3(p.count, gt_grid(p.n_all, 64, share < most ? share : most)), PL, 0, st>>>(t, nsm);
     gt_note_launches(1);
 }

@@ -986,6 +986,21 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
     const uint32_t total = gprefix[nsys];
     const uint32_t T = team_of(total, gridDim.x * NWARP), team = warp / T, first = team * T;
     uint2 *q = (uint2 *)queue + (size_t)(blockIdx.x * NWARP + first) * gt_queue_ring(qcap);
+    unsigned long long *stat = stat_sm[warp];
+    const WalkArgs &a = sargs[warp];
+    // A warp's groups are in ascending order: it looks a system up, fetches its arguments and adds to its counters only
+    // when the system changes (for every group: 64 systems of 2^12 to 2^18 particles 7225 us, now 7094).
+    int sys = -1;
+    uint32_t g0 = 0, g1 = 0;  // the system's first group and the next one's
+    if (lane < 2) stat[lane] = 0;
+    __syncwarp();
+    auto count = [&]() {
+        if (sys >= 0 && lane == 0) {
+            if (stat[0]) atomicAdd(&a.ctl->interactions, stat[0]);
+            if (stat[1]) atomicAdd(&a.ctl->mac_tests, stat[1]);
+        }
+        __syncwarp();
+    };
     for (;;) {
         uint32_t gg = 0;
         if (T == 1) {
@@ -997,36 +1012,33 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
             gg = g_sm[team];
         }
         if (gg >= total) break;
-        int sys = 0;
-        if (lane == 0) sys = system_of(gprefix, nsys, gg);
-        sys = __shfl_sync(0xffffffffu, sys, 0);
-        static_assert(sizeof(WalkArgs) % 4 == 0, "copied as words");
-        const uint32_t *src = (const uint32_t *)&args[sys];
-        uint32_t *dst = (uint32_t *)&sargs[warp];
-        for (int w = lane; w < (int)(sizeof(WalkArgs) / 4); w += 32) dst[w] = src[w];
-        unsigned long long *stat = stat_sm[warp];
-        if (lane < 2) stat[lane] = 0;
-        __syncwarp();
-        if (mac >= 0 && lane == 0) sargs[warp].mac = mac;
-        __syncwarp();
-        const WalkArgs &a = sargs[warp];
-        const uint32_t g = gg - gprefix[sys];
-        const uint32_t ngroups = gprefix[sys + 1] - gprefix[sys];
+        if (gg >= g1) {
+            count();
+            if (lane == 0) sys = system_of(gprefix, nsys, gg);
+            sys = __shfl_sync(0xffffffffu, sys, 0);
+            g0 = gprefix[sys];
+            g1 = gprefix[sys + 1];
+            static_assert(sizeof(WalkArgs) % 4 == 0, "copied as words");
+            const uint32_t *src = (const uint32_t *)&args[sys];
+            uint32_t *dst = (uint32_t *)&sargs[warp];
+            for (int w = lane; w < (int)(sizeof(WalkArgs) / 4); w += 32) dst[w] = src[w];
+            if (lane < 2) stat[lane] = 0;
+            __syncwarp();
+            if (mac >= 0 && lane == 0) sargs[warp].mac = mac;
+            __syncwarp();
+        }
         // the batch queue replaces the system's own
         if (T == 1) {
-            walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[warp], q, stat);
+            walk_group<MAC, LEVELS>(a, gg - g0, g1 - g0, list_sm[warp], q, stat);
         } else {
-            if (!team_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
-                walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat);
+            if (!team_group<MAC, LEVELS>(a, gg - g0, g1 - g0, list_sm[first], q, stat, counts_sm + first, team, T) &&
+                warp == first)
+                walk_group<MAC, LEVELS>(a, gg - g0, g1 - g0, list_sm[first], q, stat);
             team_sync(team, T);
         }
-        __syncwarp();
-        if (lane == 0) {
-            if (stat[0]) atomicAdd(&a.ctl->interactions, stat[0]);
-            if (stat[1]) atomicAdd(&a.ctl->mac_tests, stat[1]);
-        }
-        __syncwarp();
     }
+    __syncwarp();
+    count();
 }
 
 // gprefix over the systems' group counts (one warp; also resets the batch counter)
