@@ -105,6 +105,10 @@ __device__ __forceinline__ void gt_set_error(DevCtl *ctl, int code, int where) {
     if (atomicCAS(&ctl->err, 0, code) == 0) ctl->err_where = where;
 }
 
+// First in every kernel that gt_launch starts: what came before it in the stream is complete and visible from here on.
+// Blocks that come and go must all pass it, early exits too, so that the next kernel doesn't pass its own before.
+__device__ __forceinline__ void gt_grid_ready() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // FP32 values as unsigned integers in the same order (for atomic minima and maxima), and back.
 __device__ __forceinline__ unsigned int gt_ordered(float f) {
     const unsigned int b = __float_as_uint(f);
@@ -251,6 +255,27 @@ __device__ __forceinline__ unsigned int lookback_warp(unsigned long long *status
 // ---- host-side launch helpers (defined in the .cu files) --------------------
 // Every helper reports the kernels it launched (counted for gt_kernel_launches).
 void gt_note_launches(int k);
+
+// A launch whose blocks may be set up while the kernel before it in the stream still runs (they wait in
+// gt_grid_ready, so the kernel has to begin with it): as its blocks end, not earlier, where they would take the room of
+// its last ones (a sort pass told to let the next one in at its start: 1000001 keys 198 us, as it ends 157, launches the
+// ordinary way 180; a build of 2^20 particles 353, 326 and 378 us; 2^24 2700, 2635 and 2683; a force on 8192 particles
+// 212 the ordinary way, 190).  The first kernel of a call, and after another stream was waited for, is launched the
+// ordinary way.
+template <class... P, class... A>
+inline void gt_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchAttribute early;
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &early;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
 
 // Blocks of a kernel that loops over its work: one for every `per` particles, at most `most`.  (The cells of a tree
 // are fewer than its particles but for chains, so `per` bounds the blocks with work; a full grid for each of many

@@ -44,12 +44,14 @@ __device__ __forceinline__ void prepare_body(const unsigned bid, const unsigned 
 }
 
 __global__ void k_prepare(DevCtl *ctl, int begin_step) {
+    gt_grid_ready();
     prepare_body(blockIdx.x, gridDim.x, ctl, begin_step);
 }
 
 __global__ void k_set_nactive(DevCtl *ctl, unsigned int n_active) { ctl->n_active = n_active; }
 
 __global__ void k_mirror(const DevCtl *ctl, StepMirror *dst) {
+    gt_grid_ready();
     volatile StepMirror *d = dst;
     d->tnext_acc = ctl->tnext_acc;
     d->n_active = ctl->n_active;
@@ -79,6 +81,7 @@ __device__ __forceinline__ void predict2_body(const unsigned bid, const unsigned
 
 __global__ __launch_bounds__(256) void k_predict2(State s, long long n, const DevCtl *__restrict__ ctl,
         float4 *__restrict__ posm, int ahead) {
+    gt_grid_ready();
     predict2_body(blockIdx.x, gridDim.x, s, n, ctl, posm, ahead);
 }
 
@@ -99,10 +102,12 @@ __device__ __forceinline__ void predict_body(const unsigned bid, const unsigned 
 
 __global__ __launch_bounds__(256) void k_predict(State s, long long n, const DevCtl *__restrict__ ctl,
         float4 *__restrict__ posm, int ahead) {
+    gt_grid_ready();
     predict_body(blockIdx.x, gridDim.x, s, n, ctl, posm, ahead);
 }
 
 __global__ __launch_bounds__(256) void k_load(State s, long long n, float4 *__restrict__ posm) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i >= n) return;
     posm[i] = make_float4(d2f(s.rx[i]), d2f(s.ry[i]), d2f(s.rz[i]), s.mass[i]);
@@ -118,6 +123,7 @@ __global__ __launch_bounds__(256) void k_load(State s, long long n, float4 *__re
 __global__ __launch_bounds__(256) void k_load_from(State s, long long n, const double *__restrict__ pos,
                                                    const double *__restrict__ vel, const float *__restrict__ mass,
                                                    float4 *__restrict__ posm) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i >= n) return;
     const double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2];
@@ -160,6 +166,7 @@ __device__ __forceinline__ void permute_body(const unsigned bid, const unsigned 
 
 __global__ __launch_bounds__(256) void k_permute(State src, State dst, const float4 *__restrict__ pin,
         float4 *__restrict__ pout, const uint32_t *__restrict__ perm, long long n) {
+    gt_grid_ready();
     permute_body(blockIdx.x, gridDim.x, src, dst, pin, pout, perm, n);
 }
 
@@ -185,6 +192,7 @@ __device__ __forceinline__ void copy_state_body(const unsigned bid, const unsign
 
 __global__ __launch_bounds__(256) void k_copy_state(State src, State dst, const float4 *__restrict__ pin,
         float4 *__restrict__ pout, long long n) {
+    gt_grid_ready();
     copy_state_body(blockIdx.x, gridDim.x, src, dst, pin, pout, n);
 }
 
@@ -192,6 +200,7 @@ __global__ __launch_bounds__(256) void k_copy_state(State src, State dst, const 
 __global__ __launch_bounds__(256) void k_deinterleave3(const double *__restrict__ in, long long n,
                                                        double *__restrict__ x, double *__restrict__ y,
                                                        double *__restrict__ z) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i >= n) return;
     x[i] = in[3 * i];
@@ -202,6 +211,7 @@ __global__ __launch_bounds__(256) void k_deinterleave3(const double *__restrict_
 __global__ __launch_bounds__(256) void k_interleave3(const double *__restrict__ x, const double *__restrict__ y,
                                                      const double *__restrict__ z, long long n,
                                                      double *__restrict__ out) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i >= n) return;
     out[3 * i] = x[i];
@@ -212,6 +222,7 @@ __global__ __launch_bounds__(256) void k_interleave3(const double *__restrict__ 
 // state out in the caller's particle order: row id[i] of pos/vel (n x 3) <- slot i
 __global__ __launch_bounds__(256) void k_state_out(State t, long long n, double *__restrict__ pos,
                                                    double *__restrict__ vel) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i >= n) return;
     const long long j = t.id[i];
@@ -229,6 +240,7 @@ __global__ __launch_bounds__(256) void k_state_out(State t, long long n, double 
 
 __global__ __launch_bounds__(256) void k_gather_f(const float *__restrict__ in, const uint32_t *__restrict__ id,
                                                   long long n, float *__restrict__ out) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i < n) out[i] = in[id[i]];
 }
@@ -237,6 +249,7 @@ __global__ __launch_bounds__(256) void k_gather_f(const float *__restrict__ in, 
 // holds an index >= n latches GT_EINVAL (the cell grouping needs key order)
 __global__ __launch_bounds__(256) void k_scatter_flags(const uint32_t *__restrict__ active, long long na,
                                                        long long n, uint32_t *__restrict__ bits, DevCtl *ctl) {
+    gt_grid_ready();
     const long long k = blockIdx.x * 256ll + threadIdx.x;
     const uint32_t i = k < na ? active[k] : 0u;
     const bool bad = k < na && ((long long)i >= n || (k > 0 && active[k - 1] >= i)), on = k < na && !bad;
@@ -333,6 +346,7 @@ __device__ __forceinline__ void compact_body(const unsigned bid, const unsigned 
 __global__ __launch_bounds__(AT) void k_compact(long long n, const long long *__restrict__ t0,
         const uint8_t *__restrict__ level, int L, DevCtl *ctl, int ticket, uint32_t tag_slot,
         uint32_t *__restrict__ out, uint2 *__restrict__ rank, unsigned long long *status) {
+    gt_grid_ready();
     compact_body(blockIdx.x, gridDim.x, n, t0, level, L, ctl, ticket, tag_slot, out, rank, status);
 }
 
@@ -396,6 +410,7 @@ __device__ __forceinline__ void compact_bits_body(const unsigned bid, const unsi
 __global__ __launch_bounds__(AT) void k_compact_bits(long long n_host, const unsigned int *n_dev,
         uint32_t *__restrict__ bits, DevCtl *ctl, int ticket, uint32_t tag_slot, uint32_t *__restrict__ out,
         uint2 *__restrict__ rank, unsigned int *count_out, unsigned long long *status) {
+    gt_grid_ready();
     compact_bits_body(blockIdx.x, gridDim.x, n_host, n_dev, bits, ctl, ticket, tag_slot, out, rank, count_out, status);
 }
 
@@ -439,6 +454,7 @@ __device__ __forceinline__ void group_cells_body(const unsigned bid, const unsig
 template <bool ALL>
 __global__ __launch_bounds__(256) void k_group_cells(Nodes nd, long long n, long long cap,
         const uint2 *__restrict__ R, int gmax, float r_crit, uint32_t *__restrict__ marks, DevCtl *ctl) {
+    gt_grid_ready();
     group_cells_body<ALL>(blockIdx.x, gridDim.x, nd, n, cap, R, gmax, r_crit, marks, ctl);
 }
 
@@ -446,6 +462,7 @@ __global__ __launch_bounds__(256) void k_group_cells(Nodes nd, long long n, long
 __global__ __launch_bounds__(256) void k_acc_out(const float4 *__restrict__ acc, const uint32_t *__restrict__ id,
                                                  long long n, float4 *__restrict__ acc_out,
                                                  uint32_t *__restrict__ id_out) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i >= n) return;
     if (acc_out) acc_out[i] = acc[i];
@@ -453,6 +470,7 @@ __global__ __launch_bounds__(256) void k_acc_out(const float4 *__restrict__ acc,
 }
 
 __global__ __launch_bounds__(256) void k_iota(uint32_t *__restrict__ out, long long n) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i < n) out[i] = (uint32_t)i;
 }
@@ -534,6 +552,7 @@ __device__ __forceinline__ void correct_body(const unsigned bid, const unsigned 
 
 __global__ __launch_bounds__(256) void k_correct(State s, const uint32_t *__restrict__ active,
         const float4 *__restrict__ acc, DevCtl *ctl, long long n, int L, double c2) {
+    gt_grid_ready();
     correct_body(blockIdx.x, gridDim.x, s, active, acc, ctl, n, L, c2);
 }
 
@@ -544,6 +563,7 @@ __device__ __forceinline__ void aold_body(const unsigned bid, const unsigned nb,
 }
 
 __global__ __launch_bounds__(256) void k_aold(const float4 *__restrict__ acc, long long n, float *__restrict__ aold) {
+    gt_grid_ready();
     aold_body(blockIdx.x, gridDim.x, acc, n, aold);
 }
 
@@ -562,6 +582,7 @@ __device__ __forceinline__ void min_a2_body(const unsigned bid, const unsigned n
 }
 
 __global__ __launch_bounds__(256) void k_min_a2(const float4 *__restrict__ acc, long long n, DevCtl *ctl) {
+    gt_grid_ready();
     min_a2_body(blockIdx.x, gridDim.x, acc, n, ctl);
 }
 
@@ -609,11 +630,13 @@ __device__ __forceinline__ void init_levels_body(const unsigned bid, const unsig
 
 __global__ __launch_bounds__(256) void k_init_levels(State s, const float4 *__restrict__ acc, long long n, int L,
         double c2, int M_given, int have_M, DevCtl *ctl) {
+    gt_grid_ready();
     init_levels_body(blockIdx.x, gridDim.x, s, acc, n, L, c2, M_given, have_M, ctl);
 }
 
 // resume: scalars of the integration and the next block time over all particles
 __global__ void k_set_clock(DevCtl *ctl, int M, int L, long long T) {
+    gt_grid_ready();
     ctl->M = M;
     ctl->dt_max = ldexp(1.0, M);
     ctl->levels_m1 = L - 1;
@@ -628,6 +651,7 @@ __global__ void k_set_u32(unsigned int *dst, unsigned int v) { *dst = v; }
 __global__ __launch_bounds__(256) void k_tnext_all(const long long *__restrict__ t0,
                                                    const uint8_t *__restrict__ level, long long n, int L,
                                                    DevCtl *ctl) {
+    gt_grid_ready();
     unsigned long long tmin = ~0ull;
     for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += (long long)gridDim.x * 256) {
         const unsigned long long tend = (unsigned long long)t0[i] + (1ull << (L - 1 - (int)level[i]));
@@ -640,6 +664,7 @@ __global__ __launch_bounds__(256) void k_tnext_all(const long long *__restrict__
 __global__ __launch_bounds__(256) void k_gather_resume(const uint8_t *__restrict__ lv, const long long *__restrict__ t0,
                                                        const float *__restrict__ ao, const float4 *__restrict__ acc,
                                                        const uint32_t *__restrict__ id, long long n, State s) {
+    gt_grid_ready();
     const long long i = blockIdx.x * 256ll + threadIdx.x;
     if (i >= n) return;
     const uint32_t k = id[i];
@@ -650,6 +675,7 @@ __global__ __launch_bounds__(256) void k_gather_resume(const uint8_t *__restrict
 }
 
 __global__ void k_reset_start(DevCtl *ctl) {
+    gt_grid_ready();
     ctl->max_dt_bits = ~0ull;
     ctl->tnext_acc = ~0ull;
     ctl->tnext = 0;
@@ -657,6 +683,7 @@ __global__ void k_reset_start(DevCtl *ctl) {
 
 // ---- a table of systems ----
 __global__ void kg_prepare(const GroupedSys *__restrict__ t) {  // a warp each
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     prepare_body(0, 1, s.ctl, (s.flags & GT_SYS_STEP) ? 1 : 0);
     if ((s.flags & GT_SYS_START) && threadIdx.x == 0) {
@@ -667,6 +694,7 @@ __global__ void kg_prepare(const GroupedSys *__restrict__ t) {  // a warp each
 }
 
 __global__ __launch_bounds__(256) void kg_predict(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     if (!(s.flags & GT_SYS_STEP)) return;
     float4 *dst = (s.flags & GT_SYS_BUILD) ? s.posm_tmp : s.posm;
@@ -676,6 +704,7 @@ __global__ __launch_bounds__(256) void kg_predict(const GroupedSys *__restrict__
 }
 
 __global__ __launch_bounds__(256) void kg_permute(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     if (!(s.flags & GT_SYS_BUILD)) return;
     const bool tmp = (s.flags & GT_SYS_PREDICTED) != 0;
@@ -684,6 +713,7 @@ __global__ __launch_bounds__(256) void kg_permute(const GroupedSys *__restrict__
 }
 
 __global__ __launch_bounds__(256) void kg_copy_state(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     if (!(s.flags & GT_SYS_BUILD)) return;
     const bool tmp = (s.flags & GT_SYS_PREDICTED) != 0;
@@ -691,6 +721,7 @@ __global__ __launch_bounds__(256) void kg_copy_state(const GroupedSys *__restric
 }
 
 __global__ __launch_bounds__(AT) void kg_compact(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, ATILE, nsm * 4);
     if (!(s.flags & GT_SYS_STEP) || blockIdx.y >= nb) return;
@@ -699,6 +730,7 @@ __global__ __launch_bounds__(AT) void kg_compact(const GroupedSys *__restrict__ 
 }
 
 __global__ __launch_bounds__(256) void kg_group_cells(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 256, nsm * 8);
     if (blockIdx.y >= nb) return;
@@ -712,6 +744,7 @@ __global__ __launch_bounds__(256) void kg_group_cells(const GroupedSys *__restri
 }
 
 __global__ __launch_bounds__(AT) void kg_groups(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 32 * BTILE, nsm * 4);
     if (!s.cells || blockIdx.y >= nb) return;
@@ -720,17 +753,20 @@ __global__ __launch_bounds__(AT) void kg_groups(const GroupedSys *__restrict__ t
 }
 
 __global__ __launch_bounds__(256) void kg_aold(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     if (s.flags & GT_SYS_START) aold_body(blockIdx.y, gridDim.y, s.acc, s.n, s.st0.aold);
 }
 
 __global__ __launch_bounds__(256) void kg_min_a2(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 256, nsm * 4);
     if ((s.flags & GT_SYS_START) && !s.have_M && blockIdx.y < nb) min_a2_body(blockIdx.y, nb, s.acc, s.n, s.ctl);
 }
 
 __global__ __launch_bounds__(256) void kg_init_levels(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 256, nsm * 8);
     if ((s.flags & GT_SYS_START) && blockIdx.y < nb)
@@ -738,6 +774,7 @@ __global__ __launch_bounds__(256) void kg_init_levels(const GroupedSys *__restri
 }
 
 __global__ __launch_bounds__(256) void kg_correct(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 256, nsm * 8);
     if ((s.flags & GT_SYS_STEP) && blockIdx.y < nb)
@@ -760,8 +797,8 @@ void gt_launch_predict(const State &s, int64_t n, const DevCtl *ctl, float4 *pos
     if (n <= 0) return;
     const bool aligned = ((uintptr_t)s.rx | (uintptr_t)s.ry | (uintptr_t)s.rz | (uintptr_t)s.vx | (uintptr_t)s.vy |
                           (uintptr_t)s.vz | (uintptr_t)s.t0 | (uintptr_t)s.mass) % 16 == 0;
-    if (n % 2 == 0 && aligned) k_predict2<<<nblk(n / 2), 256, 0, st>>>(s, n, ctl, posm, ahead ? 1 : 0);
-    else k_predict<<<nblk(n), 256, 0, st>>>(s, n, ctl, posm, ahead ? 1 : 0);
+    if (n % 2 == 0 && aligned) gt_launch(k_predict2, nblk(n / 2), 256, 0, st, s, n, ctl, posm, ahead ? 1 : 0);
+    else gt_launch(k_predict, nblk(n), 256, 0, st, s, n, ctl, posm, ahead ? 1 : 0);
     gt_note_launches(1);
 }
 
@@ -780,12 +817,12 @@ void gt_launch_load_from(const State &s, float4 *posm, int64_t n, const double *
 
 void gt_launch_permute(const State &src, const State &dst, const float4 *posm_in, float4 *posm_out,
                        const uint32_t *perm, int64_t n, cudaStream_t st) {
-    if (n > 0) { k_permute<<<nblk(n), 256, 0, st>>>(src, dst, posm_in, posm_out, perm, n); gt_note_launches(1); }
+    if (n > 0) { gt_launch(k_permute, nblk(n), 256, 0, st, src, dst, posm_in, posm_out, perm, n); gt_note_launches(1); }
 }
 
 void gt_launch_copy_state(const State &src, const State &dst, const float4 *posm_in, float4 *posm_out,
                           int64_t n, cudaStream_t st) {
-    if (n > 0) { k_copy_state<<<nblk(n), 256, 0, st>>>(src, dst, posm_in, posm_out, n); gt_note_launches(1); }
+    if (n > 0) { gt_launch(k_copy_state, nblk(n), 256, 0, st, src, dst, posm_in, posm_out, n); gt_note_launches(1); }
 }
 
 void gt_launch_deinterleave3(const double *in, int64_t n, double *x, double *y, double *z,
@@ -808,16 +845,16 @@ void gt_launch_gather_f(const float *in, const uint32_t *id, int64_t n, float *o
 
 void gt_launch_active(const State &s, int64_t n, int L, DevCtl *ctl, uint32_t *active, uint2 *rank,
                       unsigned long long *status, int nsm, cudaStream_t st) {
-    { k_compact<<<gt_grid(n, ATILE, nsm * 4), AT, 0, st>>>(n, s.t0, s.level, L, ctl, GT_TREE_LEVELS, 30u, active, rank,
-                                                           status);
+    { gt_launch(k_compact, gt_grid(n, ATILE, nsm * 4), AT, 0, st, n, s.t0, s.level, L, ctl, GT_TREE_LEVELS, 30u,
+                active, rank, status);
       gt_note_launches(1); }
 }
 
 void gt_launch_active_from_list(const uint32_t *list, int64_t n_list, int64_t n, uint32_t *flags, DevCtl *ctl,
                                 uint32_t *active, uint2 *rank, unsigned long long *status, int nsm, cudaStream_t st) {
     if (n_list > 0) { k_scatter_flags<<<nblk(n_list), 256, 0, st>>>(list, n_list, n, flags, ctl); gt_note_launches(1); }
-    { k_compact_bits<<<gt_grid(n, 32 * BTILE, nsm * 4), AT, 0, st>>>(n, nullptr, flags, ctl, GT_TREE_LEVELS, 30u, active,
-                                                                     rank, &ctl->n_active, status);
+    { gt_launch(k_compact_bits, gt_grid(n, 32 * BTILE, nsm * 4), AT, 0, st, n, nullptr, flags, ctl, GT_TREE_LEVELS,
+                30u, active, rank, &ctl->n_active, status);
       gt_note_launches(1); }
 }
 
@@ -833,10 +870,10 @@ void gt_launch_iota(uint32_t *out, int64_t n, cudaStream_t st) {
 void gt_launch_groups(Nodes nd, int64_t cap, const uint2 *rank, int gmax, float r_crit, int64_t n, uint32_t *marks,
                       DevCtl *ctl, uint32_t *gstart, unsigned long long *status, int nsm, cudaStream_t st) {
     const unsigned grid = gt_grid(n, 256, nsm * 8);
-    if (rank) k_group_cells<false><<<grid, 256, 0, st>>>(nd, n, cap, rank, gmax, r_crit, marks, ctl);
-    else k_group_cells<true><<<grid, 256, 0, st>>>(nd, n, cap, rank, gmax, r_crit, marks, ctl);
-    k_compact_bits<<<gt_grid(n, 32 * BTILE, nsm * 4), AT, 0, st>>>(0, &ctl->n_active, marks, ctl, GT_TREE_LEVELS + 1, 31u,
-                                                                   gstart, nullptr, &ctl->n_groups, status);
+    if (rank) gt_launch(k_group_cells<false>, grid, 256, 0, st, nd, n, cap, rank, gmax, r_crit, marks, ctl);
+    else gt_launch(k_group_cells<true>, grid, 256, 0, st, nd, n, cap, rank, gmax, r_crit, marks, ctl);
+    gt_launch(k_compact_bits, gt_grid(n, 32 * BTILE, nsm * 4), AT, 0, st, 0, &ctl->n_active, marks, ctl,
+              GT_TREE_LEVELS + 1, 31u, gstart, nullptr, &ctl->n_groups, status);
     gt_note_launches(2);
 }
 
@@ -873,8 +910,8 @@ void gt_launch_gather_resume(const uint8_t *lv, const long long *t0, const float
 void gt_launch_init_levels(const State &s, const float4 *acc, int64_t n, int L, double c2, int M_given,
                            int have_M, DevCtl *ctl, int nsm, cudaStream_t st) {
     { k_reset_start<<<1, 1, 0, st>>>(ctl); gt_note_launches(1); }
-    if (!have_M && n > 0) { k_min_a2<<<gt_grid(n, 256, nsm * 4), 256, 0, st>>>(acc, n, ctl); gt_note_launches(1); }
-    { k_init_levels<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(s, acc, n, L, c2, M_given, have_M, ctl); gt_note_launches(1); }
+    if (!have_M && n > 0) { gt_launch(k_min_a2, gt_grid(n, 256, nsm * 4), 256, 0, st, acc, n, ctl); gt_note_launches(1); }
+    { gt_launch(k_init_levels, gt_grid(n, 256, nsm * 8), 256, 0, st, s, acc, n, L, c2, M_given, have_M, ctl); gt_note_launches(1); }
 }
 
 // ---- a table of systems ----
@@ -885,24 +922,24 @@ void gt_grouped_prepare(const GroupedSys *t, const GroupedPlan &p, int, cudaStre
 
 void gt_grouped_predict(const GroupedSys *t, const GroupedPlan &p, int, cudaStream_t st) {
     if (p.n_step <= 0) return;
-    kg_predict<<<dim3(p.count, nblk(p.n_step)), 256, 0, st>>>(t);
+    gt_launch(kg_predict, dim3(p.count, nblk(p.n_step)), 256, 0, st, t);
     gt_note_launches(1);
 }
 
 void gt_grouped_gather(const GroupedSys *t, const GroupedPlan &p, int, cudaStream_t st) {
     if (p.n_build <= 0) return;
-    kg_permute<<<dim3(p.count, nblk(p.n_build)), 256, 0, st>>>(t);
-    kg_copy_state<<<dim3(p.count, nblk(p.n_build)), 256, 0, st>>>(t);
+    gt_launch(kg_permute, dim3(p.count, nblk(p.n_build)), 256, 0, st, t);
+    gt_launch(kg_copy_state, dim3(p.count, nblk(p.n_build)), 256, 0, st, t);
     gt_note_launches(2);
 }
 
 void gt_grouped_groups(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
     if (p.n_step > 0) {
-        kg_compact<<<dim3(p.count, gt_grid(p.n_step, ATILE, nsm * 4)), AT, 0, st>>>(t, nsm);
+        gt_launch(kg_compact, dim3(p.count, gt_grid(p.n_step, ATILE, nsm * 4)), AT, 0, st, t, nsm);
         gt_note_launches(1);
     }
-    kg_group_cells<<<dim3(p.count, gt_grid(p.n_all, 256, nsm * 8)), 256, 0, st>>>(t, nsm);
-    kg_groups<<<dim3(p.count, gt_grid(p.n_all, 32 * BTILE, nsm * 4)), AT, 0, st>>>(t, nsm);
+    gt_launch(kg_group_cells, dim3(p.count, gt_grid(p.n_all, 256, nsm * 8)), 256, 0, st, t, nsm);
+    gt_launch(kg_groups, dim3(p.count, gt_grid(p.n_all, 32 * BTILE, nsm * 4)), AT, 0, st, t, nsm);
     gt_note_launches(2);
 }
 
@@ -915,7 +952,7 @@ void gt_grouped_aold(const GroupedSys *t, const GroupedPlan &p, int, cudaStream_
 void gt_grouped_correct(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
     if (p.n_start > 0) {
         kg_min_a2<<<dim3(p.count, gt_grid(p.n_start, 256, nsm * 4)), 256, 0, st>>>(t, nsm);
-        kg_init_levels<<<dim3(p.count, gt_grid(p.n_start, 256, nsm * 8)), 256, 0, st>>>(t, nsm);
+        gt_launch(kg_init_levels, dim3(p.count, gt_grid(p.n_start, 256, nsm * 8)), 256, 0, st, t, nsm);
         gt_note_launches(2);
     }
     if (p.n_step > 0) {

@@ -60,6 +60,7 @@ __device__ __forceinline__ void bbox_body(const unsigned bid, const unsigned nb,
 
 __global__ __launch_bounds__(BBOX_THREADS) void k_bbox(const float4 *__restrict__ posm, long long n, DevCtl *ctl,
         uint4 *__restrict__ clear, long long nclear) {
+    gt_grid_ready();
     bbox_body(blockIdx.x, gridDim.x, posm, n, ctl, clear, nclear);
 }
 
@@ -168,6 +169,7 @@ __device__ __forceinline__ void keys_body(const unsigned bid, const unsigned nb,
 
 __global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, long long n, int curve, DevCtl *ctl,
         unsigned long long *__restrict__ key, uint32_t *__restrict__ hist, uint32_t *__restrict__ base) {
+    gt_grid_ready();
     keys_body(blockIdx.x, gridDim.x, posm, n, curve, ctl, key, hist, base);
 }
 
@@ -325,6 +327,7 @@ __device__ __forceinline__ void small_sort_body(const unsigned bid, const unsign
 
 __global__ __launch_bounds__(SMALL_THREADS) void k_small_sort(const float4 *__restrict__ posm, int n, int curve,
         unsigned long long *__restrict__ key, uint32_t *__restrict__ val) {
+    gt_grid_ready();
     small_sort_body(blockIdx.x, gridDim.x, posm, n, curve, key, val);
 }
 
@@ -338,6 +341,7 @@ __host__ __device__ inline unsigned keys_blocks(long long n, int nsm) {
 }
 
 __global__ __launch_bounds__(BBOX_THREADS) void kg_bbox(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, BBOX_THREADS, nsm * 4);
     if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
@@ -345,6 +349,7 @@ __global__ __launch_bounds__(BBOX_THREADS) void kg_bbox(const GroupedSys *__rest
 }
 
 __global__ __launch_bounds__(256) void kg_keys(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = keys_blocks(s.n, nsm);
     if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
@@ -353,6 +358,7 @@ __global__ __launch_bounds__(256) void kg_keys(const GroupedSys *__restrict__ t,
 }
 
 __global__ __launch_bounds__(SMALL_THREADS) void kg_small_sort(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     if (s.flags & GT_SYS_BUILD)
         small_sort_body(0, 1, keyed(s), (int)s.n, s.curve, (unsigned long long *)s.sb.key[0], s.sb.val[0]);
@@ -363,15 +369,15 @@ __global__ __launch_bounds__(SMALL_THREADS) void kg_small_sort(const GroupedSys 
 void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, SortBufs &b, cudaStream_t st) {
     if (n <= 0) return;
     static_assert(GT_SORT_DIGITS * 4 % 16 == 0, "cleared 16 bytes at a time");
-    k_bbox<<<gt_grid(n, BBOX_THREADS, nblk), BBOX_THREADS, 0, st>>>(posm, n, ctl, (uint4 *)b.hist,
-                                                                    (long long)(gt_sort_scratch_bytes(n) / 16));
+    gt_launch(k_bbox, gt_grid(n, BBOX_THREADS, nblk), BBOX_THREADS, 0, st, posm, n, ctl, (uint4 *)b.hist,
+              (long long)(gt_sort_scratch_bytes(n) / 16));
     gt_note_launches(1);
 }
 
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st) {
     if (n <= 0) return;
-    k_keys<<<keys_blocks(n, nsm), 256, 0, st>>>(posm, n, curve, ctl, (unsigned long long *)b.key[0], b.hist,
-                                                b.digit_base);
+    gt_launch(k_keys, keys_blocks(n, nsm), 256, 0, st, posm, n, curve, ctl, (unsigned long long *)b.key[0], b.hist,
+              b.digit_base);
     gt_note_launches(1);
 }
 
@@ -382,17 +388,18 @@ void gt_keys_init() {
 
 void gt_launch_small_sort(const float4 *posm, int64_t n, int curve, SortBufs &b, cudaStream_t st) {
     if (n <= 0) return;
-    k_small_sort<<<1, SMALL_THREADS, SMALL_SMEM, st>>>(posm, (int)n, curve, (unsigned long long *)b.key[0], b.val[0]);
+    gt_launch(k_small_sort, 1, SMALL_THREADS, SMALL_SMEM, st, posm, (int)n, curve, (unsigned long long *)b.key[0],
+              b.val[0]);
     gt_note_launches(1);
 }
 
 void gt_grouped_small_sort(const GroupedSys *t, const GroupedPlan &p, cudaStream_t st) {
-    kg_small_sort<<<p.count, SMALL_THREADS, SMALL_SMEM, st>>>(t);
+    gt_launch(kg_small_sort, p.count, SMALL_THREADS, SMALL_SMEM, st, t);
     gt_note_launches(1);
 }
 
 void gt_grouped_keys(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st) {
-    kg_bbox<<<dim3(p.count, gt_grid(p.n_build, BBOX_THREADS, nsm * 4)), BBOX_THREADS, 0, st>>>(t, nsm);
-    kg_keys<<<dim3(p.count, keys_blocks(p.n_build, nsm)), 256, 0, st>>>(t, nsm);
+    gt_launch(kg_bbox, dim3(p.count, gt_grid(p.n_build, BBOX_THREADS, nsm * 4)), BBOX_THREADS, 0, st, t, nsm);
+    gt_launch(kg_keys, dim3(p.count, keys_blocks(p.n_build, nsm)), 256, 0, st, t, nsm);
     gt_note_launches(2);
 }

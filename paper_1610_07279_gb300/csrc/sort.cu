@@ -47,6 +47,7 @@ static_assert(ST >= R && ST % 32 == 0, "one thread per digit in the per-tile sca
 __global__ __launch_bounds__(HT) void k_hist_all(long long n, const unsigned long long *__restrict__ key,
                                                  uint32_t *__restrict__ hist /* PASSES x R */,
                                                  uint32_t *__restrict__ base, DevCtl *ctl) {
+    gt_grid_ready();
     __shared__ uint32_t h[PASSES][R];
     for (int p = 0; p < PASSES; p++) h[p][threadIdx.x] = 0;
     __syncthreads();
@@ -199,6 +200,7 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
         const unsigned long long *__restrict__ kin, const uint32_t *__restrict__ vin,
         unsigned long long *__restrict__ kout, uint32_t *__restrict__ vout, const uint32_t *__restrict__ digit_base,
         uint32_t *status, int ntiles, DevCtl *ctl) {
+    gt_grid_ready();
     onesweep_body<MODE>(blockIdx.x, gridDim.x, n, pass, shift, kin, vin, kout, vout, digit_base, status, ntiles, ctl);
 }
 
@@ -249,6 +251,7 @@ __device__ __forceinline__ void fix_runs_body(const unsigned bid, const unsigned
 
 __global__ __launch_bounds__(256) void k_fix_runs(long long n, int shift, unsigned long long *key, uint32_t *val,
         uint32_t *list, DevCtl *ctl) {
+    gt_grid_ready();
     fix_runs_body(blockIdx.x, gridDim.x, n, shift, key, val, list, ctl);
 }
 
@@ -384,12 +387,14 @@ __device__ __forceinline__ void fix_long_runs_body(const unsigned bid, const uns
 
 __global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, unsigned long long *key0,
         uint32_t *val0, unsigned long long *key1, uint32_t *val1, const uint32_t *__restrict__ list, DevCtl *ctl) {
+    gt_grid_ready();
     fix_long_runs_body(blockIdx.x, gridDim.x, n, shift, key0, val0, key1, val1, list, ctl);
 }
 
 // ---- a table of systems ----
 template <int MODE>
 __global__ __launch_bounds__(ST, GT_SORT_MINB) void kg_onesweep(const GroupedSys *__restrict__ t, int pass, int shift) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const int ntiles = gt_sort_tiles(s.n), src = pass & 1;
     if (!(s.flags & GT_SYS_BUILD) || (int)blockIdx.y >= ntiles) return;
@@ -402,6 +407,7 @@ __host__ __device__ inline unsigned fix_blocks(long long n, int nsm) { return gt
 __host__ __device__ inline unsigned fix_long_blocks(long long n, int nsm) { return gt_grid(n, 4 * TILE, nsm); }
 
 __global__ __launch_bounds__(256) void kg_fix_runs(const GroupedSys *__restrict__ t, int shift, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = fix_blocks(s.n, nsm);
     if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
@@ -409,6 +415,7 @@ __global__ __launch_bounds__(256) void kg_fix_runs(const GroupedSys *__restrict_
 }
 
 __global__ __launch_bounds__(ST) void kg_fix_long_runs(const GroupedSys *__restrict__ t, int shift, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = fix_long_blocks(s.n, nsm);
     if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb)
@@ -436,9 +443,9 @@ namespace {
 template <int MODE>
 void onesweep(SortBufs &b, int64_t n, DevCtl *ctl, int pass, int shift, cudaStream_t st) {
     const int ntiles = gt_sort_tiles(n), src = pass & 1;
-    k_onesweep<MODE><<<ntiles, ST, SCATTER_SMEM, st>>>(n, pass, shift, (const unsigned long long *)b.key[src], b.val[src],
-                                                       (unsigned long long *)b.key[src ^ 1], b.val[src ^ 1], b.digit_base,
-                                                       b.status + (size_t)pass * R * ntiles, ntiles, ctl);
+    gt_launch(k_onesweep<MODE>, ntiles, ST, SCATTER_SMEM, st, n, pass, shift, (const unsigned long long *)b.key[src],
+              b.val[src], (unsigned long long *)b.key[src ^ 1], b.val[src ^ 1], b.digit_base,
+              b.status + (size_t)pass * R * ntiles, ntiles, ctl);
     gt_note_launches(1);
 }
 
@@ -452,9 +459,10 @@ void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStrea
     for (int p = 3; p < PASSES; p++) onesweep<PASS_PLAIN>(b, n, ctl, p, gt_tree_digit_shift(p), st);
     const int shift = gt_tree_digit_shift(2);
     uint32_t *list = b.status;  // the look-backs are over
-    k_fix_runs<<<fix_blocks(n, nsm), 256, 0, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0], list, ctl);
-    k_fix_long_runs<<<fix_long_blocks(n, nsm), ST, SCATTER_SMEM, st>>>(n, shift, (unsigned long long *)b.key[0], b.val[0],
-                                                   (unsigned long long *)b.key[1], b.val[1], list, ctl);
+    gt_launch(k_fix_runs, fix_blocks(n, nsm), 256, 0, st, n, shift, (unsigned long long *)b.key[0], b.val[0], list,
+              ctl);
+    gt_launch(k_fix_long_runs, fix_long_blocks(n, nsm), ST, SCATTER_SMEM, st, n, shift,
+              (unsigned long long *)b.key[0], b.val[0], (unsigned long long *)b.key[1], b.val[1], list, ctl);
     gt_note_launches(2);
 }
 
@@ -573,13 +581,13 @@ void gt_grouped_sort(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStr
     }
     gt_grouped_keys(t, p, nsm, st);
     const dim3 grid(p.count, gt_sort_tiles(p.n_build));
-    kg_onesweep<PASS_LOW_FIRST><<<grid, ST, SCATTER_SMEM, st>>>(t, 0, gt_tree_digit_shift(0));
-    kg_onesweep<PASS_LOW><<<grid, ST, SCATTER_SMEM, st>>>(t, 1, gt_tree_digit_shift(1));
-    kg_onesweep<PASS_HIGH_FIRST><<<grid, ST, SCATTER_SMEM, st>>>(t, 2, gt_tree_digit_shift(2));
+    gt_launch(kg_onesweep<PASS_LOW_FIRST>, grid, ST, SCATTER_SMEM, st, t, 0, gt_tree_digit_shift(0));
+    gt_launch(kg_onesweep<PASS_LOW>, grid, ST, SCATTER_SMEM, st, t, 1, gt_tree_digit_shift(1));
+    gt_launch(kg_onesweep<PASS_HIGH_FIRST>, grid, ST, SCATTER_SMEM, st, t, 2, gt_tree_digit_shift(2));
     for (int q = 3; q < PASSES; q++)
-        kg_onesweep<PASS_PLAIN><<<grid, ST, SCATTER_SMEM, st>>>(t, q, gt_tree_digit_shift(q));
+        gt_launch(kg_onesweep<PASS_PLAIN>, grid, ST, SCATTER_SMEM, st, t, q, gt_tree_digit_shift(q));
     const int shift = gt_tree_digit_shift(2);
-    kg_fix_runs<<<dim3(p.count, fix_blocks(p.n_build, nsm)), 256, 0, st>>>(t, shift, nsm);
-    kg_fix_long_runs<<<dim3(p.count, fix_long_blocks(p.n_build, nsm)), ST, SCATTER_SMEM, st>>>(t, shift, nsm);
+    gt_launch(kg_fix_runs, dim3(p.count, fix_blocks(p.n_build, nsm)), 256, 0, st, t, shift, nsm);
+    gt_launch(kg_fix_long_runs, dim3(p.count, fix_long_blocks(p.n_build, nsm)), ST, SCATTER_SMEM, st, t, shift, nsm);
     gt_note_launches(PASSES + 2);
 }

@@ -30,6 +30,7 @@ constexpr int NPT = 1;          // cells per thread
 constexpr int BTILE = BT * NPT; // cells per tile
 
 __global__ void k_build_init(long long n, Nodes nd, DevCtl *ctl) {
+    gt_grid_ready();
     for (int b = threadIdx.x; b < GT_CELL_BUCKETS; b += blockDim.x) ctl->cell_bucket[b] = 0;
     if (threadIdx.x != 0) return;
     // root = level 0, all particles; level_start[0..1]
@@ -45,6 +46,7 @@ __global__ void k_build_init(long long n, Nodes nd, DevCtl *ctl) {
 __global__ __launch_bounds__(BT) void k_build_level(int lvl, const unsigned long long *__restrict__ skey,
                                                     int leaf_max, Nodes nd, long long cap,
                                                     unsigned long long *status, DevCtl *ctl) {
+    gt_grid_ready();
     __shared__ uint32_t tmp[BT / 32 + 1];
     __shared__ uint32_t tile_sh, excl_sh;
     const uint32_t lo = ctl->level_start[lvl], hi = ctl->level_start[lvl + 1];
@@ -249,6 +251,7 @@ __device__ __forceinline__ void flat_marks_body(const unsigned bid, const unsign
 template <int MT, int ROUNDS>
 __global__ __launch_bounds__(FB) void k_flat_marks(const unsigned long long *__restrict__ skey, long long n, int M,
         uint16_t *__restrict__ dl, uint32_t *__restrict__ cnt, int ntiles) {
+    gt_grid_ready();
     flat_marks_body<MT, ROUNDS>(blockIdx.x, gridDim.x, skey, n, M, dl, cnt, ntiles);
 }
 
@@ -301,6 +304,7 @@ __device__ __forceinline__ void flat_scan_body(const unsigned bid, const unsigne
 
 __global__ __launch_bounds__(1024) void k_flat_scan(uint32_t *__restrict__ cnt, int ntiles,
         uint32_t *__restrict__ tot, long long cap, DevCtl *ctl) {
+    gt_grid_ready();
     flat_scan_body(blockIdx.x, gridDim.x, cnt, ntiles, tot, cap, ctl);
 }
 
@@ -388,6 +392,7 @@ __device__ __forceinline__ void flat_scatter_body(const unsigned bid, const unsi
 template <int ROUNDS>
 __global__ __launch_bounds__(FB) void k_flat_scatter(const uint16_t *__restrict__ dl, long long n,
         const uint32_t *__restrict__ cnt, int ntiles, long long cap, Nodes nd, const DevCtl *__restrict__ ctl) {
+    gt_grid_ready();
     flat_scatter_body<ROUNDS>(blockIdx.x, gridDim.x, dl, n, cnt, ntiles, cap, nd, ctl);
 }
 
@@ -422,6 +427,7 @@ __device__ __forceinline__ void flat_link_body(const unsigned bid, const unsigne
 }
 
 __global__ __launch_bounds__(256) void k_flat_link(Nodes nd, long long cap, const DevCtl *__restrict__ ctl) {
+    gt_grid_ready();
     flat_link_body(blockIdx.x, gridDim.x, nd, cap, ctl);
 }
 
@@ -490,6 +496,7 @@ __device__ __forceinline__ void cell_count_body(const unsigned bid, const unsign
 }
 
 __global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, DevCtl *ctl) {
+    gt_grid_ready();
     cell_count_body(blockIdx.x, gridDim.x, nd, cap, ctl);
 }
 
@@ -523,6 +530,7 @@ __device__ __forceinline__ void cell_fill_body(const unsigned bid, const unsigne
 }
 
 __global__ __launch_bounds__(256) void k_cell_fill(Nodes nd, long long cap, DevCtl *ctl) {
+    gt_grid_ready();
     cell_fill_body(blockIdx.x, gridDim.x, nd, cap, ctl);
 }
 
@@ -853,6 +861,7 @@ __device__ __forceinline__ void pseudo_body(const unsigned bid, const unsigned n
 
 template <bool WITH_MASS>
 __global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void k_pseudo(Nodes nd, const float4 *__restrict__ posm, DevCtl *ctl) {
+    gt_grid_ready();
     pseudo_body<WITH_MASS>(blockIdx.x, gridDim.x, nd, posm, ctl);
 }
 
@@ -871,6 +880,7 @@ struct FlatScratch {
 
 template <int MT>
 __global__ __launch_bounds__(FB) void kg_flat_marks(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const FlatScratch f(s.bscratch, s.n, 2);
     if ((s.flags & GT_SYS_BUILD) && (int)blockIdx.y < f.ntiles)
@@ -879,12 +889,14 @@ __global__ __launch_bounds__(FB) void kg_flat_marks(const GroupedSys *__restrict
 }
 
 __global__ __launch_bounds__(1024) void kg_flat_scan(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const FlatScratch f(s.bscratch, s.n, 2);
     if (s.flags & GT_SYS_BUILD) flat_scan_body(blockIdx.y, NREC, f.cnt, f.ntiles, f.tot, s.cap, s.ctl);
 }
 
 __global__ __launch_bounds__(FB) void kg_flat_scatter(const GroupedSys *__restrict__ t) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const FlatScratch f(s.bscratch, s.n, 2);
     if ((s.flags & GT_SYS_BUILD) && (int)blockIdx.y < f.ntiles)
@@ -892,24 +904,28 @@ __global__ __launch_bounds__(FB) void kg_flat_scatter(const GroupedSys *__restri
 }
 
 __global__ __launch_bounds__(256) void kg_flat_link(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 256, nsm * 8);
     if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb) flat_link_body(blockIdx.y, nb, s.nd, s.cap, s.ctl);
 }
 
 __global__ __launch_bounds__(256) void kg_cell_count(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 512, nsm * 4);
     if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb) cell_count_body(blockIdx.y, nb, s.nd, s.cap, s.ctl);
 }
 
 __global__ __launch_bounds__(256) void kg_cell_fill(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = gt_grid(s.n, 1024, nsm * 2);
     if ((s.flags & GT_SYS_BUILD) && blockIdx.y < nb) cell_fill_body(blockIdx.y, nb, s.nd, s.cap, s.ctl);
 }
 
 __global__ __launch_bounds__(PL, GT_PSEUDO_MINB) void kg_pseudo(const GroupedSys *__restrict__ t, int nsm) {
+    gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     if (blockIdx.y >= gt_grid(s.n, 64, nsm * GT_PSEUDO_MINB)) return;
     if (s.flags & GT_SYS_BUILD) pseudo_body<true>(blockIdx.y, gridDim.y, s.nd, s.posm, s.ctl);
@@ -939,13 +955,13 @@ void launch_flat(const unsigned long long *k, int64_t n, int leaf_max, Nodes nd,
         case 24: marks = k_flat_marks<24, ROUNDS>; break;
         case 32: marks = k_flat_marks<32, ROUNDS>; break;
         }
-        marks<<<f.ntiles, FB, 0, st>>>(k, n, leaf_max, f.dl, f.cnt, f.ntiles);
+        gt_launch(marks, f.ntiles, FB, 0, st, k, n, leaf_max, f.dl, f.cnt, f.ntiles);
         gt_note_launches(1);
     }
-    { k_flat_scan<<<NREC, 1024, 0, st>>>(f.cnt, f.ntiles, f.tot, cap, ctl); gt_note_launches(1); }
+    { gt_launch(k_flat_scan, NREC, 1024, 0, st, f.cnt, f.ntiles, f.tot, cap, ctl); gt_note_launches(1); }
     if (f.ntiles > 0) {
-        k_flat_scatter<ROUNDS><<<f.ntiles, FB, 0, st>>>(f.dl, n, f.cnt, f.ntiles, cap, nd, ctl);
-        { k_flat_link<<<gt_grid(n, 256, nsm * 8), 256, 0, st>>>(nd, cap, ctl); }
+        gt_launch(k_flat_scatter<ROUNDS>, f.ntiles, FB, 0, st, f.dl, n, f.cnt, f.ntiles, cap, nd, ctl);
+        { gt_launch(k_flat_link, gt_grid(n, 256, nsm * 8), 256, 0, st, nd, cap, ctl); }
         gt_note_launches(2);
     }
 }
@@ -967,16 +983,16 @@ void gt_launch_build(const uint64_t *skey, int64_t n, int leaf_max, Nodes nd, in
 }
 
 void gt_launch_cell_lists(Nodes nd, int64_t n, int64_t cap, DevCtl *ctl, int nsm, cudaStream_t st) {
-    { k_cell_count<<<gt_grid(n, 512, nsm * 4), 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
-    { k_cell_fill<<<gt_grid(n, 1024, nsm * 2), 256, 0, st>>>(nd, cap, ctl); gt_note_launches(1); }
+    { gt_launch(k_cell_count, gt_grid(n, 512, nsm * 4), 256, 0, st, nd, cap, ctl); gt_note_launches(1); }
+    { gt_launch(k_cell_fill, gt_grid(n, 1024, nsm * 2), 256, 0, st, nd, cap, ctl); gt_note_launches(1); }
 }
 
 void gt_launch_pseudo(Nodes nd, int64_t n, const float4 *posm, DevCtl *ctl, int nsm, bool with_mass,
                       cudaStream_t st) {
     // the ticket and the per-level counters were cleared by gt_launch_prepare
     const unsigned grid = gt_grid(n, 64, nsm * GT_PSEUDO_MINB);
-    if (with_mass) { k_pseudo<true><<<grid, PL, 0, st>>>(nd, posm, ctl); }
-    else { k_pseudo<false><<<grid, PL, 0, st>>>(nd, posm, ctl); }
+    if (with_mass) { gt_launch(k_pseudo<true>, grid, PL, 0, st, nd, posm, ctl); }
+    else { gt_launch(k_pseudo<false>, grid, PL, 0, st, nd, posm, ctl); }
     gt_note_launches(1);
 }
 
@@ -993,12 +1009,12 @@ void gt_grouped_build(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaSt
     case 32: marks = kg_flat_marks<32>; break;
     }
     const unsigned tiles = (unsigned)((n + 2 * FB - 1) / (2 * FB));
-    marks<<<dim3(p.count, tiles), FB, 0, st>>>(t);
-    kg_flat_scan<<<dim3(p.count, NREC), 1024, 0, st>>>(t);
-    kg_flat_scatter<<<dim3(p.count, tiles), FB, 0, st>>>(t);
-    kg_flat_link<<<dim3(p.count, gt_grid(n, 256, nsm * 8)), 256, 0, st>>>(t, nsm);
-    kg_cell_count<<<dim3(p.count, gt_grid(n, 512, nsm * 4)), 256, 0, st>>>(t, nsm);
-    kg_cell_fill<<<dim3(p.count, gt_grid(n, 1024, nsm * 2)), 256, 0, st>>>(t, nsm);
+    gt_launch(marks, dim3(p.count, tiles), FB, 0, st, t);
+    gt_launch(kg_flat_scan, dim3(p.count, NREC), 1024, 0, st, t);
+    gt_launch(kg_flat_scatter, dim3(p.count, tiles), FB, 0, st, t);
+    gt_launch(kg_flat_link, dim3(p.count, gt_grid(n, 256, nsm * 8)), 256, 0, st, t, nsm);
+    gt_launch(kg_cell_count, dim3(p.count, gt_grid(n, 512, nsm * 4)), 256, 0, st, t, nsm);
+    gt_launch(kg_cell_fill, dim3(p.count, gt_grid(n, 1024, nsm * 2)), 256, 0, st, t, nsm);
     gt_note_launches(6);
 }
 
@@ -1006,6 +1022,6 @@ void gt_grouped_pseudo(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaS
     // A block of a system waits for that system's blocks only, so all systems should have some at once: the systems
     // vary fastest, and four grids' worth of blocks let those of finished systems make room for the others'.
     const int most = nsm * GT_PSEUDO_MINB, share = (4 * most + p.count - 1) / p.count;
-    kg_pseudo<<<dim3(p.count, gt_grid(p.n_all, 64, share < most ? share : most)), PL, 0, st>>>(t, nsm);
+    gt_launch(kg_pseudo, dim3(p.count, gt_grid(p.n_all, 64, share < most ? share : most)), PL, 0, st, t, nsm);
     gt_note_launches(1);
 }

@@ -929,6 +929,7 @@ __device__ __forceinline__ int system_of(const uint32_t *gprefix, int nsys, uint
 
 template <int MAC, bool LEVELS>
 __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant__ WalkArgs a) {
+    gt_grid_ready();
     __shared__ __align__(16) float list_sm[NWARP][WARP_SM];
     __shared__ unsigned long long stat_sm[NWARP][2];
     __shared__ uint2 counts_sm[NWARP];
@@ -977,6 +978,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
                                                                  const uint32_t *__restrict__ gprefix,
                                                                  unsigned int *group_next, uint32_t *queue, int qcap,
                                                                  int mac) {
+    gt_grid_ready();
     __shared__ __align__(16) float list_sm[NWARP][WARP_SM];
     __shared__ WalkArgs sargs[NWARP];
     __shared__ unsigned long long stat_sm[NWARP][2];
@@ -1044,6 +1046,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
 // gprefix over the systems' group counts (one warp; also resets the batch counter)
 __global__ void k_batch_prefix(DevCtl *const *__restrict__ ctls, const WalkArgs *__restrict__ args, int nsys,
                                uint32_t *gprefix, unsigned int *group_next) {
+    gt_grid_ready();
     uint32_t carry = 0;
     for (int s0 = 0; s0 < nsys; s0 += 32) {
         const int s = s0 + (int)threadIdx.x;
@@ -1078,7 +1081,7 @@ int gt_walk_warps_per_block() { return NWARP; }
 void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st) {
     constexpr int ACC = GT_MAC_ACCELERATION;
     const bool acc = a.mac == ACC, levels = a.inv_c2 > 0.0f;
-    auto launch = [&](auto kernel) { kernel<<<nblocks, WT, 0, st>>>(a); };
+    auto launch = [&](auto kernel) { gt_launch(kernel, nblocks, WT, 0, st, a); };
     if (levels) launch(acc ? k_walk<ACC, true> : k_walk<MAC_ANY, true>);
     else launch(acc ? k_walk<ACC, false> : k_walk<MAC_ANY, false>);
     gt_note_launches(1);
@@ -1091,7 +1094,8 @@ void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, u
     { k_batch_prefix<<<1, 32, 0, st>>>(ctls, args, nsys, gprefix, group_next); gt_note_launches(1); }
     constexpr int ACC = GT_MAC_ACCELERATION;
     const bool acc = all_acc && mac < 0;
-    auto launch = [&](auto kernel) { kernel<<<nblocks, WT, 0, st>>>(args, nsys, gprefix, group_next, queue, qcap, mac); };
+    auto launch = [&](auto kernel) { gt_launch(kernel, nblocks, WT, 0, st, args, nsys, gprefix, group_next, queue,
+                                               qcap, mac); };
     if (levels) launch(acc ? k_walk_batch<ACC, true> : k_walk_batch<MAC_ANY, true>);
     else launch(acc ? k_walk_batch<ACC, false> : k_walk_batch<MAC_ANY, false>);
     gt_note_launches(1);
