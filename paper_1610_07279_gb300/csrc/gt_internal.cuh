@@ -292,10 +292,10 @@ __host__ __device__ inline unsigned gt_grid(int64_t n, int64_t per, int64_t most
 #define GT_SORT_PASSES 8             // 64 / 8 (bit 63 is always 0)
 
 #ifndef GT_SORT_ST
-#define GT_SORT_ST 512
+#define GT_SORT_ST 256
 #endif
 #ifndef GT_SORT_IPT
-#define GT_SORT_IPT 8
+#define GT_SORT_IPT 16
 #endif
 // tiles of a pass, and the bytes of digit counts and of look-back status of every pass (passes x tiles x digits x 4 B)
 __host__ __device__ inline int gt_sort_tiles(long long n) {

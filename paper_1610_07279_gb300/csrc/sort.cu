@@ -5,7 +5,7 @@
 // the tree's keys, whose ties in those bits are then put in order (k_fix_runs); the digits of all passes are
 // counted by the kernel that makes the keys (keys.cu), or for a caller's pairs by
 //   k_hist_all     all eight digit counts in one read of the keys, and their starts   (reads 8 B/key)
-//   k_onesweep     per 4096-key tile (512 threads) taken in ticket order: a stable rank of
+//   k_onesweep     per 4096-key tile (256 threads) taken in ticket order: a stable rank of
 //                  every key inside the tile (warp-striped; a key's peers with the same
 //                  digit from nine ballots, its rank by popc), the tile's per-digit counts
 //                  published and each digit's exclusive prefix over earlier tiles found
@@ -15,7 +15,10 @@
 //                  (reads and writes 12 B/key; 4 B of status per digit and tile: two flag
 //                  bits, aggregate or inclusive prefix, and a 30-bit count; every pass has
 //                  its own status rows, all cleared once per sort)
-// HBM-bound: ~25 B per key per pass.
+// Bound by the ranking (issue and shared memory), not by its ~25 B per key of HBM: 2^24 keys 146 us a pass, 63 at the
+// copy rate.  Tiles of 256 threads with 16 keys each leave fewer warps' counts to scan than 512 with 8 (154 us); builds
+// of 2^24 with tiles of 256 x 16, 256 x 14, 512 x 8, 384 x 12, 512 x 12 (two blocks per SM) and 512 x 10 (two): 2558,
+// 2585, 2629, 2652, 2608 and 2557 us; sorts of 1000001 keys: 155, 151, 155, 161, 170 and 157.
 #include <mutex>
 
 #include "gt_internal.cuh"
@@ -137,11 +140,16 @@ __device__ __forceinline__ void onesweep_body(const unsigned bid, const unsigned
     for (int j = 0; j < IPT; j++) {
         const long long i = base + j * 32 + lane;
         k[j] = i < n ? kin[i] : 0ull;
-        v[j] = MODE == PASS_LOW_FIRST ? (uint32_t)i : (i < n ? vin[i] : 0u);
+        if (MODE == PASS_LOW_FIRST) v[j] = (uint32_t)i;
+        else if (MODE != PASS_HIGH_FIRST) v[j] = i < n ? vin[i] : 0u;
     }
-    if (MODE == PASS_HIGH_FIRST && index) {
+    if (MODE == PASS_HIGH_FIRST) {
 #pragma unroll
-        for (int j = 0; j < IPT; j++) v[j] = (uint32_t)(base + j * 32 + lane);
+        for (int j = 0; j < IPT; j++) {
+            const long long i = base + j * 32 + lane;
+            v[j] = (uint32_t)i;
+            if (!index && i < n) v[j] = vin[i];
+        }
     }
     if ((long long)(tile + 1) * TILE <= n) gt_rank_keys<true, IPT>(k, shift, 32 * IPT, wcnt + w * R, loc);
     else gt_rank_keys<false, IPT>(k, shift, (int)(n - base < 0 ? 0 : (n - base < 32 * IPT ? n - base : 32 * IPT)), wcnt + w * R, loc);
