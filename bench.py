@@ -443,7 +443,7 @@ def run_batch(g, torch, steps: int, comm: Comm | None = None):
                           "walk_queue": tune["walk_queue"], "candidates_ms": tune["ms"]},
             "batched": {"ms_per_step": ms, "interactions_per_s": inter / (ms * 1e-3),
                         "systems_per_s": 64 / (ms * 1e-3), "gpu_launches_per_step": launches,
-                        "path": "captured CUDA graph: forked builds + one persistent walk launch"},
+                        "path": "captured CUDA graph: builds (one launch per kernel) + one persistent walk launch"},
             "serial": {"ms_per_step": ms_serial, "interactions_per_s": inter_serial / (ms_serial * 1e-3),
                        "systems_per_s": 64 / (ms_serial * 1e-3),
                        "path": "gt_build_tree + gt_accel_active per system, one after another"},

@@ -404,8 +404,8 @@ GT_API int gt_sort_noalloc_status(gt_stream stream);
  *
  * A batch holds nsys systems of any sizes in one caller workspace.  One force
  * evaluation of the batch rebuilds every system's tree (A1-A5), makes every particle
- * active and cuts the groups (A6), on forked streams so that the small systems'
- * kernels overlap, then walks the groups of ALL systems in one persistent launch
+ * active and cuts the groups (A6), many small systems through one launch per kernel,
+ * others on forked streams so that their kernels overlap, then walks the groups of ALL systems in one persistent launch
  * (A7): warps take global group numbers from one counter and find their system from
  * a device-side prefix of the systems' group counts.  Each system's forces are the
  * same, bit for bit, as gt_build_tree + gt_accel_active of that system alone with the
@@ -422,7 +422,7 @@ typedef struct gt_batch gt_batch;
 GT_API int gt_batch_workspace_bytes(int nsys, const int64_t *n, const gt_params *prm, int n_prm,
                                     size_t *bytes);
 /* Create the batch inside d_ws (256-byte aligned, gt_batch_workspace_bytes long).
- * The library creates up to 32 streams of its own for the forked builds.  Every
+ * The library creates up to 32 streams of its own for such builds.  Every
  * system starts empty: load each with gt_set_state(gt_batch_system(...)). */
 GT_API int gt_batch_create(gt_batch **batch, int nsys, const int64_t *n, const gt_params *prm, int n_prm,
                            void *d_ws, size_t ws_bytes);
@@ -479,8 +479,8 @@ GT_API int gt_batch_autotune(gt_batch *batch, const gt_tune_space *space, gt_tun
  * iteration-level batching.  Each server tick enqueues, for every resident request, one
  * unit of work: the start-up (tree, opening-angle pass, a_old, first force, levels;
  * Sec. 2.2, 2.7) for a new request, one block step (predict, rebuild or pseudo j, active
- * set, correct; Sec. 2.6-2.7) for a running one.  The per-request parts run on forked
- * streams; the tree walks of all requests in the tick run in one persistent launch.
+ * set, correct; Sec. 2.6-2.7) for a running one.  The small requests share one launch
+ * per kernel, large ones run on forked streams; the tree walks of all requests in the tick run in one persistent launch.
  * Requests join and leave at tick boundaries: one submitted while others are on the
  * GPU is admitted as soon as a slot and memory are free and its work overlaps theirs.
  * A request's result does not depend on the other requests (separate buffers, the

@@ -372,7 +372,8 @@ void gt_grouped_aold(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStr
 void gt_grouped_correct(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStream_t st);  // and the starts' levels
 
 // keys.cu
-// extrema into ctl->bbox (reset by gt_launch_prepare), and the sort's counts and look-back words cleared; keys and their digit counts for gt_launch_sort_tree
+// extrema into ctl->bbox (reset by gt_launch_prepare), and the sort's counts and look-back words cleared; keys and
+// their digit counts for gt_launch_sort_tree
 void gt_launch_bbox(const float4 *posm, int64_t n, int nblk, DevCtl *ctl, SortBufs &b, cudaStream_t st);
 void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortBufs &b, int nsm, cudaStream_t st);
 // box, keys and sort of at most GT_SMALL_SORT particles in one launch

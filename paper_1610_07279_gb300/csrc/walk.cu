@@ -36,7 +36,7 @@
 // 48 KB of shared memory at three blocks per SM; members and sums wait in shared memory
 // during the traversal (held in registers they spill, and a spilling force loop costs 15 %;
 // two blocks at 95 registers 12 % more time, four at 64 10 %).  The full walk of the
-// Andromeda-like model at 2^22, leaves of 32: 2.60 ms, 0.67 warp instructions per interaction
+// Andromeda-like model at 2^22, leaves of 32: 2.55 ms, 0.69 warp instructions per interaction
 // (3.03 ms and 0.81 with a queue of single cells).
 #include <math.h>
 

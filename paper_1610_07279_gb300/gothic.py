@@ -463,7 +463,7 @@ class System:
 
 
 class Batch:
-    """Many independent systems: forked tree builds and one walk launch over all of
+    """Many independent systems: tree builds together and one walk launch over all of
     them (gt_batch_*).  The batch runs on a stream of its own (capture needs a stream
     other than the legacy default one); its members use the same stream."""
 
