@@ -41,6 +41,7 @@
 #include <math.h>
 
 #include "gt_internal.cuh"
+#include "walk_list.cuh"
 
 namespace {
 
@@ -311,7 +312,13 @@ __device__ __forceinline__ void pad_list(float *lx, uint32_t cap, uint32_t list_
     __syncwarp();
 }
 
-// The first list_n (< CHUNK) entries from quad `from` on moved to the front of the list, by one warp.
+// The warp of walk_list.cuh.
+struct Lanes {
+    __device__ __forceinline__ uint32_t lane() const { return threadIdx.x & 31u; }
+    __device__ __forceinline__ void sync() const { __syncwarp(); }
+};
+
+// A team's list: the first list_n (< CHUNK) entries from quad `from` on moved to the front of the list, by one warp.
 __device__ __forceinline__ void move_rest(float *lx, uint32_t cap, uint32_t list_n, uint32_t from) {
     const uint32_t lane = threadIdx.x & 31u;
     if (4u * lane < list_n) {
@@ -707,13 +714,7 @@ __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32
     // every full chunk of the list, then the rest moved to its front
     auto flush = [&]() {
         cp_async_wait_all();
-        __syncwarp();
-        const uint32_t full = list_n / CHUNK;
-        for (uint32_t c = 0; c < full; c++) chunk(c * (CHUNK / 4), (c + 1) * (CHUNK / 4));
-        list_n -= full * CHUNK;
-        chunks += full;
-        if (full) move_rest(lx, LIST_CAP, list_n, full * (CHUNK / 4));
-        __syncwarp();
+        chunks += flush_chunks<CHUNK>(lx, LIST_CAP, list_n, Lanes{}, chunk);
     };
     uint32_t head = 0, tail = 1;
     if (lane == 0) q[0] = make_uint2(0u, 1u);  // the root
