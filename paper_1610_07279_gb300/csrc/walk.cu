@@ -378,7 +378,7 @@ __device__ __forceinline__ void write_entries(const WalkArgs &a, const Batch &t,
                                               uint32_t cap, uint32_t to, uint32_t w0, uint32_t w1) {
     const unsigned FULL = 0xffffffffu;
     if (t.ok && excl >= w0 && excl < w1) {
-        float *e = lx + to + excl;
+        float *e = list_at(lx, to, excl);
         e[0] = t.jp.x; e[cap] = t.jp.y; e[2 * cap] = t.jp.z; e[3 * cap] = t.jp.w;
     }
     // opened leaves next to each other among one cell's children hold one range of particles: a run of them is
@@ -392,7 +392,7 @@ __device__ __forceinline__ void write_entries(const WalkArgs &a, const Batch &t,
         const float4 *p = a.posm + __shfl_sync(FULL, t.l0, src);
         for (uint32_t e = max(le, w0) + (threadIdx.x & 31u); e < e1; e += 32) {
             const float *from = (const float *)&p[e - le];
-            float *d = lx + to + e;
+            float *d = list_at(lx, to, e);
             cp_async4(d, from);
             cp_async4(d + cap, from + 1);
             cp_async4(d + 2 * cap, from + 2);
@@ -523,7 +523,7 @@ __device__ __forceinline__ void write_particles(const WalkArgs &a, const Cell &t
         const float4 *p = a.posm + __shfl_sync(FULL, t.l0, src);
         for (uint32_t e = max(le, w0) + lane; e < e1; e += 32) {
             const float *from = (const float *)&p[e - le];
-            float *d = lx + to + e;
+            float *d = list_at(lx, to, e);
             cp_async4(d, from);
             cp_async4(d + cap, from + 1);
             cp_async4(d + 2 * cap, from + 2);

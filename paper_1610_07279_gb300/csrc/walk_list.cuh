@@ -4,6 +4,10 @@
 
 #include <stdint.h>
 
+// Entry e of a window whose first entry lies at slot `to` less the entries before it: `to` may have wrapped below
+// zero, so the two are added as 32-bit numbers before they meet the pointer.
+__host__ __device__ __forceinline__ float *list_at(float *lx, uint32_t to, uint32_t e) { return lx + (uint32_t)(to + e); }
+
 // Every full chunk of the list is summed (sum(k0, k1): quads k0 to k1 by all lanes), then the rest, fewer than CHUNK
 // entries from a later quad on, is moved to the front.  The list's number of entries becomes the rest's; returns the
 // chunks summed.  A lane reads entries that other lanes wrote and writes ones that others read, so the warp meets

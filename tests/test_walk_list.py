@@ -1,5 +1,5 @@
 """The walk's interaction list (csrc/walk_list.cuh) with its lanes run one after another between barriers, on the
-host: sums of full chunks, and the move of the rest."""
+host: sums of full chunks, the move of the rest, and the slots of a window's entries."""
 import os
 import shutil
 import subprocess

@@ -79,6 +79,13 @@ int main() {
                         if (lx[a * CAP + e] != value(chunks * CHUNK + e) + 300.0f * a && bad++ < 10)
                             printf("n %u step %u down %d: entry %u is not moved\n", n0, step, down, e);
             }
+    // a window's entries: slot list_n - w0 + e, also where w0 > list_n
+    static float list[CAP];
+    for (uint32_t list_n : {0u, 5u, 127u})
+        for (uint32_t w0 : {0u, 3u, 200u, 5000u})
+            for (uint32_t e = w0; e < w0 + CAP - list_n; e++)
+                if (list_at(list, list_n - w0, e) != list + (list_n + (e - w0)) && bad++ < 20)
+                    printf("list %u window %u entry %u: another address\n", list_n, w0, e);
     printf("bad %d\n", bad);
     return bad != 0;
 }
