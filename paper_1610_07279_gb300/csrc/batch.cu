@@ -90,6 +90,13 @@ void drop_graph(gt_batch *b) {
     b->graph_kernels = 0;
 }
 
+// Host words to the batch's tables.  A copy of pageable memory may return before it has arrived, and streams that
+// don't wait for the default stream may launch kernels that read it at once: it is waited for.
+bool publish(void *dst, const void *src, size_t bytes) {
+    return cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
+           cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess;
+}
+
 // Every member's walk arguments: all particles active (identity list), a_old and the
 // force buffer of the member, the batch's queue depth.
 int upload_args(gt_batch *b) {
@@ -99,9 +106,7 @@ int upload_args(gt_batch *b) {
         b->h_args[k] = gt_sys_walk_args(s, nullptr, s->st[0].aold, s->acc_out, s->prm.mac, false);
         b->h_args[k].queue = b->queue;
     }
-    if (cudaMemcpy(b->d_args, b->h_args.data(), (size_t)b->nsys * sizeof(WalkArgs), cudaMemcpyHostToDevice) !=
-        cudaSuccess)
-        return GT_ECUDA;
+    if (!publish(b->d_args, b->h_args.data(), (size_t)b->nsys * sizeof(WalkArgs))) return GT_ECUDA;
     b->args_dirty = false;
     return GT_OK;
 }
@@ -138,9 +143,7 @@ int upload_table(gt_batch *b, int j) {
     const size_t bytes = tab.size() * sizeof(GroupedSys);
     if (tab.size() == b->h_tab[j].size() && (!bytes || !memcmp(tab.data(), b->h_tab[j].data(), bytes))) return GT_OK;
     // (earlier evaluations may still read it)
-    if (cudaDeviceSynchronize() != cudaSuccess ||
-        cudaMemcpy(b->d_tab[j], tab.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess)
-        return GT_ECUDA;
+    if (cudaDeviceSynchronize() != cudaSuccess || !publish(b->d_tab[j], tab.data(), bytes)) return GT_ECUDA;
     b->h_tab[j] = tab;
     return GT_OK;
 }
@@ -249,7 +252,7 @@ int gt_batch_create(gt_batch **out, int nsys, const int64_t *n, const gt_params 
         ctls[k] = s->ctl;
         off = align_up(off + mb[k]);
     }
-    if (cudaMemcpy(b->d_ctls, ctls.data(), (size_t)nsys * sizeof(DevCtl *), cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (!publish(b->d_ctls, ctls.data(), (size_t)nsys * sizeof(DevCtl *))) {
         gt_batch_destroy(b);
         return GT_ECUDA;
     }
