@@ -39,6 +39,7 @@ struct DevCtl {
     unsigned int n_groups;            // groups of the current force evaluation (cell grouping)
     unsigned int seg[2 * GT_TREE_LEVELS + 1];  // cell list: level l's leaves start at seg[2l], its
                                                // cells with children at seg[2l + 1]; [44] = all
+    unsigned int flat;                // the tree's cells have few children (a sheet, a filament)
     unsigned int cell_bucket[GT_CELL_BUCKETS];  // bucket sizes, then fill cursors, of the cell list
     unsigned int group_next;          // dynamic group counter of the walk
     unsigned int tile_ticket[GT_TREE_LEVELS + 4];  // dynamic tile ids: levels, actives, groups, leaves, cells
@@ -491,7 +492,8 @@ extern "C" int gt_rebuild_interval(const double *t_walk, int n, double t_make, i
                                    double *n_opt_out, double *coef_out);
 int gt_walk_warps_per_block();
 void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st);
-// one launch over the groups of nsys systems (args, ctls: device arrays of nsys entries); all_acc: every
+// one launch over the groups of nsys systems, and one over those with flat trees (args, ctls: device arrays of nsys
+// entries; gprefix: 2 (nsys + 1) words, group_next: two); all_acc: every
 // system uses the acceleration MAC; levels: some have inv_c2 > 0
 void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, uint32_t *gprefix,
                           unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, bool levels,

@@ -480,6 +480,7 @@ __device__ __forceinline__ void cell_count_body(const unsigned bid, const unsign
         v[j] = b < GT_CELL_BUCKETS ? __ldcg(&ctl->cell_bucket[b]) : 0u;
         sum += v[j];
     }
+    __shared__ uint32_t seg[2 * GT_TREE_LEVELS + 1];
     uint32_t start = block_excl_scan<256>(sum, &total, tmp);
 #pragma unroll
     for (int j = 0; j < PER; j++) {
@@ -487,12 +488,22 @@ __device__ __forceinline__ void cell_count_body(const unsigned bid, const unsign
         if (b < GT_CELL_BUCKETS) {
             ctl->cell_bucket[b] = start;
             const int q = b % GT_LEVEL_BUCKETS;
-            if (q == 0) ctl->seg[2 * (b / GT_LEVEL_BUCKETS)] = start;
-            if (q == GT_LEAF_BUCKETS) ctl->seg[2 * (b / GT_LEVEL_BUCKETS) + 1] = start;
+            if (q == 0) seg[2 * (b / GT_LEVEL_BUCKETS)] = start;
+            if (q == GT_LEAF_BUCKETS) seg[2 * (b / GT_LEVEL_BUCKETS) + 1] = start;
         }
         start += v[j];
     }
-    if (threadIdx.x == 0) ctl->seg[2 * GT_TREE_LEVELS] = total;
+    if (threadIdx.x == 0) seg[2 * GT_TREE_LEVELS] = total;
+    __syncthreads();
+    if (threadIdx.x <= 2 * GT_TREE_LEVELS) ctl->seg[threadIdx.x] = seg[threadIdx.x];
+    if (threadIdx.x >= 32) return;
+    // flat (a walk of it packs its batches): fewer than five children per cell, averaged over the levels
+    const int l = threadIdx.x;
+    const uint32_t parents = l < GT_KEY_LEVELS ? seg[2 * l + 2] - seg[2 * l + 1] : 0u;
+    const uint32_t sixteenths = parents ? (uint32_t)(16ull * (seg[2 * l + 4] - seg[2 * l + 2]) / parents) : 0u;
+    const uint32_t all = __reduce_add_sync(0xffffffffu, sixteenths);
+    const unsigned levels = __ballot_sync(0xffffffffu, parents != 0u);
+    if (l == 0) ctl->flat = all < 5u * 16u * __popc(levels) ? 1u : 0u;
 }
 
 __global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, DevCtl *ctl) {

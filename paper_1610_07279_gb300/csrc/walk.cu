@@ -13,9 +13,9 @@
 //     group is the smallest of its members';
 //   * breadth-first traversal: a ring-buffer queue in a per-warp slice of global memory, one
 //     entry (first child, number of children) per opened cell.  An octree cell of more than
-//     leaf_max particles has nearly always all eight children (7.5 to 7.95 on average on the
-//     models here), so four entries fill a batch of 32 lanes without any search for the
-//     lanes' cells, their records are read in runs, and an opened cell costs one queue
+//     leaf_max particles has nearly always all eight children in a solid body (7.5 to 7.95 on
+//     average on the models here), so four entries fill a batch of 32 lanes without any search
+//     for the lanes' cells, their records are read in runs, and an opened cell costs one queue
 //     store.  When the queue fills up, the newest entries are taken first, i.e.
 //     depth-first, which bounds its size (the order does not change the set of
 //     interactions).  The cells are tested with the MAC at distance lambda r_JI (Eqs. 2, 5-7)
@@ -335,14 +335,47 @@ struct Batch {
     bool ok;            // accepted
 };
 
-// One batch: the children of nb (at most four) queue entries from `base` on, one per lane, and what the MAC says.
-template <int MAC>
-__device__ __forceinline__ Batch test_batch(const WalkArgs &a, const Pseudo &ps, const uint2 *q, uint32_t base,
-                                            uint32_t nb, uint32_t qmask, uint32_t &tests) {
+// A batch of cells, one per lane.
+struct Take {
+    uint32_t node, nb;  // nb: queue entries taken
+    bool valid;
+};
+
+// The children of the next four queue entries, eight lanes each (sib: the lane's entry).
+__device__ __forceinline__ Take take_four(uint2 sib, uint32_t avail) {
+    const uint32_t lane = threadIdx.x & 31u, nb = min(avail, 4u);
+    const bool valid = (lane >> 3) < nb && (lane & 7u) < sib.y;
+    return Take{valid ? sib.x + (lane & 7u) : 0u, nb, valid};
+}
+
+// The children of as many whole entries from the queue's head on as fill the lanes: for flat trees (DevCtl::flat), whose
+// cells have four children on a sheet and two on a filament, so that four entries would leave half or three quarters of
+// the lanes idle.  Every particle, with four entries and packed, us: a sheet of 2^20 (leaves of 4) 887 and 762, a line
+// 1144 and 720, a sheet of 2^22 3653 and 3102, a line 6048 and 3632; solid bodies gain nothing by it (a Plummer sphere of
+// 2^22, leaves of 16: 2489 and 2692).  The line lies at five children per cell, averaged over the levels: sheets have 4,
+// slabs of a hundredth of their width 4.6 to 4.9 (2^18, leaves of 4: 365 and 353), solid models with leaves of 4 and more
+// 5.9 to 8.  Both in one kernel would cost solid bodies 2 % (batches) to 3 % (registers, code), so each has its own, and
+// the one that isn't meant ends at once (1 to 3 us a call).
+__device__ __forceinline__ Take take_packed(const uint2 *q, uint32_t head, uint32_t avail, uint32_t qmask) {
     const uint32_t lane = threadIdx.x & 31u;
-    const uint2 sib = q[(base + (lane >> 3)) & qmask];
-    bool valid = (lane >> 3) < nb && (lane & 7u) < sib.y;
-    uint32_t node = valid ? sib.x + (lane & 7u) : 0u;
+    const unsigned FULL = 0xffffffffu;
+    uint2 e = make_uint2(0u, 0u);
+    if (lane < avail) e = q[(head + lane) & qmask];
+    const uint32_t incl = warp_incl_scan(e.y), excl = incl - e.y;
+    const unsigned taken = __ballot_sync(FULL, e.y && incl <= 32u);
+    const uint32_t nb = __popc(taken);
+    // bit p: the first child of an entry has lane p
+    const unsigned m = __reduce_or_sync(FULL, e.y && incl <= 32u ? 1u << excl : 0u) & (0xffffffffu >> (31u - lane));
+    const uint32_t node = __shfl_sync(FULL, e.x, __popc(m) - 1) + lane - (31u - (uint32_t)__clz(m));
+    const bool valid = lane < __shfl_sync(FULL, incl, nb - 1u);
+    return Take{valid ? node : 0u, nb, valid};
+}
+
+// One batch: a cell per lane, and what the MAC says.
+template <int MAC>
+__device__ __forceinline__ Batch test_batch(const WalkArgs &a, const Pseudo &ps, const Take &k, uint32_t &tests) {
+    bool valid = k.valid;
+    uint32_t node = k.node;
 #if GT_DEBUG
     const uint32_t nnodes = a.ctl->level_start[GT_TREE_LEVELS];
     if (node >= nnodes) {
@@ -374,6 +407,7 @@ __device__ __forceinline__ Batch test_batch(const WalkArgs &a, const Pseudo &ps,
 
 // The entries of a batch with index in [w0, w1) into the list: entry e goes to slot to + e.  `excl`: the index
 // of the lane's first; lm: lanes with an opened leaf.
+template <bool PACK>
 __device__ __forceinline__ void write_entries(const WalkArgs &a, const Batch &t, uint32_t excl, unsigned lm, float *lx,
                                               uint32_t cap, uint32_t to, uint32_t w0, uint32_t w1) {
     const unsigned FULL = 0xffffffffu;
@@ -381,12 +415,19 @@ __device__ __forceinline__ void write_entries(const WalkArgs &a, const Batch &t,
         float *e = list_at(lx, to, excl);
         e[0] = t.jp.x; e[cap] = t.jp.y; e[2 * cap] = t.jp.z; e[3 * cap] = t.jp.w;
     }
-    // opened leaves next to each other among one cell's children hold one range of particles: a run of them is
-    // copied at a time, asynchronously
-    const unsigned starts = lm & ~((lm << 1) & 0xfefefefeu);
+    // opened leaves next to each other that hold one range of particles are copied together, asynchronously: those among
+    // one entry's children (eight lanes each), or, where entries are packed, that begin where the one before ends
+    unsigned starts = lm & ~((lm << 1) & 0xfefefefeu);
+    if (PACK) {
+        const uint32_t before = __shfl_up_sync(FULL, t.l0 + t.mine, 1);  // where the lane before ends
+        starts = lm & ~(__ballot_sync(FULL, before == t.l0) & (lm << 1));
+    }
     for (unsigned m = starts; m; m &= m - 1) {
         const int src = __ffs(m) - 1;
-        const int end = min(src + __ffs(~((lm >> src) & 0xffu)) - 2, src | 7);  // the run's last lane
+        // the run's last lane: before the next lane that is no leaf or starts a run of its own
+        const unsigned stop = (~lm | (m & (m - 1))) & (0xfffffffeu << src);
+        const int end = PACK ? (stop ? __ffs(stop) - 2 : 31)
+                             : min(src + __ffs(~((lm >> src) & 0xffu)) - 2, src | 7);
         const uint32_t le = __shfl_sync(FULL, excl, src);
         const uint32_t e1 = min(__shfl_sync(FULL, excl + t.mine, end), w1);
         const float4 *p = a.posm + __shfl_sync(FULL, t.l0, src);
@@ -690,7 +731,7 @@ __device__ __noinline__ void walk_group_ordered(const WalkArgs &a, uint32_t g, u
 
 // One group g of system a (Sec. 2.3) by one warp.  The interactions and MAC tests are added to stat[0] and
 // stat[1].  lx: the warp's WARP_SM words of shared memory.
-template <int MAC, bool LEVELS>
+template <int MAC, bool LEVELS, bool PACK>
 __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx, uint2 *q,
                                            unsigned long long *stat) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -722,15 +763,22 @@ __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32
     bool overflow = false;
     while (head != tail) {
         // breadth-first from the head while there is room, depth-first from the tail after
-        const uint32_t nb = min(tail - head, 4u);
-        uint32_t base = head;
-        if (8 * (int)(tail - head) > a.qcap - LIFO_ROOM) {
-            tail -= nb;
-            base = tail;
+        uint32_t nb = min(tail - head, 4u), base = head;
+        const bool newest = 8 * (int)(tail - head) > a.qcap - LIFO_ROOM;
+        Take k;
+        if (PACK && !newest) {
+            k = take_packed(q, head, tail - head, qmask);
+            head += k.nb;
         } else {
-            head += nb;
+            if (newest) {
+                tail -= nb;
+                base = tail;
+            } else {
+                head += nb;
+            }
+            k = take_four(q[(base + (lane >> 3)) & qmask], nb);
         }
-        const Batch t = test_batch<MAC>(a, ps, q, base, nb, qmask, tests);
+        const Batch t = test_batch<MAC>(a, ps, k, tests);
         // opened cells: their children join the queue as one entry per cell
         const unsigned om = __ballot_sync(FULL, t.nch != 0u);
         if (om) {
@@ -761,7 +809,7 @@ __device__ __forceinline__ void walk_group(const WalkArgs &a, uint32_t g, uint32
             // a window of the batch's entries at a time: what the list has room for
             for (uint32_t w0 = 0; w0 < tot;) {
                 const uint32_t w1 = min(tot, w0 + (LIST_CAP - list_n));
-                write_entries(a, t, incl - t.mine, lm, lx, LIST_CAP, list_n - w0, w0, w1);
+                write_entries<PACK>(a, t, incl - t.mine, lm, lx, LIST_CAP, list_n - w0, w0, w1);
                 list_n += w1 - w0;
                 w0 = w1;
                 if (w0 < tot) flush();
@@ -861,7 +909,7 @@ __device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32
     team_sync(team, T);
     while (head != tail) {
         const uint32_t live = tail - head, nb = min(live, 4u * T), b0 = min(4u * w, nb);
-        const Batch t = test_batch<MAC>(a, ps, q, head + b0, min(nb - b0, 4u), qmask, tests);
+        const Batch t = test_batch<MAC>(a, ps, take_four(q[(head + b0 + (lane >> 3)) & qmask], nb - b0), tests);
         head += nb;
         const unsigned om = __ballot_sync(FULL, t.nch != 0u), am = __ballot_sync(FULL, t.ok);
         const unsigned lm = __ballot_sync(FULL, t.mine != 0u) & ~am;
@@ -885,7 +933,7 @@ __device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32
         const uint32_t excl = first + incl - t.mine;
         for (uint32_t w0 = 0; w0 < tot;) {
             const uint32_t w1 = min(tot, w0 + (cap - list_n));
-            write_entries(a, t, excl, lm, lx, cap, list_n - w0, w0, w1);
+            write_entries<false>(a, t, excl, lm, lx, cap, list_n - w0, w0, w1);
             list_n += w1 - w0;
             w0 = w1;
             if (w0 < tot) flush(false);
@@ -912,8 +960,14 @@ __device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32
 // warp's time (barriers, and batches that the first levels of the tree do not fill), so it pays where the
 // longest groups, not their sum, set the time.  Whole calls in us with T = 1, 2, 4, 8 (3648 warps): 476 groups
 // 704, 509, 399, 354; 4600 groups 370, 264, 214, 238; 6080 groups 412, 368, 365, 415; 11333 groups 272, 303,
-// 380, 573; 115000 groups 2620, 3207, 4456, 7118.
+// 380, 573; 115000 groups 2620, 3207, 4456, 7118.  (The 4600 would be faster by fours, and from 4600 to 6080 it makes no
+// difference: the cut between fours and twos could lie higher.)
+// FLAT: a team's batches are four entries of each warp, which on flat trees leaves half or more of its lanes idle, so
+// teams end earlier.  Calls with T = 1, 2, 4, 8: lines, 373 groups 63, 78, 65, 56; 754 groups 70, 93, 69, 87; 1524 groups
+// 76, 108, 113, -; sheets, 256 groups 62, 62, 50, 47; 1024 groups 75, 77, 68, -; 2386 groups 107, 113, 117, -.
+template <bool FLAT>
 __device__ __forceinline__ uint32_t team_of(uint32_t ngroups, uint32_t warps) {
+    if (FLAT) return ngroups > warps / 3u ? 1u : (ngroups > warps / 8u ? 4u : 8u);
     return ngroups > 2u * warps ? 1u : (ngroups > warps ? 2u : (ngroups > warps / 4u ? 4u : 8u));
 }
 
@@ -928,9 +982,11 @@ __device__ __forceinline__ int system_of(const uint32_t *gprefix, int nsys, uint
     return lo;
 }
 
-template <int MAC, bool LEVELS>
+// FLAT: for a system whose tree is flat; one of the two kernels walks it, the other ends at once.
+template <int MAC, bool LEVELS, bool FLAT>
 __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant__ WalkArgs a) {
     gt_grid_ready();
+    if ((a.ctl->flat != 0u) != FLAT) return;
     __shared__ __align__(16) float list_sm[NWARP][WARP_SM];
     __shared__ unsigned long long stat_sm[NWARP][2];
     __shared__ uint2 counts_sm[NWARP];
@@ -939,7 +995,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant
     const uint32_t na = a.ctl->n_active;
     const uint32_t gmax = (uint32_t)a.gmax;
     const uint32_t ngroups = a.gstart ? a.ctl->n_groups : (na + gmax - 1) / gmax;
-    const uint32_t T = team_of(ngroups, gridDim.x * NWARP), team = warp / T, first = team * T;
+    const uint32_t T = team_of<FLAT>(ngroups, gridDim.x * NWARP), team = warp / T, first = team * T;
     uint2 *q = (uint2 *)a.queue + (size_t)(blockIdx.x * NWARP + first) * gt_queue_ring(a.qcap);
     unsigned long long *stat = stat_sm[warp];
     if (lane < 2) stat[lane] = 0;
@@ -950,7 +1006,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant
             if (lane == 0) g = atomicAdd(&a.ctl->group_next, 1u);
             g = __shfl_sync(0xffffffffu, g, 0);
             if (g >= ngroups) break;
-            walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[warp], q, stat);
+            walk_group<MAC, LEVELS, FLAT>(a, g, ngroups, list_sm[warp], q, stat);
         }
     } else {
         for (;;) {
@@ -959,7 +1015,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant
             const uint32_t g = g_sm[team];
             if (g >= ngroups) break;
             if (!team_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat, counts_sm + first, team, T) && warp == first)
-                walk_group<MAC, LEVELS>(a, g, ngroups, list_sm[first], q, stat);
+                walk_group<MAC, LEVELS, FLAT>(a, g, ngroups, list_sm[first], q, stat);
             team_sync(team, T);
         }
     }
@@ -973,8 +1029,9 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant
 // Many systems in one persistent launch: global group numbers run over the systems
 // in order (gprefix), every warp or team takes the next one from one counter and walks it
 // with that system's arguments (copied to shared memory).  mac >= 0 overrides every
-// system's MAC (the opening-angle start-up pass).
-template <int MAC, bool LEVELS>
+// system's MAC (the opening-angle start-up pass).  FLAT: the groups of the systems whose trees are flat, or of the others
+// (gprefix and group_next are this kind's).
+template <int MAC, bool LEVELS, bool FLAT>
 __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs *__restrict__ args, int nsys,
                                                                  const uint32_t *__restrict__ gprefix,
                                                                  unsigned int *group_next, uint32_t *queue, int qcap,
@@ -987,7 +1044,8 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
     __shared__ uint32_t g_sm[NWARP];
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     const uint32_t total = gprefix[nsys];
-    const uint32_t T = team_of(total, gridDim.x * NWARP), team = warp / T, first = team * T;
+    if (FLAT && !total) return;
+    const uint32_t T = team_of<FLAT>(total, gridDim.x * NWARP), team = warp / T, first = team * T;
     uint2 *q = (uint2 *)queue + (size_t)(blockIdx.x * NWARP + first) * gt_queue_ring(qcap);
     unsigned long long *stat = stat_sm[warp];
     const WalkArgs &a = sargs[warp];
@@ -1032,11 +1090,11 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
         }
         // the batch queue replaces the system's own
         if (T == 1) {
-            walk_group<MAC, LEVELS>(a, gg - g0, g1 - g0, list_sm[warp], q, stat);
+            walk_group<MAC, LEVELS, FLAT>(a, gg - g0, g1 - g0, list_sm[warp], q, stat);
         } else {
             if (!team_group<MAC, LEVELS>(a, gg - g0, g1 - g0, list_sm[first], q, stat, counts_sm + first, team, T) &&
                 warp == first)
-                walk_group<MAC, LEVELS>(a, gg - g0, g1 - g0, list_sm[first], q, stat);
+                walk_group<MAC, LEVELS, FLAT>(a, gg - g0, g1 - g0, list_sm[first], q, stat);
             team_sync(team, T);
         }
     }
@@ -1044,27 +1102,30 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
     count();
 }
 
-// gprefix over the systems' group counts (one warp; also resets the batch counter)
-__global__ void k_batch_prefix(DevCtl *const *__restrict__ ctls, const WalkArgs *__restrict__ args, int nsys,
-                               uint32_t *gprefix, unsigned int *group_next) {
+// gprefix over the group counts of the systems whose trees aren't flat, and behind it over those of the others (a warp
+// each; also resets the two counters)
+__global__ __launch_bounds__(64) void k_batch_prefix(DevCtl *const *__restrict__ ctls, const WalkArgs *__restrict__ args,
+                                                     int nsys, uint32_t *gprefix, unsigned int *group_next) {
     gt_grid_ready();
+    const int lane = threadIdx.x & 31, kind = threadIdx.x >> 5;
+    gprefix += kind * (nsys + 1);
     uint32_t carry = 0;
     for (int s0 = 0; s0 < nsys; s0 += 32) {
-        const int s = s0 + (int)threadIdx.x;
+        const int s = s0 + lane;
         uint32_t ng = 0;
         if (s < nsys) {
             const DevCtl *c = ctls[s];
             const uint32_t na = c->n_active;
             const uint32_t gm = (uint32_t)args[s].gmax;
-            ng = args[s].gstart ? c->n_groups : (na + gm - 1) / gm;
+            if ((c->flat != 0u) == (kind == 1)) ng = args[s].gstart ? c->n_groups : (na + gm - 1) / gm;
         }
         const uint32_t incl = warp_incl_scan(ng);
         if (s < nsys) gprefix[s] = carry + incl - ng;
         carry += __shfl_sync(0xffffffffu, incl, 31);
     }
-    if (threadIdx.x == 0) {
+    if (lane == 0) {
         gprefix[nsys] = carry;
-        *group_next = 0u;
+        group_next[kind] = 0u;
     }
 }
 
@@ -1072,7 +1133,7 @@ __global__ void k_batch_prefix(DevCtl *const *__restrict__ ctls, const WalkArgs 
 
 int gt_walk_blocks(int nsm) {
     int per = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<MAC_ANY, true>, WT, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_walk<MAC_ANY, true, false>, WT, 0);
     if (per < 1) per = 1;
     return per * nsm;
 }
@@ -1083,21 +1144,24 @@ void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st) {
     constexpr int ACC = GT_MAC_ACCELERATION;
     const bool acc = a.mac == ACC, levels = a.inv_c2 > 0.0f;
     auto launch = [&](auto kernel) { gt_launch(kernel, nblocks, WT, 0, st, a); };
-    if (levels) launch(acc ? k_walk<ACC, true> : k_walk<MAC_ANY, true>);
-    else launch(acc ? k_walk<ACC, false> : k_walk<MAC_ANY, false>);
-    gt_note_launches(1);
+    if (levels) launch(acc ? k_walk<ACC, true, false> : k_walk<MAC_ANY, true, false>);
+    else launch(acc ? k_walk<ACC, false, false> : k_walk<MAC_ANY, false, false>);
+    launch(levels ? k_walk<MAC_ANY, true, true> : k_walk<MAC_ANY, false, true>);
+    gt_note_launches(2);
 }
 
 void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, uint32_t *gprefix,
                           unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, bool levels,
                           int nblocks, cudaStream_t st) {
     if (nsys <= 0) return;
-    { k_batch_prefix<<<1, 32, 0, st>>>(ctls, args, nsys, gprefix, group_next); gt_note_launches(1); }
+    { k_batch_prefix<<<1, 64, 0, st>>>(ctls, args, nsys, gprefix, group_next); gt_note_launches(1); }
     constexpr int ACC = GT_MAC_ACCELERATION;
     const bool acc = all_acc && mac < 0;
-    auto launch = [&](auto kernel) { gt_launch(kernel, nblocks, WT, 0, st, args, nsys, gprefix, group_next, queue,
-                                               qcap, mac); };
-    if (levels) launch(acc ? k_walk_batch<ACC, true> : k_walk_batch<MAC_ANY, true>);
-    else launch(acc ? k_walk_batch<ACC, false> : k_walk_batch<MAC_ANY, false>);
-    gt_note_launches(1);
+    auto launch = [&](auto kernel, int kind) {
+        gt_launch(kernel, nblocks, WT, 0, st, args, nsys, gprefix + kind * (nsys + 1), group_next + kind, queue, qcap, mac);
+    };
+    if (levels) launch(acc ? k_walk_batch<ACC, true, false> : k_walk_batch<MAC_ANY, true, false>, 0);
+    else launch(acc ? k_walk_batch<ACC, false, false> : k_walk_batch<MAC_ANY, false, false>, 0);
+    launch(levels ? k_walk_batch<MAC_ANY, true, true> : k_walk_batch<MAC_ANY, false, true>, 1);
+    gt_note_launches(2);
 }
