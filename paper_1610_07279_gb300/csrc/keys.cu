@@ -176,8 +176,9 @@ __global__ __launch_bounds__(256) void k_keys(const float4 *__restrict__ posm, l
 // Small systems: the bounding box, the keys and the whole sort in one block, in shared memory (through the kernels
 // above: thirteen launches, of which every sort pass takes 10 us for the latency of its chain; 8192 particles ~90 us).
 // The passes move 16-bit positions only and look the digits up in the keys, which stay: the wavefronts of one SM's
-// shared memory and its ballots bound it (7 us a pass; 48 us in all, 70 with keys that move too and eight passes).  Five passes over the
-// highest 40 bits, then the short runs that agree there; a longer run that is out of order takes all eight passes.
+// shared memory and its ballots bound it (7 us a pass; 48 us in all, 70 with keys that move too and eight passes).  Five
+// passes over the highest 40 bits, then the short runs that agree there; a longer run that is out of order takes all
+// eight passes.
 constexpr int SMALL_THREADS = 1024, SMALL_WARPS = SMALL_THREADS / 32, SMALL_IPT = 8;
 static_assert(SMALL_THREADS * SMALL_IPT == GT_SMALL_SORT && SMALL_THREADS == 4 * GT_SORT_DIGITS, "one block's keys");
 constexpr size_t SMALL_SMEM = GT_SMALL_SORT * (sizeof(unsigned long long) + sizeof(uint16_t)) +
@@ -286,25 +287,36 @@ __device__ __forceinline__ void small_sort_body(const unsigned bid, const unsign
     };
     for (int shift = SMALL_SHIFT; shift < 63; shift += GT_SORT_BITS) pass(shift);
     auto same = [&](int i, int j) { return ((skey[sid[i]] ^ skey[sid[j]]) >> SMALL_SHIFT) == 0ull; };
-    for (int i = threadIdx.x; i + 1 < n; i += SMALL_THREADS) {  // runs that begin at i
-        if (!same(i, i + 1) || (i > 0 && same(i - 1, i))) continue;
-        int len = 2;
-        bool sorted = skey[sid[i]] <= skey[sid[i + 1]];
-        for (; i + len < n && same(i, i + len); len++) {
-            sorted = sorted && skey[sid[i + len - 1]] <= skey[sid[i + len]];
-            if (len > SMALL_RUN && !sorted) break;
+    // Pairs out of order within a run.  The first one of a run of at most SMALL_RUN keys has its thread put the run in
+    // order, after every thread has looked; one in a longer run (a thread looks no further than SMALL_RUN keys either way)
+    // has everything sorted again.
+    auto run_start = [&](int i) {
+        while (i > 0 && same(i - 1, i)) i--;
+        return i;
+    };
+    uint32_t mine = 0;
+    for (int j = 0, i = threadIdx.x; i + 1 < n; j++, i += SMALL_THREADS) {
+        if (!same(i, i + 1) || skey[sid[i]] <= skey[sid[i + 1]]) continue;
+        int a = i, b = i + 2;
+        bool first = true;
+        while (first && a > 0 && i - a < SMALL_RUN && same(a - 1, a)) {
+            first = skey[sid[a - 1]] <= skey[sid[a]];
+            a--;
         }
-        if (sorted) continue;
-        if (len > SMALL_RUN) {
-            redo_sh = 1;
-            continue;
-        }
-        for (int j = 1; j < len; j++) {
-            const uint16_t v = sid[i + j];
+        if (!first) continue;
+        while (b < n && b - a <= SMALL_RUN && same(i, b)) b++;
+        if (b - a > SMALL_RUN) redo_sh = 1;
+        else mine |= 1u << j;
+    }
+    __syncthreads();
+    for (uint32_t m = mine; m; m &= m - 1) {
+        const int i = (__ffs(m) - 1) * SMALL_THREADS + (int)threadIdx.x, a = run_start(i);
+        for (int j = i + 1 - a; a + j < n && same(a, a + j); j++) {
+            const uint16_t v = sid[a + j];
             const unsigned long long kv = skey[v];
             int p = j;
-            for (; p > 0 && skey[sid[i + p - 1]] > kv; p--) sid[i + p] = sid[i + p - 1];
-            sid[i + p] = v;
+            for (; p > 0 && skey[sid[a + p - 1]] > kv; p--) sid[a + p] = sid[a + p - 1];
+            sid[a + p] = v;
         }
     }
     __syncthreads();
