@@ -215,45 +215,70 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void k_onesweep(long long n, int 
 // ---- keys that agree in the sorted bits --------------------------------------------
 // The tree's keys are spread over the bounding cube by construction, so few of them agree in their highest 16 levels
 // (48 bits): six passes over those bits leave short runs of keys that differ only below, and these are put in order
-// here -- two passes fewer over all keys (2^24: 322 us of 1290) for one read of them (25 us).  The passes and all three
-// ways below are stable, so the result is that of a stable sort by the whole key.  Where the particles fill only a
-// small part of the cube (one far particle is enough), the digit of levels 11 to 13 takes few values: once one of them
-// holds a sixteenth of the keys (smooth models: a few hundredths of that share) the two low passes run as well.
+// here -- two passes fewer over all keys (2^24: 322 us of 1290) for one read of them (25 us).  The passes and all
+// ways below are stable, so the result is that of a stable sort by the whole key.  Where long runs are to be expected the
+// two low passes run as well (gt_finish_digits); what is left costs no more than they would, whatever the runs' lengths:
+// short runs are put in order by a thread, the longer ones that begin in one tile of the keys together by a block in shared
+// memory, and one that is too long for that by a block through the other buffers.  (A block for every run longer than 16
+// keys, and the choice by one digit: a Plummer sphere of 2^22 with one particle at 2500 times its radius 3854 us the
+// whole build, eight passes 1729.)
 constexpr uint32_t RUN_SHORT = 16;  // keys that one thread puts in order by insertion
-constexpr int RUN_SMEM = TILE;      // keys that a block puts in order in shared memory
+constexpr int FIX_ROUNDS = 8, FIX_TILE = 256 * FIX_ROUNDS;  // keys that a block of k_fix_runs looks at at a time
 
 __device__ __forceinline__ bool same_run(unsigned long long a, unsigned long long b, int shift) {
     return ((a ^ b) >> shift) == 0ull;
 }
 
-// One thread per key: the first key of a run of two or more has it put in order, or listed if it is longer and not in
-// order already as far as looked.
+// One thread per key: the first key of a short run of two or more has it put in order; of the longer ones that begin in a
+// tile, the first and the last begin are listed.
 __device__ __forceinline__ void fix_runs_body(const unsigned bid, const unsigned nb, long long n, int shift,
         unsigned long long *key, uint32_t *val, uint32_t *list, DevCtl *ctl) {
     if (ctl->sort_whole) return;
-    for (long long i = bid * 256ll + threadIdx.x; i < n; i += (long long)nb * 256) {
-        const unsigned long long k0 = key[i];
-        if (i + 1 >= n || !same_run(k0, key[i + 1], shift)) continue;
-        if (i > 0 && same_run(key[i - 1], k0, shift)) continue;
-        uint32_t len = 2;
-        while (len <= RUN_SHORT && i + len < n && same_run(k0, key[i + len], shift)) len++;
-        if (len > RUN_SHORT) {
-            list[atomicAdd(&ctl->run_count, 1u)] = (uint32_t)i;
-            continue;
+    __shared__ uint32_t first_sh, last_sh;
+    if (threadIdx.x == 0) first_sh = ~0u, last_sh = 0u;
+    __syncthreads();
+    for (long long t = (long long)bid * FIX_TILE; t < n; t += (long long)nb * FIX_TILE) {
+        uint32_t begins = 0;  // rounds in which this thread's key begins a run of two or more
+#pragma unroll
+        for (int r = 0; r < FIX_ROUNDS; r++) {
+            const long long i = t + 256 * r + threadIdx.x;
+            if (i + 1 >= n) continue;
+            const unsigned long long k0 = key[i], k1 = key[i + 1], kb = i > 0 ? key[i - 1] : ~k0;
+            if (same_run(k0, k1, shift) && !same_run(kb, k0, shift)) begins |= 1u << r;
         }
-        for (uint32_t j = 1; j < len; j++) {
-            const unsigned long long k = key[i + j];
-            const uint32_t v = val[i + j];
-            uint32_t p = j;
-            for (; p > 0 && key[i + p - 1] > k; p--) {
-                key[i + p] = key[i + p - 1];
-                val[i + p] = val[i + p - 1];
+        for (; begins; begins &= begins - 1) {
+            const long long i = t + 256 * (__ffs(begins) - 1) + threadIdx.x;
+            const unsigned long long k0 = key[i];
+            uint32_t len = 2;
+            while (len <= RUN_SHORT && i + len < n && same_run(k0, key[i + len], shift)) len++;
+            if (len > RUN_SHORT) {
+                atomicMin(&first_sh, (uint32_t)i);
+                atomicMax(&last_sh, (uint32_t)i);
+                continue;
             }
-            if (p != j) {
-                key[i + p] = k;
-                val[i + p] = v;
+            for (uint32_t j = 1; j < len; j++) {
+                const unsigned long long k = key[i + j];
+                const uint32_t v = val[i + j];
+                uint32_t p = j;
+                for (; p > 0 && key[i + p - 1] > k; p--) {
+                    key[i + p] = key[i + p - 1];
+                    val[i + p] = val[i + p - 1];
+                }
+                if (p != j) {
+                    key[i + p] = k;
+                    val[i + p] = v;
+                }
             }
         }
+        __syncthreads();
+        if (threadIdx.x == 0 && first_sh != ~0u) {
+            const uint32_t at = atomicAdd(&ctl->run_count, 1u);
+            list[2 * at] = first_sh;
+            list[2 * at + 1] = last_sh;
+            first_sh = ~0u;
+            last_sh = 0u;
+        }
+        __syncthreads();
     }
 }
 
@@ -263,137 +288,211 @@ __global__ __launch_bounds__(256) void k_fix_runs(long long n, int shift, unsign
     fix_runs_body(blockIdx.x, gridDim.x, n, shift, key, val, list, ctl);
 }
 
-// The listed runs, a block each: by digits in shared memory, or, beyond RUN_SMEM keys, tile by tile through the
-// other buffers.  Runs that are in order (equal keys, most of all) are left alone.
+// Shared memory of a block of k_fix_long_runs: three of them per SM.
+struct FixShared {
+    unsigned long long key[TILE];
+    uint32_t val[TILE];
+    uint16_t pos[TILE], run[TILE];  // an order of the keys, and the run of each (numbers from 0)
+    uint32_t wcnt[NW * R];          // a count per warp and digit
+    uint32_t dstart[R];             // where the next key of every digit goes
+    uint32_t scantmp[NW + 1], wruns[NW];
+};
+constexpr size_t FIX_SMEM = sizeof(FixShared);
+
+// The start of every digit's keys of the warp in its tile: the sums over the warps before, and (returned, for the
+// thread's digit) the tile's count.
+__device__ __forceinline__ uint32_t scan_warps(FixShared &sm) {
+    uint32_t cnt = 0;
+    if (threadIdx.x < R)
+        for (int ww = 0; ww < NW; ww++) {
+            const uint32_t t = sm.wcnt[ww * R + threadIdx.x];
+            sm.wcnt[ww * R + threadIdx.x] = cnt;
+            cnt += t;
+        }
+    return cnt;
+}
+
+// The first m keys in shared memory, whole runs, to global memory in the order of a stable sort by the whole key: by the
+// bits below `shift`, then by run, on the keys' positions.  Left alone if in order already.
+__device__ __forceinline__ void sort_region(FixShared &sm, int m, int shift, unsigned long long *key, uint32_t *val) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, base = w * 32 * IPT;
+    bool out = false;
+    for (int i = threadIdx.x; i + 1 < m; i += ST) out = out || sm.key[i] > sm.key[i + 1];
+    if (!__syncthreads_or(out)) return;
+    uint32_t id[IPT], runs = 0;
+#pragma unroll
+    for (int j = 0; j < IPT; j++) {
+        const int i = base + 32 * j + lane;
+        id[j] = (uint32_t)i;
+        const unsigned begins = __ballot_sync(0xffffffffu, i > 0 && i < m && !same_run(sm.key[i - 1], sm.key[i], shift));
+        if (i < m) sm.run[i] = (uint16_t)(runs + (uint32_t)__popc(begins & (lanemask_lt() | (1u << lane))));
+        runs += (uint32_t)__popc(begins);
+    }
+    if (lane == 0) sm.wruns[w] = runs;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+    for (int ww = 0; ww < NW; ww++) {
+        before += ww < w ? sm.wruns[ww] : 0u;
+        all += sm.wruns[ww];
+    }
+    for (int i = base + lane; i < base + 32 * IPT && i < m; i += 32) sm.run[i] = (uint16_t)(sm.run[i] + before);
+    __syncthreads();
+    // digits: the low bits (the last digit reaches into the run's own bits, which the runs' digits outweigh), the run
+    const int low = (shift + RB - 1) / RB, passes = low + (all == 0u ? 0 : (all < R ? 1 : 2));
+    for (int p = 0; p < passes; p++) {
+        for (int i = threadIdx.x; i < NW * R; i += ST) sm.wcnt[i] = 0;
+        __syncthreads();
+        uint32_t dig[IPT], loc[IPT];
+#pragma unroll
+        for (int j = 0; j < IPT; j++) {
+            dig[j] = R;
+            if (base + 32 * j + lane < m)
+                dig[j] = (p < low ? (uint32_t)(sm.key[id[j]] >> (RB * p)) : (uint32_t)sm.run[id[j]] >> (RB * (p - low))) & (R - 1);
+        }
+        if (base < m) {
+#pragma unroll
+            for (int j = 0; j < IPT; j++) loc[j] = gt_rank_digit<false>(dig[j], sm.wcnt + w * R);
+        }
+        __syncthreads();
+        const uint32_t cnt = scan_warps(sm);
+        uint32_t total;
+        const uint32_t e = block_excl_scan<ST>(cnt, &total, sm.scantmp);
+        if (threadIdx.x < R) sm.dstart[threadIdx.x] = e;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < IPT; j++)
+            if (dig[j] < R) sm.pos[sm.dstart[dig[j]] + sm.wcnt[w * R + dig[j]] + loc[j]] = (uint16_t)id[j];
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < IPT; j++)
+            if (dig[j] < R) id[j] = sm.pos[base + 32 * j + lane];
+    }
+#pragma unroll
+    for (int j = 0; j < IPT; j++) {
+        const int i = base + 32 * j + lane;
+        if (i < m) {
+            key[i] = sm.key[id[j]];
+            val[i] = sm.val[id[j]];
+        }
+    }
+}
+
+// A run that is longer than a tile, from key0[first] on, by one block, tile after tile through the other buffers.  Left
+// alone if in order already (equal keys, most of all).
+__device__ __forceinline__ void sort_long_run(FixShared &sm, long long first, long long n, int shift,
+        unsigned long long *key0, uint32_t *val0, unsigned long long *key1, uint32_t *val1) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned long long k0 = key0[first];
+    // its end: every round cuts what is left to a part in 256
+    long long a = first, b = n;  // key0[a] belongs to it, key0[b] (if b < n) doesn't
+    while (b - a > 1) {
+        const long long step = (b - a + ST - 1) / ST, i = a + step * threadIdx.x;
+        const int in = __syncthreads_count(i < b && same_run(k0, key0[i], shift));  // the first `in` threads
+        a += step * (in - 1);
+        b = a + step < b ? a + step : b;
+    }
+    const long long len = a + 1 - first;
+    bool out = false;
+    for (long long i = first + 1 + threadIdx.x; i < first + len && !out; i += 8 * ST) {
+        unsigned long long k[8], kb[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            const long long at = i + (long long)j * ST < first + len ? i + (long long)j * ST : i;
+            k[j] = key0[at];
+            kb[j] = key0[at - 1];
+        }
+#pragma unroll
+        for (int j = 0; j < 8; j++) out = out || kb[j] > k[j];
+    }
+    if (!__syncthreads_or(out)) return;
+    unsigned long long *ka = key0 + first, *kb = key1 + first;
+    uint32_t *va = val0 + first, *vb = val1 + first;
+    for (int s0 = 0; s0 < shift; s0 += RB) {  // (digits above the run's own bits agree: the last one may hold some)
+        if (threadIdx.x < R) sm.wcnt[threadIdx.x] = 0;  // where every digit starts
+        __syncthreads();
+        for (long long i = threadIdx.x; i < len; i += ST) atomicAdd(&sm.wcnt[(ka[i] >> s0) & (R - 1)], 1u);
+        __syncthreads();
+        uint32_t total;
+        const uint32_t e = block_excl_scan<ST>(threadIdx.x < R ? sm.wcnt[threadIdx.x] : 0u, &total, sm.scantmp);
+        if (threadIdx.x < R) sm.dstart[threadIdx.x] = e;
+        __syncthreads();
+        for (long long t0 = 0; t0 < len; t0 += TILE) {
+            for (int i = threadIdx.x; i < NW * R; i += ST) sm.wcnt[i] = 0;
+            __syncthreads();
+            const long long base = t0 + w * (32 * IPT);
+            const int m = (int)(len - base < 0 ? 0 : (len - base < 32 * IPT ? len - base : 32 * IPT));
+            unsigned long long k[IPT];
+            uint32_t v[IPT], loc[IPT];
+#pragma unroll
+            for (int j = 0; j < IPT; j++) {
+                const int i = 32 * j + lane;
+                k[j] = i < m ? ka[base + i] : 0ull;
+                v[j] = i < m ? va[base + i] : 0u;
+            }
+            gt_rank_keys<false, IPT>(k, s0, m, sm.wcnt + w * R, loc);
+            __syncthreads();
+            const uint32_t cnt = scan_warps(sm);
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < IPT; j++) {
+                if (32 * j + lane >= m) continue;
+                const uint32_t d = (uint32_t)(k[j] >> s0) & (R - 1);
+                const uint32_t pos = sm.dstart[d] + sm.wcnt[w * R + d] + loc[j];
+                kb[pos] = k[j];
+                vb[pos] = v[j];
+            }
+            __syncthreads();
+            if (threadIdx.x < R) sm.dstart[threadIdx.x] += cnt;
+            __syncthreads();
+        }
+        unsigned long long *kt = ka;
+        ka = kb;
+        kb = kt;
+        uint32_t *vt = va;
+        va = vb;
+        vb = vt;
+    }
+    if (ka != key0 + first)
+        for (long long i = threadIdx.x; i < len; i += ST) {
+            key0[first + i] = ka[i];
+            val0[first + i] = va[i];
+        }
+}
+
+// The listed tiles, a block each: from the first long run's first key to the last one's last, if it is at most TILE keys
+// on, in shared memory (runs that begin in a tile of FIX_TILE keys); a longer last run by itself.
 __device__ __forceinline__ void fix_long_runs_body(const unsigned bid, const unsigned nb, long long n, int shift,
         unsigned long long *key0, uint32_t *val0, unsigned long long *key1, uint32_t *val1,
         const uint32_t *__restrict__ list, DevCtl *ctl) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    unsigned long long *skey = (unsigned long long *)smraw;
-    uint32_t *sval = (uint32_t *)(skey + TILE);
-    uint32_t *wcnt = sval + TILE;      // NW x R
-    uint32_t *dstart = wcnt + NW * R;  // R: where the next key of every digit goes
-    uint32_t *scantmp = dstart + 2 * R;
-    __shared__ int sorted_sh;
-    __shared__ unsigned long long len_sh;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t runs = ctl->run_count;  // 0 if the whole keys were sorted
-    for (uint32_t r = bid; r < runs; r += nb) {
-        const long long first = list[r];
-        const unsigned long long k0 = key0[first];
-        if (threadIdx.x == 0) {
-            sorted_sh = 1;
-            len_sh = ~0ull;
+    static_assert(FIX_TILE <= TILE && TILE <= 65536, "the last run begins in the tile; 16-bit positions");
+    FixShared &sm = *(FixShared *)smraw;
+    const uint32_t tiles = ctl->run_count;  // 0 if the whole keys were sorted
+    for (uint32_t t = bid; t < tiles; t += nb) {
+        const long long first = list[2 * t];
+        const int last = (int)(list[2 * t + 1] - list[2 * t]);
+        const int room = n - first < TILE ? (int)(n - first) : TILE;
+        for (int i = threadIdx.x; i < room; i += ST) {
+            sm.key[i] = key0[first + i];
+            sm.val[i] = val0[first + i];
         }
         __syncthreads();
-        for (long long at = first;; at += ST) {  // the run's end, and whether its keys are in order
-            const long long i = at + threadIdx.x;
-            const bool in = i < n && same_run(k0, key0[i], shift);
-            if (!in) atomicMin(&len_sh, (unsigned long long)(i - first));
-            else if (i > first && key0[i - 1] > key0[i]) sorted_sh = 0;
-            __syncthreads();
-            const bool end = len_sh != ~0ull;
-            __syncthreads();
-            if (end) break;
+        const unsigned long long kl = sm.key[last];
+        int end = last + 1, no = room;  // the last run's end, by bisection: keys before `end` are before it
+        while (end < no) {
+            const int mid = (end + no) / 2;
+            if (same_run(kl, sm.key[mid], shift)) end = mid + 1;
+            else no = mid;
         }
-        const long long len = (long long)len_sh;
-        const bool sorted = sorted_sh != 0;
+        const bool open = end == room && first + room < n && same_run(kl, key0[first + room], shift);
+        sort_region(sm, open ? last : end, shift, key0 + first, val0 + first);
         __syncthreads();
-        if (sorted) continue;
-        unsigned long long *ka = key0 + first, *kb = key1 + first;
-        uint32_t *va = val0 + first, *vb = val1 + first;
-        const bool once = len <= RUN_SMEM;
-        for (int s0 = 0; s0 < shift; s0 += RB) {  // (digits above the run's own bits agree: the last one may hold some)
-            if (!once) {  // where every digit starts
-                if (threadIdx.x < R) wcnt[threadIdx.x] = 0;
-                __syncthreads();
-                for (long long i = threadIdx.x; i < len; i += ST) atomicAdd(&wcnt[(ka[i] >> s0) & (R - 1)], 1u);
-                __syncthreads();
-                uint32_t total;
-                const uint32_t c = threadIdx.x < R ? wcnt[threadIdx.x] : 0u;
-                const uint32_t e = block_excl_scan<ST>(c, &total, scantmp);
-                if (threadIdx.x < R) dstart[threadIdx.x] = e;
-                __syncthreads();
-            }
-            for (long long t0 = 0; t0 < len; t0 += TILE) {
-                for (int i = threadIdx.x; i < NW * R; i += ST) wcnt[i] = 0;
-                __syncthreads();
-                const long long base = t0 + w * (32 * IPT);
-                const int m = (int)(len - base < 0 ? 0 : (len - base < 32 * IPT ? len - base : 32 * IPT));
-                unsigned long long k[IPT];
-                uint32_t v[IPT], loc[IPT];
-#pragma unroll
-                for (int j = 0; j < IPT; j++) {
-                    const int i = 32 * j + lane;
-                    k[j] = 0ull;
-                    v[j] = 0u;
-                    if (i < m) {
-                        if (once && s0 > 0) {
-                            k[j] = skey[base + i];
-                            v[j] = sval[base + i];
-                        } else {
-                            k[j] = ka[base + i];
-                            v[j] = va[base + i];
-                        }
-                    }
-                }
-                gt_rank_keys<false, IPT>(k, s0, m, wcnt + w * R, loc);
-                __syncthreads();
-                uint32_t cnt = 0;
-                if (threadIdx.x < R)
-                    for (int ww = 0; ww < NW; ww++) {
-                        const uint32_t t = wcnt[ww * R + threadIdx.x];
-                        wcnt[ww * R + threadIdx.x] = cnt;
-                        cnt += t;
-                    }
-                if (once) {
-                    uint32_t total;
-                    const uint32_t e = block_excl_scan<ST>(cnt, &total, scantmp);
-                    if (threadIdx.x < R) dstart[threadIdx.x] = e;
-                }
-                __syncthreads();
-#pragma unroll
-                for (int j = 0; j < IPT; j++) {
-                    if (32 * j + lane >= m) continue;
-                    const uint32_t d = (uint32_t)(k[j] >> s0) & (R - 1);
-                    const uint32_t pos = dstart[d] + wcnt[w * R + d] + loc[j];
-                    if (once) {
-                        skey[pos] = k[j];
-                        sval[pos] = v[j];
-                    } else {
-                        kb[pos] = k[j];
-                        vb[pos] = v[j];
-                    }
-                }
-                __syncthreads();
-                if (!once && threadIdx.x < R) dstart[threadIdx.x] += cnt;
-                __syncthreads();
-            }
-            if (!once) {
-                unsigned long long *kt = ka;
-                ka = kb;
-                kb = kt;
-                uint32_t *vt = va;
-                va = vb;
-                vb = vt;
-            }
-        }
-        if (once) {
-            for (long long i = threadIdx.x; i < len; i += ST) {
-                key0[first + i] = skey[i];
-                val0[first + i] = sval[i];
-            }
-        } else if (ka != key0 + first) {
-            for (long long i = threadIdx.x; i < len; i += ST) {
-                key0[first + i] = ka[i];
-                val0[first + i] = va[i];
-            }
-        }
+        if (open) sort_long_run(sm, first + last, n, shift, key0, val0, key1, val1);
         __syncthreads();
     }
 }
 
-__global__ __launch_bounds__(ST) void k_fix_long_runs(long long n, int shift, unsigned long long *key0,
+__global__ __launch_bounds__(ST, 3) void k_fix_long_runs(long long n, int shift, unsigned long long *key0,
         uint32_t *val0, unsigned long long *key1, uint32_t *val1, const uint32_t *__restrict__ list, DevCtl *ctl) {
     gt_grid_ready();
     fix_long_runs_body(blockIdx.x, gridDim.x, n, shift, key0, val0, key1, val1, list, ctl);
@@ -411,8 +510,8 @@ __global__ __launch_bounds__(ST, GT_SORT_MINB) void kg_onesweep(const GroupedSys
                         s.sb.status + (size_t)pass * R * ntiles, ntiles, s.ctl);
 }
 
-__host__ __device__ inline unsigned fix_blocks(long long n, int nsm) { return gt_grid(n, 256, nsm * 16); }
-__host__ __device__ inline unsigned fix_long_blocks(long long n, int nsm) { return gt_grid(n, 4 * TILE, nsm); }
+__host__ __device__ inline unsigned fix_blocks(long long n, int nsm) { return gt_grid(n, FIX_TILE, nsm * 8); }
+__host__ __device__ inline unsigned fix_long_blocks(long long n, int nsm) { return gt_grid(n, TILE, nsm * 3); }
 
 __global__ __launch_bounds__(256) void kg_fix_runs(const GroupedSys *__restrict__ t, int shift, int nsm) {
     gt_grid_ready();
@@ -422,7 +521,7 @@ __global__ __launch_bounds__(256) void kg_fix_runs(const GroupedSys *__restrict_
         fix_runs_body(blockIdx.y, nb, s.n, shift, (unsigned long long *)s.sb.key[0], s.sb.val[0], s.sb.status, s.ctl);
 }
 
-__global__ __launch_bounds__(ST) void kg_fix_long_runs(const GroupedSys *__restrict__ t, int shift, int nsm) {
+__global__ __launch_bounds__(ST, 3) void kg_fix_long_runs(const GroupedSys *__restrict__ t, int shift, int nsm) {
     gt_grid_ready();
     const GroupedSys &s = t[blockIdx.x];
     const unsigned nb = fix_long_blocks(s.n, nsm);
@@ -441,8 +540,8 @@ void gt_sort_init() {
     for (auto kernel : {kg_onesweep<PASS_PLAIN>, kg_onesweep<PASS_LOW_FIRST>, kg_onesweep<PASS_LOW>,
                         kg_onesweep<PASS_HIGH_FIRST>})
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
-    cudaFuncSetAttribute(kg_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
-    cudaFuncSetAttribute(k_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+    cudaFuncSetAttribute(kg_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FIX_SMEM);
+    cudaFuncSetAttribute(k_fix_long_runs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FIX_SMEM);
 }
 
 namespace {
@@ -469,7 +568,7 @@ void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStrea
     uint32_t *list = b.status;  // the look-backs are over
     gt_launch(k_fix_runs, fix_blocks(n, nsm), 256, 0, st, n, shift, (unsigned long long *)b.key[0], b.val[0], list,
               ctl);
-    gt_launch(k_fix_long_runs, fix_long_blocks(n, nsm), ST, SCATTER_SMEM, st, n, shift,
+    gt_launch(k_fix_long_runs, fix_long_blocks(n, nsm), ST, FIX_SMEM, st, n, shift,
               (unsigned long long *)b.key[0], b.val[0], (unsigned long long *)b.key[1], b.val[1], list, ctl);
     gt_note_launches(2);
 }
@@ -596,6 +695,6 @@ void gt_grouped_sort(const GroupedSys *t, const GroupedPlan &p, int nsm, cudaStr
         gt_launch(kg_onesweep<PASS_PLAIN>, grid, ST, SCATTER_SMEM, st, t, q, gt_tree_digit_shift(q));
     const int shift = gt_tree_digit_shift(2);
     gt_launch(kg_fix_runs, dim3(p.count, fix_blocks(p.n_build, nsm)), 256, 0, st, t, shift, nsm);
-    gt_launch(kg_fix_long_runs, dim3(p.count, fix_long_blocks(p.n_build, nsm)), ST, SCATTER_SMEM, st, t, shift, nsm);
+    gt_launch(kg_fix_long_runs, dim3(p.count, fix_long_blocks(p.n_build, nsm)), ST, FIX_SMEM, st, t, shift, nsm);
     gt_note_launches(PASSES + 2);
 }

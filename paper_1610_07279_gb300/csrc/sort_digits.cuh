@@ -35,13 +35,25 @@ __device__ __forceinline__ void gt_count_digits(unsigned long long k, bool ok, u
     }
 }
 
+// Whether the tree's keys are sorted by all of their bits (eight passes) or by the highest 48 (six, and the runs of keys
+// that agree there put in order), from the six digits' counts, each the largest and the sum of squared shares:
+// - no run is longer than the smallest of the six largest counts.  From a hundredth of the keys on, the block that
+//   sorts the longest run by itself may take longer than two passes over all keys (2^24: ~0.7 ms, 0.29 ms).  (Uniform
+//   digits: 1/250 of 2^20 keys, 1/185 of 16384.)
+// - a key's run has about n times the product of the squares' sums keys, if the digits are independent.  For Plummer
+//   spheres of 2^17 to 2^22 with one particle so far off that the cells of level 16 hold several others, the estimate
+//   is 1.3 to 1.4 where a sixth of the tiles hold a run of more than 16 keys, 2.5 to 4.5 where half or more do, and at most
+//   0.2 where none do; below 10^-4 for the models.  From half of the tiles on, two passes are the faster way.
+constexpr float GT_RUN_SHARE = 0.01f, GT_RUN_MEAN = 2.0f;
+
 // The block's counts into the global ones; the last block to come turns them into every pass's digit starts (a
-// launch of its own for that took 7 to 8 us), resets the passes' tile tickets, and says whether the tree's keys crowd
-// into so small a part of the cube that they are sorted by all of their bits (n: the number of keys).
-constexpr int GT_CROWD_PASS = 3;  // the digit of levels 11 to 13
+// launch of its own for that took 7 to 8 us), resets the passes' tile tickets, and makes the choice above (n: the number
+// of keys).
 __device__ __forceinline__ void gt_finish_digits(unsigned nb, const uint32_t (*h)[GT_SORT_DIGITS], long long n,
                                                  uint32_t *hist, uint32_t *base, DevCtl *ctl) {
     __shared__ bool last;
+    __shared__ uint32_t most_sh[GT_SORT_PASSES];
+    __shared__ float squares_sh[GT_SORT_PASSES];
     __syncthreads();
     for (int p = 0; p < GT_SORT_PASSES; p++)
         if (h[p][threadIdx.x]) atomicAdd(&hist[p * GT_SORT_DIGITS + threadIdx.x], h[p][threadIdx.x]);
@@ -53,23 +65,41 @@ __device__ __forceinline__ void gt_finish_digits(unsigned nb, const uint32_t (*h
     __threadfence();
     static_assert(GT_SORT_DIGITS == 32 * GT_SORT_PASSES, "a warp per pass, eight digits per lane");
     const uint32_t p = threadIdx.x >> 5, lane = threadIdx.x & 31u;
+    const float share = 1.0f / (float)n;
     uint32_t v[8], sum = 0, most = 0;
+    float squares = 0.0f;
 #pragma unroll
     for (int j = 0; j < 8; j++) {
         v[j] = __ldcg(&hist[p * GT_SORT_DIGITS + 8 * lane + j]);
         sum += v[j];
         most = max(most, v[j]);
+        squares += (v[j] * share) * (v[j] * share);
     }
     most = __reduce_max_sync(0xffffffffu, most);
-    if (p == GT_CROWD_PASS && lane == 0) ctl->sort_whole = (long long)most * 16 >= n ? 1u : 0u;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) squares += __shfl_xor_sync(0xffffffffu, squares, o);
+    if (lane == 0) {
+        most_sh[p] = most;
+        squares_sh[p] = squares;
+    }
     uint32_t at = warp_incl_scan(sum) - sum;
 #pragma unroll
     for (int j = 0; j < 8; j++) {
         base[p * GT_SORT_DIGITS + 8 * lane + j] = at;
         at += v[j];
     }
+    __syncthreads();
     if (threadIdx.x < GT_SORT_PASSES) ctl->sort_ticket[threadIdx.x] = 0;
-    if (threadIdx.x == 0) ctl->digits_done = ctl->run_count = 0;
+    if (threadIdx.x == 0) {
+        uint32_t longest = 0xffffffffu;
+        float run = (float)n;
+        for (int k = 2; k < GT_SORT_PASSES; k++) {
+            longest = min(longest, most_sh[k]);
+            run *= squares_sh[k];
+        }
+        ctl->sort_whole = longest * share >= GT_RUN_SHARE || run >= GT_RUN_MEAN ? 1u : 0u;
+        ctl->digits_done = ctl->run_count = 0;
+    }
 }
 
 // Stable rank of a lane's digit among those that the warp has counted into cnt (a count per digit) and its lower
