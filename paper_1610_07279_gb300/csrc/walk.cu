@@ -41,6 +41,7 @@
 #include <math.h>
 
 #include "gt_internal.cuh"
+#include "walk_levels.cuh"
 #include "walk_list.cuh"
 
 namespace {
@@ -442,15 +443,6 @@ __device__ __forceinline__ void write_entries(const WalkArgs &a, const Batch &t,
     }
 }
 
-// Whether a force is so close to the threshold of a block-step level (|a|^2 / c^2 a power of 16) that the order of
-// its sums may decide: within 2^-17, some thirty times the rounding errors of the sums.
-__device__ __forceinline__ bool near_level(float4 f, float inv_c2) {
-    const float x = (f.x * f.x + f.y * f.y + f.z * f.z) * inv_c2;
-    const uint32_t b = __float_as_uint(x), e = b >> 23, m = b & 0x7fffffu;
-    if (e == 0u || e >= 255u) return false;
-    return (m < 64u && ((e - 127u) & 3u) == 0u) || (m >= 0x800000u - 64u && ((e - 126u) & 3u) == 0u);
-}
-
 // The members' sums, reduced over their lanes, to the caller's accelerations.  True (for the warp) if LEVELS, the walk
 // is one that chooses levels (inv_c2 > 0), and one of them is near a level's threshold.
 template <bool LEVELS, uint32_t MS>
@@ -472,7 +464,7 @@ __device__ __forceinline__ bool store_group(const WalkArgs &a, uint32_t a0, uint
             const float phi = fmaf(a.posm[i < a.n ? i : 0u].w, a.inv_eps, sum.w);
             const float4 f = make_float4(a.G * sum.x, a.G * sum.y, a.G * sum.z, a.G * phi);
             a.acc[k] = f;
-            if (LEVELS) near = near || near_level(f, a.inv_c2);
+            if (LEVELS) near = near || near_level((f.x * f.x + f.y * f.y + f.z * f.z) * a.inv_c2);
         }
     }
     return LEVELS && __any_sync(0xffffffffu, near);
@@ -586,9 +578,11 @@ __device__ __forceinline__ uint32_t particles_of_step(uint32_t first, uint32_t l
 // would overflow it, every chain of additions runs over the whole walk, and a second member has one lane.  Block
 // steps turn forces into discrete levels, and a particle whose |a| is within a rounding of a level's threshold
 // would get another step from any other order of the same sums (1 particle in 10^7 and step).  The groups of
-// such particles (near_level: 2 groups in 10^4) are walked a second time by this function, so that levels, and
-// with them the trajectories, don't depend on how walk_group arranges its sums.  As the only walk it would take 2.9 ms
-// against walk_group's 2.6 (every particle at 2^22).  lx: the warp's WARP_SM words of shared memory.
+// particles near a threshold (near_level: 2 groups in 10^4) are walked a second time by this function, so that their levels
+// don't depend on how walk_group arranges its sums; where a force's terms cancel so far that the rounding errors exceed
+// near_level's window, a level can still do so (walk_group's own order is fixed too: levels never depend on the teams or
+// on the run).  As the only walk it would take 2.9 ms against walk_group's 2.6 (every particle at 2^22).  lx: the warp's
+// WARP_SM words of shared memory.
 __device__ __noinline__ void walk_group_ordered(const WalkArgs &a, uint32_t g, uint32_t ngroups, float *lx, uint2 *q) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t qmask = gt_queue_ring(a.qcap) - 1u;
