@@ -204,7 +204,11 @@ GT_API int gt_build_tree(gt_system *sys, gt_stream stream);
  *   d_aold    n FP32 |a_old| by internal index (the acceleration MAC needs it),
  *             or NULL to use the system's own.
  *   d_acc     n_active x 4 FP32 output (ax, ay, az, potential), in d_active order.
- * Uses the current parameters' mac.  Requires a built tree. */
+ * Uses the current parameters' mac.  Requires a built tree.
+ * gt_start, gt_block_step and a server's requests form the sums of the groups with a force near a
+ * block-step level's threshold (within 2^-17 of it in |a|^2) in another order than this call and a
+ * batch do: the same interactions, other roundings.  A caller that passes this call's forces to
+ * gt_correct may therefore, for such a particle, choose another level than gt_block_step would. */
 GT_API int gt_accel_active(gt_system *sys, const uint32_t *d_active, int64_t n_active,
                     const float *d_aold, float *d_acc, gt_stream stream);
 
