@@ -11,6 +11,7 @@
 #include <utility>
 
 #include "gt_system.cuh"
+#include "in_place.h"
 
 static std::atomic<long long> g_launches{0};
 
@@ -347,18 +348,40 @@ void ph_sync_collect(gt_system *s, cudaStream_t st) {
 
 cudaStream_t S(gt_stream s) { return (cudaStream_t)s; }
 
-// Whether a caller's array can be read or written by a kernel in place of a copy into the system's scratch: memory
-// of this device (or managed), aligned for its elements.  Anything else is copied, as host memory is.
-bool in_place(const void *p, size_t align) {
-    if (!p || (uintptr_t)p % align) return false;
+// The driver's cuMemGetAddressRange, through the runtime (the library isn't linked against the driver's).
+typedef int (*AddressRange)(unsigned long long *base, size_t *size, unsigned long long p);
+AddressRange address_range() {
+    static const AddressRange fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (AddressRange)f;
+    }();
+    return fn;
+}
+
+// Whether a kernel can read or write the `bytes` of a caller's array in place of a copy into the system's scratch: memory
+// of this device (or managed), aligned for its elements, all of it inside one allocation.  Anything else is copied, as
+// host memory is.
+bool in_place(const void *p, size_t align, size_t bytes) {
+    if (!p) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
     int dev = -1;
-    return a.type == cudaMemoryTypeManaged ||
-           (a.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && a.device == dev);
+    MemoryAt m;
+    m.reachable = a.type == cudaMemoryTypeManaged ||
+                  (a.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && a.device == dev);
+    unsigned long long base = 0;
+    if (!m.reachable || !address_range() || address_range()(&base, &m.size, (unsigned long long)(uintptr_t)p)) return false;
+    m.base = (uintptr_t)base;
+    return covers_array(m, (uintptr_t)p, align, bytes);
 }
 
 // A1-A5 on FP32 positions posm_src (s->posm or the predicted s->posm_tmp): keys, sort,
@@ -438,7 +461,7 @@ void walk_all(gt_system *s, const float *aold, float4 *acc, int mac, bool levels
 }  // namespace
 
 // ---- helpers shared with the batch and the server ------------------------------
-bool gt_in_place(const void *p, size_t align) { return in_place(p, align); }
+bool gt_in_place(const void *p, size_t align, size_t bytes) { return in_place(p, align, bytes); }
 
 int gt_sys_check_params(const gt_params *p) { return check_params(p); }
 
@@ -731,7 +754,8 @@ int gt_set_state(gt_system *s, const double *p_pos, const double *p_vel, const f
     const int64_t n = s->n;
     State &t = s->st[0];
     if (n > 0) {
-        if (in_place(p_pos, 8) && in_place(p_vel, 8) && in_place(p_mass, 4)) {
+        const size_t N = (size_t)n;
+        if (in_place(p_pos, 8, N * 24) && in_place(p_vel, 8, N * 24) && in_place(p_mass, 4, N * 4)) {
             gt_launch_load_from(t, s->posm, n, p_pos, p_vel, p_mass, st);
         } else {
             if (cudaMemcpyAsync(s->scratch3, p_pos, (size_t)n * 24, cudaMemcpyDefault, st) != cudaSuccess) return GT_ECUDA;
@@ -885,7 +909,9 @@ int gt_set_integrator_state(gt_system *s, const uint8_t *p_level, const int64_t 
     const int L = s->prm.levels;
     State &t = s->st[0];
     if (n > 0) {
-        if (in_place(p_level, 1) && in_place(p_t0, 8) && in_place(p_aold, 4) && (!p_acc || in_place(p_acc, 16))) {
+        const size_t N = (size_t)n;
+        if (in_place(p_level, 1, N) && in_place(p_t0, 8, N * 8) && in_place(p_aold, 4, N * 4) &&
+            (!p_acc || in_place(p_acc, 16, N * 16))) {
             gt_launch_gather_resume(p_level, (const long long *)p_t0, p_aold, (const float4 *)p_acc, t, n, st);
         } else {
             // stage the caller-order arrays in scratch (24 B per particle is enough for 1+8+4 B)
@@ -1008,7 +1034,7 @@ int gt_get_state(gt_system *s, double *p_pos, double *p_vel, float *p_mass, floa
     double *to[2] = {p_pos, p_vel};
     for (int k = 0; k < 2; k++) {
         if (!to[k]) continue;
-        const bool direct = in_place(to[k], 8);
+        const bool direct = in_place(to[k], 8, (size_t)n * 24);
         gt_launch_interleave3(from[k][0], from[k][1], from[k][2], n, direct ? to[k] : s->scratch3, st);
         if (!direct && cudaMemcpyAsync(to[k], s->scratch3, (size_t)n * 24, cudaMemcpyDefault, st)) return GT_ECUDA;
     }

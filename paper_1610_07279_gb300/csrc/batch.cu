@@ -366,7 +366,8 @@ int gt_batch_get_acc(gt_batch *b, int k, float *p_acc, uint32_t *p_id, gt_stream
     gt_system *s = b->sys[k];
     cudaStream_t st = (cudaStream_t)stream;
     if (s->n > 0) {
-        if ((!p_acc || gt_in_place(p_acc, 16)) && (!p_id || gt_in_place(p_id, 4))) {  // one launch for both
+        const size_t n = (size_t)s->n;
+        if ((!p_acc || gt_in_place(p_acc, 16, 16 * n)) && (!p_id || gt_in_place(p_id, 4, 4 * n))) {  // one launch for both
             gt_launch_acc_out(s->acc_out, s->st[0].id, s->n, (float4 *)p_acc, p_id, st);
         } else {
             if (p_acc && cudaMemcpyAsync(p_acc, s->acc_out, (size_t)s->n * 16, cudaMemcpyDefault, st)) return GT_ECUDA;

@@ -108,8 +108,8 @@ struct gt_system {
 constexpr size_t GT_WS_ALIGN = 256;
 
 int gt_sys_check_params(const gt_params *p);
-// whether a kernel may take a caller's array in place (memory of this device, aligned)
-bool gt_in_place(const void *p, size_t align);
+// whether a kernel may take a caller's array in place (memory of this device, aligned, inside its allocation)
+bool gt_in_place(const void *p, size_t align, size_t bytes);
 int gt_sys_device_sms(int *dev, int *nsm);
 // Carve every buffer of a system out of base (or only measure when base == nullptr);
 // own_queue == false leaves the walk queue to the caller (a batch).
