@@ -1103,10 +1103,12 @@ int gt_sync_status(gt_system *s, gt_stream stream) {
     int err[2] = {0, 0};
     if (cudaStreamSynchronize(st) != cudaSuccess) return GT_ECUDA;
     if (cudaMemcpy(err, &s->ctl->err, sizeof(err), cudaMemcpyDeviceToHost) != cudaSuccess) return GT_ECUDA;
-    if (err[0]) {
-        const int zero[2] = {0, 0};
-        if (cudaMemcpy(&s->ctl->err, zero, sizeof(zero), cudaMemcpyHostToDevice) != cudaSuccess) return GT_ECUDA;
-    }
+    // A call that latched an error (a compaction whose wait ran out) may have left bits in the masks, which every call
+    // expects at zero: they are cleared with the error, before the stream's next call.
+    if (err[0] && (cudaMemsetAsync(&s->ctl->err, 0, sizeof(err), st) != cudaSuccess ||
+                   cudaMemsetAsync(s->flags, 0, (size_t)((char *)s->rank - (char *)s->flags), st) != cudaSuccess ||
+                   cudaStreamSynchronize(st) != cudaSuccess))
+        return GT_ECUDA;
     return err[0];
 }
 
