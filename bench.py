@@ -14,6 +14,8 @@ Reported: interactions/s of the whole job (value), seconds per block step, the
 end-to-end number through pinned host buffers, the walk kernel against the FP32
 roofline, clocks sampled during the timed region, and the CPU oracle timed on a
 bounded sample (rank 0, N = 1).  --impl reference times the CPU oracle instead.
+The accuracy sweeps' points and the batch's per-system errors go to standard error, as a
+JSON line of their own: with them the result line has 21 KB, which a reader of it may cut.
 
 Launch: python bench.py [--gpus N --steps K --warmup W]; for N > 1 under
 torch.distributed.run, one replica per GPU (the single system does not shard).
@@ -944,9 +946,27 @@ def run_ours(args):
                 "batch": batch, "serving": serving,
                 "gflops_paper_convention": {str(f): inter_all * f / (ms_max * 1e-3) / 1e9
                                             for f in (20, 24, 28, 38, round(fpi, 2))}}
+        line, tables = split_tables(line)
+        if tables:
+            print(json.dumps({"tables": tables}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()
+
+
+def split_tables(line: dict) -> tuple[dict, dict]:
+    """The result line without its long tables, and the tables."""
+    line, tables = dict(line), {}
+    if line.get("error"):
+        line["error"] = dict(line["error"])
+        if "sweeps_plummer_2p13" in line["error"]:
+            tables["sweeps_plummer_2p13"] = line["error"].pop("sweeps_plummer_2p13")
+    if (line.get("batch") or {}).get("error_vs_fp64_direct"):
+        errors = dict(line["batch"]["error_vs_fp64_direct"])
+        if "per_system" in errors:
+            tables["batch_errors_per_system"] = errors.pop("per_system")
+        line["batch"] = {**line["batch"], "error_vs_fp64_direct": errors}
+    return line, tables
 
 
 def main():
