@@ -57,7 +57,7 @@ struct DevCtl {
     int levels_m1;                    // L - 1 (finest level)
     unsigned int bbox[6];             // extrema of the positions (gt_ordered): minima, then maxima
     unsigned int digits_done;         // blocks that have added their digit counts (the sort)
-    unsigned int run_count;           // runs of equal sorted bits listed for k_fix_long_runs
+    unsigned int run_count;           // tiles of keys listed for k_fix_long_runs
     unsigned int sort_whole;          // the tree's keys are sorted by all of their bits in whole passes
     unsigned int scan_done, cells_done;  // the same for the octree's tile scan and the cell list's counts
     unsigned int spin_limit;          // bound on every spin-wait of this system; 0: GT_SPIN_LIMIT
@@ -380,9 +380,7 @@ void gt_launch_keys(const float4 *posm, int64_t n, int curve, DevCtl *ctl, SortB
 // box, keys and sort of at most GT_SMALL_SORT particles in one launch
 void gt_keys_init();
 void gt_launch_small_sort(const float4 *posm, int64_t n, int curve, SortBufs &b, cudaStream_t st);
-// sort.cu: gt_launch_sort sorts (key, val) in buffers 0; gt_launch_sort_tree the keys that gt_launch_keys made, with
-// their positions as values, into buffers 0
-void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st);
+// sort.cu: the keys that gt_launch_keys made, with their positions as values, sorted into buffers 0
 void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStream_t st);
 void gt_sort_init();
 // tree.cu

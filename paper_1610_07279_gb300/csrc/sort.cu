@@ -19,6 +19,8 @@
 // copy rate.  Tiles of 256 threads with 16 keys each leave fewer warps' counts to scan than 512 with 8 (154 us); builds
 // of 2^24 with tiles of 256 x 16, 256 x 14, 512 x 8, 384 x 12, 512 x 12 (two blocks per SM) and 512 x 10 (two): 2558,
 // 2585, 2629, 2652, 2608 and 2557 us; sorts of 1000001 keys: 155, 151, 155, 161, 170 and 157.
+#include <stddef.h>
+
 #include <mutex>
 
 #include "gt_internal.cuh"
@@ -573,35 +575,23 @@ void gt_launch_sort_tree(SortBufs &b, int64_t n, DevCtl *ctl, int nsm, cudaStrea
     gt_note_launches(2);
 }
 
-void gt_launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st) {
-    if (n <= 1) return;
-    cudaMemsetAsync(b.hist, 0, gt_sort_scratch_bytes(n), st);
-    int dev = 0, nsm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const long long blocks = (n + HT - 1) / HT;
-    k_hist_all<<<(unsigned)(blocks < nsm * 8 ? blocks : nsm * 8), HT, 0, st>>>(n, (const unsigned long long *)b.key[0],
-                                                                               b.hist, b.digit_base, ctl);
-    gt_note_launches(1);
-    for (int p = 0; p < PASSES; p++) onesweep<PASS_PLAIN>(b, n, ctl, p, RB * p, st);
-}
-
 // ---- sort without allocation (gt_sort_pairs_noalloc) -----------------------------
 // All scratch of one sort of up to GT_NOALLOC_SORT_MAX pairs lives in this array:
-// [control block | alternate keys | alternate values | digit counts | look-back status |
-// digit bases].  Host code must not use the symbol as an address: the device
+// [alternate keys | alternate values | digit bases | control block | digit counts |
+// look-back status].  Host code must not use the symbol as an address: the device
 // address is looked up once per device below.
 namespace {
 
 constexpr size_t NA_ALIGN = 256;
 constexpr size_t na_up(size_t b) { return (b + NA_ALIGN - 1) / NA_ALIGN * NA_ALIGN; }
 constexpr size_t NA_TILES = (GT_NOALLOC_SORT_MAX + TILE - 1) / TILE;
-constexpr size_t NA_OFF_KEY = na_up(sizeof(DevCtl));
-constexpr size_t NA_OFF_VAL = NA_OFF_KEY + na_up((size_t)GT_NOALLOC_SORT_MAX * sizeof(unsigned long long));
-constexpr size_t NA_OFF_HIST = NA_OFF_VAL + na_up((size_t)GT_NOALLOC_SORT_MAX * sizeof(uint32_t));
+constexpr size_t NA_OFF_VAL = na_up((size_t)GT_NOALLOC_SORT_MAX * sizeof(unsigned long long));
+constexpr size_t NA_OFF_BASE = NA_OFF_VAL + na_up((size_t)GT_NOALLOC_SORT_MAX * sizeof(uint32_t));
+constexpr size_t NA_OFF_CTL = NA_OFF_BASE + na_up(PASSES * R * sizeof(uint32_t));
+constexpr size_t NA_OFF_HIST = NA_OFF_CTL + na_up(sizeof(DevCtl));
 constexpr size_t NA_OFF_STATUS = NA_OFF_HIST + PASSES * R * sizeof(uint32_t);
-constexpr size_t NA_OFF_BASE = NA_OFF_STATUS + na_up(PASSES * R * NA_TILES * sizeof(uint32_t));
-constexpr size_t NA_BYTES = NA_OFF_BASE + na_up(PASSES * R * sizeof(uint32_t));
+constexpr size_t NA_BYTES = NA_OFF_STATUS + na_up(PASSES * R * NA_TILES * sizeof(uint32_t));
+static_assert(offsetof(DevCtl, err) < offsetof(DevCtl, digits_done), "a latched error is kept until it is read");
 
 __device__ __align__(256) unsigned char g_noalloc_sort_scratch[NA_BYTES];
 
@@ -627,6 +617,23 @@ int noalloc_scratch(char **out, bool *first_use) {
     return GT_OK;
 }
 
+// The control block lies right before the digit counts (b.hist): from its counter of finished blocks on, all is cleared
+// together, so that a sort doesn't depend on how an earlier one ended (one that another overlapped may leave the counter
+// off, and the digits' starts and the tiles' tickets would never be set again).
+void launch_sort(SortBufs &b, int64_t n, DevCtl *ctl, cudaStream_t st) {
+    if (n <= 1) return;
+    char *from = (char *)&ctl->digits_done;
+    cudaMemsetAsync(from, 0, (size_t)((char *)b.hist - from) + gt_sort_scratch_bytes(n), st);
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const long long blocks = (n + HT - 1) / HT;
+    k_hist_all<<<(unsigned)(blocks < nsm * 8 ? blocks : nsm * 8), HT, 0, st>>>(n, (const unsigned long long *)b.key[0],
+                                                                               b.hist, b.digit_base, ctl);
+    gt_note_launches(1);
+    for (int p = 0; p < PASSES; p++) onesweep<PASS_PLAIN>(b, n, ctl, p, RB * p, st);
+}
+
 }  // namespace
 
 extern "C" int gt_sort_pairs_noalloc(uint64_t *d_keys, uint32_t *d_vals, int64_t n, gt_stream stream) {
@@ -638,8 +645,8 @@ extern "C" int gt_sort_pairs_noalloc(uint64_t *d_keys, uint32_t *d_vals, int64_t
     if (rc != GT_OK) return rc;
     if (n <= 1) return GT_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    DevCtl *ctl = (DevCtl *)base;
-    // the histograms and the look-back status words are cleared by the sort itself; the
+    DevCtl *ctl = (DevCtl *)(base + NA_OFF_CTL);
+    // the histograms, the look-back status words and the counters are cleared by the sort itself; the
     // control block (tickets, error word) starts at zero once, on the first call on a
     // device, after which every call leaves it consistent for the next
     if (first_use) {
@@ -648,12 +655,12 @@ extern "C" int gt_sort_pairs_noalloc(uint64_t *d_keys, uint32_t *d_vals, int64_t
     SortBufs b;
     b.key[0] = d_keys;
     b.val[0] = d_vals;
-    b.key[1] = (uint64_t *)(base + NA_OFF_KEY);
+    b.key[1] = (uint64_t *)base;
     b.val[1] = (uint32_t *)(base + NA_OFF_VAL);
     b.status = (uint32_t *)(base + NA_OFF_STATUS);
     b.hist = (uint32_t *)(base + NA_OFF_HIST);
     b.digit_base = (uint32_t *)(base + NA_OFF_BASE);
-    gt_launch_sort(b, n, ctl, st);  // an even number of passes leaves the result in d_keys/d_vals
+    launch_sort(b, n, ctl, st);  // an even number of passes leaves the result in d_keys/d_vals
     return cudaGetLastError() == cudaSuccess ? GT_OK : GT_ECUDA;
 }
 
@@ -669,7 +676,7 @@ extern "C" int gt_sort_noalloc_status(gt_stream stream) {
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaStreamSynchronize(st) != cudaSuccess) return GT_ECUDA;
     if (!base) return GT_OK;  // no sort has run on this device
-    DevCtl *ctl = (DevCtl *)base;
+    DevCtl *ctl = (DevCtl *)(base + NA_OFF_CTL);
     int err = 0;
     if (cudaMemcpyAsync(&err, &ctl->err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
