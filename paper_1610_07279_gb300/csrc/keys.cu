@@ -15,7 +15,8 @@ namespace {
 
 constexpr int BBOX_THREADS = 256;
 // Blocks per SM of the key pass: every block adds up to 2048 counts to the global ones, which below ~2^22 keys costs
-// more than the warps hide (2^20: 407 us the whole build at 4, 413 at 8; 2^24: 3009 and 3001).
+// more than the warps hide (whole builds with 4 and with 8: 2^19 203 and 208 us, 2^20 291 and 302, 2^21 442 and 442, 2^22
+// 761 and 761; an earlier 2^24 3009 and 3001).
 constexpr int64_t KEYS_MANY = 1 << 22;
 
 __device__ __forceinline__ void bbox_body(const unsigned bid, const unsigned nb, const float4 *__restrict__ posm,

@@ -165,7 +165,9 @@ __global__ __launch_bounds__(BT) void k_build_level(int lvl, const unsigned long
 constexpr int FLAT_LWIN = GT_FLAT_LEAF_MAX;              // the largest leaf_max of this build
 constexpr int FB = 256;                    // threads per block
 // Particles per tile: a block takes its tile's rounds of FB particles one after another, so that small systems,
-// which fill few blocks, get short tiles (8192 particles: k_flat_scatter 15.6 us with 8 rounds).
+// which fill few blocks, get short tiles (8192 particles: k_flat_scatter 15.6 us with 8 rounds).  Whole builds with two
+// and with eight: 2^20 291 and 296 us, 2^20.5 355 and 352, 2^21 443 and 444, 2^21.5 562 and 562, 2^22 769 and 761, 2^23
+// 1423 and 1409.
 #ifndef GT_FLAT_SMALL
 #define GT_FLAT_SMALL (1 << 21)            // systems up to this size take tiles of two rounds, larger ones of eight
 #endif
@@ -578,7 +580,7 @@ __device__ __forceinline__ void pseudo_leaf(const Nodes &nd, const float4 *__res
     const uint32_t f = nd.first[c];
     const uint32_t k = nd.count[c];
     double m = WITH_MASS ? 0.0 : nd.sum[c].m, sx = 0.0, sy = 0.0, sz = 0.0;
-    // in particle order; the loads of four particles go out before their sums
+    // in particle order; the loads of PU particles go out before their sums
     // (m x is exact in FP64, so the fused form rounds once like + does)
     for (uint32_t i0 = f; i0 < f + k; i0 += PU) {
         float4 p[PU];
@@ -639,7 +641,7 @@ __device__ __forceinline__ CellInfo cell_info(const Nodes &nd, uint32_t p) {
 
 // Cell p with children: its children's FP64 sums added in child order.  The children
 // were written by other blocks of this launch: they are read through L2 (__ldcg), an
-// SM's L1 may hold a line of them from before they were written.  Loads go out four
+// SM's L1 may hold a line of them from before they were written.  Loads go out CU
 // children at a time, so a level costs few L2 round trips.
 template <bool WITH_MASS>
 __device__ __forceinline__ void pseudo_cell(const Nodes &nd, const CellInfo &ci) {

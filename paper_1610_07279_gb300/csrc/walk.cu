@@ -35,7 +35,9 @@
 // cycles, 4 rsqrt, 4 loads); the node records (32 B per cell) stay in L2.  80 registers and
 // 48 KB of shared memory at three blocks per SM; members and sums wait in shared memory
 // during the traversal (held in registers they spill, and a spilling force loop costs 15 %;
-// two blocks at 95 registers 12 % more time, four at 64 10 %).  The full walk of the
+// two blocks at 95 registers 12 % more time, four at 64 10 %).  What still spills is outside of
+// the force loop: 12 B of stores and 36 B of loads in k_walk (44 and 36 with levels, and 44 and 116
+// in walk_group_ordered), 64 and 116 in k_walk_batch.  The full walk of the
 // Andromeda-like model at 2^22, leaves of 32: 2.55 ms, 0.69 warp instructions per interaction
 // (3.03 ms and 0.81 with a queue of single cells).
 #include <math.h>
