@@ -499,13 +499,16 @@ __device__ __forceinline__ void cell_count_body(const unsigned bid, const unsign
     __syncthreads();
     if (threadIdx.x <= 2 * GT_TREE_LEVELS) ctl->seg[threadIdx.x] = seg[threadIdx.x];
     if (threadIdx.x >= 32) return;
-    // flat (a walk of it packs its batches): fewer than five children per cell, averaged over the levels
+    // flat (a walk of it packs its batches): fewer than five children per cell, and fewer than 4.5 averaged over the levels
     const int l = threadIdx.x;
     const uint32_t parents = l < GT_KEY_LEVELS ? seg[2 * l + 2] - seg[2 * l + 1] : 0u;
-    const uint32_t sixteenths = parents ? (uint32_t)(16ull * (seg[2 * l + 4] - seg[2 * l + 2]) / parents) : 0u;
-    const uint32_t all = __reduce_add_sync(0xffffffffu, sixteenths);
+    const uint32_t children = parents ? seg[2 * l + 4] - seg[2 * l + 2] : 0u;
+    const uint32_t sixteenths = parents ? (uint32_t)(16ull * children / parents) : 0u;
     const unsigned levels = __ballot_sync(0xffffffffu, parents != 0u);
-    if (l == 0) ctl->flat = all < 5u * 16u * __popc(levels) ? 1u : 0u;
+    const uint32_t by_level = __reduce_add_sync(0xffffffffu, sixteenths);
+    const uint32_t all_parents = __reduce_add_sync(0xffffffffu, parents);
+    const uint32_t all_children = __reduce_add_sync(0xffffffffu, children);
+    if (l == 0) ctl->flat = all_children < 5ull * all_parents && by_level < 72u * __popc(levels) ? 1u : 0u;
 }
 
 __global__ __launch_bounds__(256) void k_cell_count(Nodes nd, long long cap, DevCtl *ctl) {

@@ -355,10 +355,13 @@ __device__ __forceinline__ Take take_four(uint2 sib, uint32_t avail) {
 // cells have four children on a sheet and two on a filament, so that four entries would leave half or three quarters of
 // the lanes idle.  Every particle, with four entries and packed, us: a sheet of 2^20 (leaves of 4) 887 and 762, a line
 // 1144 and 720, a sheet of 2^22 3653 and 3102, a line 6048 and 3632; solid bodies gain nothing by it (a Plummer sphere of
-// 2^22, leaves of 16: 2489 and 2692).  The line lies at five children per cell, averaged over the levels: sheets have 4,
-// slabs of a hundredth of their width 4.6 to 4.9 (2^18, leaves of 4: 365 and 353), solid models with leaves of 4 and more
-// 5.9 to 8.  Both in one kernel would cost solid bodies 2 % (batches) to 3 % (registers, code), so each has its own, and
-// the one that isn't meant ends at once (1 to 3 us a call).
+// 2^22, leaves of 16: 2489 and 2692), nor do filaments and slabs that are solid at the scale of the groups (2^18, a
+// hundredth thick, leaves of 16: 1361 and 1480, 354 and 356).  So a tree is flat if its cells have fewer than five children,
+// on average over all cells (sheets up to 4, slabs of a thousandth at 2^22 4.3, thicker ones and filaments 5 to 8) and
+// fewer than 4.5 on average over the levels (solid models with leaves of one or two particles have 3 to 4.3 over all
+// cells, most of which are the last two levels', but 4.5 and more over the levels from 2^16 on).  Both in one kernel would
+// cost solid bodies 2 % (batches) to 3 % (registers, code), so each has its own, and the one that isn't meant ends at
+// once (1 to 3 us a call).
 __device__ __forceinline__ Take take_packed(const uint2 *q, uint32_t head, uint32_t avail, uint32_t qmask) {
     const uint32_t lane = threadIdx.x & 31u;
     const unsigned FULL = 0xffffffffu;
