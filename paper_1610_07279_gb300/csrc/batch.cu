@@ -58,7 +58,7 @@ size_t plan(int nsys, const int64_t *n, const gt_params *prm, int n_prm, int nsm
     off = align_up(off + (size_t)nsys * sizeof(WalkArgs));
     off = align_up(off + (size_t)nsys * sizeof(DevCtl *));
     off = align_up(off + 2 * (size_t)(nsys + 1) * sizeof(uint32_t));
-    off = align_up(off + 2 * sizeof(unsigned int));
+    off = align_up(off + 4 * sizeof(unsigned int));
     off = align_up(off + 2 * (size_t)nsys * sizeof(GroupedSys));
     off = align_up(off + warps * gt_queue_words(qcap) * sizeof(uint32_t));
     if (member_bytes) member_bytes->clear();
@@ -230,7 +230,7 @@ int gt_batch_create(gt_batch **out, int nsys, const int64_t *n, const gt_params 
     b->d_gprefix = (uint32_t *)(base + off);
     off = align_up(off + 2 * (size_t)(nsys + 1) * sizeof(uint32_t));
     b->d_next = (unsigned int *)(base + off);
-    off = align_up(off + 2 * sizeof(unsigned int));
+    off = align_up(off + 4 * sizeof(unsigned int));
     for (int j = 0; j < 2; j++) b->d_tab[j] = (GroupedSys *)(base + off) + (size_t)j * nsys;
     off = align_up(off + 2 * (size_t)nsys * sizeof(GroupedSys));
     const size_t warps = (size_t)b->walk_blocks * (size_t)gt_walk_warps_per_block();

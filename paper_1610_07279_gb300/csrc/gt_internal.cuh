@@ -491,7 +491,7 @@ extern "C" int gt_rebuild_interval(const double *t_walk, int n, double t_make, i
 int gt_walk_warps_per_block();
 void gt_launch_walk(const WalkArgs &a, int nblocks, cudaStream_t st);
 // one launch over the groups of nsys systems, and one over those with flat trees (args, ctls: device arrays of nsys
-// entries; gprefix: 2 (nsys + 1) words, group_next: two); all_acc: every
+// entries; gprefix: 2 (nsys + 1) words, group_next: four); all_acc: every
 // system uses the acceleration MAC; levels: some have inv_c2 > 0
 void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, uint32_t *gprefix,
                           unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, bool levels,

@@ -327,7 +327,7 @@ int gt_server_create(gt_server **out, size_t hbm_cap, int max_slots, int walk_qu
     const size_t o_tctl = off; off = align_up(off + (size_t)max_slots * sizeof(DevCtl *));
     const size_t o_ent = off; off = align_up(off + 2 * (size_t)max_slots * sizeof(GroupedSys));
     const size_t o_gpre = off; off = align_up(off + 2 * (size_t)(max_slots + 1) * sizeof(uint32_t));
-    const size_t o_next = off; off = align_up(off + 2 * sizeof(unsigned int));
+    const size_t o_next = off; off = align_up(off + 4 * sizeof(unsigned int));
     const size_t o_queue = off; off = align_up(off + warps * gt_queue_words(walk_queue) * sizeof(uint32_t));
     if (off > hbm_cap) { delete v; return GT_ENOMEM; }
     v->region = alloc_fn(off, ctx);

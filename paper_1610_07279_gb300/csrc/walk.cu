@@ -40,6 +40,7 @@
 // in walk_group_ordered), 64 and 116 in k_walk_batch.  The full walk of the
 // Andromeda-like model at 2^22, leaves of 32: 2.55 ms, 0.69 warp instructions per interaction
 // (3.03 ms and 0.81 with a queue of single cells).
+#include <limits.h>
 #include <math.h>
 
 #include "gt_internal.cuh"
@@ -964,9 +965,11 @@ __device__ __forceinline__ bool team_group(const WalkArgs &a, uint32_t g, uint32
 // FLAT: a team's batches are four entries of each warp, which on flat trees leaves half or more of its lanes idle, so
 // teams end earlier.  Calls with T = 1, 2, 4, 8: lines, 373 groups 63, 78, 65, 56; 754 groups 70, 93, 69, 87; 1524 groups
 // 76, 108, 113, -; sheets, 256 groups 62, 62, 50, 47; 1024 groups 75, 77, 68, -; 2386 groups 107, 113, 117, -.
-template <bool FLAT>
-__device__ __forceinline__ uint32_t team_of(uint32_t ngroups, uint32_t warps) {
-    if (FLAT) return ngroups > warps / 3u ? 1u : (ngroups > warps / 8u ? 4u : 8u);
+// A queue that is depth-first from the start (qcap) has a team hand every group back to one warp, the others idle: no
+// teams.  65536 particles of a Plummer sphere, 3618 groups, a queue of 4096: 162 with teams, 115 without.
+__device__ __forceinline__ uint32_t team_of(bool flat, uint32_t ngroups, uint32_t warps, int qcap) {
+    if (qcap <= LIFO_ROOM) return 1u;
+    if (flat) return ngroups > warps / 3u ? 1u : (ngroups > warps / 8u ? 4u : 8u);
     return ngroups > 2u * warps ? 1u : (ngroups > warps ? 2u : (ngroups > warps / 4u ? 4u : 8u));
 }
 
@@ -994,7 +997,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk(const __grid_constant
     const uint32_t na = a.ctl->n_active;
     const uint32_t gmax = (uint32_t)a.gmax;
     const uint32_t ngroups = a.gstart ? a.ctl->n_groups : (na + gmax - 1) / gmax;
-    const uint32_t T = team_of<FLAT>(ngroups, gridDim.x * NWARP), team = warp / T, first = team * T;
+    const uint32_t T = team_of(FLAT, ngroups, gridDim.x * NWARP, a.qcap), team = warp / T, first = team * T;
     uint2 *q = (uint2 *)a.queue + (size_t)(blockIdx.x * NWARP + first) * gt_queue_ring(a.qcap);
     unsigned long long *stat = stat_sm[warp];
     if (lane < 2) stat[lane] = 0;
@@ -1044,7 +1047,7 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     const uint32_t total = gprefix[nsys];
     if (FLAT && !total) return;
-    const uint32_t T = team_of<FLAT>(total, gridDim.x * NWARP), team = warp / T, first = team * T;
+    const uint32_t T = group_next[2], team = warp / T, first = team * T;  // (k_batch_prefix)
     uint2 *q = (uint2 *)queue + (size_t)(blockIdx.x * NWARP + first) * gt_queue_ring(qcap);
     unsigned long long *stat = stat_sm[warp];
     const WalkArgs &a = sargs[warp];
@@ -1102,13 +1105,15 @@ __global__ __launch_bounds__(WT, GT_WALK_MINB) void k_walk_batch(const WalkArgs 
 }
 
 // gprefix over the group counts of the systems whose trees aren't flat, and behind it over those of the others (a warp
-// each; also resets the two counters)
+// each; also resets the two counters and chooses the teams' sizes, behind them)
 __global__ __launch_bounds__(64) void k_batch_prefix(DevCtl *const *__restrict__ ctls, const WalkArgs *__restrict__ args,
-                                                     int nsys, uint32_t *gprefix, unsigned int *group_next) {
+                                                     int nsys, uint32_t *gprefix, unsigned int *group_next,
+                                                     uint32_t walk_warps) {
     gt_grid_ready();
     const int lane = threadIdx.x & 31, kind = threadIdx.x >> 5;
     gprefix += kind * (nsys + 1);
     uint32_t carry = 0;
+    int qcap = INT_MAX;  // the smallest queue
     for (int s0 = 0; s0 < nsys; s0 += 32) {
         const int s = s0 + lane;
         uint32_t ng = 0;
@@ -1117,14 +1122,17 @@ __global__ __launch_bounds__(64) void k_batch_prefix(DevCtl *const *__restrict__
             const uint32_t na = c->n_active;
             const uint32_t gm = (uint32_t)args[s].gmax;
             if ((c->flat != 0u) == (kind == 1)) ng = args[s].gstart ? c->n_groups : (na + gm - 1) / gm;
+            if (ng) qcap = min(qcap, args[s].qcap);
         }
         const uint32_t incl = warp_incl_scan(ng);
         if (s < nsys) gprefix[s] = carry + incl - ng;
         carry += __shfl_sync(0xffffffffu, incl, 31);
     }
+    qcap = __reduce_min_sync(0xffffffffu, qcap);
     if (lane == 0) {
         gprefix[nsys] = carry;
         group_next[kind] = 0u;
+        group_next[2 + kind] = team_of(kind == 1, carry, walk_warps, qcap);
     }
 }
 
@@ -1153,7 +1161,7 @@ void gt_launch_walk_batch(DevCtl *const *ctls, const WalkArgs *args, int nsys, u
                           unsigned int *group_next, uint32_t *queue, int qcap, int mac, bool all_acc, bool levels,
                           int nblocks, cudaStream_t st) {
     if (nsys <= 0) return;
-    { k_batch_prefix<<<1, 64, 0, st>>>(ctls, args, nsys, gprefix, group_next); gt_note_launches(1); }
+    { k_batch_prefix<<<1, 64, 0, st>>>(ctls, args, nsys, gprefix, group_next, (uint32_t)(nblocks * NWARP)); gt_note_launches(1); }
     constexpr int ACC = GT_MAC_ACCELERATION;
     const bool acc = all_acc && mac < 0;
     auto launch = [&](auto kernel, int kind) {
